@@ -19,7 +19,7 @@ LIB = os.path.join(BUILD, "libpf.so")
 SOURCES = ["pf_zelastic.cu", "pf_zfwd.cu", "pf_ypass.cu", "pf_xpass_f32.cu", "pf_xpass_f64.cu",
            "pf_zfinal_f64.cu", "pf_zstage_f64.cu", "pf_fno.cu", "pf_api.cu", "pf_misc.cu",
            "pf_plan.cu", "pf_noalloc.cu", "pf_hc.cu", "pf_zelastic_unf.cu",
-           "pf_zelastic_cl.cu"]
+           "pf_zelastic_cl.cu", "pf_fno_fused.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

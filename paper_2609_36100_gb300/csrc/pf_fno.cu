@@ -9,11 +9,13 @@
 //                     z = V_l a_l + v_l + s,  a_{l+1} = GELU(z) (not after the last layer)
 //   h = GELU(Q1 a_L + q1), out = Q2 h + q2
 //
-// Truncated transforms and their adjoints are small dense contractions along
-// one axis (kernel k_axis with precomputed complex matrices).  The per-mode
-// channel mix is a batch-1 32x32 complex matvec per retained mode: it streams
-// the weights once per pass (weight-bandwidth bound), so it runs on CUDA cores
-// from BF16 storage rather than through the tensor cores.
+// Two paths.  In BF16 mode, for the sizes fno_fused_ok names, the layers run
+// in the fused kernels of pf_fno_fused.cu.  Everything else (the FP32 checking
+// mode, wider channels or more modes, short or very long rows) runs the
+// kernels of this file, one operation each: truncated transforms and their
+// adjoints as small dense contractions along one axis (k_axis with
+// precomputed complex matrices), the per-mode channel mix as a batch-1 complex
+// matvec per retained mode.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -23,6 +25,7 @@
 #include <vector>
 
 #include "pf.h"
+#include "pf_fno.cuh"
 #include "pf_internal.h"
 
 using namespace pf;
@@ -42,11 +45,6 @@ struct FnoDims {
 // ---------------------------------------------------------------------------
 // kernels
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_g(float z) {
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
-}
-
 // out[o][k][i] (=|+=) sum_j M[k][j] in[o][j][i]; complex M [nk][nj]
 template <bool IN_REAL, bool OUT_REAL, bool ACCUM>
 __global__ void k_axis(const void* __restrict__ inp, void* __restrict__ outp, const float2* __restrict__ M, int nk,
@@ -86,17 +84,19 @@ __global__ void k_axis(const void* __restrict__ inp, void* __restrict__ outp, co
     }
 }
 
-// spectral weight (re, im) of mode k, row c, column d
-__device__ __forceinline__ float2 wget(const float2* w32, const __nv_bfloat162* w16, long long e) {
+// spectral weight (re, im) of mode k, row c, column d.  Spectral weights and
+// their gradients start at an odd float of the parameter vector when C is odd,
+// so (re, im) pairs are read and written as two floats.
+__device__ __forceinline__ float2 wget(const float* w32, const __nv_bfloat162* w16, long long e) {
     if (w16) {
         const __nv_bfloat162 b = w16[e];
         return make_float2(__bfloat162float(b.x), __bfloat162float(b.y));
     }
-    return w32[e];
+    return make_float2(w32[2 * e], w32[2 * e + 1]);
 }
 
 // O[c][k] = sum_d W[k][c][d] A[d][k]
-__global__ void k_mix(const float2* __restrict__ A, float2* __restrict__ O, const float2* __restrict__ w32,
+__global__ void k_mix(const float2* __restrict__ A, float2* __restrict__ O, const float* __restrict__ w32,
                       const __nv_bfloat162* __restrict__ w16, int C, int K) {
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < (long long)C * K;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -116,7 +116,7 @@ __global__ void k_mix(const float2* __restrict__ A, float2* __restrict__ O, cons
 // backward of the mix: GA[d][k] = sum_c conj(W[k][c][d]) GO[c][k];
 // GW[k][c][d] = GO[c][k] conj(A[d][k])
 __global__ void k_mix_bwd(const float2* __restrict__ GO, const float2* __restrict__ A, float2* __restrict__ GA,
-                          float2* __restrict__ GW, const float2* __restrict__ w32,
+                          float* __restrict__ GW, const float* __restrict__ w32,
                           const __nv_bfloat162* __restrict__ w16, int C, int K) {
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < (long long)C * K;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -129,7 +129,8 @@ __global__ void k_mix_bwd(const float2* __restrict__ GO, const float2* __restric
             const float2 g = GO[(long long)c * K + k];
             ar += w.x * g.x + w.y * g.y;  // conj(w) g
             ai += w.x * g.y - w.y * g.x;
-            GW[e] = make_float2(g.x * a.x + g.y * a.y, g.y * a.x - g.x * a.y);  // g conj(a)
+            GW[2 * e] = g.x * a.x + g.y * a.y;  // g conj(a)
+            GW[2 * e + 1] = g.y * a.x - g.x * a.y;
         }
         GA[idx] = make_float2(ar, ai);
     }
@@ -258,9 +259,9 @@ __global__ void k_adam(float* __restrict__ th, const float* __restrict__ g, floa
     }
 }
 
-__global__ void k_to_bf16(const float2* __restrict__ w, __nv_bfloat162* __restrict__ o, long long n) {
+__global__ void k_to_bf16(const float* __restrict__ w, __nv_bfloat162* __restrict__ o, long long n) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        o[i] = __floats2bfloat162_rn(w[i].x, w[i].y);
+        o[i] = __floats2bfloat162_rn(w[2 * i], w[2 * i + 1]);
 }
 
 // real-space state (FP64, [4][N]) -> normalised FP32 network input
@@ -367,28 +368,6 @@ __global__ void k_wrms_dist(const double* __restrict__ a, const double* __restri
 // cost the weights' and activations' FP32 copies no accuracy beyond the BF16
 // spectral weights of this mode.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// two FP32 values -> their BF16 leading parts packed (first value in the low
-// half) and the BF16 roundings of their remainders
-__device__ __forceinline__ void split2(float x0, float x1, unsigned& hi, unsigned& lo) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
-    const __nv_bfloat162 l = __floats2bfloat162_rn(x0 - __bfloat162float(h.x), x1 - __bfloat162float(h.y));
-    hi = *reinterpret_cast<const unsigned*>(&h);
-    lo = *reinterpret_cast<const unsigned*>(&l);
-}
-__device__ __forceinline__ void mma3(float (&d)[4], const unsigned (&ah)[4], const unsigned (&al)[4], unsigned bh0,
-                                     unsigned bh1, unsigned bl0, unsigned bl1) {
-    mma_bf16_16816(d, ah, bh0, bh1);
-    mma_bf16_16816(d, ah, bl0, bl1);
-    mma_bf16_16816(d, al, bh0, bh1);
-}
-
 constexpr int kMmaWarps = 4;
 
 // y[m][p] = act(sum_k W'[m][k] x[k][p] + bias[m] (+ add[m][p])), W' = W (M x K
@@ -567,6 +546,8 @@ struct pf_fno {
     double* realbuf = nullptr;  // real-space FP64 state [4][N]: the proposal
     double* realbuf2 = nullptr; // real-space FP64 state [4][N]: the verified integration
     float* tgt = nullptr;       // training target [4][N]
+    bool fused = false;         // the kernels of pf_fno_fused.cu (chosen at creation)
+    FnoTables tab;
     char err[256] = "no error";
 };
 
@@ -593,7 +574,8 @@ cudaError_t falloc(P** p, size_t bytes) {
 void fno_free(pf_fno* f) {
     void* ps[] = {f->theta, f->grad, f->am, f->av, f->wbf, f->Mx, f->Mxw, f->My, f->Mz, f->IXw, f->IX1, f->IY,
                   f->IZ, f->x, f->act, f->zs, f->hpre, f->hh, f->out, f->Ak, f->T1, f->T2, f->Ok, f->Gk,
-                  f->sbuf, f->da, f->dz, f->dh, f->dout, f->part, f->dpart, f->realbuf, f->realbuf2, f->tgt};
+                  f->sbuf, f->da, f->dz, f->dh, f->dout, f->part, f->dpart, f->realbuf, f->realbuf2, f->tgt,
+                  f->tab.xc, f->tab.xs, f->tab.xcw, f->tab.xsw, f->tab.y, f->tab.z};
     for (void* p : ps) cudaFree(p);
     if (f->hsum) cudaFreeHost(f->hsum);
 }
@@ -698,11 +680,65 @@ void dense_t(pf_fno* f, const float* dy, float* dx, const float* Mw, int A, int 
     k_dense_t<<<grid_for(f->d.N), kT, sm, f->s>>>(dy, dx, Mw, A, B, f->d.N, accum);
 }
 
-int fno_forward(pf_fno* f, const float* x) {
+FnoFusedDims fused_dims(const FnoDims& d) { return {d.nx, d.ny, d.nz, d.C, d.m, d.H, d.L, d.N}; }
+FnoWork fused_work(const pf_fno* f) { return {f->T1, f->T2, f->Ok, f->Gk, f->part, f->dpart}; }
+
+int fused_forward(pf_fno* f, float* out) {
+    const FnoDims& d = f->d;
+    const FnoFusedDims fd = fused_dims(d);
+    const FnoWork w = fused_work(f);
+    const float *th = f->theta, *P = th + f->oP, *p = th + f->op;
+    cudaError_t e = fno_row_lift(fd, f->tab, w, f->x, P, p, f->s);
+    for (int l = 0; l < d.L && e == cudaSuccess; ++l) {
+        const float* zprev = l ? f->zs + (size_t)(l - 1) * d.C * d.N : nullptr;
+        e = fno_spectral_fwd(fd, f->tab, w, f->Ak + (size_t)l * d.C * d.K, f->wbf + (size_t)l * f->nW, f->s);
+        if (e == cudaSuccess)
+            e = fno_row_layer(fd, f->tab, w, zprev, f->x, P, p, th + f->oV[l], th + f->ov[l],
+                              f->zs + (size_t)l * d.C * d.N, l == d.L - 1, f->s);
+    }
+    if (e == cudaSuccess && out)
+        e = fno_project(fd, f->zs + (size_t)(d.L - 1) * d.C * d.N, th + f->oQ1, th + f->oq1, th + f->oQ2,
+                        th + f->oq2, out, f->s);
+    return e == cudaSuccess ? PF_OK : ffail(f, PF_ECUDA, "fno forward", e);
+}
+
+int fused_backward(pf_fno* f, const float* tgt, double* loss) {
+    const FnoDims& d = f->d;
+    const FnoFusedDims fd = fused_dims(d);
+    const FnoWork w = fused_work(f);
+    const float* th = f->theta;
+    float* G = f->grad;
+    int nb = 0;
+    cudaError_t e = fno_project_bwd(fd, w, f->zs + (size_t)(d.L - 1) * d.C * d.N, tgt, th + f->oQ1, th + f->oq1,
+                                    th + f->oQ2, th + f->oq2, f->dz, G + f->oQ1, G + f->oq1, G + f->oQ2, G + f->oq2,
+                                    &nb, f->s);
+    if (e == cudaSuccess) e = fno_row_raw(fd, f->tab, w, f->dz, f->s);
+    for (int l = d.L - 1; l >= 0 && e == cudaSuccess; --l) {
+        const float* zprev = l ? f->zs + (size_t)(l - 1) * d.C * d.N : nullptr;
+        e = fno_spectral_bwd(fd, f->tab, w, f->Ak + (size_t)l * d.C * d.K, f->wbf + (size_t)l * f->nW,
+                             reinterpret_cast<float2*>(G + f->oW[l]), f->s);
+        if (e == cudaSuccess)
+            e = fno_row_layer_bwd(fd, f->tab, w, f->dz, zprev, f->x, th + f->oP, th + f->op, th + f->oV[l],
+                                  G + f->oV[l], G + f->ov[l], G + f->oP, G + f->op, f->s);
+    }
+    if (e == cudaSuccess && loss) {
+        double* tot = f->dpart + nb;
+        launch_reduce(f->dpart, nb, 1.0 / (4.0 * (double)d.N), tot, f->s);
+        e = cudaMemcpyAsync(f->hsum, tot, sizeof(double), cudaMemcpyDeviceToHost, f->s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(f->s);
+        if (e == cudaSuccess) *loss = f->hsum[0];
+    }
+    if (e == cudaSuccess) e = cudaGetLastError();
+    return e == cudaSuccess ? PF_OK : ffail(f, PF_ECUDA, "fno backward", e);
+}
+
+// forward pass of x; `out` null: only what the backward pass reads
+int fno_forward(pf_fno* f, const float* x, float* out) {
     const FnoDims& d = f->d;
     const long long N = d.N;
     cudaStream_t s = f->s;
     if (x != f->x) cudaMemcpyAsync(f->x, x, sizeof(float) * 4 * N, cudaMemcpyDeviceToDevice, s);
+    if (f->fused) return fused_forward(f, out);
     float* a0 = f->act;
     dense(f, f->x, a0, nullptr, f->theta + f->oP, f->theta + f->op, nullptr, d.C, d.cin, 0);
     for (int l = 0; l < d.L; ++l) {
@@ -710,7 +746,7 @@ int fno_forward(pf_fno* f, const float* x) {
         float* an = f->act + (size_t)(l + 1) * d.C * N;
         float2* A = f->Ak + (size_t)l * d.C * d.K;
         trunc_dft(f, a, A, f->Mx);
-        const float2* w32 = reinterpret_cast<const float2*>(f->theta + f->oW[l]);
+        const float* w32 = f->theta + f->oW[l];
         const __nv_bfloat162* w16 = f->bf16 ? f->wbf + (size_t)l * f->nW : nullptr;
         k_mix<<<grid_for((long long)d.C * d.K), kT, 0, s>>>(A, f->Ok, w32, w16, d.C, d.K);
         trunc_inv(f, f->Ok, f->sbuf, f->IXw, false);
@@ -720,11 +756,13 @@ int fno_forward(pf_fno* f, const float* x) {
     float* aL = f->act + (size_t)d.L * d.C * N;
     dense(f, aL, f->hh, f->hpre, f->theta + f->oQ1, f->theta + f->oq1, nullptr, d.H, d.C, 1);
     dense(f, f->hh, f->out, nullptr, f->theta + f->oQ2, f->theta + f->oq2, nullptr, d.cin, d.H, 0);
+    if (out && out != f->out) cudaMemcpyAsync(out, f->out, sizeof(float) * 4 * N, cudaMemcpyDeviceToDevice, s);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PF_OK : ffail(f, PF_ECUDA, "fno forward", e);
 }
 
 int fno_backward(pf_fno* f, const float* tgt, double* loss) {
+    if (f->fused) return fused_backward(f, tgt, loss);
     const FnoDims& d = f->d;
     const long long N = d.N;
     cudaStream_t s = f->s;
@@ -749,10 +787,10 @@ int fno_backward(pf_fno* f, const float* tgt, double* loss) {
         dense_t(f, f->dz, f->da, f->theta + f->oV[l], d.C, d.C, 0);
         // spectral: GO = (w/N) F(dz); GW, GA; da += Re F^-1 (GA) (unweighted)
         trunc_dft(f, f->dz, f->Gk, f->Mxw);
-        const float2* w32 = reinterpret_cast<const float2*>(f->theta + f->oW[l]);
+        const float* w32 = f->theta + f->oW[l];
         const __nv_bfloat162* w16 = f->bf16 ? f->wbf + (size_t)l * f->nW : nullptr;
         float2* A = f->Ak + (size_t)l * d.C * d.K;
-        k_mix_bwd<<<grid_for((long long)d.C * d.K), kT, 0, s>>>(f->Gk, A, f->Ok, reinterpret_cast<float2*>(G + f->oW[l]),
+        k_mix_bwd<<<grid_for((long long)d.C * d.K), kT, 0, s>>>(f->Gk, A, f->Ok, G + f->oW[l],
                                                                 w32, w16, d.C, d.K);
         trunc_inv(f, f->Ok, f->da, f->IX1, true);
     }
@@ -772,7 +810,7 @@ int fno_backward(pf_fno* f, const float* tgt, double* loss) {
 
 void refresh_bf16(pf_fno* f) {
     for (int l = 0; l < f->d.L; ++l)
-        k_to_bf16<<<grid_for(f->nW), kT, 0, f->s>>>(reinterpret_cast<const float2*>(f->theta + f->oW[l]),
+        k_to_bf16<<<grid_for(f->nW), kT, 0, f->s>>>(f->theta + f->oW[l],
                                                    f->wbf + (size_t)l * f->nW, f->nW);
 }
 
@@ -874,44 +912,57 @@ int pf_fno_create(int nx, int ny, int nz, int C, int modes, int H, int L, int bf
     A(&f->am, sizeof(float) * f->npar);
     A(&f->av, sizeof(float) * f->npar);
     A(&f->wbf, sizeof(__nv_bfloat162) * f->nW * L);
+    f->fused = bf16 && fno_fused_ok(fused_dims(d));
     A(&f->x, sizeof(float) * 4 * N);
-    A(&f->act, sizeof(float) * (size_t)(L + 1) * C * N);
     A(&f->zs, sizeof(float) * (size_t)L * C * N);
-    A(&f->hpre, sizeof(float) * (size_t)H * N);
-    A(&f->hh, sizeof(float) * (size_t)H * N);
     A(&f->out, sizeof(float) * 4 * N);
     A(&f->Ak, sizeof(float2) * (size_t)L * C * d.K);
     A(&f->T1, sizeof(float2) * (size_t)C * nz * ny * modes);
     A(&f->T2, sizeof(float2) * (size_t)C * nz * 2 * modes * modes);
     A(&f->Ok, sizeof(float2) * (size_t)C * d.K);
     A(&f->Gk, sizeof(float2) * (size_t)C * d.K);
-    A(&f->sbuf, sizeof(float) * (size_t)C * N);
-    A(&f->da, sizeof(float) * (size_t)C * N);
     A(&f->dz, sizeof(float) * (size_t)C * N);
-    A(&f->dh, sizeof(float) * (size_t)H * N);
-    A(&f->dout, sizeof(float) * 4 * N);
     A(&f->tgt, sizeof(float) * 4 * N);
-    A(&f->part, sizeof(float) * (size_t)f->npart_blk * (size_t)(H * C > C * C ? H * C : C * C));
     A(&f->dpart, sizeof(double) * (152 * 4 * 16 + 32));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&f->hsum, sizeof(double) * 2);
-    std::vector<float2> Mx, Mxw, My, Mz, IXw, IX1, IY, IZ;
-    build_matrices(f, Mx, Mxw, My, Mz, IXw, IX1, IY, IZ);
-    A(&f->Mx, Mx.size() * sizeof(float2));
-    A(&f->Mxw, Mxw.size() * sizeof(float2));
-    A(&f->My, My.size() * sizeof(float2));
-    A(&f->Mz, Mz.size() * sizeof(float2));
-    A(&f->IXw, IXw.size() * sizeof(float2));
-    A(&f->IX1, IX1.size() * sizeof(float2));
-    A(&f->IY, IY.size() * sizeof(float2));
-    A(&f->IZ, IZ.size() * sizeof(float2));
-    if (e == cudaSuccess) {
+    if (f->fused) {
+        const FnoFusedDims fd = fused_dims(d);
+        const size_t nt = fno_fused_xtab_len(fd), nyt = (size_t)(ny / 2 + 1) * (modes + 1),
+                     nzt = (size_t)(nz / 2 + 1) * (modes + 1);
+        A(&f->part, sizeof(float) * fno_fused_part_len(fd));
+        std::vector<float> xt(4 * nt);
+        std::vector<float2> yt(nyt), zt(nzt);
+        fno_fused_tables(fd, xt.data(), xt.data() + nt, xt.data() + 2 * nt, xt.data() + 3 * nt, yt.data(), zt.data());
+        float** xs[] = {&f->tab.xc, &f->tab.xs, &f->tab.xcw, &f->tab.xsw};
+        for (int q = 0; q < 4; ++q) {
+            A(xs[q], nt * sizeof(float));
+            if (e == cudaSuccess) e = cudaMemcpy(*xs[q], xt.data() + q * nt, nt * sizeof(float), cudaMemcpyHostToDevice);
+        }
+        A(&f->tab.y, nyt * sizeof(float2));
+        A(&f->tab.z, nzt * sizeof(float2));
+        if (e == cudaSuccess) e = cudaMemcpy(f->tab.y, yt.data(), nyt * sizeof(float2), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(f->tab.z, zt.data(), nzt * sizeof(float2), cudaMemcpyHostToDevice);
+    } else {
+        A(&f->act, sizeof(float) * (size_t)(L + 1) * C * N);
+        A(&f->hpre, sizeof(float) * (size_t)H * N);
+        A(&f->hh, sizeof(float) * (size_t)H * N);
+        A(&f->sbuf, sizeof(float) * (size_t)C * N);
+        A(&f->da, sizeof(float) * (size_t)C * N);
+        A(&f->dh, sizeof(float) * (size_t)H * N);
+        A(&f->dout, sizeof(float) * 4 * N);
+        A(&f->part, sizeof(float) * (size_t)f->npart_blk * (size_t)(H * C > C * C ? H * C : C * C));
+        std::vector<float2> Mx, Mxw, My, Mz, IXw, IX1, IY, IZ;
+        build_matrices(f, Mx, Mxw, My, Mz, IXw, IX1, IY, IZ);
         struct {
-            float2* d;
+            float2** d;
             std::vector<float2>* h;
-        } cp[] = {{f->Mx, &Mx}, {f->Mxw, &Mxw}, {f->My, &My}, {f->Mz, &Mz},
-                  {f->IXw, &IXw}, {f->IX1, &IX1}, {f->IY, &IY}, {f->IZ, &IZ}};
-        for (auto& c : cp)
-            if (e == cudaSuccess) e = cudaMemcpy(c.d, c.h->data(), c.h->size() * sizeof(float2), cudaMemcpyHostToDevice);
+        } cp[] = {{&f->Mx, &Mx}, {&f->Mxw, &Mxw}, {&f->My, &My}, {&f->Mz, &Mz},
+                  {&f->IXw, &IXw}, {&f->IX1, &IX1}, {&f->IY, &IY}, {&f->IZ, &IZ}};
+        for (auto& c : cp) {
+            A(c.d, c.h->size() * sizeof(float2));
+            if (e == cudaSuccess)
+                e = cudaMemcpy(*c.d, c.h->data(), c.h->size() * sizeof(float2), cudaMemcpyHostToDevice);
+        }
     }
     if (e == cudaSuccess) e = cudaMemset(f->am, 0, sizeof(float) * f->npar);
     if (e == cudaSuccess) e = cudaMemset(f->av, 0, sizeof(float) * f->npar);
@@ -978,10 +1029,8 @@ int pf_fno_set_norm(pf_fno* f, const float* in_mean, const float* in_std, const 
 int pf_fno_forward(pf_fno* f, const float* x_dev, float* out_dev) {
     if (!f || !x_dev) return ffail(f, PF_EINVAL, "pf_fno_forward: NULL argument");
     cudaSetDevice(f->dev);
-    int rc = fno_forward(f, x_dev);
+    int rc = fno_forward(f, x_dev, out_dev);
     if (rc) return rc;
-    if (out_dev)
-        cudaMemcpyAsync(out_dev, f->out, sizeof(float) * 4 * f->d.N, cudaMemcpyDeviceToDevice, f->s);
     cudaError_t e = cudaStreamSynchronize(f->s);
     return e == cudaSuccess ? PF_OK : ffail(f, PF_ECUDA, "pf_fno_forward", e);
 }
@@ -1009,7 +1058,7 @@ int pf_fno_adam(pf_fno* f, float lr, float b1, float b2, float eps) {
 int pf_fno_train_step(pf_fno* f, const float* x_dev, const float* target_dev, float lr, double* loss_out) {
     if (!f || !x_dev || !target_dev) return ffail(f, PF_EINVAL, "pf_fno_train_step: NULL argument");
     cudaSetDevice(f->dev);
-    int rc = fno_forward(f, x_dev);
+    int rc = fno_forward(f, x_dev, nullptr);
     if (!rc) rc = pf_fno_backward(f, target_dev, loss_out);
     if (!rc) rc = pf_fno_adam(f, lr, 0.9f, 0.999f, 1e-8f);
     return rc;
@@ -1052,7 +1101,7 @@ int pf_fno_train_pair(pf_fno* f, const float* s0_dev, const float* s1_dev, float
     const float4 io = make_float4(1.f / f->out_std.x, 1.f / f->out_std.y, 1.f / f->out_std.z, 1.f / f->out_std.w);
     k_pair_prep<<<grid_for(4 * f->d.N), kT, 0, f->s>>>(s0_dev, s1_dev, f->x, f->tgt, f->d.N, f->in_mean, f->in_istd,
                                                       io);
-    int rc = fno_forward(f, f->x);
+    int rc = fno_forward(f, f->x, nullptr);
     if (!rc) rc = pf_fno_backward(f, f->tgt, loss_out);
     if (!rc) rc = pf_fno_adam(f, lr, 0.9f, 0.999f, 1e-8f);
     return rc;
@@ -1086,7 +1135,7 @@ int pf_surrogate_step(pf_ctx* ctx, pf_fno* f, double tau, double h, double rtol,
     rc = pf_get_state(ctx, f->realbuf, 1);
     if (rc) return rc;
     k_norm_in<<<grid_for(4 * N), kT, 0, f->s>>>(f->realbuf, f->x, N, f->in_mean, f->in_istd);
-    rc = fno_forward(f, f->x);
+    rc = fno_forward(f, f->x, f->out);
     if (rc) return rc;
     k_apply_delta<<<grid_for(4 * N), kT, 0, f->s>>>(f->realbuf, f->out, N, f->out_std);
     e = cudaStreamSynchronize(f->s);

@@ -1,0 +1,1285 @@
+// Fused kernels of the Fourier neural operator surrogate (BF16 mode).
+//
+// One layer is two kinds of work: pointwise channel products and truncated
+// transforms along the rows of the grid, both of which need all channels of a
+// row, and transforms along y and z of the few retained x modes.  The row
+// kernels do everything of the first kind in one pass over the activations:
+// a warp holds one row of all channels in shared memory, applies GELU to the
+// previous pre-activation, the channel product on the tensor cores, adds the
+// inverse x transform of the layer's spectral part, stores the
+// pre-activation, and leaves the x transform of its GELU for the next layer.
+// So a layer reads one [C][N] array and writes one; activations are
+// recomputed from pre-activations instead of stored.  The transforms use the
+// symmetry of cosines and sines under x -> n - x, which halves their products.
+//
+// Layout of the partial transforms: channels and x modes innermost,
+// T1 [z][y][c][kx], T2 [z][jy][c][kx], A [jz][jy][c][kx] (jy, jz: 0..m-1, then
+// -m..-1), so that every transform along y and z is a contraction over the
+// middle index with a contiguous inner one.
+#include <cmath>
+#include <type_traits>
+
+#include "pf_fno.cuh"
+
+namespace pf {
+
+namespace {
+
+constexpr int kSMs = 152;
+constexpr int kSmemMax = 227 * 1024;
+constexpr int kMaxModes = 16;  // x modes a lane group of the row kernels covers
+constexpr int kMaxRow = 256;   // points of a row
+constexpr int kFoldIter = (kMaxRow / 2 + 4 + 31) / 32;
+
+__host__ __device__ inline int up(int a, int b) { return (a + b - 1) / b * b; }
+// padded half row, row pitch (16-byte units odd: rows 0..7 fall on different
+// banks, also as the k rows 2t of a B fragment), padded inverse positions
+__host__ __device__ inline int half_pad(int nx) { return up(nx / 2 + 1, 4); }
+__host__ __device__ inline int row_pitch(int nx) {
+    int r = 2 * half_pad(nx);
+    if (r < up(nx, 8)) r = up(nx, 8);
+    while (r % 8 != 4) r += 4;
+    return r;
+}
+__host__ __device__ inline int inv_pad(int nx) { return up((nx + 1) / 2, 16); }
+inline int chan_pad(int C) { return C <= 16 ? 16 : 32; }
+inline int modes_pad(int m) { return up(m, 4); }
+
+struct RowArgs {
+    const float* zprev;  // previous pre-activation (GELU applied), raw field, or null (lift of x)
+    const float* x;      // network input [4][N]
+    const float *P, *pb; // lift
+    const float *V, *vb;
+    float2* T1;
+    float* z;            // forward: pre-activation out; backward: dz in and out
+    const float *fc, *fs, *ic, *is;  // forward and inverse x tables
+    float* part;
+    int nx, C, m;
+    int dense;  // forward: the layer (else only the x transform)
+    int raw;    // zprev is taken as it is
+    int last;   // forward: no x transform afterwards
+    long long N, rows;
+};
+
+// shared memory of the row kernels, in floats
+struct RowSmem {
+    int tf, ti, sp, frag, bias, lift, warp, perwarp;
+};
+__host__ __device__ inline RowSmem row_smem(int nx, int CP, int MP) {
+    RowSmem o;
+    const int HP = half_pad(nx), XQ = inv_pad(nx), T = CP / 16;
+    o.tf = 0;
+    o.ti = o.tf + 2 * MP * HP;
+    o.sp = o.ti + 2 * MP * XQ;
+    o.frag = o.sp + MP;
+    o.bias = o.frag + T * T * 256;
+    o.lift = o.bias + CP;
+    o.warp = o.lift + 5 * CP;
+    o.perwarp = CP * row_pitch(nx) + 2 * MP * (CP + 4);
+    return o;
+}
+
+template <int CPL>
+__device__ __forceinline__ void ld_chan(float (&v)[CPL], const float* p) {
+    if constexpr (CPL == 4) {
+        const float4 t = *reinterpret_cast<const float4*>(p);
+        v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+    } else {
+        const float2 t = *reinterpret_cast<const float2*>(p);
+        v[0] = t.x, v[1] = t.y;
+    }
+}
+
+// tables, fragments of V (or its transpose), bias and lift into shared memory
+template <int CP, int MP, bool TRANS>
+__device__ __forceinline__ void row_setup(const RowArgs& a, float* sm, const RowSmem& L) {
+    const int HP = half_pad(a.nx), XQ = inv_pad(a.nx), XL = (a.nx + 1) / 2, C = a.C;
+    for (int e = threadIdx.x; e < MP * HP; e += blockDim.x) {
+        sm[L.tf + e] = a.fc[e];
+        sm[L.tf + MP * HP + e] = a.fs[e];
+    }
+    // inverse positions in the order a lane group takes them: four positions
+    // spaced by 4 are one 16-byte load
+    for (int e = threadIdx.x; e < MP * XQ; e += blockDim.x) {
+        const int k = e / XQ, q = e - k * XQ, r = q & 15, x = (q & ~15) + (r >> 2) + 4 * (r & 3);
+        sm[L.ti + e] = x < XL ? a.ic[k * HP + x] : 0.f;
+        sm[L.ti + MP * XQ + e] = x < XL ? a.is[k * HP + x] : 0.f;
+    }
+    for (int e = threadIdx.x; e < MP; e += blockDim.x) sm[L.sp + e] = a.ic[e * HP + a.nx / 2];
+    if (a.V) {
+        constexpr int T = CP / 16;
+        unsigned* w = reinterpret_cast<unsigned*>(sm + L.frag);
+        for (int e = threadIdx.x; e < T * T * 32; e += blockDim.x) {
+            const int lane = e & 31, tile = e >> 5, mt = tile / T, kt = tile - mt * T, g = lane >> 2, t = lane & 3;
+            auto wv = [&](int mm, int kk) -> float {
+                if (mm >= C || kk >= C) return 0.f;
+                return TRANS ? a.V[kk * C + mm] : a.V[mm * C + kk];
+            };
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int mm = mt * 16 + g + ((r & 1) ? 8 : 0), kk = kt * 16 + 2 * t + ((r & 2) ? 8 : 0);
+                split2(wv(mm, kk), wv(mm, kk + 1), w[tile * 256 + lane * 4 + r], w[tile * 256 + 128 + lane * 4 + r]);
+            }
+        }
+    }
+    for (int e = threadIdx.x; e < CP; e += blockDim.x) {
+        sm[L.bias + e] = a.vb && e < C ? a.vb[e] : 0.f;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) sm[L.lift + 4 * e + f] = a.P && e < C ? a.P[e * 4 + f] : 0.f;
+        sm[L.lift + 4 * CP + e] = a.pb && e < C ? a.pb[e] : 0.f;
+    }
+    // padded channels stay zero in every row
+    for (int e = L.warp + threadIdx.x; e < L.warp + (int)(blockDim.x >> 5) * L.perwarp; e += blockDim.x) sm[e] = 0.f;
+}
+
+// the row's retained x modes: T1 -> [kx][channel], channels of a lane adjacent
+template <int CP, int MP>
+__device__ __forceinline__ void row_load_modes(const RowArgs& a, long long row, float* T) {
+    constexpr int CPL = CP / 8, TS = CP + 4;
+    const float2* src = a.T1 + row * a.C * a.m;
+    const int lane = threadIdx.x & 31;
+#pragma unroll 4
+    for (int e = lane; e < MP * CP; e += 32) {
+        const int c = e / MP, k = e - c * MP;
+        const float2 t = c < a.C && k < a.m ? src[c * a.m + k] : make_float2(0.f, 0.f);
+        const int o = k * TS + (c & 7) * CPL + (c >> 3);
+        T[o] = t.x;
+        T[MP * TS + o] = t.y;
+    }
+}
+
+// A <- W A column tile by column tile on the tensor cores (W's fragments in shared memory)
+template <int CP>
+__device__ __forceinline__ void row_dense(float* A, int RS, int nx, const unsigned* w) {
+    constexpr int T = CP / 16;
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    unsigned ah[T][T][4], al[T][T][4];
+#pragma unroll
+    for (int i = 0; i < T; ++i)
+#pragma unroll
+        for (int j = 0; j < T; ++j) {
+            const uint4 h = *reinterpret_cast<const uint4*>(w + (i * T + j) * 256 + lane * 4);
+            const uint4 l = *reinterpret_cast<const uint4*>(w + (i * T + j) * 256 + 128 + lane * 4);
+            ah[i][j][0] = h.x, ah[i][j][1] = h.y, ah[i][j][2] = h.z, ah[i][j][3] = h.w;
+            al[i][j][0] = l.x, al[i][j][1] = l.y, al[i][j][2] = l.z, al[i][j][3] = l.w;
+        }
+    for (int n0 = 0; n0 < nx; n0 += 8) {
+        float acc[T][4] = {};
+#pragma unroll
+        for (int j = 0; j < T; ++j) {
+            const float* b = A + (j * 16 + 2 * t) * RS + n0 + g;
+            unsigned bh0, bl0, bh1, bl1;
+            split2(b[0], b[RS], bh0, bl0);
+            split2(b[8 * RS], b[9 * RS], bh1, bl1);
+#pragma unroll
+            for (int i = 0; i < T; ++i) mma3(acc[i], ah[i][j], al[i][j], bh0, bh1, bl0, bl1);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < T; ++i) {
+            float* o = A + (i * 16 + g) * RS + n0 + 2 * t;
+            *reinterpret_cast<float2*>(o) = make_float2(acc[i][0], acc[i][1]);
+            *reinterpret_cast<float2*>(o + 8 * RS) = make_float2(acc[i][2], acc[i][3]);
+        }
+        __syncwarp();
+    }
+}
+
+// A += bias + inverse x transform of the modes in T: a lane takes CP/8
+// channels at four positions x and their mirrors n - x
+template <int CP, int MP>
+__device__ __forceinline__ void row_inverse_add(float* A, int RS, int nx, const float* T, const float* tic,
+                                                const float* tis, const float* sp, const float* bias) {
+    constexpr int CPL = CP / 8, TS = CP + 4;
+    const int lane = threadIdx.x & 31, g = lane & 7, xg = lane >> 3;
+    const int XL = (nx + 1) / 2, XQ = inv_pad(nx);
+    for (int x0 = 0; x0 < XQ; x0 += 16) {
+        float c[CPL][4] = {}, s[CPL][4] = {};
+#pragma unroll
+        for (int k = 0; k < MP; ++k) {
+            float tr[CPL], ti[CPL];
+            ld_chan<CPL>(tr, T + k * TS + g * CPL);
+            ld_chan<CPL>(ti, T + (MP + k) * TS + g * CPL);
+            const float4 cc = *reinterpret_cast<const float4*>(tic + k * XQ + x0 + xg * 4);
+            const float4 ss = *reinterpret_cast<const float4*>(tis + k * XQ + x0 + xg * 4);
+            const float cv[4] = {cc.x, cc.y, cc.z, cc.w}, sv[4] = {ss.x, ss.y, ss.z, ss.w};
+#pragma unroll
+            for (int i = 0; i < CPL; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    c[i][j] = fmaf(tr[i], cv[j], c[i][j]);
+                    s[i][j] = fmaf(ti[i], sv[j], s[i][j]);
+                }
+        }
+#pragma unroll
+        for (int i = 0; i < CPL; ++i) {
+            float* r = A + (g + 8 * i) * RS;
+            const float b = bias[g + 8 * i];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int x = x0 + xg + 4 * j;
+                if (x < XL) {
+                    r[x] += c[i][j] - s[i][j] + b;
+                    if (x > 0) r[nx - x] += c[i][j] + s[i][j] + b;
+                }
+            }
+        }
+    }
+    if ((nx & 1) == 0 && lane < CP) {  // the position that is its own mirror
+        const int slot = (lane & 7) * CPL + (lane >> 3);
+        float v = bias[lane];
+#pragma unroll
+        for (int k = 0; k < MP; ++k) v = fmaf(T[k * TS + slot], sp[k], v);
+        A[lane * RS + nx / 2] += v;
+    }
+}
+
+// T1 <- forward x transform of the folded rows (sums at [0, HP), differences
+// at [HP, 2 HP)): a lane takes CP/8 channels and MP/4 modes
+template <int CP, int MP>
+__device__ __forceinline__ void row_forward(const RowArgs& a, long long row, const float* A, int RS, float* T,
+                                            const float* tfc, const float* tfs) {
+    constexpr int CPL = CP / 8, KPL = MP / 4;
+    const int lane = threadIdx.x & 31, g = lane & 7, kg = lane >> 3, HP = half_pad(a.nx);
+    float re[CPL][KPL] = {}, im[CPL][KPL] = {};
+    for (int x = 0; x < HP; x += 4) {
+        float4 c[KPL], s[KPL];
+#pragma unroll
+        for (int j = 0; j < KPL; ++j) {
+            c[j] = *reinterpret_cast<const float4*>(tfc + (kg * KPL + j) * HP + x);
+            s[j] = *reinterpret_cast<const float4*>(tfs + (kg * KPL + j) * HP + x);
+        }
+#pragma unroll
+        for (int i = 0; i < CPL; ++i) {
+            const float4 e = *reinterpret_cast<const float4*>(A + (g + 8 * i) * RS + x);
+            const float4 o = *reinterpret_cast<const float4*>(A + (g + 8 * i) * RS + HP + x);
+#pragma unroll
+            for (int j = 0; j < KPL; ++j) {
+                re[i][j] = fmaf(e.w, c[j].w, fmaf(e.z, c[j].z, fmaf(e.y, c[j].y, fmaf(e.x, c[j].x, re[i][j]))));
+                im[i][j] = fmaf(o.w, s[j].w, fmaf(o.z, s[j].z, fmaf(o.y, s[j].y, fmaf(o.x, s[j].x, im[i][j]))));
+            }
+        }
+    }
+    // through shared memory (the modes of this row are used up) for a contiguous store
+    float2* st = reinterpret_cast<float2*>(T);
+#pragma unroll
+    for (int i = 0; i < CPL; ++i)
+#pragma unroll
+        for (int j = 0; j < KPL; ++j) {
+            const int c = g + 8 * i, k = kg * KPL + j;
+            if (c < a.C && k < a.m) st[c * a.m + k] = make_float2(re[i][j], -im[i][j]);
+        }
+    __syncwarp();
+    float2* dst = a.T1 + row * a.C * a.m;
+    for (int e = lane; e < a.C * a.m; e += 32) dst[e] = st[e];
+    __syncwarp();
+}
+
+// in place: a row's values -> sums and differences under x -> n - x, through
+// val(channel, x, value) (which may store and change the value)
+template <class F>
+__device__ __forceinline__ void row_fold(float* A, int RS, int nx, int C, F val) {
+    const int lane = threadIdx.x & 31, HP = half_pad(nx), Hx = nx / 2 + 1;
+#pragma unroll 2
+    for (int c = 0; c < C; ++c) {
+        float* r = A + c * RS;
+        float e[kFoldIter], o[kFoldIter];
+#pragma unroll
+        for (int q = 0; q < kFoldIter; ++q) {
+            const int x = lane + 32 * q;
+            e[q] = o[q] = 0.f;
+            if (x < Hx) {
+                const float v = val(c, x, r[x]);
+                e[q] = v;
+                if (x > 0 && 2 * x != nx) {
+                    const float u = val(c, nx - x, r[nx - x]);
+                    e[q] = v + u;
+                    o[q] = v - u;
+                }
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < kFoldIter; ++q) {
+            const int x = lane + 32 * q;
+            if (x < HP) {
+                r[x] = e[q];
+                r[HP + x] = o[q];
+            }
+        }
+    }
+    __syncwarp();
+}
+
+// lift of the row's input: a_0 = P x + p
+template <int CP>
+__device__ __forceinline__ void row_lift(const RowArgs& a, long long r0, float* A, int RS, const float* lift) {
+    for (int x = threadIdx.x & 31; x < a.nx; x += 32) {
+        float v[4];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) v[f] = a.x[f * a.N + r0 + x];
+        for (int c = 0; c < a.C; ++c) {
+            const float4 w = *reinterpret_cast<const float4*>(lift + 4 * c);
+            A[c * RS + x] = fmaf(w.w, v[3], fmaf(w.z, v[2], fmaf(w.y, v[1], fmaf(w.x, v[0], lift[4 * CP + c]))));
+        }
+    }
+}
+
+template <int CP, int MP>
+__global__ void __launch_bounds__(512, 1) k_fno_row(RowArgs a) {
+    extern __shared__ __align__(16) float sm[];
+    const RowSmem L = row_smem(a.nx, CP, MP);
+    row_setup<CP, MP, false>(a, sm, L);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int nx = a.nx, C = a.C, RS = row_pitch(nx), HP = half_pad(nx), XQ = inv_pad(nx);
+    float* A = sm + L.warp + warp * L.perwarp;
+    float* T = A + CP * RS;
+    for (long long row = blockIdx.x * (long long)nw + warp; row < a.rows; row += (long long)gridDim.x * nw) {
+        const long long r0 = row * nx;
+        if (a.dense) row_load_modes<CP, MP>(a, row, T);
+        if (!a.zprev) {
+            row_lift<CP>(a, r0, A, RS, sm + L.lift);
+        } else {
+            for (int x = lane; x < nx; x += 32) {
+                const float* src = a.zprev + r0 + x;
+#pragma unroll 8
+                for (int c = 0; c < C; ++c) {
+                    const float v = src[(long long)c * a.N];
+                    A[c * RS + x] = a.raw ? v : gelu_f(v);
+                }
+            }
+        }
+        __syncwarp();
+        if (a.dense) {
+            row_dense<CP>(A, RS, nx, reinterpret_cast<const unsigned*>(sm + L.frag));
+            row_inverse_add<CP, MP>(A, RS, nx, T, sm + L.ti, sm + L.ti + MP * XQ, sm + L.sp, sm + L.bias);
+            __syncwarp();
+        }
+        if (a.last) {
+            for (int x = lane; x < nx; x += 32)
+#pragma unroll 8
+                for (int c = 0; c < C; ++c) a.z[(long long)c * a.N + r0 + x] = A[c * RS + x];
+            __syncwarp();
+            continue;
+        }
+        if (a.dense) {
+            row_fold(A, RS, nx, C, [&](int c, int x, float v) {
+                a.z[(long long)c * a.N + r0 + x] = v;
+                return gelu_f(v);
+            });
+        } else {
+            row_fold(A, RS, nx, C, [](int, int, float v) { return v; });
+        }
+        row_forward<CP, MP>(a, row, A, RS, T, sm + L.tf, sm + L.tf + MP * HP);
+    }
+}
+
+// Partial sums of a block of k_fno_row_bwd: [C C] V, [C] v, [4 C] P, [C] p
+__host__ __device__ inline int row_part_len(int C) { return C * C + 6 * C; }
+
+template <int CP, int MP>
+__global__ void __launch_bounds__(384, 1) k_fno_row_bwd(RowArgs a) {
+    extern __shared__ __align__(16) float sm[];
+    const RowSmem L = row_smem(a.nx, CP, MP);
+    row_setup<CP, MP, true>(a, sm, L);
+    __syncthreads();
+    constexpr int MT = CP / 16, NT = CP / 8;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, g = lane >> 2, t = lane & 3;
+    const int nx = a.nx, C = a.C, RS = row_pitch(nx), HP = half_pad(nx), XQ = inv_pad(nx);
+    const bool first = a.zprev == nullptr;
+    float* A = sm + L.warp + warp * L.perwarp;
+    float* T = A + CP * RS;
+    const float* lift = sm + L.lift;
+    float gV[MT][NT][4] = {}, gP[MT][4] = {}, sv[MT][2] = {}, sp[MT][2] = {};
+    // A fragments (rows = channels of the shared-memory row, k = 16 points) and the row sums
+    auto rows_frag = [&](int p, unsigned (&ah)[MT][4], unsigned (&al)[MT][4], float (&sum)[MT][2]) {
+#pragma unroll
+        for (int i = 0; i < MT; ++i) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int q = p + ((r & 2) ? 8 : 0);
+                float2 u = *reinterpret_cast<const float2*>(A + (i * 16 + g + ((r & 1) ? 8 : 0)) * RS + (q < nx ? q : 0));
+                if (q >= nx) u.x = 0.f;
+                if (q + 1 >= nx) u.y = 0.f;
+                sum[i][r & 1] += u.x + u.y;
+                split2(u.x, u.y, ah[i][r], al[i][r]);
+            }
+        }
+    };
+    for (long long row = blockIdx.x * (long long)nw + warp; row < a.rows; row += (long long)gridDim.x * nw) {
+        const long long r0 = row * nx;
+        row_load_modes<CP, MP>(a, row, T);
+        for (int x = lane; x < nx; x += 32) {
+            const float* src = a.z + r0 + x;
+#pragma unroll 8
+            for (int c = 0; c < C; ++c) A[c * RS + x] = src[(long long)c * a.N];
+        }
+        __syncwarp();
+        // gradient of V: dz a^T over the row's points, a in fragments straight from global memory
+        for (int k0 = 0; k0 < nx; k0 += 16) {
+            const int p = k0 + 2 * t;
+            float av[NT][4];
+            if (!first) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const int d = j * 8 + g, q = p + (r & 1) + ((r & 2) ? 8 : 0);
+                        av[j][r] = d < C && q < nx ? a.zprev[(long long)d * a.N + r0 + q] : 0.f;
+                    }
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) av[j][r] = gelu_f(av[j][r]);
+            } else {
+                float xv[4][4];
+#pragma unroll
+                for (int f = 0; f < 4; ++f)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const int q = p + (r & 1) + ((r & 2) ? 8 : 0);
+                        xv[f][r] = q < nx ? a.x[f * a.N + r0 + q] : 0.f;
+                    }
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    const float4 w = *reinterpret_cast<const float4*>(lift + 4 * (j * 8 + g));
+                    const float b = lift[4 * CP + j * 8 + g];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+                        av[j][r] = fmaf(w.w, xv[3][r], fmaf(w.z, xv[2][r], fmaf(w.y, xv[1][r], fmaf(w.x, xv[0][r], b))));
+                }
+            }
+            unsigned ah[MT][4], al[MT][4];
+            rows_frag(p, ah, al, sv);
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                unsigned bh0, bl0, bh1, bl1;
+                split2(av[j][0], av[j][1], bh0, bl0);
+                split2(av[j][2], av[j][3], bh1, bl1);
+#pragma unroll
+                for (int i = 0; i < MT; ++i) mma3(gV[i][j], ah[i], al[i], bh0, bh1, bl0, bl1);
+            }
+        }
+        __syncwarp();
+        row_dense<CP>(A, RS, nx, reinterpret_cast<const unsigned*>(sm + L.frag));
+        row_inverse_add<CP, MP>(A, RS, nx, T, sm + L.ti, sm + L.ti + MP * XQ, sm + L.sp, sm + L.bias);
+        __syncwarp();
+        if (first) {
+            // gradients of the lift: da x^T and the row sums
+            for (int k0 = 0; k0 < nx; k0 += 16) {
+                const int p = k0 + 2 * t;
+                float xv[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int q = p + (r & 1) + ((r & 2) ? 8 : 0);
+                    xv[r] = g < 4 && q < nx ? a.x[g * a.N + r0 + q] : 0.f;
+                }
+                unsigned ah[MT][4], al[MT][4], bh0, bl0, bh1, bl1;
+                rows_frag(p, ah, al, sp);
+                split2(xv[0], xv[1], bh0, bl0);
+                split2(xv[2], xv[3], bh1, bl1);
+#pragma unroll
+                for (int i = 0; i < MT; ++i) mma3(gP[i], ah[i], al[i], bh0, bh1, bl0, bl1);
+            }
+            __syncwarp();
+            continue;
+        }
+        row_fold(A, RS, nx, C, [&](int c, int x, float v) {
+            const long long i = (long long)c * a.N + r0 + x;
+            const float d = v * gelu_g(a.zprev[i]);
+            a.z[i] = d;
+            return d;
+        });
+        row_forward<CP, MP>(a, row, A, RS, T, sm + L.tf, sm + L.tf + MP * HP);
+    }
+    // warps -> block, in warp order
+    const int E = row_part_len(C);
+    __syncthreads();
+    float* own = sm + L.warp + warp * L.perwarp;  // at least CP (2 half_pad) floats: CP CP + 6 CP fit from nx = 32 on
+#pragma unroll
+    for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int c = i * 16 + g + ((r & 2) ? 8 : 0);
+            if (c < C) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    const int d = j * 8 + 2 * t + (r & 1);
+                    if (d < C) own[c * C + d] = gV[i][j][r];
+                }
+                if (2 * t + (r & 1) < 4) own[C * C + C + c * 4 + 2 * t + (r & 1)] = gP[i][r];
+            }
+        }
+#pragma unroll
+    for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            float u = sv[i][r], w = sp[i][r];
+            u += __shfl_xor_sync(0xffffffffu, u, 1);
+            u += __shfl_xor_sync(0xffffffffu, u, 2);
+            w += __shfl_xor_sync(0xffffffffu, w, 1);
+            w += __shfl_xor_sync(0xffffffffu, w, 2);
+            const int c = i * 16 + g + 8 * r;
+            if (t == 0 && c < C) {
+                own[C * C + c] = u;
+                own[C * C + 5 * C + c] = w;
+            }
+        }
+    __syncthreads();
+    for (int e = threadIdx.x; e < E; e += blockDim.x) {
+        float v = 0.f;
+        for (int w = 0; w < nw; ++w) v += sm[L.warp + w * L.perwarp + e];
+        a.part[(long long)blockIdx.x * E + e] = v;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// transforms along y or z of the retained modes: modes 0..m-1 and -m..-1.
+// With E(j) = v(j) + v(J - j), O(j) = v(j) - v(J - j), the sums
+// P_k = sum_j E cos, Q_k = sum_j O sin give F(+-k) = P_k -+ i Q_k, a quarter
+// of the products of the plain contraction.  tab[j][k] = (cos, sin), k <= m.
+// ---------------------------------------------------------------------------
+template <int MP>
+__global__ void __launch_bounds__(64) k_dft_modes(const float2* __restrict__ in, float2* __restrict__ out,
+                                                  const float2* __restrict__ tab, int J, int m, int I) {
+    extern __shared__ __align__(16) float2 st[];  // [J/2 + 1][MP + 2]
+    constexpr int TP = MP + 2;
+    for (int e = threadIdx.x; e < (J / 2 + 1) * TP; e += blockDim.x) {
+        const int j = e / TP, k = e - j * TP;
+        st[e] = k <= m ? tab[j * (m + 1) + k] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= I) return;
+    const float2* src = in + (long long)blockIdx.y * J * I + i;
+    float2 P[MP + 1], Q[MP + 1];
+#pragma unroll
+    for (int k = 0; k <= MP; ++k) P[k] = Q[k] = make_float2(0.f, 0.f);
+    auto add = [&](int j, float2 e, float2 o) {
+        const float4* row = reinterpret_cast<const float4*>(st + j * TP);
+#pragma unroll
+        for (int k2 = 0; k2 < TP / 2; ++k2) {
+            const float4 w = row[k2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int k = 2 * k2 + h;
+                if (k <= MP) {
+                    const float c = h ? w.z : w.x, s = h ? w.w : w.y;
+                    P[k].x = fmaf(c, e.x, P[k].x);
+                    P[k].y = fmaf(c, e.y, P[k].y);
+                    Q[k].x = fmaf(s, o.x, Q[k].x);
+                    Q[k].y = fmaf(s, o.y, Q[k].y);
+                }
+            }
+        }
+    };
+    const float2 z = make_float2(0.f, 0.f);
+    add(0, src[0], z);
+    const int pairs = (J - 1) / 2;
+    int j = 1;
+    for (; j + 3 <= pairs; j += 4) {
+        float2 a[4], b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            a[u] = src[(long long)(j + u) * I];
+            b[u] = src[(long long)(J - j - u) * I];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            add(j + u, make_float2(a[u].x + b[u].x, a[u].y + b[u].y), make_float2(a[u].x - b[u].x, a[u].y - b[u].y));
+    }
+    for (; j <= pairs; ++j) {
+        const float2 a = src[(long long)j * I], b = src[(long long)(J - j) * I];
+        add(j, make_float2(a.x + b.x, a.y + b.y), make_float2(a.x - b.x, a.y - b.y));
+    }
+    if ((J & 1) == 0) add(J / 2, src[(long long)(J / 2) * I], z);
+    float2* dst = out + (long long)blockIdx.y * 2 * m * I + i;
+#pragma unroll
+    for (int k = 0; k <= MP; ++k) {
+        if (k < m) dst[(long long)k * I] = make_float2(P[k].x + Q[k].y, P[k].y - Q[k].x);
+        if (k > 0 && k <= m) dst[(long long)(2 * m - k) * I] = make_float2(P[k].x - Q[k].y, P[k].y + Q[k].x);
+    }
+}
+
+// out(j) = sum over the modes of in e^{+2 pi i k j / J}, positions j and J - j
+// together, blockIdx.z-th part of the positions
+template <int MP>
+__global__ void __launch_bounds__(64) k_dft_modes_inv(const float2* __restrict__ in, float2* __restrict__ out,
+                                                      const float2* __restrict__ tab, int J, int m, int I) {
+    extern __shared__ __align__(16) float2 st[];
+    constexpr int TP = MP + 2;
+    const int half = J / 2 + 1, per = (half + gridDim.z - 1) / gridDim.z;
+    const int j0 = blockIdx.z * per, j1 = min(half, j0 + per);
+    for (int e = threadIdx.x; e < (j1 - j0) * TP; e += blockDim.x) {
+        const int j = e / TP, k = e - j * TP;
+        st[e] = k <= m ? tab[(j0 + j) * (m + 1) + k] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= I) return;
+    const float2* src = in + (long long)blockIdx.y * 2 * m * I + i;
+    float2 U[MP + 1], V[MP + 1];
+#pragma unroll
+    for (int k = 0; k <= MP; ++k) {
+        const float2 a = k < m ? src[(long long)k * I] : make_float2(0.f, 0.f);
+        const float2 b = k > 0 && k <= m ? src[(long long)(2 * m - k) * I] : make_float2(0.f, 0.f);
+        U[k] = make_float2(a.x + b.x, a.y + b.y);
+        V[k] = make_float2(a.x - b.x, a.y - b.y);
+    }
+    float2* dst = out + (long long)blockIdx.y * J * I + i;
+    for (int j = j0; j < j1; ++j) {
+        const float4* row = reinterpret_cast<const float4*>(st + (j - j0) * TP);
+        float2 P = make_float2(0.f, 0.f), Q = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k2 = 0; k2 < TP / 2; ++k2) {
+            const float4 w = row[k2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int k = 2 * k2 + h;
+                if (k <= MP) {
+                    const float c = h ? w.z : w.x, s = h ? w.w : w.y;
+                    P.x = fmaf(c, U[k].x, P.x);
+                    P.y = fmaf(c, U[k].y, P.y);
+                    Q.x = fmaf(s, V[k].x, Q.x);
+                    Q.y = fmaf(s, V[k].y, Q.y);
+                }
+            }
+        }
+        dst[(long long)j * I] = make_float2(P.x - Q.y, P.y + Q.x);
+        if (j > 0 && 2 * j != J) dst[(long long)(J - j) * I] = make_float2(P.x + Q.y, P.y - Q.x);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// per-mode channel mix: one block per (jz, jy), a warp per kx.
+// O[c] = sum_d W[c][d] A[d]: a lane takes row c of the mode's matrix, in
+// 16-byte pieces where rows are 16-byte aligned (C a multiple of 4)
+// ---------------------------------------------------------------------------
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_mix_modes(const float2* __restrict__ A, float2* __restrict__ O,
+                                                   const __nv_bfloat162* __restrict__ w16, int C, int m) {
+    extern __shared__ __align__(16) float2 st[];  // [C m] in, [C m] out
+    const long long b = blockIdx.x;
+    float2* so = st + C * m;
+    for (int e = threadIdx.x; e < C * m; e += blockDim.x) st[e] = A[b * C * m + e];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int kx = threadIdx.x >> 5; kx < m; kx += blockDim.x >> 5) {
+        if (lane < C) {
+            const __nv_bfloat162* w = w16 + ((b * m + kx) * C + lane) * C;
+            float ar = 0.f, ai = 0.f;
+            auto add = [&](unsigned u, int d) {
+                const float wx = __uint_as_float(u << 16), wy = __uint_as_float(u & 0xffff0000u);
+                const float2 v = st[d * m + kx];
+                ar = fmaf(-wy, v.y, fmaf(wx, v.x, ar));
+                ai = fmaf(wy, v.x, fmaf(wx, v.y, ai));
+            };
+            if constexpr (VEC) {
+#pragma unroll 8
+                for (int d = 0; d < C; d += 4) {
+                    const uint4 u = __ldg(reinterpret_cast<const uint4*>(w + d));
+                    add(u.x, d);
+                    add(u.y, d + 1);
+                    add(u.z, d + 2);
+                    add(u.w, d + 3);
+                }
+            } else {
+                for (int d = 0; d < C; ++d) add(*reinterpret_cast<const unsigned*>(w + d), d);
+            }
+            so[lane * m + kx] = make_float2(ar, ai);
+        }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < C * m; e += blockDim.x) O[b * C * m + e] = so[e];
+}
+
+// GA[d] = sum_c conj(W[c][d]) GO[c]; GW[c][d] = GO[c] conj(A[d]): a lane takes column d
+__global__ void __launch_bounds__(256) k_mix_modes_bwd(const float2* __restrict__ GO, const float2* __restrict__ A,
+                                                       float2* __restrict__ GA, float2* __restrict__ GW,
+                                                       const __nv_bfloat162* __restrict__ w16, int C, int m) {
+    extern __shared__ __align__(16) float2 st[];  // [C m] GO, A, GA
+    const long long b = blockIdx.x;
+    float2 *sa = st + C * m, *so = sa + C * m;
+    for (int e = threadIdx.x; e < C * m; e += blockDim.x) {
+        st[e] = GO[b * C * m + e];
+        sa[e] = A[b * C * m + e];
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int kx = threadIdx.x >> 5; kx < m; kx += blockDim.x >> 5) {
+        if (lane < C) {
+            const long long w0 = (b * m + kx) * C * C + lane;
+            const float2 a = sa[lane * m + kx];
+            float ar = 0.f, ai = 0.f;
+#pragma unroll 8
+            for (int c = 0; c < C; ++c) {
+                const unsigned u = *reinterpret_cast<const unsigned*>(w16 + w0 + c * C);
+                const float wx = __uint_as_float(u << 16), wy = __uint_as_float(u & 0xffff0000u);
+                const float2 g = st[c * m + kx];
+                ar = fmaf(wy, g.y, fmaf(wx, g.x, ar));
+                ai = fmaf(-wy, g.x, fmaf(wx, g.y, ai));
+                GW[w0 + c * C] = make_float2(g.x * a.x + g.y * a.y, g.y * a.x - g.x * a.y);
+            }
+            so[lane * m + kx] = make_float2(ar, ai);
+        }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < C * m; e += blockDim.x) GA[b * C * m + e] = so[e];
+}
+
+// ---------------------------------------------------------------------------
+// projection: tiles of 64 points; a warp owns 16 of the H rows.
+// ---------------------------------------------------------------------------
+constexpr int kPts = 64, kPS = 68;
+__host__ __device__ inline int proj_part_len(int C, int H) { return H * C + 5 * H + 4; }
+struct ProjArgs {
+    const float *a, *tgt, *Q1, *q1, *Q2, *q2;
+    float *out, *da, *part;
+    double* dpart;
+    int C, H;
+    long long N;
+    float sc;  // 2 / (4 N)
+};
+template <int CP, int NW, bool TRAIN>
+constexpr int proj_smem() {
+    constexpr int HP = 16 * NW, KT = CP / 16;
+    return (CP * kPS + HP * kPS + 4 * kPS + 5 * HP + 4 + NW * KT * 256 + (TRAIN ? NW * KT * 256 : 0)) * 4;
+}
+
+template <int CP, int NW, bool TRAIN>
+__global__ void __launch_bounds__(32 * NW, (CP == 32 && NW == 8 && TRAIN) ? 2 : 1) k_fno_project(ProjArgs p) {
+    constexpr int HP = 16 * NW, KT = CP / 16, NT = kPts / 8;
+    extern __shared__ __align__(16) float sm[];
+    float* sa = sm;               // [CP][kPS]
+    float* sh = sa + CP * kPS;    // [HP][kPS]: h, then dh
+    float* sd = sh + HP * kPS;    // [4][kPS]: d out
+    float* sq2 = sd + 4 * kPS;    // [HP][4]
+    float* sq1 = sq2 + 4 * HP;    // [HP]
+    float* sb2 = sq1 + HP;        // [4]
+    unsigned* w1 = reinterpret_cast<unsigned*>(sb2 + 4);  // Q1 fragments [NW][KT]
+    unsigned* wt = w1 + NW * KT * 256;                    // Q1^T fragments [KT][NW]
+    const int C = p.C, H = p.H;
+    auto q1v = [&](int h, int c) -> float { return h < H && c < C ? p.Q1[h * C + c] : 0.f; };
+    for (int e = threadIdx.x; e < NW * KT * 32; e += blockDim.x) {
+        const int lane = e & 31, tile = e >> 5, g = lane >> 2, t = lane & 3;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int mm = g + ((r & 1) ? 8 : 0), kk = 2 * t + ((r & 2) ? 8 : 0);
+            const int mt = tile / KT, kt = tile - mt * KT;
+            split2(q1v(mt * 16 + mm, kt * 16 + kk), q1v(mt * 16 + mm, kt * 16 + kk + 1), w1[tile * 256 + lane * 4 + r],
+                   w1[tile * 256 + 128 + lane * 4 + r]);
+            if (TRAIN) {
+                const int ct = tile / NW, ht = tile - ct * NW;
+                split2(q1v(ht * 16 + kk, ct * 16 + mm), q1v(ht * 16 + kk + 1, ct * 16 + mm),
+                       wt[tile * 256 + lane * 4 + r], wt[tile * 256 + 128 + lane * 4 + r]);
+            }
+        }
+    }
+    for (int e = threadIdx.x; e < HP; e += blockDim.x) {
+#pragma unroll
+        for (int f = 0; f < 4; ++f) sq2[4 * e + f] = e < H ? p.Q2[f * H + e] : 0.f;
+        sq1[e] = e < H ? p.q1[e] : 0.f;
+    }
+    if (threadIdx.x < 4) sb2[threadIdx.x] = p.q2[threadIdx.x];
+    for (int e = threadIdx.x; e < CP * kPS; e += blockDim.x) sa[e] = 0.f;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const long long tiles = (p.N + kPts - 1) / kPts;
+    // gradients kept over the block's tiles
+    float gQ1[CP / 8][4] = {}, gq1[2] = {}, gQ2[4] = {};
+    float gq2 = 0.f;
+    double loss = 0.0;
+    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const long long p0 = tile * kPts;
+        const int np = (int)min((long long)kPts, p.N - p0);
+#pragma unroll 4
+        for (int e = threadIdx.x; e < C * kPts; e += blockDim.x) {
+            const int c = e / kPts, q = e - c * kPts;
+            sa[c * kPS + q] = q < np ? p.a[(long long)c * p.N + p0 + q] : 0.f;
+        }
+        __syncthreads();
+        // h = GELU(Q1 a + q1) of this warp's rows; its derivative stays in registers
+        const int h0 = warp * 16;
+        float gp[TRAIN ? NT : 1][4];
+        {
+            unsigned ah[KT][4], al[KT][4];
+#pragma unroll
+            for (int k = 0; k < KT; ++k) {
+                const unsigned* w = w1 + (warp * KT + k) * 256 + lane * 4;
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    ah[k][r] = w[r];
+                    al[k][r] = w[128 + r];
+                }
+            }
+            const float b0 = sq1[h0 + g], b1 = sq1[h0 + g + 8];
+#pragma unroll
+            for (int n = 0; n < NT; ++n) {
+                float acc[4] = {b0, b0, b1, b1};
+#pragma unroll
+                for (int k = 0; k < KT; ++k) {
+                    const float* b = sa + (k * 16 + 2 * t) * kPS + n * 8 + g;
+                    unsigned bh0, bl0, bh1, bl1;
+                    split2(b[0], b[kPS], bh0, bl0);
+                    split2(b[8 * kPS], b[9 * kPS], bh1, bl1);
+                    mma3(acc, ah[k], al[k], bh0, bh1, bl0, bl1);
+                }
+                float hv[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float z = acc[r];
+                    const float cdf = 0.5f * (1.0f + erff(z * 0.70710678118654752f));
+                    hv[r] = z * cdf;
+                    if (TRAIN) gp[n][r] = cdf + z * expf(-0.5f * z * z) * 0.39894228040143268f;
+                }
+                float* o = sh + (h0 + g) * kPS + n * 8 + 2 * t;
+                *reinterpret_cast<float2*>(o) = make_float2(hv[0], hv[1]);
+                *reinterpret_cast<float2*>(o + 8 * kPS) = make_float2(hv[2], hv[3]);
+            }
+        }
+        __syncthreads();
+        // out = Q2 h + q2, one (field, point) a thread at a time
+        for (int e = threadIdx.x; e < 4 * kPts; e += blockDim.x) {
+            const int f = e / kPts, q = e - f * kPts;
+            float v0 = sb2[f], v1 = 0.f, v2 = 0.f, v3 = 0.f;
+#pragma unroll 8
+            for (int h = 0; h < HP; h += 4) {
+                v0 = fmaf(sq2[4 * h + f], sh[h * kPS + q], v0);
+                v1 = fmaf(sq2[4 * h + 4 + f], sh[(h + 1) * kPS + q], v1);
+                v2 = fmaf(sq2[4 * h + 8 + f], sh[(h + 2) * kPS + q], v2);
+                v3 = fmaf(sq2[4 * h + 12 + f], sh[(h + 3) * kPS + q], v3);
+            }
+            const float v = (v0 + v1) + (v2 + v3);
+            if constexpr (TRAIN) {
+                float d = 0.f;
+                if (q < np) {
+                    d = v - p.tgt[(long long)f * p.N + p0 + q];
+                    loss += (double)d * d;
+                    d *= p.sc;
+                }
+                sd[f * kPS + q] = d;
+            } else if (q < np) {
+                p.out[(long long)f * p.N + p0 + q] = v;
+            }
+        }
+        __syncthreads();
+        if constexpr (TRAIN) {
+            // gradients of Q2 (four fields per row h, rows over the threads) and q2
+            {
+                constexpr int G = 32 * NW / HP;  // threads per row: 2, each two fields
+                const int h = threadIdx.x % HP, f0 = threadIdx.x / HP * (4 / G);
+                const float* hr = sh + h * kPS;
+#pragma unroll 4
+                for (int q = 0; q < kPts; q += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(hr + q);
+#pragma unroll
+                    for (int u = 0; u < 4 / G; ++u) {
+                        const float4 d = *reinterpret_cast<const float4*>(sd + (f0 + u) * kPS + q);
+                        gQ2[u] = fmaf(v.w, d.w, fmaf(v.z, d.z, fmaf(v.y, d.y, fmaf(v.x, d.x, gQ2[u]))));
+                    }
+                }
+                if (threadIdx.x < 4) {
+                    float s = 0.f;
+                    for (int q = 0; q < kPts; ++q) s += sd[threadIdx.x * kPS + q];
+                    gq2 += s;
+                }
+            }
+            __syncthreads();
+            // dh = GELU' (Q2^T d out) over h
+            {
+                float4 qa = *reinterpret_cast<const float4*>(sq2 + 4 * (h0 + g));
+                float4 qb = *reinterpret_cast<const float4*>(sq2 + 4 * (h0 + g + 8));
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                    const float* d = sd + n * 8 + 2 * t;
+                    const float2 d0 = *reinterpret_cast<const float2*>(d), d1 = *reinterpret_cast<const float2*>(d + kPS);
+                    const float2 d2 = *reinterpret_cast<const float2*>(d + 2 * kPS);
+                    const float2 d3 = *reinterpret_cast<const float2*>(d + 3 * kPS);
+                    const float v0 = gp[n][0] * (qa.x * d0.x + qa.y * d1.x + qa.z * d2.x + qa.w * d3.x);
+                    const float v1 = gp[n][1] * (qa.x * d0.y + qa.y * d1.y + qa.z * d2.y + qa.w * d3.y);
+                    const float v2 = gp[n][2] * (qb.x * d0.x + qb.y * d1.x + qb.z * d2.x + qb.w * d3.x);
+                    const float v3 = gp[n][3] * (qb.x * d0.y + qb.y * d1.y + qb.z * d2.y + qb.w * d3.y);
+                    gq1[0] += v0 + v1;
+                    gq1[1] += v2 + v3;
+                    float* o = sh + (h0 + g) * kPS + n * 8 + 2 * t;
+                    *reinterpret_cast<float2*>(o) = make_float2(v0, v1);
+                    *reinterpret_cast<float2*>(o + 8 * kPS) = make_float2(v2, v3);
+                }
+            }
+            __syncthreads();
+            // gradient of Q1: dh a^T over the tile's points
+#pragma unroll
+            for (int k = 0; k < kPts / 16; ++k) {
+                unsigned ah[4], al[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float2 u = *reinterpret_cast<const float2*>(sh + (h0 + g + ((r & 1) ? 8 : 0)) * kPS + k * 16 +
+                                                                      2 * t + ((r & 2) ? 8 : 0));
+                    split2(u.x, u.y, ah[r], al[r]);
+                }
+#pragma unroll
+                for (int j = 0; j < CP / 8; ++j) {
+                    const float* b = sa + (j * 8 + g) * kPS + k * 16 + 2 * t;
+                    const float2 u0 = *reinterpret_cast<const float2*>(b), u1 = *reinterpret_cast<const float2*>(b + 8);
+                    unsigned bh0, bl0, bh1, bl1;
+                    split2(u0.x, u0.y, bh0, bl0);
+                    split2(u1.x, u1.y, bh1, bl1);
+                    mma3(gQ1[j], ah, al, bh0, bh1, bl0, bl1);
+                }
+            }
+            // da = Q1^T dh, column tiles over the warps
+            for (int n = warp; n < NT; n += NW) {
+                float acc[KT][4] = {};
+#pragma unroll
+                for (int k = 0; k < NW; ++k) {
+                    const float* b = sh + (k * 16 + 2 * t) * kPS + n * 8 + g;
+                    unsigned bh0, bl0, bh1, bl1;
+                    split2(b[0], b[kPS], bh0, bl0);
+                    split2(b[8 * kPS], b[9 * kPS], bh1, bl1);
+#pragma unroll
+                    for (int i = 0; i < KT; ++i) {
+                        const uint4 hv = *reinterpret_cast<const uint4*>(wt + (i * NW + k) * 256 + lane * 4);
+                        const uint4 lv = *reinterpret_cast<const uint4*>(wt + (i * NW + k) * 256 + 128 + lane * 4);
+                        const unsigned ah[4] = {hv.x, hv.y, hv.z, hv.w}, al[4] = {lv.x, lv.y, lv.z, lv.w};
+                        mma3(acc[i], ah, al, bh0, bh1, bl0, bl1);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < KT; ++i)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const int c = i * 16 + g + ((r & 2) ? 8 : 0), q = n * 8 + 2 * t + (r & 1);
+                        if (c < C && q < np) p.da[(long long)c * p.N + p0 + q] = acc[i][r];
+                    }
+            }
+            __syncthreads();
+        }
+    }
+    if constexpr (TRAIN) {
+        // block partials: [H C] Q1, [H] q1, [4 H] Q2, [4] q2; the loss in FP64
+        float* o = p.part + (long long)blockIdx.x * proj_part_len(C, H);
+        const int h0 = warp * 16;
+#pragma unroll
+        for (int j = 0; j < CP / 8; ++j)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int h = h0 + g + ((r & 2) ? 8 : 0), c = j * 8 + 2 * t + (r & 1);
+                if (h < H && c < C) o[h * C + c] = gQ1[j][r];
+            }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            float v = gq1[r];
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            const int h = h0 + g + 8 * r;
+            if (t == 0 && h < H) o[H * C + h] = v;
+        }
+        {
+            constexpr int G = 32 * NW / HP;
+            const int h = threadIdx.x % HP, f0 = threadIdx.x / HP * (4 / G);
+#pragma unroll
+            for (int u = 0; u < 4 / G; ++u)
+                if (h < H) o[H * C + H + (f0 + u) * H + h] = gQ2[u];
+        }
+        if (threadIdx.x < 4) o[H * C + 5 * H + threadIdx.x] = gq2;
+        __shared__ double red[NW];
+        for (int s = 16; s > 0; s >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, s);
+        if (lane == 0) red[warp] = loss;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double v = 0.0;
+            for (int w = 0; w < NW; ++w) v += red[w];
+            p.dpart[blockIdx.x] = v;
+        }
+    }
+}
+
+// sums of the blocks' partials in a fixed order: 32 entries a block, eight
+// warps over the partial blocks, up to four destinations
+struct SumSeg {
+    int off[4], len[4];
+    float* dst[4];
+    int n;
+};
+__global__ void __launch_bounds__(256) k_part_sum(const float* __restrict__ part, int nblk, int E, SumSeg sg) {
+    __shared__ float red[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+    float v = 0.f;
+    if (e < E)
+        for (int b = warp; b < nblk; b += 8) v += part[(long long)b * E + e];
+    red[warp][lane] = v;
+    __syncthreads();
+    if (warp == 0 && e < E) {
+        v = 0.f;
+        for (int w = 0; w < 8; ++w) v += red[w][lane];
+        for (int s = 0; s < sg.n; ++s)
+            if (e >= sg.off[s] && e < sg.off[s] + sg.len[s]) sg.dst[s][e - sg.off[s]] = v;
+    }
+}
+
+template <typename F>
+void with_modes(int m, F f) {
+    switch (modes_pad(m)) {
+        case 4: f(std::integral_constant<int, 4>{}); break;
+        case 8: f(std::integral_constant<int, 8>{}); break;
+        case 12: f(std::integral_constant<int, 12>{}); break;
+        default: f(std::integral_constant<int, 16>{}); break;
+    }
+}
+
+// warps of a row block: as many rows as its shared memory holds
+int row_warps(const FnoFusedDims& d, int most) {
+    const RowSmem L = row_smem(d.nx, chan_pad(d.C), modes_pad(d.m));
+    const int w = (kSmemMax / 4 - L.warp) / L.perwarp;
+    return w > most ? most : w;
+}
+
+cudaError_t row_launch(const FnoFusedDims& d, RowArgs& a, bool bwd, cudaStream_t s) {
+    a.nx = d.nx;
+    a.C = d.C;
+    a.m = d.m;
+    a.N = d.N;
+    a.rows = (long long)d.nz * d.ny;
+    const int CP = chan_pad(d.C), nw = row_warps(d, bwd ? 12 : 16);
+    const RowSmem L = row_smem(d.nx, CP, modes_pad(d.m));
+    const int sm = (L.warp + nw * L.perwarp) * 4;
+    long long grid = (a.rows + nw - 1) / nw;
+    if (grid > kSMs) grid = kSMs;
+    cudaError_t e = cudaSuccess;
+    with_modes(d.m, [&](auto M) {
+        constexpr int MP = decltype(M)::value;
+        auto k = bwd ? (CP == 16 ? k_fno_row_bwd<16, MP> : k_fno_row_bwd<32, MP>)
+                     : (CP == 16 ? k_fno_row<16, MP> : k_fno_row<32, MP>);
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        if (e == cudaSuccess) k<<<(int)grid, 32 * nw, sm, s>>>(a);
+    });
+    return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
+template <bool TRAIN>
+cudaError_t project_launch(const FnoFusedDims& d, ProjArgs& p, int* blocks, cudaStream_t s) {
+    p.C = d.C;
+    p.H = d.H;
+    p.N = d.N;
+    p.sc = 2.0f / (float)(4 * d.N);
+    const long long tiles = (d.N + kPts - 1) / kPts;
+    cudaError_t e = cudaSuccess;
+    auto go = [&](auto cp, auto nwc) {
+        constexpr int CP = decltype(cp)::value, NW = decltype(nwc)::value;
+        constexpr int sm = proj_smem<CP, NW, TRAIN>();
+        auto k = k_fno_project<CP, NW, TRAIN>;
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        if (e != cudaSuccess) return;
+        const int per = 2;  // 83 KB a block at C = 32, H = 128
+        const long long grid = tiles < per * kSMs ? tiles : per * kSMs;
+        if (blocks) *blocks = (int)grid;
+        k<<<(int)grid, 32 * NW, sm, s>>>(p);
+    };
+    using I16 = std::integral_constant<int, 16>;
+    using I32 = std::integral_constant<int, 32>;
+    using I4 = std::integral_constant<int, 4>;
+    using I8 = std::integral_constant<int, 8>;
+    if (chan_pad(d.C) == 16)
+        d.H <= 64 ? go(I16{}, I4{}) : go(I16{}, I8{});
+    else
+        d.H <= 64 ? go(I32{}, I4{}) : go(I32{}, I8{});
+    return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
+void dft_fwd(const float2* in, float2* out, const float2* tab, int J, int m, int I, int O, cudaStream_t s) {
+    with_modes(m, [&](auto M) {
+        constexpr int MP = decltype(M)::value;
+        const size_t sm = (size_t)(J / 2 + 1) * (MP + 2) * sizeof(float2);
+        if (sm > 48 * 1024)
+            cudaFuncSetAttribute(k_dft_modes<MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        k_dft_modes<MP><<<dim3((I + 63) / 64, O), 64, sm, s>>>(in, out, tab, J, m, I);
+    });
+}
+void dft_inv(const float2* in, float2* out, const float2* tab, int J, int m, int I, int O, cudaStream_t s) {
+    with_modes(m, [&](auto M) {
+        constexpr int MP = decltype(M)::value;
+        // parts of the positions: about eight resident blocks an SM
+        const long long blocks = (long long)((I + 63) / 64) * O;
+        int parts = (int)((8 * kSMs + blocks - 1) / blocks);
+        const int half = J / 2 + 1;
+        if (parts > (half + 7) / 8) parts = (half + 7) / 8;
+        if (parts < 1) parts = 1;
+        const size_t sm = (size_t)((half + parts - 1) / parts) * (MP + 2) * sizeof(float2);
+        if (sm > 48 * 1024)
+            cudaFuncSetAttribute(k_dft_modes_inv<MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        k_dft_modes_inv<MP><<<dim3((I + 63) / 64, O, parts), 64, sm, s>>>(in, out, tab, J, m, I);
+    });
+}
+
+}  // namespace
+
+// The rule: one warp row of every channel has to fit a warp's share of shared
+// memory (C <= 32, rows of 32 to 256 points), a lane group's registers cover
+// the modes (m <= 16) and the projection's row tiles the hidden width (H <= 128).
+// Shorter rows leave most lanes of a warp idle; longer ones few warps an SM.
+// With an odd C the spectral weights are not aligned to (re, im) pairs.
+bool fno_fused_ok(const FnoFusedDims& d) {
+    return d.C <= 32 && d.C % 2 == 0 && d.H <= 128 && d.m <= kMaxModes && d.nx >= 32 && d.nx <= kMaxRow && d.nz <= 65535;
+}
+
+size_t fno_fused_xtab_len(const FnoFusedDims& d) { return (size_t)modes_pad(d.m) * half_pad(d.nx); }
+
+void fno_fused_tables(const FnoFusedDims& d, float* xc, float* xs, float* xcw, float* xsw, float2* y, float2* z) {
+    const double tp = 6.283185307179586476925286766559;
+    const int HP = half_pad(d.nx);
+    for (int k = 0; k < modes_pad(d.m); ++k)
+        for (int x = 0; x < HP; ++x) {
+            const bool in = k < d.m && x <= d.nx / 2;
+            const double th = tp * (double)((long long)k * x % d.nx) / d.nx, w = (k == 0 ? 1.0 : 2.0) / (double)d.N;
+            const double c = in ? std::cos(th) : 0.0, s = in ? std::sin(th) : 0.0;
+            xc[k * HP + x] = (float)c;
+            xs[k * HP + x] = (float)s;
+            xcw[k * HP + x] = (float)(c * w);
+            xsw[k * HP + x] = (float)(s * w);
+        }
+    auto axis = [&](int n, float2* o) {
+        for (int j = 0; j <= n / 2; ++j)
+            for (int k = 0; k <= d.m; ++k) {
+                const double th = tp * (double)((long long)k * j % n) / n;
+                o[j * (d.m + 1) + k] = make_float2((float)std::cos(th), (float)std::sin(th));
+            }
+    };
+    axis(d.ny, y);
+    axis(d.nz, z);
+}
+
+size_t fno_fused_part_len(const FnoFusedDims& d) {
+    const size_t a = (size_t)kSMs * row_part_len(d.C), b = (size_t)2 * kSMs * proj_part_len(d.C, d.H);
+    return a > b ? a : b;
+}
+
+cudaError_t fno_spectral_fwd(const FnoFusedDims& d, const FnoTables& t, const FnoWork& w, float2* A,
+                             const __nv_bfloat162* w16, cudaStream_t s) {
+    const int I = d.C * d.m, m2 = 2 * d.m;
+    dft_fwd(w.T1, w.T2, t.y, d.ny, d.m, I, d.nz, s);
+    dft_fwd(w.T2, A, t.z, d.nz, d.m, m2 * I, 1, s);
+    const size_t sm = 2 * (size_t)I * sizeof(float2);
+    if (d.C % 4 == 0)
+        k_mix_modes<true><<<m2 * m2, 256, sm, s>>>(A, w.Ok, w16, d.C, d.m);
+    else
+        k_mix_modes<false><<<m2 * m2, 256, sm, s>>>(A, w.Ok, w16, d.C, d.m);
+    dft_inv(w.Ok, w.T2, t.z, d.nz, d.m, m2 * I, 1, s);
+    dft_inv(w.T2, w.T1, t.y, d.ny, d.m, I, d.nz, s);
+    return cudaGetLastError();
+}
+
+cudaError_t fno_spectral_bwd(const FnoFusedDims& d, const FnoTables& t, const FnoWork& w, const float2* A,
+                             const __nv_bfloat162* w16, float2* GW, cudaStream_t s) {
+    const int I = d.C * d.m, m2 = 2 * d.m;
+    dft_fwd(w.T1, w.T2, t.y, d.ny, d.m, I, d.nz, s);
+    dft_fwd(w.T2, w.Gk, t.z, d.nz, d.m, m2 * I, 1, s);
+    k_mix_modes_bwd<<<m2 * m2, 256, 3 * (size_t)I * sizeof(float2), s>>>(w.Gk, A, w.Ok, GW, w16, d.C, d.m);
+    dft_inv(w.Ok, w.T2, t.z, d.nz, d.m, m2 * I, 1, s);
+    dft_inv(w.T2, w.T1, t.y, d.ny, d.m, I, d.nz, s);
+    return cudaGetLastError();
+}
+
+cudaError_t fno_row_lift(const FnoFusedDims& d, const FnoTables& t, const FnoWork& w, const float* x, const float* P,
+                         const float* p, cudaStream_t s) {
+    RowArgs a{};
+    a.x = x;
+    a.P = P;
+    a.pb = p;
+    a.T1 = w.T1;
+    a.fc = a.ic = t.xc;
+    a.fs = a.is = t.xs;
+    return row_launch(d, a, false, s);
+}
+
+cudaError_t fno_row_raw(const FnoFusedDims& d, const FnoTables& t, const FnoWork& w, const float* g, cudaStream_t s) {
+    RowArgs a{};
+    a.zprev = g;
+    a.raw = 1;
+    a.T1 = w.T1;
+    a.fc = a.ic = t.xcw;
+    a.fs = a.is = t.xsw;
+    return row_launch(d, a, false, s);
+}
+
+cudaError_t fno_row_layer(const FnoFusedDims& d, const FnoTables& t, const FnoWork& w, const float* zprev,
+                          const float* x, const float* P, const float* p, const float* V, const float* v, float* z,
+                          bool last, cudaStream_t s) {
+    RowArgs a{};
+    a.zprev = zprev;
+    a.x = x;
+    a.P = P;
+    a.pb = p;
+    a.V = V;
+    a.vb = v;
+    a.T1 = w.T1;
+    a.z = z;
+    a.fc = t.xc;
+    a.fs = t.xs;
+    a.ic = t.xcw;
+    a.is = t.xsw;
+    a.dense = 1;
+    a.last = last ? 1 : 0;
+    return row_launch(d, a, false, s);
+}
+
+cudaError_t fno_row_layer_bwd(const FnoFusedDims& d, const FnoTables& t, const FnoWork& w, float* dz,
+                              const float* zprev, const float* x, const float* P, const float* p, const float* V,
+                              float* gV, float* gv, float* gP, float* gp, cudaStream_t s) {
+    RowArgs a{};
+    a.zprev = zprev;
+    a.x = x;
+    a.P = P;
+    a.pb = p;
+    a.V = V;
+    a.T1 = w.T1;
+    a.z = dz;
+    a.fc = t.xcw;
+    a.fs = t.xsw;
+    a.ic = t.xc;
+    a.is = t.xs;
+    a.part = w.part;
+    cudaError_t e = row_launch(d, a, true, s);
+    if (e != cudaSuccess) return e;
+    const int C = d.C, nw = row_warps(d, 12);
+    const long long nb = (a.rows + nw - 1) / nw;
+    SumSeg sg{{0, C * C, C * C + C, C * C + 5 * C}, {C * C, C, 4 * C, C}, {gV, gv, gP, gp}, zprev ? 2 : 4};
+    const int E = row_part_len(C);
+    k_part_sum<<<(E + 31) / 32, 256, 0, s>>>(w.part, (int)(nb < kSMs ? nb : kSMs), E, sg);
+    return cudaGetLastError();
+}
+
+cudaError_t fno_project(const FnoFusedDims& d, const float* a, const float* Q1, const float* q1, const float* Q2,
+                        const float* q2, float* out, cudaStream_t s) {
+    ProjArgs p{};
+    p.a = a;
+    p.Q1 = Q1;
+    p.q1 = q1;
+    p.Q2 = Q2;
+    p.q2 = q2;
+    p.out = out;
+    return project_launch<false>(d, p, nullptr, s);
+}
+
+cudaError_t fno_project_bwd(const FnoFusedDims& d, const FnoWork& w, const float* a, const float* tgt,
+                            const float* Q1, const float* q1, const float* Q2, const float* q2, float* da, float* gQ1,
+                            float* gq1, float* gQ2, float* gq2, int* blocks, cudaStream_t s) {
+    ProjArgs p{};
+    p.a = a;
+    p.tgt = tgt;
+    p.Q1 = Q1;
+    p.q1 = q1;
+    p.Q2 = Q2;
+    p.q2 = q2;
+    p.da = da;
+    p.part = w.part;
+    p.dpart = w.dpart;
+    cudaError_t e = project_launch<true>(d, p, blocks, s);
+    if (e != cudaSuccess) return e;
+    const int C = d.C, H = d.H, E = proj_part_len(C, H);
+    SumSeg sg{{0, H * C, H * C + H, H * C + 5 * H}, {H * C, H, 4 * H, 4}, {gQ1, gq1, gQ2, gq2}, 4};
+    k_part_sum<<<(E + 31) / 32, 256, 0, s>>>(w.part, *blocks, E, sg);
+    return cudaGetLastError();
+}
+
+}  // namespace pf

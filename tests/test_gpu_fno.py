@@ -77,6 +77,57 @@ def test_forward_and_gradients_vs_oracle(pfg, bf16, tol_out, tol_g):
         net.close()
 
 
+# the fused layers' edges: the shortest and longest rows, odd rows and sides, padded channels, modes and hidden widths,
+# one mode, one layer, modes up to the Nyquist plane of an axis
+@pytest.mark.parametrize("shape,dims", [
+    ((8, 6, 32), dict(C=32, modes=3, H=128, L=2)),
+    ((18, 19, 36), dict(C=4, modes=9, H=128, L=2)),
+    ((9, 11, 33), dict(C=18, modes=4, H=100, L=2)),
+    ((4, 4, 256), dict(C=8, modes=1, H=16, L=2)),
+    ((26, 27, 63), dict(C=2, modes=13, H=64, L=1)),
+    ((8, 9, 150), dict(C=30, modes=4, H=65, L=2)),
+    ((7, 9, 40), dict(C=5, modes=3, H=20, L=2)),  # odd channel counts run the unfused kernels
+])
+def test_fused_layers_vs_oracle(pfg, shape, dims):
+    """Spectral weights that BF16 holds exactly, so that only the products' split (about 2^-16 relative for each of the
+    contractions in a row: at most 2 L + 3 of them forward and as many back) and FP32 rounding separate the two."""
+    import torch
+    d = ofno.Dims(shape, C=dims["C"], m=dims["modes"], H=dims["H"], L=dims["L"])
+    theta = ofno.init_params(d, 7).astype(np.float32)
+    P = ofno.unpack(d, theta)
+    for l in range(d.L):
+        w = torch.from_numpy(P["W%d" % l] * np.float32(20.0))
+        P["W%d" % l][...] = w.bfloat16().float().numpy()
+    rng = np.random.default_rng(3)
+    x, tgt = rng.standard_normal((4,) + shape), rng.standard_normal((4,) + shape) * 0.1
+    x, tgt = x.astype(np.float32).astype(np.float64), tgt.astype(np.float32).astype(np.float64)
+    out_ref, acts = ofno.forward(d, theta.astype(np.float64), x, cache=True)
+    g_ref = ofno.backward(d, theta.astype(np.float64), acts, out_ref, tgt)
+    net = pfg.FNO(shape, bf16=True, **dims)
+    try:
+        net.set_params(theta)
+        xt, tt = torch.from_numpy(x.astype(np.float32)).cuda(), torch.from_numpy(tgt.astype(np.float32)).cuda()
+        bound = (2 * d.L + 3) * 2.0 ** -16
+        out = net.forward(xt).cpu().numpy()
+        assert np.linalg.norm(out - out_ref) <= bound * np.linalg.norm(out_ref)
+        loss = net.backward(tt)
+        assert loss == pytest.approx(ofno.loss(out_ref, tgt), rel=bound)
+        o, bad = 0, {}
+        got = net.grads().astype(np.float64)
+        for name, s in ofno.layout(d):
+            k = int(np.prod(s))
+            e = np.linalg.norm(got[o:o + k] - g_ref[o:o + k]) / max(np.linalg.norm(g_ref[o:o + k]), 1e-30)
+            if not e <= 2 * bound:
+                bad[name] = e
+            o += k
+        assert not bad, bad
+        # a training step leaves the same gradients without computing the output
+        assert net.train_step(xt, tt, 0.0) == loss
+        assert np.array_equal(net.grads().astype(np.float64), got)
+    finally:
+        net.close()
+
+
 def test_adam_training_reduces_loss(pfg):
     import torch
     d = odims()
