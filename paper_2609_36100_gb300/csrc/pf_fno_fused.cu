@@ -29,7 +29,7 @@ constexpr int kSMs = 152;
 constexpr int kSmemMax = 227 * 1024;
 constexpr int kMaxModes = 16;  // x modes a lane group of the row kernels covers
 constexpr int kMaxRow = 256;   // points of a row
-constexpr int kFoldIter = (kMaxRow / 2 + 4 + 31) / 32;
+constexpr int kFoldIter = (kMaxRow / 2 + 31) / 32;
 
 __host__ __device__ inline int up(int a, int b) { return (a + b - 1) / b * b; }
 // padded half row, row pitch (16-byte units odd: rows 0..7 fall on different
@@ -58,6 +58,7 @@ struct RowArgs {
     int dense;  // forward: the layer (else only the x transform)
     int raw;    // zprev is taken as it is
     int last;   // forward: no x transform afterwards
+    int vec;    // rows of the [C][N] arrays start on 16-byte boundaries
     long long N, rows;
 };
 
@@ -132,19 +133,48 @@ __device__ __forceinline__ void row_setup(const RowArgs& a, float* sm, const Row
     for (int e = L.warp + threadIdx.x; e < L.warp + (int)(blockDim.x >> 5) * L.perwarp; e += blockDim.x) sm[e] = 0.f;
 }
 
+// asynchronous global -> shared copies: a warp has a whole row in flight
+// without holding it in registers (loaded through registers, 8 channels at a
+// time, a row cost 16 trips to memory one after another)
+__device__ __forceinline__ void cp4(float* dst, const float* src, bool valid) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp16(float* dst, const float* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // the row's retained x modes: T1 -> [kx][channel], channels of a lane adjacent
+// (zeros at the padded ones)
 template <int CP, int MP>
 __device__ __forceinline__ void row_load_modes(const RowArgs& a, long long row, float* T) {
     constexpr int CPL = CP / 8, TS = CP + 4;
-    const float2* src = a.T1 + row * a.C * a.m;
+    const float* src = reinterpret_cast<const float*>(a.T1 + row * a.C * a.m);
     const int lane = threadIdx.x & 31;
 #pragma unroll 4
     for (int e = lane; e < MP * CP; e += 32) {
         const int c = e / MP, k = e - c * MP;
-        const float2 t = c < a.C && k < a.m ? src[c * a.m + k] : make_float2(0.f, 0.f);
+        const bool in = c < a.C && k < a.m;
+        const float* t = src + (in ? 2 * (c * a.m + k) : 0);
         const int o = k * TS + (c & 7) * CPL + (c >> 3);
-        T[o] = t.x;
-        T[MP * TS + o] = t.y;
+        cp4(T + o, t, in);
+        cp4(T + MP * TS + o, t + 1, in);
+    }
+}
+
+// a row of C channels of src [C][N] into A
+__device__ __forceinline__ void row_load(const RowArgs& a, const float* src, long long r0, float* A, int RS) {
+    const int lane = threadIdx.x & 31;
+    if (a.vec) {  // rows start on 16-byte boundaries
+        for (int x = 4 * lane; x < a.nx; x += 128)
+#pragma unroll 8
+            for (int c = 0; c < a.C; ++c) cp16(A + c * RS + x, src + (long long)c * a.N + r0 + x);
+    } else {
+        for (int x = lane; x < a.nx; x += 32)
+#pragma unroll 8
+            for (int c = 0; c < a.C; ++c) cp4(A + c * RS + x, src + (long long)c * a.N + r0 + x, true);
     }
 }
 
@@ -163,24 +193,33 @@ __device__ __forceinline__ void row_dense(float* A, int RS, int nx, const unsign
             ah[i][j][0] = h.x, ah[i][j][1] = h.y, ah[i][j][2] = h.z, ah[i][j][3] = h.w;
             al[i][j][0] = l.x, al[i][j][1] = l.y, al[i][j][2] = l.z, al[i][j][3] = l.w;
         }
-    for (int n0 = 0; n0 < nx; n0 += 8) {
-        float acc[T][4] = {};
+    // two column tiles at a time: their chains of products overlap
+    for (int n0 = 0; n0 < nx; n0 += 16) {
+        const bool two = n0 + 8 < nx;
+        float acc[2][T][4] = {};
 #pragma unroll
-        for (int j = 0; j < T; ++j) {
-            const float* b = A + (j * 16 + 2 * t) * RS + n0 + g;
-            unsigned bh0, bl0, bh1, bl1;
-            split2(b[0], b[RS], bh0, bl0);
-            split2(b[8 * RS], b[9 * RS], bh1, bl1);
+        for (int u = 0; u < 2; ++u) {
+            const float* col = A + n0 + (u && two ? 8 : 0) + g;
 #pragma unroll
-            for (int i = 0; i < T; ++i) mma3(acc[i], ah[i][j], al[i][j], bh0, bh1, bl0, bl1);
+            for (int j = 0; j < T; ++j) {
+                const float* b = col + (j * 16 + 2 * t) * RS;
+                unsigned bh0, bl0, bh1, bl1;
+                split2(b[0], b[RS], bh0, bl0);
+                split2(b[8 * RS], b[9 * RS], bh1, bl1);
+#pragma unroll
+                for (int i = 0; i < T; ++i) mma3(acc[u][i], ah[i][j], al[i][j], bh0, bh1, bl0, bl1);
+            }
         }
         __syncwarp();
 #pragma unroll
-        for (int i = 0; i < T; ++i) {
-            float* o = A + (i * 16 + g) * RS + n0 + 2 * t;
-            *reinterpret_cast<float2*>(o) = make_float2(acc[i][0], acc[i][1]);
-            *reinterpret_cast<float2*>(o + 8 * RS) = make_float2(acc[i][2], acc[i][3]);
-        }
+        for (int u = 0; u < 2; ++u)
+            if (u == 0 || two)
+#pragma unroll
+                for (int i = 0; i < T; ++i) {
+                    float* o = A + (i * 16 + g) * RS + n0 + 8 * u + 2 * t;
+                    *reinterpret_cast<float2*>(o) = make_float2(acc[u][i][0], acc[u][i][1]);
+                    *reinterpret_cast<float2*>(o + 8 * RS) = make_float2(acc[u][i][2], acc[u][i][3]);
+                }
         __syncwarp();
     }
 }
@@ -275,37 +314,58 @@ __device__ __forceinline__ void row_forward(const RowArgs& a, long long row, con
     __syncwarp();
 }
 
-// in place: a row's values -> sums and differences under x -> n - x, through
-// val(channel, x, value) (which may store and change the value)
-template <class F>
-__device__ __forceinline__ void row_fold(float* A, int RS, int nx, int C, F val) {
-    const int lane = threadIdx.x & 31, HP = half_pad(nx), Hx = nx / 2 + 1;
-#pragma unroll 2
-    for (int c = 0; c < C; ++c) {
-        float* r = A + c * RS;
-        float e[kFoldIter], o[kFoldIter];
+// in place: a row's values -> sums and differences under x -> n - x, after
+// val(channel, x, value, pre(channel, x)).  The two positions that are their
+// own mirrors, 0 and n/2, share a lane.  CB channels at a time: first every
+// pre (a load, say), then the values.
+template <int CB, class G, class F>
+__device__ __forceinline__ void row_fold(float* A, int RS, int nx, int C, G pre, F val) {
+    const int lane = threadIdx.x & 31, HP = half_pad(nx), Hx = nx / 2 + 1, XL = (nx + 1) / 2;
+    const bool even = (nx & 1) == 0;
+    for (int c0 = 0; c0 < C; c0 += CB) {
+        float v[CB][kFoldIter], u[CB][kFoldIter];
+        using P = decltype(pre(0, 0));
+        P pv[CB][kFoldIter], pu[CB][kFoldIter];
 #pragma unroll
-        for (int q = 0; q < kFoldIter; ++q) {
-            const int x = lane + 32 * q;
-            e[q] = o[q] = 0.f;
-            if (x < Hx) {
-                const float v = val(c, x, r[x]);
-                e[q] = v;
-                if (x > 0 && 2 * x != nx) {
-                    const float u = val(c, nx - x, r[nx - x]);
-                    e[q] = v + u;
-                    o[q] = v - u;
+        for (int b = 0; b < CB; ++b)
+#pragma unroll
+            for (int q = 0; q < kFoldIter; ++q) {
+                const int x = lane + 32 * q, y = x ? nx - x : nx / 2;
+                if (c0 + b < C && x < XL) {
+                    pv[b][q] = pre(c0 + b, x);
+                    if (x || even) pu[b][q] = pre(c0 + b, y);
                 }
             }
-        }
+#pragma unroll
+        for (int b = 0; b < CB; ++b)
+#pragma unroll
+            for (int q = 0; q < kFoldIter; ++q) {
+                const int x = lane + 32 * q, y = x ? nx - x : nx / 2;
+                v[b][q] = u[b][q] = 0.f;
+                if (c0 + b < C && x < XL) {
+                    const float* r = A + (c0 + b) * RS;
+                    v[b][q] = val(c0 + b, x, r[x], pv[b][q]);
+                    if (x || even) u[b][q] = val(c0 + b, y, r[y], pu[b][q]);
+                }
+            }
         __syncwarp();
 #pragma unroll
-        for (int q = 0; q < kFoldIter; ++q) {
-            const int x = lane + 32 * q;
-            if (x < HP) {
-                r[x] = e[q];
-                r[HP + x] = o[q];
+        for (int b = 0; b < CB; ++b) {
+            if (c0 + b >= C) break;
+            float* r = A + (c0 + b) * RS;
+#pragma unroll
+            for (int q = 0; q < kFoldIter; ++q) {
+                const int x = lane + 32 * q;
+                if (x < XL) {
+                    r[x] = x ? v[b][q] + u[b][q] : v[b][q];
+                    r[HP + x] = x ? v[b][q] - u[b][q] : 0.f;
+                    if (x == 0 && even) {
+                        r[nx / 2] = u[b][q];
+                        r[HP + nx / 2] = 0.f;
+                    }
+                }
             }
+            if (lane < HP - Hx) r[Hx + lane] = r[HP + Hx + lane] = 0.f;
         }
     }
     __syncwarp();
@@ -325,6 +385,60 @@ __device__ __forceinline__ void row_lift(const RowArgs& a, long long r0, float* 
     }
 }
 
+// T1 of the lifted input: the x transform of the four input fields, then
+// P X + p (whose transform is p nx at kx = 0), a warp per row
+template <int MP>
+__global__ void __launch_bounds__(256) k_fno_lift_modes(RowArgs a) {
+    extern __shared__ __align__(16) float sm[];
+    const int HP = half_pad(a.nx), RS = row_pitch(a.nx), nx = a.nx;
+    float *tc = sm, *ts = tc + MP * HP, *lift = ts + MP * HP;  // lift: [32][4] P, [32] p
+    for (int e = threadIdx.x; e < MP * HP; e += blockDim.x) {
+        tc[e] = a.fc[e];
+        ts[e] = a.fs[e];
+    }
+    for (int e = threadIdx.x; e < 32; e += blockDim.x) {
+#pragma unroll
+        for (int f = 0; f < 4; ++f) lift[4 * e + f] = e < a.C ? a.P[e * 4 + f] : 0.f;
+        lift[128 + e] = e < a.C ? a.pb[e] * (float)nx : 0.f;
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    float* A = lift + 160 + warp * (4 * RS + 8 * MP);
+    float2* X = reinterpret_cast<float2*>(A + 4 * RS);  // [4][MP]
+    for (long long row = blockIdx.x * (long long)nw + warp; row < a.rows; row += (long long)gridDim.x * nw) {
+        for (int x = lane; x < nx; x += 32)
+#pragma unroll
+            for (int f = 0; f < 4; ++f) cp4(A + f * RS + x, a.x + f * a.N + row * nx + x, true);
+        cp_wait();
+        __syncwarp();
+        row_fold<4>(
+            A, RS, nx, 4, [](int, int) { return 0; }, [](int, int, float v, int) { return v; });
+        const int f = lane & 3;
+        for (int k = lane >> 2; k < a.m; k += 8) {
+            float re = 0.f, im = 0.f;
+            for (int x = 0; x < HP; x += 4) {
+                const float4 c = *reinterpret_cast<const float4*>(tc + k * HP + x);
+                const float4 s = *reinterpret_cast<const float4*>(ts + k * HP + x);
+                const float4 e = *reinterpret_cast<const float4*>(A + f * RS + x);
+                const float4 o = *reinterpret_cast<const float4*>(A + f * RS + HP + x);
+                re = fmaf(e.w, c.w, fmaf(e.z, c.z, fmaf(e.y, c.y, fmaf(e.x, c.x, re))));
+                im = fmaf(o.w, s.w, fmaf(o.z, s.z, fmaf(o.y, s.y, fmaf(o.x, s.x, im))));
+            }
+            X[f * MP + k] = make_float2(re, -im);
+        }
+        __syncwarp();
+        float2* dst = a.T1 + row * a.C * a.m;
+        for (int e = lane; e < a.C * a.m; e += 32) {
+            const int c = e / a.m, k = e - c * a.m;
+            const float4 w = *reinterpret_cast<const float4*>(lift + 4 * c);
+            const float2 x0 = X[k], x1 = X[MP + k], x2 = X[2 * MP + k], x3 = X[3 * MP + k];
+            dst[e] = make_float2(fmaf(w.w, x3.x, fmaf(w.z, x2.x, fmaf(w.y, x1.x, fmaf(w.x, x0.x, k ? 0.f : lift[128 + c])))),
+                                 fmaf(w.w, x3.y, fmaf(w.z, x2.y, fmaf(w.y, x1.y, w.x * x0.y))));
+        }
+        __syncwarp();
+    }
+}
+
 template <int CP, int MP>
 __global__ void __launch_bounds__(512, 1) k_fno_row(RowArgs a) {
     extern __shared__ __align__(16) float sm[];
@@ -338,17 +452,15 @@ __global__ void __launch_bounds__(512, 1) k_fno_row(RowArgs a) {
     for (long long row = blockIdx.x * (long long)nw + warp; row < a.rows; row += (long long)gridDim.x * nw) {
         const long long r0 = row * nx;
         if (a.dense) row_load_modes<CP, MP>(a, row, T);
+        if (a.zprev) row_load(a, a.zprev, r0, A, RS);
+        cp_wait();
+        __syncwarp();
         if (!a.zprev) {
             row_lift<CP>(a, r0, A, RS, sm + L.lift);
-        } else {
-            for (int x = lane; x < nx; x += 32) {
-                const float* src = a.zprev + r0 + x;
+        } else if (!a.raw) {
+            for (int x = lane; x < nx; x += 32)
 #pragma unroll 8
-                for (int c = 0; c < C; ++c) {
-                    const float v = src[(long long)c * a.N];
-                    A[c * RS + x] = a.raw ? v : gelu_f(v);
-                }
-            }
+                for (int c = 0; c < C; ++c) A[c * RS + x] = gelu_f(A[c * RS + x]);
         }
         __syncwarp();
         if (a.dense) {
@@ -364,12 +476,15 @@ __global__ void __launch_bounds__(512, 1) k_fno_row(RowArgs a) {
             continue;
         }
         if (a.dense) {
-            row_fold(A, RS, nx, C, [&](int c, int x, float v) {
-                a.z[(long long)c * a.N + r0 + x] = v;
-                return gelu_f(v);
-            });
+            row_fold<2>(
+                A, RS, nx, C, [](int, int) { return 0; },
+                [&](int c, int x, float v, int) {
+                    a.z[(long long)c * a.N + r0 + x] = v;
+                    return gelu_f(v);
+                });
         } else {
-            row_fold(A, RS, nx, C, [](int, int, float v) { return v; });
+            row_fold<2>(
+                A, RS, nx, C, [](int, int) { return 0; }, [](int, int, float v, int) { return v; });
         }
         row_forward<CP, MP>(a, row, A, RS, T, sm + L.tf, sm + L.tf + MP * HP);
     }
@@ -410,13 +525,16 @@ __global__ void __launch_bounds__(384, 1) k_fno_row_bwd(RowArgs a) {
     for (long long row = blockIdx.x * (long long)nw + warp; row < a.rows; row += (long long)gridDim.x * nw) {
         const long long r0 = row * nx;
         row_load_modes<CP, MP>(a, row, T);
-        for (int x = lane; x < nx; x += 32) {
-            const float* src = a.z + r0 + x;
-#pragma unroll 8
-            for (int c = 0; c < C; ++c) A[c * RS + x] = src[(long long)c * a.N];
-        }
+        row_load(a, a.z, r0, A, RS);
+        if (!first)  // the row of zprev on its way while dz arrives
+            for (int e = lane; e < C * ((nx + 31) / 32 + 1); e += 32) {
+                const int c = e % C, x = min(32 * (e / C), nx - 1);
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(a.zprev + (long long)c * a.N + r0 + x));
+            }
+        cp_wait();
         __syncwarp();
         // gradient of V: dz a^T over the row's points, a in fragments straight from global memory
+#pragma unroll 2
         for (int k0 = 0; k0 < nx; k0 += 16) {
             const int p = k0 + 2 * t;
             float av[NT][4];
@@ -485,12 +603,13 @@ __global__ void __launch_bounds__(384, 1) k_fno_row_bwd(RowArgs a) {
             __syncwarp();
             continue;
         }
-        row_fold(A, RS, nx, C, [&](int c, int x, float v) {
-            const long long i = (long long)c * a.N + r0 + x;
-            const float d = v * gelu_g(a.zprev[i]);
-            a.z[i] = d;
-            return d;
-        });
+        row_fold<4>(
+            A, RS, nx, C, [&](int c, int x) { return a.zprev[(long long)c * a.N + r0 + x]; },
+            [&](int c, int x, float v, float z) {
+                const float d = v * gelu_g(z);
+                a.z[(long long)c * a.N + r0 + x] = d;
+                return d;
+            });
         row_forward<CP, MP>(a, row, A, RS, T, sm + L.tf, sm + L.tf + MP * HP);
     }
     // warps -> block, in warp order
@@ -578,15 +697,17 @@ __global__ void __launch_bounds__(64) k_dft_modes(const float2* __restrict__ in,
     add(0, src[0], z);
     const int pairs = (J - 1) / 2;
     int j = 1;
-    for (; j + 3 <= pairs; j += 4) {
-        float2 a[4], b[4];
+    // eight pairs' loads in flight: a thread's trips to memory, not its
+    // products, set the time
+    for (; j + 7 <= pairs; j += 8) {
+        float2 a[8], b[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 8; ++u) {
             a[u] = src[(long long)(j + u) * I];
             b[u] = src[(long long)(J - j - u) * I];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < 8; ++u)
             add(j + u, make_float2(a[u].x + b[u].x, a[u].y + b[u].y), make_float2(a[u].x - b[u].x, a[u].y - b[u].y));
     }
     for (; j <= pairs; ++j) {
@@ -744,19 +865,24 @@ struct ProjArgs {
 template <int CP, int NW, bool TRAIN>
 constexpr int proj_smem() {
     constexpr int HP = 16 * NW, KT = CP / 16;
-    return (CP * kPS + HP * kPS + 4 * kPS + 5 * HP + 4 + NW * KT * 256 + (TRAIN ? NW * KT * 256 : 0)) * 4;
+    return (2 * CP * kPS + HP * kPS + 4 * kPS + NW * 128 + 4 * HP + HP + 4 + NW * KT * 256 +
+            (TRAIN ? NW * KT * 256 : 0)) * 4;
 }
 
+// The products of a tile run on the tensor cores; what bounds the kernel is
+// the error function of its H x 64 hidden values.  The next tile's columns of
+// a are copied in while this one is worked on.
 template <int CP, int NW, bool TRAIN>
-__global__ void __launch_bounds__(32 * NW, (CP == 32 && NW == 8 && TRAIN) ? 2 : 1) k_fno_project(ProjArgs p) {
+__global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
     constexpr int HP = 16 * NW, KT = CP / 16, NT = kPts / 8;
     extern __shared__ __align__(16) float sm[];
-    float* sa = sm;               // [CP][kPS]
-    float* sh = sa + CP * kPS;    // [HP][kPS]: h, then dh
-    float* sd = sh + HP * kPS;    // [4][kPS]: d out
-    float* sq2 = sd + 4 * kPS;    // [HP][4]
-    float* sq1 = sq2 + 4 * HP;    // [HP]
-    float* sb2 = sq1 + HP;        // [4]
+    float* sa0 = sm;                  // [2][CP][kPS]
+    float* sh = sa0 + 2 * CP * kPS;   // [HP][kPS]: h, then dh
+    float* sd = sh + HP * kPS;        // [4][kPS]: d out
+    uint4* w2 = reinterpret_cast<uint4*>(sd + 4 * kPS);  // Q2 fragments [NW][32]: rows 0..3, leading and remainder
+    float* sq2 = sd + 4 * kPS + NW * 128;  // [HP][4]
+    float* sq1 = sq2 + 4 * HP;             // [HP]
+    float* sb2 = sq1 + HP;                 // [4]
     unsigned* w1 = reinterpret_cast<unsigned*>(sb2 + 4);  // Q1 fragments [NW][KT]
     unsigned* wt = w1 + NW * KT * 256;                    // Q1^T fragments [KT][NW]
     const int C = p.C, H = p.H;
@@ -776,42 +902,74 @@ __global__ void __launch_bounds__(32 * NW, (CP == 32 && NW == 8 && TRAIN) ? 2 : 
             }
         }
     }
+    for (int e = threadIdx.x; e < NW * 32; e += blockDim.x) {
+        const int g = (e & 31) >> 2, h = (e >> 5) * 16 + 2 * (e & 3);
+        auto v = [&](int hh) -> float { return g < 4 && hh < H ? p.Q2[g * H + hh] : 0.f; };
+        uint4 w;
+        split2(v(h), v(h + 1), w.x, w.z);
+        split2(v(h + 8), v(h + 9), w.y, w.w);
+        w2[e] = w;
+    }
     for (int e = threadIdx.x; e < HP; e += blockDim.x) {
 #pragma unroll
         for (int f = 0; f < 4; ++f) sq2[4 * e + f] = e < H ? p.Q2[f * H + e] : 0.f;
         sq1[e] = e < H ? p.q1[e] : 0.f;
     }
     if (threadIdx.x < 4) sb2[threadIdx.x] = p.q2[threadIdx.x];
-    for (int e = threadIdx.x; e < CP * kPS; e += blockDim.x) sa[e] = 0.f;
+    for (int e = threadIdx.x; e < 2 * CP * kPS; e += blockDim.x) sa0[e] = 0.f;
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const long long tiles = (p.N + kPts - 1) / kPts;
+    auto load = [&](long long tile, float* dst) {
+        const long long p0 = tile * kPts;
+        if (p.N % 4 == 0 && p0 + kPts <= p.N) {
+            for (int e = threadIdx.x; e < C * (kPts / 4); e += blockDim.x) {
+                const int c = e / (kPts / 4), q = 4 * (e % (kPts / 4));
+                cp16(dst + c * kPS + q, p.a + (long long)c * p.N + p0 + q);
+            }
+        } else {
+            for (int e = threadIdx.x; e < C * kPts; e += blockDim.x) {
+                const int c = e / kPts, q = e % kPts;
+                const bool in = p0 + q < p.N;
+                cp4(dst + c * kPS + q, p.a + (long long)c * p.N + (in ? p0 + q : 0), in);
+            }
+        }
+    };
     // gradients kept over the block's tiles
     float gQ1[CP / 8][4] = {}, gq1[2] = {}, gQ2[4] = {};
     float gq2 = 0.f;
     double loss = 0.0;
-    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int h0 = warp * 16;
+    int cur = 0;
+    if (blockIdx.x < tiles) load(blockIdx.x, sa0);
+    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x, cur ^= 1) {
         const long long p0 = tile * kPts;
         const int np = (int)min((long long)kPts, p.N - p0);
-#pragma unroll 4
-        for (int e = threadIdx.x; e < C * kPts; e += blockDim.x) {
-            const int c = e / kPts, q = e - c * kPts;
-            sa[c * kPS + q] = q < np ? p.a[(long long)c * p.N + p0 + q] : 0.f;
-        }
+        const float* sa = sa0 + cur * CP * kPS;
+        cp_wait();
         __syncthreads();
+        if (tile + gridDim.x < tiles) load(tile + gridDim.x, sa0 + (cur ^ 1) * CP * kPS);
+        // this warp's targets: fields 0..3 on the first 16 lanes
+        float tg[TRAIN ? NT / NW + 1 : 1][2] = {};
+        if constexpr (TRAIN) {
+#pragma unroll
+            for (int u = 0; u < NT / NW; ++u)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const int q = (warp + u * NW) * 8 + 2 * t + r;
+                    if (g < 4 && q < np) tg[u][r] = p.tgt[(long long)g * p.N + p0 + q];
+                }
+        }
         // h = GELU(Q1 a + q1) of this warp's rows; its derivative stays in registers
-        const int h0 = warp * 16;
         float gp[TRAIN ? NT : 1][4];
         {
             unsigned ah[KT][4], al[KT][4];
 #pragma unroll
             for (int k = 0; k < KT; ++k) {
-                const unsigned* w = w1 + (warp * KT + k) * 256 + lane * 4;
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    ah[k][r] = w[r];
-                    al[k][r] = w[128 + r];
-                }
+                const uint4 hv = *reinterpret_cast<const uint4*>(w1 + (warp * KT + k) * 256 + lane * 4);
+                const uint4 lv = *reinterpret_cast<const uint4*>(w1 + (warp * KT + k) * 256 + 128 + lane * 4);
+                ah[k][0] = hv.x, ah[k][1] = hv.y, ah[k][2] = hv.z, ah[k][3] = hv.w;
+                al[k][0] = lv.x, al[k][1] = lv.y, al[k][2] = lv.z, al[k][3] = lv.w;
             }
             const float b0 = sq1[h0 + g], b1 = sq1[h0 + g + 8];
 #pragma unroll
@@ -839,57 +997,66 @@ __global__ void __launch_bounds__(32 * NW, (CP == 32 && NW == 8 && TRAIN) ? 2 : 
             }
         }
         __syncthreads();
-        // out = Q2 h + q2, one (field, point) a thread at a time
-        for (int e = threadIdx.x; e < 4 * kPts; e += blockDim.x) {
-            const int f = e / kPts, q = e - f * kPts;
-            float v0 = sb2[f], v1 = 0.f, v2 = 0.f, v3 = 0.f;
-#pragma unroll 8
-            for (int h = 0; h < HP; h += 4) {
-                v0 = fmaf(sq2[4 * h + f], sh[h * kPS + q], v0);
-                v1 = fmaf(sq2[4 * h + 4 + f], sh[(h + 1) * kPS + q], v1);
-                v2 = fmaf(sq2[4 * h + 8 + f], sh[(h + 2) * kPS + q], v2);
-                v3 = fmaf(sq2[4 * h + 12 + f], sh[(h + 3) * kPS + q], v3);
-            }
-            const float v = (v0 + v1) + (v2 + v3);
-            if constexpr (TRAIN) {
-                float d = 0.f;
-                if (q < np) {
-                    d = v - p.tgt[(long long)f * p.N + p0 + q];
-                    loss += (double)d * d;
-                    d *= p.sc;
-                }
-                sd[f * kPS + q] = d;
-            } else if (q < np) {
-                p.out[(long long)f * p.N + p0 + q] = v;
-            }
-        }
-        __syncthreads();
-        if constexpr (TRAIN) {
-            // gradients of Q2 (four fields per row h, rows over the threads) and q2
-            {
-                constexpr int G = 32 * NW / HP;  // threads per row: 2, each two fields
-                const int h = threadIdx.x % HP, f0 = threadIdx.x / HP * (4 / G);
-                const float* hr = sh + h * kPS;
-#pragma unroll 4
-                for (int q = 0; q < kPts; q += 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(hr + q);
+        // out = Q2 h + q2, eight points a warp at a time
 #pragma unroll
-                    for (int u = 0; u < 4 / G; ++u) {
-                        const float4 d = *reinterpret_cast<const float4*>(sd + (f0 + u) * kPS + q);
-                        gQ2[u] = fmaf(v.w, d.w, fmaf(v.z, d.z, fmaf(v.y, d.y, fmaf(v.x, d.x, gQ2[u]))));
+        for (int u = 0; u < NT / NW; ++u) {
+            const int n = warp + u * NW;
+            const float b = g < 4 ? sb2[g] : 0.f;
+            float acc[2][4] = {{b, b, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+            for (int k = 0; k < NW; ++k) {
+                const float* hb = sh + (k * 16 + 2 * t) * kPS + n * 8 + g;
+                unsigned bh0, bl0, bh1, bl1;
+                split2(hb[0], hb[kPS], bh0, bl0);
+                split2(hb[8 * kPS], hb[9 * kPS], bh1, bl1);
+                const uint4 w = w2[k * 32 + lane];
+                const unsigned ah[4] = {w.x, 0u, w.y, 0u}, al[4] = {w.z, 0u, w.w, 0u};
+                mma3(acc[k & 1], ah, al, bh0, bh1, bl0, bl1);
+            }
+            if (g < 4) {
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const int q = n * 8 + 2 * t + r;
+                    const float v = acc[0][r] + acc[1][r];
+                    if constexpr (TRAIN) {
+                        float d = 0.f;
+                        if (q < np) {
+                            d = v - tg[u][r];
+                            loss += (double)d * d;
+                            d *= p.sc;
+                        }
+                        sd[g * kPS + q] = d;
+                        gq2 += d;
+                    } else if (q < np) {
+                        p.out[(long long)g * p.N + p0 + q] = v;
                     }
                 }
-                if (threadIdx.x < 4) {
-                    float s = 0.f;
-                    for (int q = 0; q < kPts; ++q) s += sd[threadIdx.x * kPS + q];
-                    gq2 += s;
-                }
             }
+        }
+        if constexpr (TRAIN) {
             __syncthreads();
+            // gradient of Q2 (transposed: rows h, columns the fields): h d out^T
+#pragma unroll
+            for (int k = 0; k < kPts / 16; ++k) {
+                unsigned ah[4], al[4], bh0, bl0, bh1, bl1;
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float2 u = *reinterpret_cast<const float2*>(sh + (h0 + g + ((r & 1) ? 8 : 0)) * kPS + k * 16 +
+                                                                      2 * t + ((r & 2) ? 8 : 0));
+                    split2(u.x, u.y, ah[r], al[r]);
+                }
+                const float* d = sd + (g & 3) * kPS + k * 16 + 2 * t;
+                float2 d0 = *reinterpret_cast<const float2*>(d), d1 = *reinterpret_cast<const float2*>(d + 8);
+                if (g >= 4) d0 = d1 = make_float2(0.f, 0.f);
+                split2(d0.x, d0.y, bh0, bl0);
+                split2(d1.x, d1.y, bh1, bl1);
+                mma3(gQ2, ah, al, bh0, bh1, bl0, bl1);
+            }
+            __syncwarp();
             // dh = GELU' (Q2^T d out) over h
             {
-                float4 qa = *reinterpret_cast<const float4*>(sq2 + 4 * (h0 + g));
-                float4 qb = *reinterpret_cast<const float4*>(sq2 + 4 * (h0 + g + 8));
+                const float4 qa = *reinterpret_cast<const float4*>(sq2 + 4 * (h0 + g));
+                const float4 qb = *reinterpret_cast<const float4*>(sq2 + 4 * (h0 + g + 8));
 #pragma unroll
                 for (int n = 0; n < NT; ++n) {
                     const float* d = sd + n * 8 + 2 * t;
@@ -929,7 +1096,9 @@ __global__ void __launch_bounds__(32 * NW, (CP == 32 && NW == 8 && TRAIN) ? 2 : 
                 }
             }
             // da = Q1^T dh, column tiles over the warps
-            for (int n = warp; n < NT; n += NW) {
+#pragma unroll
+            for (int v = 0; v < NT / NW; ++v) {
+                const int n = warp + v * NW;
                 float acc[KT][4] = {};
 #pragma unroll
                 for (int k = 0; k < NW; ++k) {
@@ -953,13 +1122,11 @@ __global__ void __launch_bounds__(32 * NW, (CP == 32 && NW == 8 && TRAIN) ? 2 : 
                         if (c < C && q < np) p.da[(long long)c * p.N + p0 + q] = acc[i][r];
                     }
             }
-            __syncthreads();
         }
     }
     if constexpr (TRAIN) {
         // block partials: [H C] Q1, [H] q1, [4 H] Q2, [4] q2; the loss in FP64
         float* o = p.part + (long long)blockIdx.x * proj_part_len(C, H);
-        const int h0 = warp * 16;
 #pragma unroll
         for (int j = 0; j < CP / 8; ++j)
 #pragma unroll
@@ -968,6 +1135,11 @@ __global__ void __launch_bounds__(32 * NW, (CP == 32 && NW == 8 && TRAIN) ? 2 : 
                 if (h < H && c < C) o[h * C + c] = gQ1[j][r];
             }
 #pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int h = h0 + g + ((r & 2) ? 8 : 0), f = 2 * t + (r & 1);
+            if (h < H && f < 4) o[H * C + H + f * H + h] = gQ2[r];
+        }
+#pragma unroll
         for (int r = 0; r < 2; ++r) {
             float v = gq1[r];
             v += __shfl_xor_sync(0xffffffffu, v, 1);
@@ -975,18 +1147,19 @@ __global__ void __launch_bounds__(32 * NW, (CP == 32 && NW == 8 && TRAIN) ? 2 : 
             const int h = h0 + g + 8 * r;
             if (t == 0 && h < H) o[H * C + h] = v;
         }
-        {
-            constexpr int G = 32 * NW / HP;
-            const int h = threadIdx.x % HP, f0 = threadIdx.x / HP * (4 / G);
-#pragma unroll
-            for (int u = 0; u < 4 / G; ++u)
-                if (h < H) o[H * C + H + (f0 + u) * H + h] = gQ2[u];
-        }
-        if (threadIdx.x < 4) o[H * C + 5 * H + threadIdx.x] = gq2;
         __shared__ double red[NW];
+        __shared__ float red2[NW][4];
+        gq2 += __shfl_xor_sync(0xffffffffu, gq2, 1);
+        gq2 += __shfl_xor_sync(0xffffffffu, gq2, 2);
+        if (t == 0 && g < 4) red2[warp][g] = gq2;
         for (int s = 16; s > 0; s >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, s);
         if (lane == 0) red[warp] = loss;
         __syncthreads();
+        if (threadIdx.x < 4) {
+            float v = 0.f;
+            for (int w = 0; w < NW; ++w) v += red2[w][threadIdx.x];
+            o[H * C + 5 * H + threadIdx.x] = v;
+        }
         if (threadIdx.x == 0) {
             double v = 0.0;
             for (int w = 0; w < NW; ++w) v += red[w];
@@ -1041,6 +1214,7 @@ cudaError_t row_launch(const FnoFusedDims& d, RowArgs& a, bool bwd, cudaStream_t
     a.m = d.m;
     a.N = d.N;
     a.rows = (long long)d.nz * d.ny;
+    a.vec = d.nx % 4 == 0 ? 1 : 0;  // N is then a multiple of 4 too; the arrays are the library's own
     const int CP = chan_pad(d.C), nw = row_warps(d, bwd ? 12 : 16);
     const RowSmem L = row_smem(d.nx, CP, modes_pad(d.m));
     const int sm = (L.warp + nw * L.perwarp) * 4;
@@ -1071,7 +1245,7 @@ cudaError_t project_launch(const FnoFusedDims& d, ProjArgs& p, int* blocks, cuda
         auto k = k_fno_project<CP, NW, TRAIN>;
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
         if (e != cudaSuccess) return;
-        const int per = 2;  // 83 KB a block at C = 32, H = 128
+        const int per = 2;  // 93 KB a block at C = 32, H = 128
         const long long grid = tiles < per * kSMs ? tiles : per * kSMs;
         if (blocks) *blocks = (int)grid;
         k<<<(int)grid, 32 * NW, sm, s>>>(p);
@@ -1187,9 +1361,23 @@ cudaError_t fno_row_lift(const FnoFusedDims& d, const FnoTables& t, const FnoWor
     a.P = P;
     a.pb = p;
     a.T1 = w.T1;
-    a.fc = a.ic = t.xc;
-    a.fs = a.is = t.xs;
-    return row_launch(d, a, false, s);
+    a.fc = t.xc;
+    a.fs = t.xs;
+    a.nx = d.nx;
+    a.C = d.C;
+    a.m = d.m;
+    a.N = d.N;
+    a.rows = (long long)d.nz * d.ny;
+    long long grid = (a.rows + 7) / 8;
+    if (grid > 4 * kSMs) grid = 4 * kSMs;
+    cudaError_t e = cudaSuccess;
+    with_modes(d.m, [&](auto M) {
+        constexpr int MP = decltype(M)::value;
+        const int sm = (2 * MP * half_pad(d.nx) + 160 + 8 * (4 * row_pitch(d.nx) + 8 * MP)) * 4;
+        e = cudaFuncSetAttribute(k_fno_lift_modes<MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        if (e == cudaSuccess) k_fno_lift_modes<MP><<<(int)grid, 256, sm, s>>>(a);
+    });
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 cudaError_t fno_row_raw(const FnoFusedDims& d, const FnoTables& t, const FnoWork& w, const float* g, cudaStream_t s) {
