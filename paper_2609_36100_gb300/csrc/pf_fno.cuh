@@ -12,6 +12,40 @@ __device__ __forceinline__ float gelu_g(float z) {
     return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
 }
 
+// Normal distribution function Phi(z) = (1 + erf(z / sqrt 2)) / 2 of GELU(z) =
+// z Phi(z), with e = exp(-z^2 / 2) for the derivative Phi(z) + z e / sqrt(2 pi).
+// The tail Phi(-|z|) is e times a polynomial in t = 1 / (1 + p |z|), the form of
+// Hastings' approximations of the error function, here of degree eight with
+// coefficients fitted to 9e-8 relative over |z| <= 14.  In FP32 the error of
+// GELU (2.1e-7 at most, 4.0e-8 rms for |z| < 3) is that of the formula with
+// the library's erff (2.5e-7, 4.4e-8): there 1 + erf cancels for negative z.
+// One exponential serves both values: 16 instructions for GELU and 19 with its
+// derivative, against about 31 and 60 with erff and expf.
+__device__ __forceinline__ float gauss_cdf(float z, float& e) {
+    float t;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(fabsf(z), 0.30452660f, 1.0f)));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * z * -0.72134752f));
+    float q = 0.036764109f;
+    q = fmaf(q, t, -0.15403491f);
+    q = fmaf(q, t, 0.18868711f);
+    q = fmaf(q, t, -0.040320144f);
+    q = fmaf(q, t, 0.12216621f);
+    q = fmaf(q, t, 0.10296576f);
+    q = fmaf(q, t, 0.12232373f);
+    q = fmaf(q, t, 0.12144818f);
+    const float tail = q * t * e;
+    return z < 0.f ? tail : 1.0f - tail;
+}
+__device__ __forceinline__ float gelu_fast(float z) {
+    float e;
+    return z * gauss_cdf(z, e);
+}
+__device__ __forceinline__ float gelu_fast_g(float z) {
+    float e;
+    const float c = gauss_cdf(z, e);
+    return fmaf(z * 0.39894228f, e, c);
+}
+
 // D += A B on one 16x8x16 BF16 tile, FP32 accumulation
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
     asm volatile(

@@ -4,10 +4,10 @@
 // transforms along the rows of the grid, both of which need all channels of a
 // row, and transforms along y and z of the few retained x modes.  The row
 // kernels do everything of the first kind in one pass over the activations:
-// a warp holds one row of all channels in shared memory, applies GELU to the
-// previous pre-activation, the channel product on the tensor cores, adds the
-// inverse x transform of the layer's spectral part, stores the
-// pre-activation, and leaves the x transform of its GELU for the next layer.
+// two warps hold one row of all channels in shared memory, apply GELU to the
+// previous pre-activation, the channel product on the tensor cores, add the
+// inverse x transform of the layer's spectral part, store the
+// pre-activation, and leave the x transform of its GELU for the next layer.
 // So a layer reads one [C][N] array and writes one; activations are
 // recomputed from pre-activations instead of stored.  The transforms use the
 // symmetry of cosines and sines under x -> n - x, which halves their products.
@@ -80,6 +80,20 @@ __host__ __device__ inline RowSmem row_smem(int nx, int CP, int MP) {
     return o;
 }
 
+// The warps of a row: `part` 0..W-1 of W, synchronised by a named barrier
+// (W = 2) or within the warp.  Shared memory holds about ten rows an SM; with
+// one warp a row that left two warps a scheduler.
+template <int W>
+struct Team {
+    int part, id;
+    __device__ __forceinline__ void sync() const {
+        if constexpr (W == 1)
+            __syncwarp();
+        else
+            asm volatile("bar.sync %0, %1;" ::"r"(id + 1), "n"(32 * W) : "memory");
+    }
+};
+
 template <int CPL>
 __device__ __forceinline__ void ld_chan(float (&v)[CPL], const float* p) {
     if constexpr (CPL == 4) {
@@ -130,7 +144,7 @@ __device__ __forceinline__ void row_setup(const RowArgs& a, float* sm, const Row
         sm[L.lift + 4 * CP + e] = a.pb && e < C ? a.pb[e] : 0.f;
     }
     // padded channels stay zero in every row
-    for (int e = L.warp + threadIdx.x; e < L.warp + (int)(blockDim.x >> 5) * L.perwarp; e += blockDim.x) sm[e] = 0.f;
+    for (int e = L.warp + threadIdx.x; e < L.warp + (int)(blockDim.x / 64) * L.perwarp; e += blockDim.x) sm[e] = 0.f;
 }
 
 // asynchronous global -> shared copies: a warp has a whole row in flight
@@ -148,13 +162,13 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::
 
 // the row's retained x modes: T1 -> [kx][channel], channels of a lane adjacent
 // (zeros at the padded ones)
-template <int CP, int MP>
-__device__ __forceinline__ void row_load_modes(const RowArgs& a, long long row, float* T) {
+template <int CP, int MP, int W>
+__device__ __forceinline__ void row_load_modes(const RowArgs& a, long long row, float* T, Team<W> tm) {
     constexpr int CPL = CP / 8, TS = CP + 4;
     const float* src = reinterpret_cast<const float*>(a.T1 + row * a.C * a.m);
     const int lane = threadIdx.x & 31;
 #pragma unroll 4
-    for (int e = lane; e < MP * CP; e += 32) {
+    for (int e = lane + 32 * tm.part; e < MP * CP; e += 32 * W) {
         const int c = e / MP, k = e - c * MP;
         const bool in = c < a.C && k < a.m;
         const float* t = src + (in ? 2 * (c * a.m + k) : 0);
@@ -165,22 +179,24 @@ __device__ __forceinline__ void row_load_modes(const RowArgs& a, long long row, 
 }
 
 // a row of C channels of src [C][N] into A
-__device__ __forceinline__ void row_load(const RowArgs& a, const float* src, long long r0, float* A, int RS) {
+template <int W>
+__device__ __forceinline__ void row_load(const RowArgs& a, const float* src, long long r0, float* A, int RS,
+                                         Team<W> tm) {
     const int lane = threadIdx.x & 31;
     if (a.vec) {  // rows start on 16-byte boundaries
         for (int x = 4 * lane; x < a.nx; x += 128)
 #pragma unroll 8
-            for (int c = 0; c < a.C; ++c) cp16(A + c * RS + x, src + (long long)c * a.N + r0 + x);
+            for (int c = tm.part; c < a.C; c += W) cp16(A + c * RS + x, src + (long long)c * a.N + r0 + x);
     } else {
         for (int x = lane; x < a.nx; x += 32)
 #pragma unroll 8
-            for (int c = 0; c < a.C; ++c) cp4(A + c * RS + x, src + (long long)c * a.N + r0 + x, true);
+            for (int c = tm.part; c < a.C; c += W) cp4(A + c * RS + x, src + (long long)c * a.N + r0 + x, true);
     }
 }
 
 // A <- W A column tile by column tile on the tensor cores (W's fragments in shared memory)
-template <int CP>
-__device__ __forceinline__ void row_dense(float* A, int RS, int nx, const unsigned* w) {
+template <int CP, int W>
+__device__ __forceinline__ void row_dense(float* A, int RS, int nx, const unsigned* w, Team<W> tm) {
     constexpr int T = CP / 16;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     unsigned ah[T][T][4], al[T][T][4];
@@ -194,7 +210,7 @@ __device__ __forceinline__ void row_dense(float* A, int RS, int nx, const unsign
             al[i][j][0] = l.x, al[i][j][1] = l.y, al[i][j][2] = l.z, al[i][j][3] = l.w;
         }
     // two column tiles at a time: their chains of products overlap
-    for (int n0 = 0; n0 < nx; n0 += 16) {
+    for (int n0 = 16 * tm.part; n0 < nx; n0 += 16 * W) {
         const bool two = n0 + 8 < nx;
         float acc[2][T][4] = {};
 #pragma unroll
@@ -226,13 +242,13 @@ __device__ __forceinline__ void row_dense(float* A, int RS, int nx, const unsign
 
 // A += bias + inverse x transform of the modes in T: a lane takes CP/8
 // channels at four positions x and their mirrors n - x
-template <int CP, int MP>
+template <int CP, int MP, int W>
 __device__ __forceinline__ void row_inverse_add(float* A, int RS, int nx, const float* T, const float* tic,
-                                                const float* tis, const float* sp, const float* bias) {
+                                                const float* tis, const float* sp, const float* bias, Team<W> tm) {
     constexpr int CPL = CP / 8, TS = CP + 4;
     const int lane = threadIdx.x & 31, g = lane & 7, xg = lane >> 3;
     const int XL = (nx + 1) / 2, XQ = inv_pad(nx);
-    for (int x0 = 0; x0 < XQ; x0 += 16) {
+    for (int x0 = 16 * tm.part; x0 < XQ; x0 += 16 * W) {
         float c[CPL][4] = {}, s[CPL][4] = {};
 #pragma unroll
         for (int k = 0; k < MP; ++k) {
@@ -264,7 +280,7 @@ __device__ __forceinline__ void row_inverse_add(float* A, int RS, int nx, const 
             }
         }
     }
-    if ((nx & 1) == 0 && lane < CP) {  // the position that is its own mirror
+    if ((nx & 1) == 0 && lane < CP && tm.part == W - 1) {  // the position that is its own mirror
         const int slot = (lane & 7) * CPL + (lane >> 3);
         float v = bias[lane];
 #pragma unroll
@@ -274,13 +290,14 @@ __device__ __forceinline__ void row_inverse_add(float* A, int RS, int nx, const 
 }
 
 // T1 <- forward x transform of the folded rows (sums at [0, HP), differences
-// at [HP, 2 HP)): a lane takes CP/8 channels and MP/4 modes
-template <int CP, int MP>
+// at [HP, 2 HP)): a lane takes CP/(8 W) channels and MP/4 modes
+template <int CP, int MP, int W>
 __device__ __forceinline__ void row_forward(const RowArgs& a, long long row, const float* A, int RS, float* T,
-                                            const float* tfc, const float* tfs) {
-    constexpr int CPL = CP / 8, KPL = MP / 4;
-    const int lane = threadIdx.x & 31, g = lane & 7, kg = lane >> 3, HP = half_pad(a.nx);
+                                            const float* tfc, const float* tfs, Team<W> tm) {
+    constexpr int CPL = CP / (8 * W), KPL = MP / 4;
+    const int lane = threadIdx.x & 31, g = (lane & 7) + 8 * CPL * tm.part, kg = lane >> 3, HP = half_pad(a.nx);
     float re[CPL][KPL] = {}, im[CPL][KPL] = {};
+#pragma unroll 2
     for (int x = 0; x < HP; x += 4) {
         float4 c[KPL], s[KPL];
 #pragma unroll
@@ -308,21 +325,21 @@ __device__ __forceinline__ void row_forward(const RowArgs& a, long long row, con
             const int c = g + 8 * i, k = kg * KPL + j;
             if (c < a.C && k < a.m) st[c * a.m + k] = make_float2(re[i][j], -im[i][j]);
         }
-    __syncwarp();
+    tm.sync();
     float2* dst = a.T1 + row * a.C * a.m;
-    for (int e = lane; e < a.C * a.m; e += 32) dst[e] = st[e];
-    __syncwarp();
+    for (int e = lane + 32 * tm.part; e < a.C * a.m; e += 32 * W) dst[e] = st[e];
+    tm.sync();
 }
 
 // in place: a row's values -> sums and differences under x -> n - x, after
 // val(channel, x, value, pre(channel, x)).  The two positions that are their
 // own mirrors, 0 and n/2, share a lane.  CB channels at a time: first every
 // pre (a load, say), then the values.
-template <int CB, class G, class F>
-__device__ __forceinline__ void row_fold(float* A, int RS, int nx, int C, G pre, F val) {
+template <int CB, int W, class G, class F>
+__device__ __forceinline__ void row_fold(float* A, int RS, int nx, int C, Team<W> tm, G pre, F val) {
     const int lane = threadIdx.x & 31, HP = half_pad(nx), Hx = nx / 2 + 1, XL = (nx + 1) / 2;
     const bool even = (nx & 1) == 0;
-    for (int c0 = 0; c0 < C; c0 += CB) {
+    for (int c0 = CB * tm.part; c0 < C; c0 += CB * W) {
         float v[CB][kFoldIter], u[CB][kFoldIter];
         using P = decltype(pre(0, 0));
         P pv[CB][kFoldIter], pu[CB][kFoldIter];
@@ -368,13 +385,14 @@ __device__ __forceinline__ void row_fold(float* A, int RS, int nx, int C, G pre,
             if (lane < HP - Hx) r[Hx + lane] = r[HP + Hx + lane] = 0.f;
         }
     }
-    __syncwarp();
+    tm.sync();
 }
 
 // lift of the row's input: a_0 = P x + p
-template <int CP>
-__device__ __forceinline__ void row_lift(const RowArgs& a, long long r0, float* A, int RS, const float* lift) {
-    for (int x = threadIdx.x & 31; x < a.nx; x += 32) {
+template <int CP, int W>
+__device__ __forceinline__ void row_lift(const RowArgs& a, long long r0, float* A, int RS, const float* lift,
+                                         Team<W> tm) {
+    for (int x = (threadIdx.x & 31) + 32 * tm.part; x < a.nx; x += 32 * W) {
         float v[4];
 #pragma unroll
         for (int f = 0; f < 4; ++f) v[f] = a.x[f * a.N + r0 + x];
@@ -412,7 +430,7 @@ __global__ void __launch_bounds__(256) k_fno_lift_modes(RowArgs a) {
         cp_wait();
         __syncwarp();
         row_fold<4>(
-            A, RS, nx, 4, [](int, int) { return 0; }, [](int, int, float v, int) { return v; });
+            A, RS, nx, 4, Team<1>{0, 0}, [](int, int) { return 0; }, [](int, int, float v, int) { return v; });
         const int f = lane & 3;
         for (int k = lane >> 2; k < a.m; k += 8) {
             float re = 0.f, im = 0.f;
@@ -439,54 +457,58 @@ __global__ void __launch_bounds__(256) k_fno_lift_modes(RowArgs a) {
     }
 }
 
+constexpr int kTeam = 2;  // warps of a row
+
 template <int CP, int MP>
-__global__ void __launch_bounds__(512, 1) k_fno_row(RowArgs a) {
+__global__ void __launch_bounds__(640, 1) k_fno_row(RowArgs a) {
     extern __shared__ __align__(16) float sm[];
     const RowSmem L = row_smem(a.nx, CP, MP);
     row_setup<CP, MP, false>(a, sm, L);
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nt = blockDim.x / (32 * kTeam);
+    const Team<kTeam> tm{warp % kTeam, warp / kTeam};
     const int nx = a.nx, C = a.C, RS = row_pitch(nx), HP = half_pad(nx), XQ = inv_pad(nx);
-    float* A = sm + L.warp + warp * L.perwarp;
+    float* A = sm + L.warp + tm.id * L.perwarp;
     float* T = A + CP * RS;
-    for (long long row = blockIdx.x * (long long)nw + warp; row < a.rows; row += (long long)gridDim.x * nw) {
+    for (long long row = blockIdx.x * (long long)nt + tm.id; row < a.rows; row += (long long)gridDim.x * nt) {
         const long long r0 = row * nx;
-        if (a.dense) row_load_modes<CP, MP>(a, row, T);
-        if (a.zprev) row_load(a, a.zprev, r0, A, RS);
+        if (a.dense) row_load_modes<CP, MP>(a, row, T, tm);
+        if (a.zprev) row_load(a, a.zprev, r0, A, RS, tm);
         cp_wait();
-        __syncwarp();
+        tm.sync();
         if (!a.zprev) {
-            row_lift<CP>(a, r0, A, RS, sm + L.lift);
+            row_lift<CP>(a, r0, A, RS, sm + L.lift, tm);
         } else if (!a.raw) {
             for (int x = lane; x < nx; x += 32)
 #pragma unroll 8
-                for (int c = 0; c < C; ++c) A[c * RS + x] = gelu_f(A[c * RS + x]);
+                for (int c = tm.part; c < C; c += kTeam) A[c * RS + x] = gelu_fast(A[c * RS + x]);
         }
-        __syncwarp();
+        tm.sync();
         if (a.dense) {
-            row_dense<CP>(A, RS, nx, reinterpret_cast<const unsigned*>(sm + L.frag));
-            row_inverse_add<CP, MP>(A, RS, nx, T, sm + L.ti, sm + L.ti + MP * XQ, sm + L.sp, sm + L.bias);
-            __syncwarp();
+            row_dense<CP>(A, RS, nx, reinterpret_cast<const unsigned*>(sm + L.frag), tm);
+            tm.sync();
+            row_inverse_add<CP, MP>(A, RS, nx, T, sm + L.ti, sm + L.ti + MP * XQ, sm + L.sp, sm + L.bias, tm);
+            tm.sync();
         }
         if (a.last) {
             for (int x = lane; x < nx; x += 32)
 #pragma unroll 8
-                for (int c = 0; c < C; ++c) a.z[(long long)c * a.N + r0 + x] = A[c * RS + x];
-            __syncwarp();
+                for (int c = tm.part; c < C; c += kTeam) a.z[(long long)c * a.N + r0 + x] = A[c * RS + x];
+            tm.sync();
             continue;
         }
         if (a.dense) {
             row_fold<2>(
-                A, RS, nx, C, [](int, int) { return 0; },
+                A, RS, nx, C, tm, [](int, int) { return 0; },
                 [&](int c, int x, float v, int) {
                     a.z[(long long)c * a.N + r0 + x] = v;
-                    return gelu_f(v);
+                    return gelu_fast(v);
                 });
         } else {
             row_fold<2>(
-                A, RS, nx, C, [](int, int) { return 0; }, [](int, int, float v, int) { return v; });
+                A, RS, nx, C, tm, [](int, int) { return 0; }, [](int, int, float v, int) { return v; });
         }
-        row_forward<CP, MP>(a, row, A, RS, T, sm + L.tf, sm + L.tf + MP * HP);
+        row_forward<CP, MP>(a, row, A, RS, T, sm + L.tf, sm + L.tf + MP * HP, tm);
     }
 }
 
@@ -494,16 +516,18 @@ __global__ void __launch_bounds__(512, 1) k_fno_row(RowArgs a) {
 __host__ __device__ inline int row_part_len(int C) { return C * C + 6 * C; }
 
 template <int CP, int MP>
-__global__ void __launch_bounds__(384, 1) k_fno_row_bwd(RowArgs a) {
+__global__ void __launch_bounds__(512, 1) k_fno_row_bwd(RowArgs a) {
     extern __shared__ __align__(16) float sm[];
     const RowSmem L = row_smem(a.nx, CP, MP);
     row_setup<CP, MP, true>(a, sm, L);
     __syncthreads();
     constexpr int MT = CP / 16, NT = CP / 8;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, g = lane >> 2, t = lane & 3;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nt = blockDim.x / (32 * kTeam);
+    const int g = lane >> 2, t = lane & 3;
+    const Team<kTeam> tm{warp % kTeam, warp / kTeam};
     const int nx = a.nx, C = a.C, RS = row_pitch(nx), HP = half_pad(nx), XQ = inv_pad(nx);
     const bool first = a.zprev == nullptr;
-    float* A = sm + L.warp + warp * L.perwarp;
+    float* A = sm + L.warp + tm.id * L.perwarp;
     float* T = A + CP * RS;
     const float* lift = sm + L.lift;
     float gV[MT][NT][4] = {}, gP[MT][4] = {}, sv[MT][2] = {}, sp[MT][2] = {};
@@ -522,20 +546,19 @@ __global__ void __launch_bounds__(384, 1) k_fno_row_bwd(RowArgs a) {
             }
         }
     };
-    for (long long row = blockIdx.x * (long long)nw + warp; row < a.rows; row += (long long)gridDim.x * nw) {
+    for (long long row = blockIdx.x * (long long)nt + tm.id; row < a.rows; row += (long long)gridDim.x * nt) {
         const long long r0 = row * nx;
-        row_load_modes<CP, MP>(a, row, T);
-        row_load(a, a.z, r0, A, RS);
+        row_load_modes<CP, MP>(a, row, T, tm);
+        row_load(a, a.z, r0, A, RS, tm);
         if (!first)  // the row of zprev on its way while dz arrives
-            for (int e = lane; e < C * ((nx + 31) / 32 + 1); e += 32) {
+            for (int e = lane + 32 * tm.part; e < C * ((nx + 31) / 32 + 1); e += 32 * kTeam) {
                 const int c = e % C, x = min(32 * (e / C), nx - 1);
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(a.zprev + (long long)c * a.N + r0 + x));
             }
         cp_wait();
-        __syncwarp();
+        tm.sync();
         // gradient of V: dz a^T over the row's points, a in fragments straight from global memory
-#pragma unroll 2
-        for (int k0 = 0; k0 < nx; k0 += 16) {
+        for (int k0 = 16 * tm.part; k0 < nx; k0 += 16 * kTeam) {
             const int p = k0 + 2 * t;
             float av[NT][4];
             if (!first) {
@@ -549,7 +572,7 @@ __global__ void __launch_bounds__(384, 1) k_fno_row_bwd(RowArgs a) {
 #pragma unroll
                 for (int j = 0; j < NT; ++j)
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) av[j][r] = gelu_f(av[j][r]);
+                    for (int r = 0; r < 4; ++r) av[j][r] = gelu_fast(av[j][r]);
             } else {
                 float xv[4][4];
 #pragma unroll
@@ -579,13 +602,14 @@ __global__ void __launch_bounds__(384, 1) k_fno_row_bwd(RowArgs a) {
                 for (int i = 0; i < MT; ++i) mma3(gV[i][j], ah[i], al[i], bh0, bh1, bl0, bl1);
             }
         }
-        __syncwarp();
-        row_dense<CP>(A, RS, nx, reinterpret_cast<const unsigned*>(sm + L.frag));
-        row_inverse_add<CP, MP>(A, RS, nx, T, sm + L.ti, sm + L.ti + MP * XQ, sm + L.sp, sm + L.bias);
-        __syncwarp();
+        tm.sync();
+        row_dense<CP>(A, RS, nx, reinterpret_cast<const unsigned*>(sm + L.frag), tm);
+        tm.sync();
+        row_inverse_add<CP, MP>(A, RS, nx, T, sm + L.ti, sm + L.ti + MP * XQ, sm + L.sp, sm + L.bias, tm);
+        tm.sync();
         if (first) {
             // gradients of the lift: da x^T and the row sums
-            for (int k0 = 0; k0 < nx; k0 += 16) {
+            for (int k0 = 16 * tm.part; k0 < nx; k0 += 16 * kTeam) {
                 const int p = k0 + 2 * t;
                 float xv[4];
 #pragma unroll
@@ -600,55 +624,64 @@ __global__ void __launch_bounds__(384, 1) k_fno_row_bwd(RowArgs a) {
 #pragma unroll
                 for (int i = 0; i < MT; ++i) mma3(gP[i], ah[i], al[i], bh0, bh1, bl0, bl1);
             }
-            __syncwarp();
+            tm.sync();
             continue;
         }
         row_fold<4>(
-            A, RS, nx, C, [&](int c, int x) { return a.zprev[(long long)c * a.N + r0 + x]; },
+            A, RS, nx, C, tm, [&](int c, int x) { return a.zprev[(long long)c * a.N + r0 + x]; },
             [&](int c, int x, float v, float z) {
-                const float d = v * gelu_g(z);
+                const float d = v * gelu_fast_g(z);
                 a.z[(long long)c * a.N + r0 + x] = d;
                 return d;
             });
-        row_forward<CP, MP>(a, row, A, RS, T, sm + L.tf, sm + L.tf + MP * HP);
+        row_forward<CP, MP>(a, row, A, RS, T, sm + L.tf, sm + L.tf + MP * HP, tm);
     }
-    // warps -> block, in warp order
+    // the warps of a row add up in its shared memory one after another, then
+    // the rows, each in order
     const int E = row_part_len(C);
-    __syncthreads();
-    float* own = sm + L.warp + warp * L.perwarp;  // at least CP (2 half_pad) floats: CP CP + 6 CP fit from nx = 32 on
-#pragma unroll
-    for (int i = 0; i < MT; ++i)
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int c = i * 16 + g + ((r & 2) ? 8 : 0);
-            if (c < C) {
-#pragma unroll
-                for (int j = 0; j < NT; ++j) {
-                    const int d = j * 8 + 2 * t + (r & 1);
-                    if (d < C) own[c * C + d] = gV[i][j][r];
-                }
-                if (2 * t + (r & 1) < 4) own[C * C + C + c * 4 + 2 * t + (r & 1)] = gP[i][r];
-            }
-        }
+    float* own = A;  // CP row_pitch + 2 MP (CP + 4) floats: E of them from nx = 32 on
 #pragma unroll
     for (int i = 0; i < MT; ++i)
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            float u = sv[i][r], w = sp[i][r];
-            u += __shfl_xor_sync(0xffffffffu, u, 1);
-            u += __shfl_xor_sync(0xffffffffu, u, 2);
-            w += __shfl_xor_sync(0xffffffffu, w, 1);
-            w += __shfl_xor_sync(0xffffffffu, w, 2);
-            const int c = i * 16 + g + 8 * r;
-            if (t == 0 && c < C) {
-                own[C * C + c] = u;
-                own[C * C + 5 * C + c] = w;
-            }
+            sv[i][r] += __shfl_xor_sync(0xffffffffu, sv[i][r], 1);
+            sv[i][r] += __shfl_xor_sync(0xffffffffu, sv[i][r], 2);
+            sp[i][r] += __shfl_xor_sync(0xffffffffu, sp[i][r], 1);
+            sp[i][r] += __shfl_xor_sync(0xffffffffu, sp[i][r], 2);
         }
+    for (int w = 0; w < kTeam; ++w) {
+        __syncthreads();
+        if (tm.part != w) continue;
+        auto put = [&](int e, float v) { own[e] = w ? own[e] + v : v; };
+#pragma unroll
+        for (int i = 0; i < MT; ++i)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int c = i * 16 + g + ((r & 2) ? 8 : 0);
+                if (c < C) {
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) {
+                        const int d = j * 8 + 2 * t + (r & 1);
+                        if (d < C) put(c * C + d, gV[i][j][r]);
+                    }
+                    if (2 * t + (r & 1) < 4) put(C * C + C + c * 4 + 2 * t + (r & 1), gP[i][r]);
+                }
+            }
+#pragma unroll
+        for (int i = 0; i < MT; ++i)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int c = i * 16 + g + 8 * r;
+                if (t == 0 && c < C) {
+                    put(C * C + c, sv[i][r]);
+                    put(C * C + 5 * C + c, sp[i][r]);
+                }
+            }
+    }
     __syncthreads();
     for (int e = threadIdx.x; e < E; e += blockDim.x) {
         float v = 0.f;
-        for (int w = 0; w < nw; ++w) v += sm[L.warp + w * L.perwarp + e];
+        for (int w = 0; w < nt; ++w) v += sm[L.warp + w * L.perwarp + e];
         a.part[(long long)blockIdx.x * E + e] = v;
     }
 }
@@ -870,7 +903,7 @@ constexpr int proj_smem() {
 }
 
 // The products of a tile run on the tensor cores; what bounds the kernel is
-// the error function of its H x 64 hidden values.  The next tile's columns of
+// the instructions around them, GELU of its H x 64 hidden values first.  The next tile's columns of
 // a are copied in while this one is worked on.
 template <int CP, int NW, bool TRAIN>
 __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
@@ -987,9 +1020,10 @@ __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     const float z = acc[r];
-                    const float cdf = 0.5f * (1.0f + erff(z * 0.70710678118654752f));
+                    float e;
+                    const float cdf = gauss_cdf(z, e);
                     hv[r] = z * cdf;
-                    if (TRAIN) gp[n][r] = cdf + z * expf(-0.5f * z * z) * 0.39894228040143268f;
+                    if (TRAIN) gp[n][r] = fmaf(z * 0.39894228f, e, cdf);
                 }
                 float* o = sh + (h0 + g) * kPS + n * 8 + 2 * t;
                 *reinterpret_cast<float2*>(o) = make_float2(hv[0], hv[1]);
@@ -1201,8 +1235,10 @@ void with_modes(int m, F f) {
     }
 }
 
-// warps of a row block: as many rows as its shared memory holds
-int row_warps(const FnoFusedDims& d, int most) {
+// rows of a block: as many as its shared memory holds, up to what its
+// registers allow (640 threads of 96 forward, 512 of 128 backward)
+int row_teams(const FnoFusedDims& d, bool bwd) {
+    const int most = (bwd ? 512 : 640) / (32 * kTeam);
     const RowSmem L = row_smem(d.nx, chan_pad(d.C), modes_pad(d.m));
     const int w = (kSmemMax / 4 - L.warp) / L.perwarp;
     return w > most ? most : w;
@@ -1215,7 +1251,7 @@ cudaError_t row_launch(const FnoFusedDims& d, RowArgs& a, bool bwd, cudaStream_t
     a.N = d.N;
     a.rows = (long long)d.nz * d.ny;
     a.vec = d.nx % 4 == 0 ? 1 : 0;  // N is then a multiple of 4 too; the arrays are the library's own
-    const int CP = chan_pad(d.C), nw = row_warps(d, bwd ? 12 : 16);
+    const int CP = chan_pad(d.C), nw = row_teams(d, bwd);
     const RowSmem L = row_smem(d.nx, CP, modes_pad(d.m));
     const int sm = (L.warp + nw * L.perwarp) * 4;
     long long grid = (a.rows + nw - 1) / nw;
@@ -1226,7 +1262,7 @@ cudaError_t row_launch(const FnoFusedDims& d, RowArgs& a, bool bwd, cudaStream_t
         auto k = bwd ? (CP == 16 ? k_fno_row_bwd<16, MP> : k_fno_row_bwd<32, MP>)
                      : (CP == 16 ? k_fno_row<16, MP> : k_fno_row<32, MP>);
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        if (e == cudaSuccess) k<<<(int)grid, 32 * nw, sm, s>>>(a);
+        if (e == cudaSuccess) k<<<(int)grid, 32 * kTeam * nw, sm, s>>>(a);
     });
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
@@ -1429,7 +1465,7 @@ cudaError_t fno_row_layer_bwd(const FnoFusedDims& d, const FnoTables& t, const F
     a.part = w.part;
     cudaError_t e = row_launch(d, a, true, s);
     if (e != cudaSuccess) return e;
-    const int C = d.C, nw = row_warps(d, 12);
+    const int C = d.C, nw = row_teams(d, true);
     const long long nb = (a.rows + nw - 1) / nw;
     SumSeg sg{{0, C * C, C * C + C, C * C + 5 * C}, {C * C, C, 4 * C, C}, {gV, gv, gP, gp}, zprev ? 2 : 4};
     const int E = row_part_len(C);
