@@ -270,23 +270,35 @@ static int strided_tile(int n, int nbuf, int budget) {
     return tx;
 }
 
-template <typename T>
-static int tile_cols(const Geo& g, int n, int nbuf, int budget) {
-    int tx = strided_tile<T>(n, nbuf, budget);
-    // no wider than the (odd) half-spectrum row
-    while (tx > 1 && tx / 2 >= g.nxh) tx >>= 1;
-    return tx;
-}
-
 // tuned width (0 = untuned) capped by what fits the shared-memory budget
 template <typename T>
-static int tuned_cols(const Geo& g, int tuned, int n, int nbuf, int budget) {
-    if (tuned <= 0) return tile_cols<T>(g, n, nbuf, nbuf == 4 ? 64 * 1024 : 96 * 1024);
-    const int cap = tile_cols<T>(g, n, nbuf, budget);
+static int tuned_cols(int tuned, int n, int nbuf, int budget) {
+    if (tuned <= 0) return strided_tile<T>(n, nbuf, nbuf == 4 ? 64 * 1024 : 96 * 1024);
+    const int cap = strided_tile<T>(n, nbuf, budget);
     int tx = 1;
     while (tx * 2 <= tuned && tx * 2 <= 16) tx *= 2;
     return tx < cap ? tx : cap;
 }
+
+// The column a thread of a y or z pass works on: TX consecutive ones per CTA
+// of the columns of a whole field, counted along kx and on into the next row
+// (plane), since a row of nx/2 + 1 columns leaves the last tile of a row
+// mostly empty (33 columns in three tiles of 16 at nx = 64: 69 % used).  Every
+// loop over a tile strides by a multiple of TX, so a thread keeps its column.
+// Columns of a z pass are also contiguous across rows: tiles start on 128-byte
+// lines wherever ny (nx/2 + 1) is a multiple of 16.
+template <int TX>
+struct Column {
+    int row, kx;  // ky of a z pass, kz of a y pass
+    bool ok;
+    __device__ __forceinline__ Column(int nxh, int rows) {
+        const int q = blockIdx.x * TX + (int)(threadIdx.x & (TX - 1));
+        ok = q < rows * nxh;
+        row = ok ? q / nxh : 0;
+        kx = ok ? q - row * nxh : 0;
+    }
+};
+inline unsigned column_tiles(int nxh, int rows, int TX) { return (unsigned)((rows * nxh + TX - 1) / TX); }
 
 template <typename K>
 static void set_smem(K kern, size_t bytes) {

@@ -15,13 +15,12 @@ __global__ void __launch_bounds__(kThreads) k_y_pass(Geo g, typename Cx<T>::t* _
     extern __shared__ __align__(16) unsigned char smraw[];
     T2* A = reinterpret_cast<T2*>(smraw);
     T2* B = A + TX * g.ny;
-    const int f = blockIdx.z, kz = blockIdx.y, kx0 = blockIdx.x * TX;
-    const int ncol = min(TX, g.nxh - kx0);
-    T2* base = buf + (long long)f * g.NK + (long long)kz * g.ny * g.nxh + kx0;
+    const Column<TX> c(g.nxh, g.nz);
+    T2* base = buf + (long long)blockIdx.y * g.NK + (long long)c.row * g.ny * g.nxh + c.kx;
     const int ys = g.nxh;
-    auto src = [&](int ky, int col) -> T2 { return col < ncol ? base[ky * ys + col] : T2{0, 0}; };
-    auto dst = [&](int ky, int col, T2 v) {
-        if (col < ncol) base[ky * ys + col] = v;
+    auto src = [&](int ky, int) -> T2 { return c.ok ? base[ky * ys] : T2{0, 0}; };
+    auto dst = [&](int ky, int, T2 v) {
+        if (c.ok) base[ky * ys] = v;
     };
     cols_fft<SIGN, TX, true, 0, R16, PID, true>(g.py, A, B, src, dst);
 }
@@ -29,13 +28,13 @@ __global__ void __launch_bounds__(kThreads) k_y_pass(Geo g, typename Cx<T>::t* _
 template <typename T>
 void launch_y_pass(const Geo& g, void* buf, int nf, int sign, cudaStream_t s) {
     using T2 = typename Cx<T>::t;
-    const int TX = tuned_cols<T>(g, g.tx_y, g.ny, 2, 128 * 1024);
+    const int TX = tuned_cols<T>(g.tx_y, g.ny, 2, 128 * 1024);
     // a transform of at most two stages never touches its second buffer
     // (stage 0 reads global, the last stage writes global), and a compiled
     // plan runs its middle stages in place: half the shared memory, more
     // CTAs per SM
     const size_t sm = col_buffers<T>(g.py, TX) * (size_t)TX * g.ny * sizeof(T2);
-    dim3 grid((g.nxh + TX - 1) / TX, g.nz, nf);
+    dim3 grid(column_tiles(g.nxh, g.nz, TX), nf);
     if (sign > 0) {
         PF_COL_SWITCH(T, g.py, TX, set_smem(k_y_pass<T, 1, TXC, R16C, PIDC>, sm);
                       k_y_pass<T, 1, TXC, R16C, PIDC><<<grid, kThreads, sm, s>>>(g, reinterpret_cast<T2*>(buf)));
@@ -56,13 +55,12 @@ __global__ void __launch_bounds__(kThreads) k_z_pass(Geo g, typename Cx<T>::t* _
     extern __shared__ __align__(16) unsigned char smraw[];
     T2* A = reinterpret_cast<T2*>(smraw);
     T2* B = A + TX * g.nz;
-    const int f = blockIdx.z, ky = blockIdx.y, kx0 = blockIdx.x * TX;
-    const int ncol = min(TX, g.nxh - kx0);
-    T2* base = buf + (long long)f * g.NK + (long long)ky * g.nxh + kx0;
+    const Column<TX> c(g.nxh, g.ny);
+    T2* base = buf + (long long)blockIdx.y * g.NK + (long long)c.row * g.nxh + c.kx;
     const long long zs = (long long)g.ny * g.nxh;
-    auto src = [&](int kz, int col) -> T2 { return col < ncol ? base[kz * zs + col] : T2{0, 0}; };
-    auto dst = [&](int kz, int col, T2 v) {
-        if (col < ncol) base[kz * zs + col] = v;
+    auto src = [&](int kz, int) -> T2 { return c.ok ? base[kz * zs] : T2{0, 0}; };
+    auto dst = [&](int kz, int, T2 v) {
+        if (c.ok) base[kz * zs] = v;
     };
     cols_fft<SIGN, TX, true, 0, R16, PID, true>(g.pz, A, B, src, dst);
 }
@@ -70,9 +68,9 @@ __global__ void __launch_bounds__(kThreads) k_z_pass(Geo g, typename Cx<T>::t* _
 template <typename T>
 void launch_z_pass(const Geo& g, void* buf, int nf, int sign, cudaStream_t s) {
     using T2 = typename Cx<T>::t;
-    const int TX = tuned_cols<T>(g, g.tx_zf, g.nz, 2, 128 * 1024);
+    const int TX = tuned_cols<T>(g.tx_zf, g.nz, 2, 128 * 1024);
     const size_t sm = col_buffers<T>(g.pz, TX) * (size_t)TX * g.nz * sizeof(T2);  // as in the y pass
-    dim3 grid((g.nxh + TX - 1) / TX, g.ny, nf);
+    dim3 grid(column_tiles(g.nxh, g.ny, TX), nf);
     if (sign > 0) {
         PF_COL_SWITCH(T, g.pz, TX, set_smem(k_z_pass<T, 1, TXC, R16C, PIDC>, sm);
                       k_z_pass<T, 1, TXC, R16C, PIDC><<<grid, kThreads, sm, s>>>(g, reinterpret_cast<T2*>(buf)));
@@ -97,24 +95,24 @@ __global__ void __launch_bounds__(kThreads) k_z_fwd(Geo g, Phys ph, const typena
     extern __shared__ __align__(16) unsigned char smraw[];
     T2* A = reinterpret_cast<T2*>(smraw);
     T2* B = A + TX * g.nz;
-    const int f = blockIdx.z, ky = blockIdx.y, kx0 = blockIdx.x * TX;
-    const int ncol = min(TX, g.nxh - kx0);
-    const long long base = (long long)f * g.NK + (long long)ky * g.nxh + kx0;
+    const Column<TX> c(g.nxh, g.ny);
+    const int f = blockIdx.y;
+    const long long base = (long long)f * g.NK + (long long)c.row * g.nxh + c.kx;
     const long long zs = (long long)g.ny * g.nxh;
     const double invN = g.invN;
     const T mN = phys_t<T>(ph).mN, lN = phys_t<T>(ph).lN;
-    const T kyv = kval<T>(g, 1, ky);
-    auto src = [&](int kz, int col) -> T2 { return col < ncol ? W[base + kz * zs + col] : T2{0, 0}; };
-    auto dst = [&](int kz, int col, T2 v) {
-        if (col >= ncol) return;
-        const long long gi = base + kz * zs + col;
+    const T kx = kval<T>(g, 0, c.kx), kyv = kval<T>(g, 1, c.row), kxy2 = kx * kx + kyv * kyv;
+    auto src = [&](int kz, int) -> T2 { return c.ok ? W[base + kz * zs] : T2{0, 0}; };
+    auto dst = [&](int kz, int, T2 v) {
+        if (!c.ok) return;
+        const long long gi = base + kz * zs;
         if (mode == 0) {
             out[gi] = OT2{(OT)((double)v.x * invN), (OT)((double)v.y * invN)};
         } else {
             T sc;
             if (f == 0) {
-                const T kx = kval<T>(g, 0, kx0 + col), kzv = kval<T>(g, 2, kz);
-                sc = mN * (kx * kx + kyv * kyv + kzv * kzv);
+                const T kzv = kval<T>(g, 2, kz);
+                sc = mN * (kxy2 + kzv * kzv);
             } else {
                 sc = lN;
             }
@@ -127,11 +125,11 @@ __global__ void __launch_bounds__(kThreads) k_z_fwd(Geo g, Phys ph, const typena
 template <typename T>
 void launch_z_fwd(const Geo& g, const Phys& ph, const void* W, void* out, int scale_mode, cudaStream_t s, int nf) {
     using T2 = typename Cx<T>::t;
-    const int TX = tuned_cols<T>(g, g.tx_zf, g.nz, 2, 128 * 1024);
+    const int TX = tuned_cols<T>(g.tx_zf, g.nz, 2, 128 * 1024);
     // modes 0/2 run the generic stages (two buffers for three or more stages)
     const size_t sm = (scale_mode == 1 ? col_buffers<T>(g.pz, TX) : (g.pz.nst <= 2 ? 1 : 2)) * (size_t)TX * g.nz *
                       sizeof(T2);
-    dim3 grid((g.nxh + TX - 1) / TX, g.ny, nf);
+    dim3 grid(column_tiles(g.nxh, g.ny, TX), nf);
     if (scale_mode == 1) {
         PF_COL_SWITCH(T, g.pz, TX, set_smem(k_z_fwd<T, T2, TXC, R16C, PIDC>, sm);
                       k_z_fwd<T, T2, TXC, R16C, PIDC><<<grid, kThreads, sm, s>>>(
@@ -155,9 +153,8 @@ __global__ void __launch_bounds__(kThreads) k_z_elastic(Geo g, Phys ph, typename
     slot[1] = slot[0] + tile;
     slot[2] = slot[1] + tile;
     T2* E = slot[2] + tile;
-    const int ky = blockIdx.y, kx0 = blockIdx.x * TX;
-    const int ncol = min(TX, g.nxh - kx0);
-    const long long rowoff = (long long)ky * g.nxh + kx0;
+    const Column<TX> c(g.nxh, g.ny);
+    const long long rowoff = (long long)c.row * g.nxh + c.kx;
     const long long zs = (long long)g.ny * g.nxh;
     bool nst_even;
     if constexpr (PID > 0)
@@ -170,7 +167,7 @@ __global__ void __launch_bounds__(kThreads) k_z_elastic(Geo g, Phys ph, typename
     for (int f = 0; f < 3; ++f) {
         T2* S = slot[f];
         const long long fb = (long long)f * g.NK + rowoff;
-        auto src = [&](int kz, int col) -> T2 { return col < ncol ? H[fb + kz * zs + col] : T2{0, 0}; };
+        auto src = [&](int kz, int) -> T2 { return c.ok ? H[fb + kz * zs] : T2{0, 0}; };
         auto dst = [&](int kz, int col, T2 v) { S[kz * TX + col] = v; };
         if (nst_even)
             cols_fft<-1, TX, false, 0, R16, PID>(g.pz, E, S, src, dst);
@@ -180,19 +177,19 @@ __global__ void __launch_bounds__(kThreads) k_z_elastic(Geo g, Phys ph, typename
     }
     const T invN = std::is_same<T, float>::value ? (T)g.invN32 : (T)g.invN;
     const PhysT<T>& pt = phys_t<T>(ph);
-    const T kyv = kval<T>(g, 1, ky);
+    const T kxv = kval<T>(g, 0, c.kx), kyv = kval<T>(g, 1, c.row);
     // FP32 contexts with diagonal eigenstrains read B/N from the octant table
     const float* bt = sizeof(T) == 4 ? g.btab : nullptr;
     const int hy = g.ny / 2 + 1;
     const long long tn = (long long)(g.nz / 2 + 1) * hy * g.nxh;
-    const long long trow = (long long)(ky <= g.ny / 2 ? ky : g.ny - ky) * g.nxh + kx0;
+    const long long trow = (long long)(c.row <= g.ny / 2 ? c.row : g.ny - c.row) * g.nxh + c.kx;
     for (int r = threadIdx.x; r < tile; r += blockDim.x) {
-        const int col = r & (TX - 1), kz = r / TX;
-        if (col >= ncol) continue;
+        const int kz = r / TX;
+        if (!c.ok) continue;
         T Bm[3][3];
         T sc = invN;
         if (bt) {
-            const long long ti = (long long)(kz <= g.nz / 2 ? kz : g.nz - kz) * hy * g.nxh + trow + col;
+            const long long ti = (long long)(kz <= g.nz / 2 ? kz : g.nz - kz) * hy * g.nxh + trow;
             Bm[0][0] = (T)__ldg(bt + ti);
             Bm[0][1] = Bm[1][0] = (T)__ldg(bt + tn + ti);
             Bm[0][2] = Bm[2][0] = (T)__ldg(bt + 2 * tn + ti);
@@ -201,7 +198,7 @@ __global__ void __launch_bounds__(kThreads) k_z_elastic(Geo g, Phys ph, typename
             Bm[2][2] = (T)__ldg(bt + 5 * tn + ti);
             sc = (T)1;
         } else {
-            elastic_kernel<T>(pt, kval<T>(g, 0, kx0 + col), kyv, kval<T>(g, 2, kz), Bm);
+            elastic_kernel<T>(pt, kxv, kyv, kval<T>(g, 2, kz), Bm);
         }
         const T2 h0 = slot[0][r], h1 = slot[1][r], h2 = slot[2][r];
         slot[0][r] = T2{(Bm[0][0] * h0.x + Bm[0][1] * h1.x + Bm[0][2] * h2.x) * sc,
@@ -219,8 +216,8 @@ __global__ void __launch_bounds__(kThreads) k_z_elastic(Geo g, Phys ph, typename
         T2* S = slot[f];
         const long long fb = (long long)f * g.NK + rowoff;
         auto src = [&](int kz, int col) -> T2 { return S[kz * TX + col]; };
-        auto dst = [&](int kz, int col, T2 v) {
-            if (col < ncol) H[fb + kz * zs + col] = v;
+        auto dst = [&](int kz, int, T2 v) {
+            if (c.ok) H[fb + kz * zs] = v;
         };
         cols_fft<+1, TX, false, 0, R16, PID>(g.pz, E, S, src, dst);
         __syncthreads();
@@ -291,15 +288,14 @@ __global__ void __launch_bounds__(NT, elastic_min_blocks<T, PID, NT>())
     static_assert(NT == TX * M, "one thread per (column, j) of the fused stage");
     extern __shared__ __align__(16) unsigned char smraw[];
     T2* S = reinterpret_cast<T2*>(smraw);  // [3][N][TX]
-    const int ky = blockIdx.y, kx0 = blockIdx.x * TX;
-    const int ncol = min(TX, g.nxh - kx0);
-    const long long rowoff = (long long)ky * g.nxh + kx0;
+    const Column<TX> c(g.nxh, g.ny);
+    const long long rowoff = (long long)c.row * g.nxh + c.kx;
     const long long zs = (long long)g.ny * g.nxh;
     const T2* tw = twiddles<T2>(g.pz);
     // forward stage 1: global -> tile
     {
-        auto ld = [&](int f, int kz, int col) -> T2 {
-            return col < ncol ? H[(long long)f * g.NK + rowoff + kz * zs + col] : T2{0, 0};
+        auto ld = [&](int f, int kz, int) -> T2 {
+            return c.ok ? H[(long long)f * g.NK + rowoff + kz * zs] : T2{0, 0};
         };
         auto st = [&](int f, int kz, int col, T2 v) { S[f * (N * TX) + kz * TX + col] = v; };
         tile_stage_io<RF, -1, TX, N, 1, 3, NT>(tw, ld, st);
@@ -322,13 +318,13 @@ __global__ void __launch_bounds__(NT, elastic_min_blocks<T, PID, NT>())
         __syncthreads();
         const T invN = std::is_same<T, float>::value ? (T)g.invN32 : (T)g.invN;
         const PhysT<T>& pt = phys_t<T>(ph);
-        const T kxv = kval<T>(g, 0, kx0 + (col < ncol ? col : 0)), kyv = kval<T>(g, 1, ky);
+        const T kxv = kval<T>(g, 0, c.kx), kyv = kval<T>(g, 1, c.row);
         // FP32 contexts with diagonal eigenstrains read B/N from the table
         // (held in L2 across the tiles); otherwise B is formed per wave vector
         const float* bt = sizeof(T) == 4 ? g.btab : nullptr;
         const int hy = g.ny / 2 + 1, hz = g.nz / 2 + 1;
         const long long tn = (long long)hz * hy * g.nxh;
-        const long long trow = (long long)(ky <= g.ny / 2 ? ky : g.ny - ky) * g.nxh + kx0 + (col < ncol ? col : 0);
+        const long long trow = (long long)(c.row <= g.ny / 2 ? c.row : g.ny - c.row) * g.nxh + c.kx;
 #pragma unroll
         for (int t = 0; t < RL; ++t) {
             T Bm[3][3];
@@ -346,11 +342,11 @@ __global__ void __launch_bounds__(NT, elastic_min_blocks<T, PID, NT>())
             } else {
                 elastic_kernel<T>(pt, kxv, kyv, kval<T>(g, 2, j + t * M), Bm);
             }
-            const T2 a = h[0][t], b = h[1][t], c = h[2][t];
+            const T2 a0 = h[0][t], a1 = h[1][t], a2 = h[2][t];
 #pragma unroll
             for (int v = 0; v < 3; ++v)
-                h[v][t] = T2{(Bm[v][0] * a.x + Bm[v][1] * b.x + Bm[v][2] * c.x) * sc,
-                             (Bm[v][0] * a.y + Bm[v][1] * b.y + Bm[v][2] * c.y) * sc};
+                h[v][t] = T2{(Bm[v][0] * a0.x + Bm[v][1] * a1.x + Bm[v][2] * a2.x) * sc,
+                             (Bm[v][0] * a0.y + Bm[v][1] * a1.y + Bm[v][2] * a2.y) * sc};
         }
 #pragma unroll
         for (int f = 0; f < 3; ++f) {
@@ -365,8 +361,8 @@ __global__ void __launch_bounds__(NT, elastic_min_blocks<T, PID, NT>())
     tile_stages_inplace<+1, TX, N, RL, 3, NT>(S, tw, typename PlanInner<Inv>::type{});
     {
         auto ld = [&](int f, int kz, int col) -> T2 { return S[f * (N * TX) + kz * TX + col]; };
-        auto st = [&](int f, int kz, int col, T2 v) {
-            if (col < ncol) H[(long long)f * g.NK + rowoff + kz * zs + col] = v;
+        auto st = [&](int f, int kz, int, T2 v) {
+            if (c.ok) H[(long long)f * g.NK + rowoff + kz * zs] = v;
         };
         tile_stage_io<RF, +1, TX, N, N / RF, 3, NT>(tw, ld, st);
     }
@@ -391,14 +387,13 @@ __global__ void __launch_bounds__(NT) k_z_elastic_stages(Geo g, Phys ph, typenam
     constexpr int RF = RadInfo<Fwd>::first, RL = RadInfo<Fwd>::last;
     extern __shared__ __align__(16) unsigned char smraw[];
     T2* S = reinterpret_cast<T2*>(smraw);  // [3][N][TX]
-    const int ky = blockIdx.y, kx0 = blockIdx.x * TX;
-    const int ncol = min(TX, g.nxh - kx0);
-    const long long rowoff = (long long)ky * g.nxh + kx0;
+    const Column<TX> c(g.nxh, g.ny);
+    const long long rowoff = (long long)c.row * g.nxh + c.kx;
     const long long zs = (long long)g.ny * g.nxh;
     const T2* tw = twiddles<T2>(g.pz);
     {
-        auto ld = [&](int f, int kz, int col) -> T2 {
-            return col < ncol ? H[(long long)f * g.NK + rowoff + kz * zs + col] : T2{0, 0};
+        auto ld = [&](int f, int kz, int) -> T2 {
+            return c.ok ? H[(long long)f * g.NK + rowoff + kz * zs] : T2{0, 0};
         };
         auto st = [&](int f, int kz, int col, T2 v) { S[f * (N * TX) + kz * TX + col] = v; };
         tile_stage_io<RF, -1, TX, N, 1, 3, NT>(tw, ld, st);
@@ -409,18 +404,18 @@ __global__ void __launch_bounds__(NT) k_z_elastic_stages(Geo g, Phys ph, typenam
     {
         const T invN = std::is_same<T, float>::value ? (T)g.invN32 : (T)g.invN;
         const PhysT<T>& pt = phys_t<T>(ph);
-        const T kyv = kval<T>(g, 1, ky);
+        const T kxv = kval<T>(g, 0, c.kx), kyv = kval<T>(g, 1, c.row);
         const float* bt = sizeof(T) == 4 ? g.btab : nullptr;
         const int hy = g.ny / 2 + 1;
         const long long tn = (long long)(g.nz / 2 + 1) * hy * g.nxh;
-        const long long trow = (long long)(ky <= g.ny / 2 ? ky : g.ny - ky) * g.nxh + kx0;
+        const long long trow = (long long)(c.row <= g.ny / 2 ? c.row : g.ny - c.row) * g.nxh + c.kx;
         for (int e = threadIdx.x; e < N * TX; e += NT) {
-            const int kz = e / TX, col = e - kz * TX;
-            if (col >= ncol) continue;
+            const int kz = e / TX;
+            if (!c.ok) continue;
             T Bm[3][3];
             T sc = invN;
             if (bt) {
-                const long long ti = (long long)(kz <= g.nz / 2 ? kz : g.nz - kz) * hy * g.nxh + trow + col;
+                const long long ti = (long long)(kz <= g.nz / 2 ? kz : g.nz - kz) * hy * g.nxh + trow;
                 Bm[0][0] = (T)__ldg(bt + ti);
                 Bm[0][1] = Bm[1][0] = (T)__ldg(bt + tn + ti);
                 Bm[0][2] = Bm[2][0] = (T)__ldg(bt + 2 * tn + ti);
@@ -429,13 +424,13 @@ __global__ void __launch_bounds__(NT) k_z_elastic_stages(Geo g, Phys ph, typenam
                 Bm[2][2] = (T)__ldg(bt + 5 * tn + ti);
                 sc = (T)1;
             } else {
-                elastic_kernel<T>(pt, kval<T>(g, 0, kx0 + col), kyv, kval<T>(g, 2, kz), Bm);
+                elastic_kernel<T>(pt, kxv, kyv, kval<T>(g, 2, kz), Bm);
             }
-            const T2 a = S[e], b = S[N * TX + e], c = S[2 * N * TX + e];
+            const T2 a0 = S[e], a1 = S[N * TX + e], a2 = S[2 * N * TX + e];
 #pragma unroll
             for (int v = 0; v < 3; ++v)
-                S[v * N * TX + e] = T2{(Bm[v][0] * a.x + Bm[v][1] * b.x + Bm[v][2] * c.x) * sc,
-                                       (Bm[v][0] * a.y + Bm[v][1] * b.y + Bm[v][2] * c.y) * sc};
+                S[v * N * TX + e] = T2{(Bm[v][0] * a0.x + Bm[v][1] * a1.x + Bm[v][2] * a2.x) * sc,
+                                       (Bm[v][0] * a0.y + Bm[v][1] * a1.y + Bm[v][2] * a2.y) * sc};
         }
     }
     __syncthreads();
@@ -445,8 +440,8 @@ __global__ void __launch_bounds__(NT) k_z_elastic_stages(Geo g, Phys ph, typenam
     tile_stages_inplace<+1, TX, N, RL, 3, NT>(S, tw, typename PlanInner<Inv>::type{});
     {
         auto ld = [&](int f, int kz, int col) -> T2 { return S[f * (N * TX) + kz * TX + col]; };
-        auto st = [&](int f, int kz, int col, T2 v) {
-            if (col < ncol) H[(long long)f * g.NK + rowoff + kz * zs + col] = v;
+        auto st = [&](int f, int kz, int, T2 v) {
+            if (c.ok) H[(long long)f * g.NK + rowoff + kz * zs] = v;
         };
         tile_stage_io<RF, +1, TX, N, N / RF, 3, NT>(tw, ld, st);
     }
@@ -480,13 +475,13 @@ static bool launch_z_elastic_fused(const Geo& g, const Phys& ph, void* H, int tu
             if (fits(tx) && (TX == 0 || (tuned > 0 && tx == tuned))) TX = tx;
         if (tuned <= 0)
             for (int tx : {16, 8, 4, 2})
-                if (fits(tx) && tx / 2 < g.nxh) {
+                if (fits(tx)) {
                     TX = tx;
                     break;
                 }
         if (TX == 0) return false;
         const size_t sm = 3 * (size_t)TX * N * sizeof(T2);
-        dim3 grid((g.nxh + TX - 1) / TX, g.ny, 1);
+        const unsigned grid = column_tiles(g.nxh, g.ny, TX);
 #define PF_ELF(TXC)                                                                                       if constexpr ((TXC) * M <= 1024) {                                                                        set_smem(k_z_elastic_fused<T, TXC, PID, (TXC) * M>, sm);                                              k_z_elastic_fused<T, TXC, PID, (TXC) * M><<<grid, (TXC) * M, sm, s>>>(g, ph, reinterpret_cast<T2*>(H));     }
         switch (TX) {
             case 16: PF_ELF(16); break;
@@ -515,13 +510,13 @@ static bool launch_z_elastic_unf(const Geo& g, const Phys& ph, void* H, int tune
             if (fits(tx) && (TX == 0 || (tuned > 0 && tx == tuned))) TX = tx;
         if (tuned <= 0)
             for (int tx : {16, 8, 4, 2})
-                if (fits(tx) && tx / 2 < g.nxh) {
+                if (fits(tx)) {
                     TX = tx;
                     break;
                 }
         if (TX == 0) return false;
         const size_t sm = 3 * (size_t)TX * N * sizeof(T2);
-        dim3 grid((g.nxh + TX - 1) / TX, g.ny, 1);
+        const unsigned grid = column_tiles(g.nxh, g.ny, TX);
 #define PF_ELU(TXC)                                                                                   \
     {                                                                                                 \
         constexpr int NTU = elastic_stage_threads<PID, TXC>();                                        \
@@ -584,9 +579,9 @@ void launch_z_elastic(const Geo& g, const Phys& ph, void* H, cudaStream_t s) {
         }
     }
     if (done) return;
-    const int TX = tuned_cols<T>(g, g.tx_el, g.nz, 4, 128 * 1024);
+    const int TX = tuned_cols<T>(g.tx_el, g.nz, 4, 128 * 1024);
     const size_t sm = 4 * (size_t)TX * g.nz * sizeof(T2);
-    dim3 grid((g.nxh + TX - 1) / TX, g.ny, 1);
+    const unsigned grid = column_tiles(g.nxh, g.ny, TX);
     PF_COL_SWITCH8(T, g.pz, TX, set_smem(k_z_elastic<T, TXC, R16C, PIDC>, sm);
                   k_z_elastic<T, TXC, R16C, PIDC><<<grid, kThreads, sm, s>>>(g, ph, reinterpret_cast<T2*>(H)));
 }

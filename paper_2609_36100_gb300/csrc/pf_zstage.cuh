@@ -42,18 +42,18 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) k_z_stage(Ge
     extern __shared__ __align__(16) unsigned char smraw[];
     T2* A = reinterpret_cast<T2*>(smraw);
     T2* B = A + TX * g.nz;
-    const int f = blockIdx.z, ky = blockIdx.y, kx0 = blockIdx.x * TX;
-    const int ncol = min(TX, g.nxh - kx0);
-    const long long base = (long long)f * g.NK + (long long)ky * g.nxh + kx0;
+    const Column<TX> c(g.nxh, g.ny);
+    const int f = blockIdx.y;
+    const long long base = (long long)f * g.NK + (long long)c.row * g.nxh + c.kx;
     const long long zs = (long long)g.ny * g.nxh;
-    const double kyv = g.ky[ky];
+    const double kxv = g.kx[c.kx], kyv = g.ky[c.row];
     static_assert(sizeof(T) == 8, "the FP32-bulk form assembles its stages in k_stage_assemble_df");
-    auto src = [&](int kz, int col) -> T2 {
-        if (col >= ncol) return T2{0, 0};
-        const long long gi = base + kz * zs + col;
+    auto src = [&](int kz, int) -> T2 {
+        if (!c.ok) return T2{0, 0};
+        const long long gi = base + kz * zs;
         // every load first (independent, all in flight together), then the sums
         const double2 yv = __ldg(y + gi);
-        const double lam = lam_at(g, ph, f, gi, g.kx[kx0 + col], kyv, g.kz[kz]);
+        const double lam = lam_at(g, ph, f, gi, kxv, kyv, g.kz[kz]);
         const double qv = (st.has_gamma && st.qin) ? __ldg(st.qin + gi) : 1.0;
         const unsigned mz = st.mI & ~st.mY;
         double2 zv[kMaxStages], fv[kMaxStages];
@@ -84,8 +84,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) k_z_stage(Ge
         if (zout) zout[gi] = r;
         return r;
     };
-    auto dst = [&](int kz, int col, T2 v) {
-        if (col < ncol) W[base + kz * zs + col] = v;
+    auto dst = [&](int kz, int, T2 v) {
+        if (c.ok) W[base + kz * zs] = v;
     };
     // few terms: few registers per element, so several elements' loads go out together
     cols_fft<+1, TX, false, (MAXT == 0 ? 4 : (MAXT <= 2 ? 2 : 1)), R16, PID>(g.pz, A, B, src, dst);
@@ -95,9 +95,9 @@ template <typename T>
 void launch_z_stage(const Geo& g, const Phys& ph, const double2* y, const StageTerms& st, double2* zout, void* W,
                     cudaStream_t s) {
     using T2 = typename Cx<T>::t;
-    const int TX = tuned_cols<T>(g, g.tx_z, g.nz, 2, 128 * 1024);
+    const int TX = tuned_cols<T>(g.tx_z, g.nz, 2, 128 * 1024);
     const size_t sm = 2 * (size_t)TX * g.nz * sizeof(T2);
-    dim3 grid((g.nxh + TX - 1) / TX, g.ny, 4);
+    dim3 grid(column_tiles(g.nxh, g.ny, TX), 4);
     constexpr int MT = kMaxStages;
     PF_COL_SWITCH(T, g.pz, TX, set_smem(k_z_stage<T, TXC, R16C, PIDC, MT>, sm);
                   k_z_stage<T, TXC, R16C, PIDC, MT><<<grid, kThreads, sm, s>>>(g, ph, y, st, zout,
@@ -123,20 +123,20 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) k_z_final(Ge
     extern __shared__ __align__(16) unsigned char smraw[];
     T2* A = reinterpret_cast<T2*>(smraw);
     T2* B = A + TX * g.nz;
-    const int f = blockIdx.z, ky = blockIdx.y, kx0 = blockIdx.x * TX;
-    const int ncol = min(TX, g.nxh - kx0);
-    const long long base = (long long)f * g.NK + (long long)ky * g.nxh + kx0;
+    const Column<TX> c(g.nxh, g.ny);
+    const int f = blockIdx.y;
+    const long long base = (long long)f * g.NK + (long long)c.row * g.nxh + c.kx;
     const long long zs = (long long)g.ny * g.nxh;
-    const double kyv = g.ky[ky];
+    const double kxv = g.kx[c.kx], kyv = g.ky[c.row];
     static_assert(sizeof(T) == 8, "the FP32-bulk form completes its steps in k_step_complete_df");
-    auto combine = [&](int kz, int col) -> T2 {
-        if (col >= ncol) return T2{0, 0};
-        const long long gi = base + kz * zs + col;
+    auto combine = [&](int kz, int) -> T2 {
+        if (!c.ok) return T2{0, 0};
+        const long long gi = base + kz * zs;
         const unsigned lmI = want_lte ? dt.mI : 0u, lmE = want_lte ? dt.mE : 0u;
         const unsigned mI = bt.mI | lmI, mE = bt.mE | lmE, mz = mI & ~bt.mY;
         // every load first, then the sums
         const double2 yv = __ldg(y + gi);
-        const double lam = lam_at(g, ph, f, gi, g.kx[kx0 + col], kyv, g.kz[kz]);
+        const double lam = lam_at(g, ph, f, gi, kxv, kyv, g.kz[kz]);
         double2 zv[kMaxStages], fv[kMaxStages];
 #pragma unroll
         for (int j = 0; j < kMaxStages; ++j) {
@@ -168,8 +168,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) k_z_final(Ge
         for (int e = threadIdx.x; e < TX * g.nz; e += blockDim.x) combine(e / TX, e & (TX - 1));
         return;
     }
-    auto dst = [&](int kz, int col, T2 v) {
-        if (col < ncol) W[base + kz * zs + col] = v;
+    auto dst = [&](int kz, int, T2 v) {
+        if (c.ok) W[base + kz * zs] = v;
     };
     cols_fft<+1, TX, false, 1, R16, PID>(g.pz, A, B, combine, dst);
 }
@@ -178,9 +178,9 @@ template <typename T>
 void launch_z_final(const Geo& g, const Phys& ph, const double2* y, const StageTerms& bterm, const StageTerms& dterm,
                     int want_lte, double2* ynew, void* W, cudaStream_t s) {
     using T2 = typename Cx<T>::t;
-    const int TX = tuned_cols<T>(g, g.tx_z, g.nz, 2, 128 * 1024);
+    const int TX = tuned_cols<T>(g.tx_z, g.nz, 2, 128 * 1024);
     const size_t sm = 2 * (size_t)TX * g.nz * sizeof(T2);
-    dim3 grid((g.nxh + TX - 1) / TX, g.ny, 4);
+    dim3 grid(column_tiles(g.nxh, g.ny, TX), 4);
     PF_COL_SWITCH(T, g.pz, TX, set_smem(k_z_final<T, TXC, R16C, PIDC>, sm);
                   k_z_final<T, TXC, R16C, PIDC><<<grid, kThreads, sm, s>>>(g, ph, y, bterm, dterm, want_lte, ynew,
                                                                         reinterpret_cast<T2*>(W)));
