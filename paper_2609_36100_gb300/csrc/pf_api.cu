@@ -214,7 +214,7 @@ struct pf_ctx {
     void* R1 = nullptr;
     double* lam = nullptr;   // [4][NK] lambda(k), FP64
     float2* lamdf = nullptr;  // [4][NK] lambda(k), double-float (FP32-bulk contexts)
-    float* btab = nullptr;    // FP32 elastic-kernel table (FP32-bulk contexts with diagonal eigenstrains)
+    void* btab = nullptr;     // elastic-kernel table in the compute type (diagonal eigenstrains)
     double2* xsave = nullptr;  // the composition's k-space field across the obstacle projection (barrier = 1)
     double* qtab = nullptr;  // [4][NK] 1/(1 - dt gamma lambda) of the current step (ESDIRK diagonal)
     double gdiag = 0.0;      // common nonzero implicit diagonal entry, or 0
@@ -301,6 +301,10 @@ void typed_phys(const Phys& ph, double invN, PhysT<T>& o) {
     o.obst = ph.obst;
     o.ie = (T)(1.0 / ph.pair_eps);
     o.twoAm = (T)(2.0 * ph.Am);
+    o.dB = (T)(ph.Bv - ph.Bm);
+    o.dinv = (T)(ph.inv2Av - ph.inv2Am);
+    o.dA0 = (T)(ph.A0v - ph.A0m);
+    o.dq = (T)(0.25 / ph.Am - 0.25 / ph.Av);
     o.C44 = (T)ph.C44;
     o.Cm = (T)ph.Cmix;
     o.Ca = (T)ph.Caniso;
@@ -948,15 +952,15 @@ int pf_create(const pf_grid* grid, const pf_params* params, void* cuda_stream, p
     rc = rc ? rc : dalloc(c, &c->R1, 4 * (size_t)g.N * tsz);
     rc = rc ? rc : dalloc(c, &c->lam, nk4 * sizeof(double));
     if (c->fp32) rc = rc ? rc : dalloc(c, &c->lamdf, nk4 * sizeof(float2));
-    // elastic-kernel table: FP32-bulk, homogeneous modulus, diagonal
-    // eigenstrains (B even in each wave-number component), at most 1 GB (794 MB
-    // at 640^3)
+    // elastic-kernel table: homogeneous modulus, diagonal eigenstrains (B even
+    // in each wave-number component), at most 1 GB (FP32: 794 MB at 640^3; FP64:
+    // 103 MB at 256^3)
     bool diag = true;
     for (int v = 0; v < 3; ++v)
         for (int a = 3; a < 6; ++a) diag = diag && params->eps_star[v][a] == 0.0;
     const long long tabn = (long long)(g.nz / 2 + 1) * (g.ny / 2 + 1) * g.nxh;
-    if (c->fp32 && c->ph.elastic && !c->inhom && diag && 6 * tabn * (long long)sizeof(float) <= (1LL << 30))
-        rc = rc ? rc : dalloc(c, &c->btab, 6 * (size_t)tabn * sizeof(float));
+    if (c->ph.elastic && !c->inhom && diag && 6 * tabn * (long long)tsz <= (1LL << 30))
+        rc = rc ? rc : dalloc(c, &c->btab, 6 * (size_t)tabn * tsz);
     rc = rc ? rc : dalloc(c, &c->qtab, nk4 * sizeof(double));
     if (params->barrier == 1) rc = rc ? rc : dalloc(c, &c->xsave, (size_t)g.NK * sizeof(double2));
     // worst case over any tuned rows-per-CTA setting (one row pair per CTA)
@@ -1025,7 +1029,7 @@ int pf_create(const pf_grid* grid, const pf_params* params, void* cuda_stream, p
             g.lam2 = same ? 1 : 0;
         }
         launch_lambda_table(g, c->ph, c->lam, c->lamdf, c->stream);
-        if (c->btab) launch_btab(g, c->ph, c->btab, c->stream);
+        if (c->btab) launch_btab(g, c->ph, c->btab, !c->fp32, c->stream);
         e = cudaGetLastError();
         g.lam = c->lam;
         g.lamdf = c->lamdf;

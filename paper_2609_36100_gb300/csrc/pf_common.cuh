@@ -270,10 +270,15 @@ static int strided_tile(int n, int nbuf, int budget) {
     return tx;
 }
 
-// tuned width (0 = untuned) capped by what fits the shared-memory budget
+// tuned width (0 = untuned) capped by what fits the shared-memory budget;
+// untuned, the widest up to 16, but 8 where tiles of 16 of the `cols` columns
+// are fewer than two an SM
 template <typename T>
-static int tuned_cols(int tuned, int n, int nbuf, int budget) {
-    if (tuned <= 0) return strided_tile<T>(n, nbuf, nbuf == 4 ? 64 * 1024 : 96 * 1024);
+static int tuned_cols(int tuned, int n, int nbuf, int budget, long long cols) {
+    if (tuned <= 0) {
+        const int tx = strided_tile<T>(n, nbuf, nbuf == 4 ? 64 * 1024 : 96 * 1024);
+        return tx == 16 && cols < 2LL * 152 * 16 ? 8 : tx;
+    }
     const int cap = strided_tile<T>(n, nbuf, budget);
     int tx = 1;
     while (tx * 2 <= tuned && tx * 2 <= 16) tx *= 2;

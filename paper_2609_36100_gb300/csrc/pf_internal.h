@@ -66,8 +66,8 @@ struct Geo {
     int el_unfused;          // form of the compiled-plan elastic pass: 0 fuses the last forward / first inverse
                              // stage, 1 runs every stage (and the contraction) over the three fields in place,
                              // 2 runs a cluster of three CTAs, one field each (FP32 contexts)
-    const float* btab;       // FP32 elastic kernel B(k) / N over kx >= 0, |ky| <= ny/2, |kz| <= nz/2 (six
-                             // symmetric entries, [6][nz/2+1][ny/2+1][nx/2+1]), or null: computed per k
+    const void* btab;        // elastic kernel B(k) / N in the compute type over kx >= 0, |ky| <= ny/2, |kz| <= nz/2
+                             // (six symmetric entries, [6][nz/2+1][ny/2+1][nx/2+1]), or null: computed per k
 };
 
 // Model constants of the real-space and elastic terms in one compute type,
@@ -82,6 +82,11 @@ struct PhysT {
     int obst; // 1: the literal obstacle barrier omega_bar S (1 - S)
     T ie;     // 1 / pair_eps
     T twoAm;  // 2 A^m
+    // the KKS potential and driving force with the constants gathered
+    T dB;     // B^v - B^m
+    T dinv;   // 1/(2 A^v) - 1/(2 A^m), 0 with equal curvatures
+    T dA0;    // A0^v - A0^m
+    T dq;     // 1/(4 A^m) - 1/(4 A^v)
     T w[3][3];
     T C44, Cm, Ca;
     T sig[3][6];
@@ -232,7 +237,8 @@ void launch_solve(const Geo& g, const Phys& ph, double gamma, const double2* r, 
 void launch_lambda_table(const Geo& g, const Phys& ph, double* lam, float2* lamdf, cudaStream_t s);
 // FP32 table of the elastic kernel B_vq(k)/N (diagonal eigenstrains: B is
 // even in each wave-number component, so |ky| and |kz| index it)
-void launch_btab(const Geo& g, const Phys& ph, float* btab, cudaStream_t s);
+// table of the elastic kernel in double (fp64) or float
+void launch_btab(const Geo& g, const Phys& ph, void* btab, bool fp64, cudaStream_t s);
 void launch_clamp_phi(double* real, long long N, cudaStream_t s);
 // FP32-bulk stage assembly as a streaming pass (double-float z_i out, FP32
 // transform input W out); the inverse z transform follows as launch_z_pass

@@ -241,9 +241,10 @@ __global__ void k_lambda_table(Geo g, Phys ph, double* __restrict__ lam, float2*
     }
 }
 
-// B_vq(k) / N in FP64, rounded to FP32, over kx in [0, nx/2], ky, kz in
+// B_vq(k) / N in FP64, rounded to T, over kx in [0, nx/2], ky, kz in
 // [0, n/2] (the kernel is even in each component for diagonal eigenstrains)
-__global__ void k_btab(Geo g, Phys ph, float* __restrict__ tab) {
+template <typename T>
+__global__ void k_btab(Geo g, Phys ph, T* __restrict__ tab) {
     const int hy = g.ny / 2 + 1, hz = g.nz / 2 + 1;
     const long long n = (long long)hz * hy * g.nxh;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -253,17 +254,20 @@ __global__ void k_btab(Geo g, Phys ph, float* __restrict__ tab) {
         double Bm[3][3];
         elastic_kernel<double>(ph.t64, g.kx[kx], g.ky[ky], g.kz[kz], Bm);
         const double s = g.invN;
-        tab[0 * n + i] = (float)(Bm[0][0] * s);
-        tab[1 * n + i] = (float)(Bm[0][1] * s);
-        tab[2 * n + i] = (float)(Bm[0][2] * s);
-        tab[3 * n + i] = (float)(Bm[1][1] * s);
-        tab[4 * n + i] = (float)(Bm[1][2] * s);
-        tab[5 * n + i] = (float)(Bm[2][2] * s);
+        tab[0 * n + i] = (T)(Bm[0][0] * s);
+        tab[1 * n + i] = (T)(Bm[0][1] * s);
+        tab[2 * n + i] = (T)(Bm[0][2] * s);
+        tab[3 * n + i] = (T)(Bm[1][1] * s);
+        tab[4 * n + i] = (T)(Bm[1][2] * s);
+        tab[5 * n + i] = (T)(Bm[2][2] * s);
     }
 }
 
-void launch_btab(const Geo& g, const Phys& ph, float* btab, cudaStream_t s) {
-    k_btab<<<152 * 8, 256, 0, s>>>(g, ph, btab);
+void launch_btab(const Geo& g, const Phys& ph, void* btab, bool fp64, cudaStream_t s) {
+    if (fp64)
+        k_btab<<<152 * 8, 256, 0, s>>>(g, ph, static_cast<double*>(btab));
+    else
+        k_btab<<<152 * 8, 256, 0, s>>>(g, ph, static_cast<float*>(btab));
 }
 
 // the obstacle barrier's bound: real-space order parameters (fields 1-3 of a

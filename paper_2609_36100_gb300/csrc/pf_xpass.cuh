@@ -22,28 +22,46 @@ __device__ __forceinline__ T xdiv(T a, T b) {
         return a / b;
 }
 
+// x clipped to [-1, 1]; in FP64 by the exponent field, off the FP64 pipe
+// (two FP64 comparisons a value there).  A NaN stays a NaN in FP64; every term
+// it meets is one already.
+template <typename T>
+__device__ __forceinline__ T clip1(T x) {
+    if constexpr (sizeof(T) == 4) {
+        return fminf(1.f, fmaxf(-1.f, x));
+    } else {
+        const int hi = __double2hiint(x), mag = hi & 0x7fffffff;
+        const bool clip = mag >= 0x3ff00000 && (mag < 0x7ff00000 || (mag == 0x7ff00000 && __double2loint(x) == 0));
+        return clip ? __hiloint2double((hi & (int)0x80000000) | 0x3ff00000, 0) : x;
+    }
+}
+
 struct Pt {
     // real-space physics at one point (Sec. 4.1); returns q and g_v.  OBST:
     // the literal obstacle barrier instead of the double well (a compile-time
-    // choice, so that the default path carries none of its instructions)
+    // choice, so that the default path carries none of its instructions).
+    // With X^p - B^p = mu / (2 A^p) the driving force f^v - f^m - mu (X^v - X^m)
+    // is dA0 - mu dB + dq mu^2 (dq = 1/(4 A^m) - 1/(4 A^v)), and the pairwise
+    // barrier's clipped products are shared by both variants of a pair: the
+    // FP64 passes run at the FP64 pipe's rate, the FP32 ones at the issue rate.
     template <typename T, bool OBST = false>
     __device__ __forceinline__ static void rhs(const PhysT<T>& pt, T X, const T* p, const T* e, T& q, T* gv) {
         T h[3], hp[3];
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
-            const T f = p[v];
-            h[v] = f * f * f * ((T)6 * f * f - (T)15 * f + (T)10);
-            hp[v] = (T)30 * f * f * ((T)1 - f) * ((T)1 - f);
+            const T f = p[v], f2 = f * f, u = (T)1 - f;
+            h[v] = f2 * f * (f * ((T)6 * f - (T)15) + (T)10);
+            hp[v] = (T)30 * f2 * (u * u);
         }
         const T H = h[0] + h[1] + h[2];
-        const T Bv = pt.Bv, Bm = pt.Bm;
-        const T denom = H * pt.inv2Av + ((T)1 - H) * pt.inv2Am;
-        const T mu = xdiv<T>(X - H * Bv - ((T)1 - H) * Bm, denom);
-        const T Xm = mu * pt.inv2Am + Bm;
-        const T Xv = mu * pt.inv2Av + Bv;
-        const T fm = pt.A0m + pt.Am * (Xm - Bm) * (Xm - Bm);
-        const T fv = pt.A0v + pt.Av * (Xv - Bv) * (Xv - Bv);
-        const T drive = fv - fm - mu * (Xv - Xm);
+        const T num = X - pt.Bm - H * pt.dB;
+        // equal curvatures (the same for every point): the denominator is 1/(2 A^m)
+        const T mu = pt.dinv == (T)0 ? num * pt.twoAm : xdiv<T>(num, pt.inv2Am + H * pt.dinv);
+        const T drive = pt.dA0 + mu * (pt.dq * mu - pt.dB);
+        const T s01 = pt.w[0][1] * clip1<T>(p[0] * p[1] * pt.ie);
+        const T s02 = pt.w[0][2] * clip1<T>(p[0] * p[2] * pt.ie);
+        const T s12 = pt.w[1][2] * clip1<T>(p[1] * p[2] * pt.ie);
+        const T pair[3] = {s01 * p[1] + s02 * p[2], s01 * p[0] + s12 * p[2], s02 * p[0] + s12 * p[1]};
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
             const T f = p[v];
@@ -52,20 +70,14 @@ struct Pt {
                 d = pt.wb * ((T)1 - (T)2 * (p[0] + p[1] + p[2]));  // d/dphi_v of omega_bar S (1 - S)
             else
                 d = pt.wb2 * f * ((T)1 - f) * ((T)1 - (T)2 * f);
-#pragma unroll
-            for (int qq = 0; qq < 3; ++qq)
-                if (qq != v) {
-                    const T sl = fmin((T)1, fmax((T)-1, f * p[qq] * pt.ie));
-                    d += pt.w[v][qq] * sl * p[qq];
-                }
-            gv[v] = d + hp[v] * drive + hp[v] * e[v];
+            gv[v] = d + pair[v] + hp[v] * (drive + e[v]);
         }
         q = mu - pt.twoAm * X;
     }
 };
 
 template <typename T>
-__device__ __forceinline__ T hfun(T f) { return f * f * f * ((T)6 * f * f - (T)15 * f + (T)10); }
+__device__ __forceinline__ T hfun(T f) { return f * f * f * (f * ((T)6 * f - (T)15) + (T)10); }
 
 // line length nx and half-spectrum length nx/2+1 along x, compile-time when
 // NX > 0, and the divisions by them

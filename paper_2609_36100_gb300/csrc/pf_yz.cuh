@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(kThreads) k_y_pass(Geo g, typename Cx<T>::t* _
 template <typename T>
 void launch_y_pass(const Geo& g, void* buf, int nf, int sign, cudaStream_t s) {
     using T2 = typename Cx<T>::t;
-    const int TX = tuned_cols<T>(g.tx_y, g.ny, 2, 128 * 1024);
+    const int TX = tuned_cols<T>(g.tx_y, g.ny, 2, 128 * 1024, (long long)nf * g.nz * g.nxh);
     // a transform of at most two stages never touches its second buffer
     // (stage 0 reads global, the last stage writes global), and a compiled
     // plan runs its middle stages in place: half the shared memory, more
@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kThreads) k_z_pass(Geo g, typename Cx<T>::t* _
 template <typename T>
 void launch_z_pass(const Geo& g, void* buf, int nf, int sign, cudaStream_t s) {
     using T2 = typename Cx<T>::t;
-    const int TX = tuned_cols<T>(g.tx_zf, g.nz, 2, 128 * 1024);
+    const int TX = tuned_cols<T>(g.tx_zf, g.nz, 2, 128 * 1024, (long long)nf * g.ny * g.nxh);
     const size_t sm = col_buffers<T>(g.pz, TX) * (size_t)TX * g.nz * sizeof(T2);  // as in the y pass
     dim3 grid(column_tiles(g.nxh, g.ny, TX), nf);
     if (sign > 0) {
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kThreads) k_z_fwd(Geo g, Phys ph, const typena
 template <typename T>
 void launch_z_fwd(const Geo& g, const Phys& ph, const void* W, void* out, int scale_mode, cudaStream_t s, int nf) {
     using T2 = typename Cx<T>::t;
-    const int TX = tuned_cols<T>(g.tx_zf, g.nz, 2, 128 * 1024);
+    const int TX = tuned_cols<T>(g.tx_zf, g.nz, 2, 128 * 1024, (long long)nf * g.ny * g.nxh);
     // modes 0/2 run the generic stages (two buffers for three or more stages)
     const size_t sm = (scale_mode == 1 ? col_buffers<T>(g.pz, TX) : (g.pz.nst <= 2 ? 1 : 2)) * (size_t)TX * g.nz *
                       sizeof(T2);
@@ -178,8 +178,10 @@ __global__ void __launch_bounds__(kThreads) k_z_elastic(Geo g, Phys ph, typename
     const T invN = std::is_same<T, float>::value ? (T)g.invN32 : (T)g.invN;
     const PhysT<T>& pt = phys_t<T>(ph);
     const T kxv = kval<T>(g, 0, c.kx), kyv = kval<T>(g, 1, c.row);
-    // FP32 contexts with diagonal eigenstrains read B/N from the octant table
-    const float* bt = sizeof(T) == 4 ? g.btab : nullptr;
+    // contexts with diagonal eigenstrains read B/N from the octant table (formed
+    // per wave vector in FP64 it was more than half of the pass: 94 of 168 FP64
+    // instructions a point)
+    const T* bt = static_cast<const T*>(g.btab);
     const int hy = g.ny / 2 + 1;
     const long long tn = (long long)(g.nz / 2 + 1) * hy * g.nxh;
     const long long trow = (long long)(c.row <= g.ny / 2 ? c.row : g.ny - c.row) * g.nxh + c.kx;
@@ -190,12 +192,12 @@ __global__ void __launch_bounds__(kThreads) k_z_elastic(Geo g, Phys ph, typename
         T sc = invN;
         if (bt) {
             const long long ti = (long long)(kz <= g.nz / 2 ? kz : g.nz - kz) * hy * g.nxh + trow;
-            Bm[0][0] = (T)__ldg(bt + ti);
-            Bm[0][1] = Bm[1][0] = (T)__ldg(bt + tn + ti);
-            Bm[0][2] = Bm[2][0] = (T)__ldg(bt + 2 * tn + ti);
-            Bm[1][1] = (T)__ldg(bt + 3 * tn + ti);
-            Bm[1][2] = Bm[2][1] = (T)__ldg(bt + 4 * tn + ti);
-            Bm[2][2] = (T)__ldg(bt + 5 * tn + ti);
+            Bm[0][0] = __ldg(bt + ti);
+            Bm[0][1] = Bm[1][0] = __ldg(bt + tn + ti);
+            Bm[0][2] = Bm[2][0] = __ldg(bt + 2 * tn + ti);
+            Bm[1][1] = __ldg(bt + 3 * tn + ti);
+            Bm[1][2] = Bm[2][1] = __ldg(bt + 4 * tn + ti);
+            Bm[2][2] = __ldg(bt + 5 * tn + ti);
             sc = (T)1;
         } else {
             elastic_kernel<T>(pt, kxv, kyv, kval<T>(g, 2, kz), Bm);
@@ -319,9 +321,9 @@ __global__ void __launch_bounds__(NT, elastic_min_blocks<T, PID, NT>())
         const T invN = std::is_same<T, float>::value ? (T)g.invN32 : (T)g.invN;
         const PhysT<T>& pt = phys_t<T>(ph);
         const T kxv = kval<T>(g, 0, c.kx), kyv = kval<T>(g, 1, c.row);
-        // FP32 contexts with diagonal eigenstrains read B/N from the table
-        // (held in L2 across the tiles); otherwise B is formed per wave vector
-        const float* bt = sizeof(T) == 4 ? g.btab : nullptr;
+        // contexts with diagonal eigenstrains read B/N from the table (held in
+        // L2 across the tiles); otherwise B is formed per wave vector
+        const T* bt = static_cast<const T*>(g.btab);
         const int hy = g.ny / 2 + 1, hz = g.nz / 2 + 1;
         const long long tn = (long long)hz * hy * g.nxh;
         const long long trow = (long long)(c.row <= g.ny / 2 ? c.row : g.ny - c.row) * g.nxh + c.kx;
@@ -332,12 +334,12 @@ __global__ void __launch_bounds__(NT, elastic_min_blocks<T, PID, NT>())
             if (bt) {
                 const int kz = j + t * M;
                 const long long ti = (long long)(kz <= g.nz / 2 ? kz : g.nz - kz) * hy * g.nxh + trow;
-                Bm[0][0] = (T)__ldg(bt + ti);
-                Bm[0][1] = Bm[1][0] = (T)__ldg(bt + tn + ti);
-                Bm[0][2] = Bm[2][0] = (T)__ldg(bt + 2 * tn + ti);
-                Bm[1][1] = (T)__ldg(bt + 3 * tn + ti);
-                Bm[1][2] = Bm[2][1] = (T)__ldg(bt + 4 * tn + ti);
-                Bm[2][2] = (T)__ldg(bt + 5 * tn + ti);
+                Bm[0][0] = __ldg(bt + ti);
+                Bm[0][1] = Bm[1][0] = __ldg(bt + tn + ti);
+                Bm[0][2] = Bm[2][0] = __ldg(bt + 2 * tn + ti);
+                Bm[1][1] = __ldg(bt + 3 * tn + ti);
+                Bm[1][2] = Bm[2][1] = __ldg(bt + 4 * tn + ti);
+                Bm[2][2] = __ldg(bt + 5 * tn + ti);
                 sc = (T)1;
             } else {
                 elastic_kernel<T>(pt, kxv, kyv, kval<T>(g, 2, j + t * M), Bm);
@@ -405,7 +407,7 @@ __global__ void __launch_bounds__(NT) k_z_elastic_stages(Geo g, Phys ph, typenam
         const T invN = std::is_same<T, float>::value ? (T)g.invN32 : (T)g.invN;
         const PhysT<T>& pt = phys_t<T>(ph);
         const T kxv = kval<T>(g, 0, c.kx), kyv = kval<T>(g, 1, c.row);
-        const float* bt = sizeof(T) == 4 ? g.btab : nullptr;
+        const T* bt = static_cast<const T*>(g.btab);
         const int hy = g.ny / 2 + 1;
         const long long tn = (long long)(g.nz / 2 + 1) * hy * g.nxh;
         const long long trow = (long long)(c.row <= g.ny / 2 ? c.row : g.ny - c.row) * g.nxh + c.kx;
@@ -416,12 +418,12 @@ __global__ void __launch_bounds__(NT) k_z_elastic_stages(Geo g, Phys ph, typenam
             T sc = invN;
             if (bt) {
                 const long long ti = (long long)(kz <= g.nz / 2 ? kz : g.nz - kz) * hy * g.nxh + trow;
-                Bm[0][0] = (T)__ldg(bt + ti);
-                Bm[0][1] = Bm[1][0] = (T)__ldg(bt + tn + ti);
-                Bm[0][2] = Bm[2][0] = (T)__ldg(bt + 2 * tn + ti);
-                Bm[1][1] = (T)__ldg(bt + 3 * tn + ti);
-                Bm[1][2] = Bm[2][1] = (T)__ldg(bt + 4 * tn + ti);
-                Bm[2][2] = (T)__ldg(bt + 5 * tn + ti);
+                Bm[0][0] = __ldg(bt + ti);
+                Bm[0][1] = Bm[1][0] = __ldg(bt + tn + ti);
+                Bm[0][2] = Bm[2][0] = __ldg(bt + 2 * tn + ti);
+                Bm[1][1] = __ldg(bt + 3 * tn + ti);
+                Bm[1][2] = Bm[2][1] = __ldg(bt + 4 * tn + ti);
+                Bm[2][2] = __ldg(bt + 5 * tn + ti);
                 sc = (T)1;
             } else {
                 elastic_kernel<T>(pt, kxv, kyv, kval<T>(g, 2, kz), Bm);
@@ -579,7 +581,7 @@ void launch_z_elastic(const Geo& g, const Phys& ph, void* H, cudaStream_t s) {
         }
     }
     if (done) return;
-    const int TX = tuned_cols<T>(g.tx_el, g.nz, 4, 128 * 1024);
+    const int TX = tuned_cols<T>(g.tx_el, g.nz, 4, 128 * 1024, (long long)g.ny * g.nxh);
     const size_t sm = 4 * (size_t)TX * g.nz * sizeof(T2);
     const unsigned grid = column_tiles(g.nxh, g.ny, TX);
     PF_COL_SWITCH8(T, g.pz, TX, set_smem(k_z_elastic<T, TXC, R16C, PIDC>, sm);

@@ -66,7 +66,7 @@ __global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(NT, elastic_cluster_
         const float invN = g.invN32;
         const PhysT<float>& pt = phys_t<float>(ph);
         const float kyv = kval<float>(g, 1, ky);
-        const float* bt = g.btab;
+        const float* bt = static_cast<const float*>(g.btab);
         const int hy = g.ny / 2 + 1;
         const long long tn = (long long)(g.nz / 2 + 1) * hy * g.nxh;
         const long long trow = (long long)(ky <= g.ny / 2 ? ky : g.ny - ky) * g.nxh + kx0;

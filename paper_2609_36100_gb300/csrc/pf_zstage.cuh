@@ -95,7 +95,7 @@ template <typename T>
 void launch_z_stage(const Geo& g, const Phys& ph, const double2* y, const StageTerms& st, double2* zout, void* W,
                     cudaStream_t s) {
     using T2 = typename Cx<T>::t;
-    const int TX = tuned_cols<T>(g.tx_z, g.nz, 2, 128 * 1024);
+    const int TX = tuned_cols<T>(g.tx_z, g.nz, 2, 128 * 1024, 4LL * g.ny * g.nxh);
     const size_t sm = 2 * (size_t)TX * g.nz * sizeof(T2);
     dim3 grid(column_tiles(g.nxh, g.ny, TX), 4);
     constexpr int MT = kMaxStages;
@@ -178,7 +178,7 @@ template <typename T>
 void launch_z_final(const Geo& g, const Phys& ph, const double2* y, const StageTerms& bterm, const StageTerms& dterm,
                     int want_lte, double2* ynew, void* W, cudaStream_t s) {
     using T2 = typename Cx<T>::t;
-    const int TX = tuned_cols<T>(g.tx_z, g.nz, 2, 128 * 1024);
+    const int TX = tuned_cols<T>(g.tx_z, g.nz, 2, 128 * 1024, 4LL * g.ny * g.nxh);
     const size_t sm = 2 * (size_t)TX * g.nz * sizeof(T2);
     dim3 grid(column_tiles(g.nxh, g.ny, TX), 4);
     PF_COL_SWITCH(T, g.pz, TX, set_smem(k_z_final<T, TXC, R16C, PIDC>, sm);
