@@ -253,7 +253,7 @@ const char* pf_kernel_name(int kind);
 /* Launch schedule of a context: tuned tile widths of the z stage-assembly
  * and completion / y / elastic passes, rows per CTA of the x passes (0 =
  * built-in heuristic), the radix order of each axis (count + up to 10 radices
- * in {2,3,4,5,8,16}, for x, y, z: ints 4-36), the tile width of the forward
+ * in {2,3,4,5,6,8,9,10,12,15,16}, for x, y, z: ints 4-36), the tile width of the forward
  * z pass (int 37), the compiled radix plan of the elastic pass (int 38;
  * 0 = the z axis's own plan, -1 = no compiled elastic plan: the z axis's
  * column transforms, one field after another), whether the FP32 x passes run the staged kernel instead of the
@@ -262,9 +262,10 @@ const char* pf_kernel_name(int kind);
  * transform stage and the contraction over the three fields in place, 2 runs
  * a cluster of three CTAs, one h field each, sharing the contraction through
  * distributed shared memory; FP32 contexts, FP64 contexts run 0 for 2;
- * other values are refused with PF_EINVAL), whether the FP32 fused x pass of the right-hand side copies its stored
- * real fields into shared memory with its input rows (int 41) and whether the
- * FP32 fused x passes run every stage in place in one shared buffer (int 42).
+ * other values are refused with PF_EINVAL; the compiled plans of the common
+ * sizes beyond the first eleven have form 1 only, at its own tile width).  Ints
+ * 41 and 42 once chose other forms of the FP32 fused x passes; they are kept
+ * as they are set, and every value runs the one form there is.
  * PF_TUNE_LEN ints. */
 #define PF_TUNE_LEN 43
 int pf_get_tuning(pf_ctx* ctx, int* cfg, int n);

@@ -16,10 +16,11 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libpf.so")
-SOURCES = ["pf_zelastic.cu", "pf_zfwd.cu", "pf_ypass.cu", "pf_xpass_f32.cu", "pf_xpass_f64.cu",
-           "pf_zfinal_f64.cu", "pf_zstage_f64.cu", "pf_fno.cu", "pf_api.cu", "pf_misc.cu",
-           "pf_plan.cu", "pf_noalloc.cu", "pf_hc.cu", "pf_zelastic_unf.cu",
-           "pf_zelastic_cl.cu", "pf_fno_fused.cu"]
+SOURCES = ["pf_zelastic.cu", "pf_zelastic_f64.cu", "pf_zelastic_unf.cu", "pf_zfwd.cu", "pf_zpass.cu",
+           "pf_ypass_fwd.cu", "pf_ypass_inv.cu", "pf_ypass.cu", "pf_xfused_a.cu", "pf_xfused_b.cu",
+           "pf_xfused_c.cu", "pf_xfused_d.cu", "pf_xpass_f32.cu", "pf_xpass_f64.cu", "pf_fno_fused.cu",
+           "pf_zelastic_cl.cu", "pf_zfinal_f64.cu", "pf_zstage_f64.cu", "pf_fno.cu", "pf_api.cu", "pf_misc.cu",
+           "pf_plan.cu", "pf_noalloc.cu", "pf_hc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

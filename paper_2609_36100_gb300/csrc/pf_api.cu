@@ -615,7 +615,7 @@ int enqueue_step(pf_ctx* c, double dt, bool want_lte, const StageCoefDev* dcoef 
             }
             {
                 ProfScope p(c, PF_K_Z_IFFT, 4 * NK * 2 * cb);
-                launch_z_pass<T>(g, c->W, 4, +1, s);
+                launch_z_pass<T>(g, c->W, 4, s);
             }
         } else {
             ProfScope p(c, PF_K_Z_STAGE, 4 * NK * (16.0 + terms + (zout ? 16.0 : 0.0) + cb));
@@ -711,7 +711,7 @@ int enqueue_step(pf_ctx* c, double dt, bool want_lte, const StageCoefDev* dcoef 
         }
         if (lte) {
             ProfScope p(c, PF_K_Z_IFFT, 4 * NK * 2 * cb);
-            launch_z_pass<T>(g, c->W, 4, +1, s);
+            launch_z_pass<T>(g, c->W, 4, s);
         }
     } else {
         ProfScope p(c, PF_K_Z_FINAL, 4 * NK * (16.0 + fterms + 16.0 + (lte ? cb : 0.0)));
@@ -785,7 +785,7 @@ int rhs_explicit_t(pf_ctx* c, const double2* yh, double2* out) {
     StageTerms none{};
     if constexpr (sizeof(T) == 4) {
         launch_stage_assemble(g, yh, none, nullptr, c->W, s);
-        launch_z_pass<T>(g, c->W, 4, +1, s);
+        launch_z_pass<T>(g, c->W, 4, s);
     } else {
         launch_z_stage<T>(g, ph, yh, none, nullptr, c->W, s);
     }
@@ -929,6 +929,11 @@ int pf_create(const pf_grid* grid, const pf_params* params, void* cuda_stream, p
             delete c;
             return fail(nullptr, PF_EUNSUPPORTED, "cannot factor %d", ns[a]);
         }
+    }
+    // schedule slots as they run untuned (see pf_get_tuning)
+    if (c->fp32) {
+        g.el_unfused = default_elastic_form(g.pz);
+        g.el_pid = default_elastic_plan(g.pz);
     }
     const size_t nk4 = 4 * (size_t)g.NK;
     const size_t tsz = c->fp32 ? sizeof(float) : sizeof(double);
@@ -1791,20 +1796,6 @@ int pf_autotune(pf_ctx* c, int reps, double* ms_before, double* ms_after) {
             cfg[39] = v;
             trial(cfg);
         }
-        // fused x passes with two shared buffers or one (in place)
-        if (c->fp32)
-            for (int v : {0, 1}) {
-                std::memcpy(cfg, best, sizeof cfg);
-                cfg[42] = v;
-                trial(cfg);
-            }
-        // real fields of the right-hand-side x pass read from global or staged
-        if (c->fp32 && c->ph.elastic)
-            for (int v : {0, 1}) {
-                std::memcpy(cfg, best, sizeof cfg);
-                cfg[41] = v;
-                trial(cfg);
-            }
         // elastic pass with the fused stage, with every stage over the three
         // fields, or as a three-CTA cluster (FP32)
         if (c->ph.elastic && !c->inhom) {

@@ -347,30 +347,63 @@ __device__ __forceinline__ void cp_async_wait_all() {
             __VA_ARGS__;                    \
         }                                   \
     } break;
-#define PF_COL_SWITCH(T_, plan, tx, ...)                                                          \
-    do {                                                                                          \
-        int pid_ = 0;                                                                             \
-        if (sizeof(T_) == 4 && ((tx) == 8 || (tx) == 16)) pid_ = fixed_plan_id(plan);              \
-        if constexpr (sizeof(T_) == 4) {                                                          \
-            switch (pid_) {                                                                       \
-                PF_PID_CASE(1, tx, __VA_ARGS__)                                                   \
-                PF_PID_CASE(2, tx, __VA_ARGS__)                                                   \
-                PF_PID_CASE(3, tx, __VA_ARGS__)                                                   \
-                PF_PID_CASE(4, tx, __VA_ARGS__)                                                   \
-                PF_PID_CASE(5, tx, __VA_ARGS__)                                                   \
-                PF_PID_CASE(6, tx, __VA_ARGS__)                                                   \
-                PF_PID_CASE(7, tx, __VA_ARGS__)                                                   \
-                PF_PID_CASE(8, tx, __VA_ARGS__)                                                   \
-                PF_PID_CASE(9, tx, __VA_ARGS__)                                                   \
-                PF_PID_CASE(10, tx, __VA_ARGS__)                                                  \
-                PF_PID_CASE(11, tx, __VA_ARGS__)                                                  \
-                default: break;                                                                   \
-            }                                                                                     \
-        }                                                                                         \
-        if (pid_ == 0) {                                                                          \
-            constexpr int PIDC = 0;                                                               \
-            PF_R16_SWITCH((plan).has16, PF_TX_SWITCH(tx, __VA_ARGS__));                            \
-        }                                                                                         \
+#define PF_PID_CASE1(K_, ...)                                   \
+    case K_: {                                                  \
+        constexpr int PIDC = K_;                                \
+        constexpr bool R16C = false;                            \
+        constexpr int TXC = plan_width(FixedPlan<PIDC>::N);     \
+        __VA_ARGS__;                                            \
+    } break;
+#define PF_COL_SWITCH(T_, plan, tx, ...) \
+    do { \
+        int pid_ = 0; \
+        if (sizeof(T_) == 4) pid_ = fixed_plan_id(plan); \
+        if (!plan_has_width(pid_, (plan).n, tx)) pid_ = 0; \
+        if constexpr (sizeof(T_) == 4) { \
+            switch (pid_) { \
+                PF_PID_CASE(1, tx, __VA_ARGS__) \
+                PF_PID_CASE(2, tx, __VA_ARGS__) \
+                PF_PID_CASE(3, tx, __VA_ARGS__) \
+                PF_PID_CASE(4, tx, __VA_ARGS__) \
+                PF_PID_CASE(5, tx, __VA_ARGS__) \
+                PF_PID_CASE(6, tx, __VA_ARGS__) \
+                PF_PID_CASE(7, tx, __VA_ARGS__) \
+                PF_PID_CASE(8, tx, __VA_ARGS__) \
+                PF_PID_CASE(9, tx, __VA_ARGS__) \
+                PF_PID_CASE(10, tx, __VA_ARGS__) \
+                PF_PID_CASE(11, tx, __VA_ARGS__) \
+                PF_PID_CASE1(12, __VA_ARGS__) \
+                PF_PID_CASE1(13, __VA_ARGS__) \
+                PF_PID_CASE1(14, __VA_ARGS__) \
+                PF_PID_CASE1(15, __VA_ARGS__) \
+                PF_PID_CASE1(16, __VA_ARGS__) \
+                PF_PID_CASE1(17, __VA_ARGS__) \
+                PF_PID_CASE1(18, __VA_ARGS__) \
+                PF_PID_CASE1(19, __VA_ARGS__) \
+                PF_PID_CASE1(20, __VA_ARGS__) \
+                PF_PID_CASE1(21, __VA_ARGS__) \
+                PF_PID_CASE1(22, __VA_ARGS__) \
+                PF_PID_CASE1(23, __VA_ARGS__) \
+                PF_PID_CASE1(24, __VA_ARGS__) \
+                PF_PID_CASE1(25, __VA_ARGS__) \
+                PF_PID_CASE1(26, __VA_ARGS__) \
+                PF_PID_CASE1(27, __VA_ARGS__) \
+                PF_PID_CASE1(28, __VA_ARGS__) \
+                PF_PID_CASE1(29, __VA_ARGS__) \
+                PF_PID_CASE1(30, __VA_ARGS__) \
+                PF_PID_CASE1(31, __VA_ARGS__) \
+                PF_PID_CASE1(32, __VA_ARGS__) \
+                PF_PID_CASE1(33, __VA_ARGS__) \
+                PF_PID_CASE1(34, __VA_ARGS__) \
+                PF_PID_CASE1(35, __VA_ARGS__) \
+                PF_PID_CASE1(36, __VA_ARGS__) \
+                default: break; \
+            } \
+        } \
+        if (pid_ == 0) { \
+            constexpr int PIDC = 0; \
+            PF_R16_SWITCH((plan).has16, PF_TX_SWITCH(tx, __VA_ARGS__)); \
+        } \
     } while (0)
 
 // as PF_COL_SWITCH, with compiled plans for tile width 8 only (passes whose
@@ -386,6 +419,7 @@ __device__ __forceinline__ void cp_async_wait_all() {
     do {                                                                                          \
         int pid_ = 0;                                                                             \
         if (sizeof(T_) == 4 && (tx) == 8) pid_ = fixed_plan_id(plan);                             \
+        if (pid_ > kBothWidths) pid_ = 0;                                                         \
         if constexpr (sizeof(T_) == 4) {                                                          \
             switch (pid_) {                                                                       \
                 PF_PID_CASE8(1, __VA_ARGS__)                                                      \

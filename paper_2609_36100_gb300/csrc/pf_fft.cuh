@@ -1,4 +1,4 @@
-// Shared-memory mixed-radix (2,3,4,5,8,16) Stockham FFT used by every pass of
+// Shared-memory mixed-radix (2..6, 8..10, 12, 15, 16) Stockham FFT used by every pass of
 // the pseudospectral right-hand side.  A CTA transforms `nl` lines of length
 // n held in shared memory; element e of line l sits at l*ls + e*es.  Stages
 // ping-pong between two buffers; each butterfly reads R inputs strided by n/R,
@@ -168,6 +168,181 @@ struct Bfly<16, SIGN, T2> {
     }
 };
 
+// Coprime factors N = N1 N2 need no twiddles between them (Good's prime-factor
+// mapping): input N2 n1 + N1 n2 (mod N), output k with k = k1 (mod N1), k = k2
+// (mod N2).
+template <int N1, int N2, int SIGN, typename T2>
+struct BflyPF {
+    // 1 (mod N1), 0 (mod N2) and the other way round
+    static constexpr int unit(int n, int m) {
+        int k = m;
+        while (k % n != 1) k += m;
+        return k;
+    }
+    static constexpr int U1 = unit(N1, N2), U2 = unit(N2, N1);
+    __device__ __forceinline__ static void run(T2* v) {
+        T2 a[N2][N1];
+#pragma unroll
+        for (int n2 = 0; n2 < N2; ++n2) {
+#pragma unroll
+            for (int n1 = 0; n1 < N1; ++n1) a[n2][n1] = v[(N2 * n1 + N1 * n2) % (N1 * N2)];
+            Bfly<N1, SIGN, T2>::run(a[n2]);
+        }
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) {
+            T2 q[N2];
+#pragma unroll
+            for (int n2 = 0; n2 < N2; ++n2) q[n2] = a[n2][k1];
+            Bfly<N2, SIGN, T2>::run(q);
+#pragma unroll
+            for (int k2 = 0; k2 < N2; ++k2) v[(k1 * U1 + k2 * U2) % (N1 * N2)] = q[k2];
+        }
+    }
+};
+template <int SIGN, typename T2>
+struct Bfly<6, SIGN, T2> : BflyPF<2, 3, SIGN, T2> {};
+template <int SIGN, typename T2>
+struct Bfly<10, SIGN, T2> : BflyPF<2, 5, SIGN, T2> {};
+template <int SIGN, typename T2>
+struct Bfly<12, SIGN, T2> : BflyPF<4, 3, SIGN, T2> {};
+template <int SIGN, typename T2>
+struct Bfly<15, SIGN, T2> : BflyPF<3, 5, SIGN, T2> {};
+// 9 = 3 x 3 with twiddles exp(SIGN 2 pi i m / 9), m = 1, 2, 4
+template <int SIGN, typename T2>
+struct Bfly<9, SIGN, T2> {
+    __device__ __forceinline__ static void run(T2* v) {
+        using T = decltype(v[0].x);
+        T2 a[3][3];
+#pragma unroll
+        for (int n2 = 0; n2 < 3; ++n2) {
+            a[n2][0] = v[n2];
+            a[n2][1] = v[3 + n2];
+            a[n2][2] = v[6 + n2];
+            Bfly<3, SIGN, T2>::run(a[n2]);
+        }
+        const T2 w1 = T2{(T)0.7660444431189781, SIGN * (T)0.6427876096865394};   // cos, sin of 40 degrees
+        const T2 w2 = T2{(T)0.17364817766693041, SIGN * (T)0.984807753012208};   // 80
+        const T2 w4 = T2{(T)(-0.9396926207859083), SIGN * (T)0.3420201433256689};  // 160
+        a[1][1] = cmul(a[1][1], w1);
+        a[1][2] = cmul(a[1][2], w2);
+        a[2][1] = cmul(a[2][1], w2);
+        a[2][2] = cmul(a[2][2], w4);
+#pragma unroll
+        for (int k1 = 0; k1 < 3; ++k1) {
+            T2 q[3] = {a[0][k1], a[1][k1], a[2][k1]};
+            Bfly<3, SIGN, T2>::run(q);
+#pragma unroll
+            for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = q[k2];
+        }
+    }
+};
+
+// ---------------------------------------------------------------------------
+// Twiddled butterfly of a power-of-two radix with the twiddles merged into its
+// radix-2 levels (decimation in time): X_k = E_k + c_k O_k, X_{k+R/2} = E_k -
+// c_k O_k with c_k = w w_R^k, E and O the halves over the even and the odd
+// inputs with w^2 in the place of w.  a + c b is four FMAs and a - c b = 2 a -
+// (a + c b) two more, so a radix-16 butterfly with its 15 twiddles is 192
+// instructions (238 with products first: 4 a twiddle, 160 for the butterfly
+// and its constants), a radix-8 one 72 (84), a radix-4 one 24 (28).  c_{k+R/4}
+// is c_k turned by a quarter, so R/2 twiddles are read, all of them rounded
+// table entries: w^(R/2), ..., w^2, w and their eighth and sixteenth turns.
+// ---------------------------------------------------------------------------
+template <typename T2>
+__device__ __forceinline__ void bf2_tw(T2& a, T2& b, T2 c) {
+    using T = decltype(a.x);
+    const T sx = fma(c.x, b.x, fma(-c.y, b.y, a.x)), sy = fma(c.x, b.y, fma(c.y, b.x, a.y));
+    b = T2{fma((T)2, a.x, -sx), fma((T)2, a.y, -sy)};
+    a = T2{sx, sy};
+}
+// X[0..3] (natural order) of the inputs x[0], x[S], x[2S], x[3S] in place of
+// x[0..3 S]: w1 = w, w2 = w^2
+template <int SIGN, typename T2>
+__device__ __forceinline__ void bf4_tw(T2& x0, T2& x1, T2& x2, T2& x3, T2 w1, T2 w2) {
+    bf2_tw(x0, x2, w2);  // E_0, E_1
+    bf2_tw(x1, x3, w2);  // O_0, O_1
+    bf2_tw(x0, x1, w1);  // X_0, X_2
+    bf2_tw(x2, x3, mul_si<SIGN>(w1));  // X_1, X_3
+    const T2 t = x1;
+    x1 = x2;
+    x2 = t;
+}
+template <int SIGN, typename T2>
+__device__ __forceinline__ void bf8_tw(T2* v, T2 w1, T2 w1e, T2 w2, T2 w4) {
+    T2 e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+    bf4_tw<SIGN>(e[0], e[1], e[2], e[3], w2, w4);
+    bf4_tw<SIGN>(o[0], o[1], o[2], o[3], w2, w4);
+    bf2_tw(e[0], o[0], w1);
+    bf2_tw(e[1], o[1], w1e);
+    bf2_tw(e[2], o[2], mul_si<SIGN>(w1));
+    bf2_tw(e[3], o[3], mul_si<SIGN>(w1e));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        v[k] = e[k];
+        v[k + 4] = o[k];
+    }
+}
+
+// radix-R stage of a transform of length n: v[t] *= w^t, then the butterfly;
+// w = tw[st] (SIGN < 0) or its conjugate
+template <int R, int SIGN, typename T2>
+__device__ __forceinline__ void tw_bfly(T2* v, const T2* __restrict__ tw, int st, int n) {
+    auto ld = [&](int i) {
+        const T2 w = __ldg(tw + i);
+        return SIGN < 0 ? w : T2{w.x, -w.y};
+    };
+    if constexpr (R == 2) {
+        bf2_tw(v[0], v[1], ld(st));
+    } else if constexpr (R == 4) {
+        bf4_tw<SIGN>(v[0], v[1], v[2], v[3], ld(st), ld(2 * st));
+    } else if constexpr (R == 8) {
+        bf8_tw<SIGN>(v, ld(st), ld(st + n / 8), ld(2 * st), ld(4 * st));
+    } else if constexpr (R == 16) {
+        T2 e[8] = {v[0], v[2], v[4], v[6], v[8], v[10], v[12], v[14]};
+        T2 o[8] = {v[1], v[3], v[5], v[7], v[9], v[11], v[13], v[15]};
+        const T2 w2 = ld(2 * st), w2e = ld(2 * st + n / 8), w4 = ld(4 * st), w8 = ld(8 * st);
+        bf8_tw<SIGN>(e, w2, w2e, w4, w8);
+        bf8_tw<SIGN>(o, w2, w2e, w4, w8);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const T2 w = ld(st + k * (n / 16));
+            bf2_tw(e[k], o[k], w);
+            bf2_tw(e[k + 4], o[k + 4], mul_si<SIGN>(w));
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            v[k] = e[k];
+            v[k + 8] = o[k];
+        }
+    } else {
+#pragma unroll
+        for (int t = 1; t < R; ++t) {
+            const T2 w = ld(t * st);
+            v[t] = cmul(v[t], w);
+        }
+        Bfly<R, SIGN, T2>::run(v);
+    }
+}
+
+// butterfly of a generic (run-time plan) stage: FP64 stages, bound by the FP64
+// pipe, merge the twiddles; FP32 ones, bound by address arithmetic, gained
+// nothing from it (a second form of every radix: 480^3 1 % slower) and multiply
+template <int R, int SIGN, typename T2>
+__device__ __forceinline__ void generic_bfly(T2* v, const T2* __restrict__ tw, int st, int n, bool turn) {
+    if (sizeof(T2) == 16 && turn) {
+        tw_bfly<R, SIGN>(v, tw, st, n);
+        return;
+    }
+    if (turn) {
+#pragma unroll
+        for (int t = 1; t < R; ++t) {
+            const T2 w = __ldg(tw + t * st);
+            v[t] = SIGN < 0 ? cmul(v[t], w) : cmulc(v[t], w);
+        }
+    }
+    Bfly<R, SIGN, T2>::run(v);
+}
+
 template <typename T2>
 __device__ __forceinline__ const T2* twiddles(const AxisPlan& p);
 template <>
@@ -228,15 +403,7 @@ __device__ __forceinline__ void fft_stage(const T2* __restrict__ src, T2* __rest
         for (int t = 0; t < R; ++t) v[t] = s[skew<SKEW>((j + t * m) * es)];
         const int jq = (int)divN.div((unsigned)j);
         const int k = j - jq * Ns;
-        if (Ns > 1) {
-            const int st = k * tws;
-#pragma unroll
-            for (int t = 1; t < R; ++t) {
-                const T2 w = __ldg(tw + t * st);
-                v[t] = SIGN < 0 ? cmul(v[t], w) : cmulc(v[t], w);
-            }
-        }
-        Bfly<R, SIGN, T2>::run(v);
+        generic_bfly<R, SIGN>(v, tw, k * tws, n, Ns > 1);
         const int base = jq * Ns * R + k;
         T2* d = dst + line * ls;
 #pragma unroll
@@ -254,44 +421,6 @@ __device__ __forceinline__ void fft_stage(const T2* __restrict__ src, T2* __rest
 // ---------------------------------------------------------------------------
 template <int... Rs>
 struct Radices {};
-
-// v[t] *= w^t (SIGN < 0) or conj(w)^t, w = tw[st], t = 1..R-1.  FP32 radix-8
-// and radix-16 stages load w, w^2, w^4 (and w^8) from the table and form the
-// other powers by at most three complex products (a few ulp, against the
-// ulp-level rounding of the table itself), trading up to 11 dependent L1
-// loads per butterfly for FMAs; FP64 stages (whose FMA pipe is the narrow
-// one) load every power.
-template <int R, int SIGN, typename T2>
-__device__ __forceinline__ void apply_twiddles(T2* v, const T2* __restrict__ tw, int st) {
-    auto mul = [](T2& x, T2 w) { x = SIGN < 0 ? cmul(x, w) : cmulc(x, w); };
-    if constexpr (sizeof(T2) == 8 && (R == 8 || R == 16)) {
-        // each power applied as soon as it is formed (few live registers)
-        const T2 w1 = __ldg(tw + st), w2 = __ldg(tw + 2 * st), w4 = __ldg(tw + 4 * st);
-        mul(v[1], w1);
-        mul(v[2], w2);
-        const T2 w3 = cmul(w2, w1);
-        mul(v[3], w3);
-        mul(v[4], w4);
-        mul(v[5], cmul(w4, w1));
-        mul(v[6], cmul(w4, w2));
-        mul(v[7], cmul(w4, w3));
-        if constexpr (R == 16) {
-            const T2 w8 = __ldg(tw + 8 * st);
-            mul(v[8], w8);
-            mul(v[9], cmul(w8, w1));
-            mul(v[10], cmul(w8, w2));
-            mul(v[11], cmul(w8, w3));
-            const T2 w12 = cmul(w8, w4);
-            mul(v[12], w12);
-            mul(v[13], cmul(w12, w1));
-            mul(v[14], cmul(w12, w2));
-            mul(v[15], cmul(w12, w3));
-        }
-    } else {
-#pragma unroll
-        for (int t = 1; t < R; ++t) mul(v[t], __ldg(tw + t * st));
-    }
-}
 
 template <int R, int SIGN, int N, int NS, typename T2>
 __device__ __forceinline__ void fft_stage_fixed(const T2* __restrict__ src, T2* __restrict__ dst, int nl, int ls,
@@ -314,10 +443,10 @@ __device__ __forceinline__ void fft_stage_fixed(const T2* __restrict__ src, T2* 
             for (int t = 0; t < R; ++t) v[t] = s[skew<true>(j + t * M)];
         }
         const int jq = j / NS, k = j - jq * NS;
-        if constexpr (NS > 1) {
-            apply_twiddles<R, SIGN>(v, tw, k * TWS);
-        }
-        Bfly<R, SIGN, T2>::run(v);
+        if constexpr (NS > 1)
+            tw_bfly<R, SIGN>(v, tw, k * TWS, N);
+        else
+            Bfly<R, SIGN, T2>::run(v);
         T2* d = dst + line * ls;
         const int a = jq * NS * R;  // output block start; outputs at a + k + t NS
         if constexpr ((NS * R) % 16 == 0 && NS % 16 == 0) {
@@ -355,9 +484,9 @@ __device__ __forceinline__ T2* fft_fixed_run(T2* src, T2* dst, int nl, int ls, c
     return fft_fixed_run<SIGN, N, NS * R>(dst, src, nl, ls, tw, Radices<Rest...>{});
 }
 
-// Full transform of the lines in `a` (b is scratch).  Radix-16 stages are
-// compiled in only with R16 (they raise the register count of the whole
-// kernel); the launcher picks R16 from the plan (AxisPlan::has16).  Callers synchronise
+// Full transform of the lines in `a` (b is scratch).  Stages of radix 9 and
+// more are compiled in only with R16 (they raise the register count of the
+// whole kernel); the launcher picks R16 from the plan (AxisPlan::has16).  Callers synchronise
 // before; returns the buffer holding the result (synchronised).  NL > 0 fixes
 // the line count at compile time (strided tiles of NL columns).
 template <int SIGN, bool LINE_FAST, int NL = 0, bool SKEW = false, bool R16 = false, typename T2>
@@ -374,9 +503,14 @@ __device__ T2* fft_lines(T2* a, T2* b, const AxisPlan& p, int nl, int es, int ls
             case 3: fft_stage<3, SIGN, LINE_FAST, NL, SKEW>(src, dst, p.n, nl, es, ls, Ns, tw, dm, dN, divl); break;
             case 4: fft_stage<4, SIGN, LINE_FAST, NL, SKEW>(src, dst, p.n, nl, es, ls, Ns, tw, dm, dN, divl); break;
             case 5: fft_stage<5, SIGN, LINE_FAST, NL, SKEW>(src, dst, p.n, nl, es, ls, Ns, tw, dm, dN, divl); break;
-            case 16:
-                if constexpr (R16) fft_stage<16, SIGN, LINE_FAST, NL, SKEW>(src, dst, p.n, nl, es, ls, Ns, tw, dm, dN, divl);
-                break;
+            case 6: fft_stage<6, SIGN, LINE_FAST, NL, SKEW>(src, dst, p.n, nl, es, ls, Ns, tw, dm, dN, divl); break;
+#define PF_WIDE(R_)                                                                                                  \
+    case R_:                                                                                                         \
+        if constexpr (R16)                                                                                           \
+            fft_stage<R_, SIGN, LINE_FAST, NL, SKEW>(src, dst, p.n, nl, es, ls, Ns, tw, dm, dN, divl);               \
+        break;
+            PF_WIDE(9) PF_WIDE(10) PF_WIDE(12) PF_WIDE(15) PF_WIDE(16)
+#undef PF_WIDE
             default: fft_stage<8, SIGN, LINE_FAST, NL, SKEW>(src, dst, p.n, nl, es, ls, Ns, tw, dm, dN, divl); break;
         }
         __syncthreads();
@@ -417,15 +551,7 @@ __device__ __forceinline__ void col_stage(int n, int Ns, FastDiv dN, const T2* _
         }
         const int jq = (int)dN.div((unsigned)j);
         const int k = j - jq * Ns;
-        if (Ns > 1) {
-            const int st = k * tws;
-#pragma unroll
-            for (int t = 1; t < R; ++t) {
-                const T2 w = __ldg(tw + t * st);
-                v[t] = SIGN < 0 ? cmul(v[t], w) : cmulc(v[t], w);
-            }
-        }
-        Bfly<R, SIGN, T2>::run(v);
+        generic_bfly<R, SIGN>(v, tw, k * tws, n, Ns > 1);
         const int base = jq * Ns * R + k;
         if (last) {
 #pragma unroll
@@ -467,6 +593,19 @@ __device__ void fft_cols(const AxisPlan& p, T2* P, T2* Q, Src src, Dst dst) {
                 case 3: col_stage<3, SIGN, TX>(n, Ns, dN, in, out, false, last, tw, none, dst); break;
                 case 4: col_stage<4, SIGN, TX>(n, Ns, dN, in, out, false, last, tw, none, dst); break;
                 case 5: col_stage<5, SIGN, TX>(n, Ns, dN, in, out, false, last, tw, none, dst); break;
+                case 6: col_stage<6, SIGN, TX>(n, Ns, dN, in, out, false, last, tw, none, dst); break;
+                case 9:
+                    if constexpr (R16) col_stage<9, SIGN, TX>(n, Ns, dN, in, out, false, last, tw, none, dst);
+                    break;
+                case 10:
+                    if constexpr (R16) col_stage<10, SIGN, TX>(n, Ns, dN, in, out, false, last, tw, none, dst);
+                    break;
+                case 12:
+                    if constexpr (R16) col_stage<12, SIGN, TX>(n, Ns, dN, in, out, false, last, tw, none, dst);
+                    break;
+                case 15:
+                    if constexpr (R16) col_stage<15, SIGN, TX>(n, Ns, dN, in, out, false, last, tw, none, dst);
+                    break;
                 case 16:
                     if constexpr (R16) col_stage<16, SIGN, TX>(n, Ns, dN, in, out, false, last, tw, none, dst);
                     break;
@@ -489,6 +628,19 @@ __device__ void fft_cols(const AxisPlan& p, T2* P, T2* Q, Src src, Dst dst) {
             case 3: col_stage<3, SIGN, TX>(n, 1, dN, P, P, true, true, tw, src, toP); break;
             case 4: col_stage<4, SIGN, TX>(n, 1, dN, P, P, true, true, tw, src, toP); break;
             case 5: col_stage<5, SIGN, TX>(n, 1, dN, P, P, true, true, tw, src, toP); break;
+            case 6: col_stage<6, SIGN, TX>(n, 1, dN, P, P, true, true, tw, src, toP); break;
+            case 9:
+                if constexpr (R16) col_stage<9, SIGN, TX>(n, 1, dN, P, P, true, true, tw, src, toP);
+                break;
+            case 10:
+                if constexpr (R16) col_stage<10, SIGN, TX>(n, 1, dN, P, P, true, true, tw, src, toP);
+                break;
+            case 12:
+                if constexpr (R16) col_stage<12, SIGN, TX>(n, 1, dN, P, P, true, true, tw, src, toP);
+                break;
+            case 15:
+                if constexpr (R16) col_stage<15, SIGN, TX>(n, 1, dN, P, P, true, true, tw, src, toP);
+                break;
             case 16:
                 if constexpr (R16) col_stage<16, SIGN, TX>(n, 1, dN, P, P, true, true, tw, src, toP);
                 break;
@@ -509,6 +661,19 @@ __device__ void fft_cols(const AxisPlan& p, T2* P, T2* Q, Src src, Dst dst) {
             case 3: col_stage<3, SIGN, TX>(n, Ns, dN, in, out, first, last, tw, src, dst); break;
             case 4: col_stage<4, SIGN, TX>(n, Ns, dN, in, out, first, last, tw, src, dst); break;
             case 5: col_stage<5, SIGN, TX>(n, Ns, dN, in, out, first, last, tw, src, dst); break;
+            case 6: col_stage<6, SIGN, TX>(n, Ns, dN, in, out, first, last, tw, src, dst); break;
+            case 9:
+                if constexpr (R16) col_stage<9, SIGN, TX>(n, Ns, dN, in, out, first, last, tw, src, dst);
+                break;
+            case 10:
+                if constexpr (R16) col_stage<10, SIGN, TX>(n, Ns, dN, in, out, first, last, tw, src, dst);
+                break;
+            case 12:
+                if constexpr (R16) col_stage<12, SIGN, TX>(n, Ns, dN, in, out, first, last, tw, src, dst);
+                break;
+            case 15:
+                if constexpr (R16) col_stage<15, SIGN, TX>(n, Ns, dN, in, out, first, last, tw, src, dst);
+                break;
             case 16:
                 if constexpr (R16) col_stage<16, SIGN, TX>(n, Ns, dN, in, out, first, last, tw, src, dst);
                 break;
@@ -525,8 +690,10 @@ __device__ void fft_cols(const AxisPlan& p, T2* P, T2* Q, Src src, Dst dst) {
 // ---------------------------------------------------------------------------
 // Plans compiled with a constant length and radix order (PID > 0), shared by
 // the line (x) and column (y, z) transforms; any other plan runs the generic
-// stages (PID 0).  The list holds the default plans of the grid sizes of the
-// workloads (FP32 plans prefer radix 16, FP64 plans radix 8).
+// stages (PID 0).  The list: PIDs 1 to 11 every pass compiles, at both tile
+// widths; from 12 on the default FP32 plans of common sizes up to 640, which the
+// y and z passes compile at their default tile width and the elastic pass in
+// the form with every stage over the three fields.
 // ---------------------------------------------------------------------------
 template <int PID>
 struct FixedPlan {
@@ -550,8 +717,33 @@ PF_FIXED_PLAN(8, 96, 8, 4, 3)
 PF_FIXED_PLAN(9, 120, 8, 3, 5)
 PF_FIXED_PLAN(10, 192, 16, 4, 3)
 PF_FIXED_PLAN(11, 640, 16, 8, 5)
+PF_FIXED_PLAN(12, 32, 8, 4)
+PF_FIXED_PLAN(13, 48, 8, 6)
+PF_FIXED_PLAN(14, 72, 12, 6)
+PF_FIXED_PLAN(15, 80, 10, 8)
+PF_FIXED_PLAN(16, 96, 12, 8)
+PF_FIXED_PLAN(17, 100, 10, 10)
+PF_FIXED_PLAN(18, 108, 12, 9)
+PF_FIXED_PLAN(19, 120, 15, 8)
+PF_FIXED_PLAN(20, 144, 12, 12)
+PF_FIXED_PLAN(21, 160, 16, 10)
+PF_FIXED_PLAN(22, 180, 15, 12)
+PF_FIXED_PLAN(23, 192, 16, 12)
+PF_FIXED_PLAN(24, 200, 10, 10, 2)
+PF_FIXED_PLAN(25, 216, 12, 6, 3)
+PF_FIXED_PLAN(26, 240, 16, 15)
+PF_FIXED_PLAN(27, 288, 12, 12, 2)
+PF_FIXED_PLAN(28, 300, 15, 10, 2)
+PF_FIXED_PLAN(29, 320, 10, 8, 4)
+PF_FIXED_PLAN(30, 360, 15, 12, 2)
+PF_FIXED_PLAN(31, 384, 12, 8, 4)
+PF_FIXED_PLAN(32, 400, 10, 10, 4)
+PF_FIXED_PLAN(33, 432, 12, 12, 3)
+PF_FIXED_PLAN(34, 480, 15, 8, 4)
+PF_FIXED_PLAN(35, 512, 8, 8, 8)
+PF_FIXED_PLAN(36, 640, 10, 8, 8)
 #undef PF_FIXED_PLAN
-constexpr int kFixedPlans = 11;
+constexpr int kFixedPlans = 36;
 
 template <int... Rs>
 inline bool plan_is(const AxisPlan& p, int n, Radices<Rs...>) {
@@ -560,6 +752,16 @@ inline bool plan_is(const AxisPlan& p, int n, Radices<Rs...>) {
     for (int s = 0; s < p.nst; ++s)
         if (p.rad[s] != r[s]) return false;
     return true;
+}
+
+constexpr int kBothWidths = 11;  // plans up to here are compiled for tiles of 8 and 16 columns
+
+// tile width a column pass compiles plan PID >= 12 for (its untuned width:
+// two buffers of 16 columns in 96 KB, or 8; grids of up to 48 have too few
+// columns for wide tiles)
+constexpr int plan_width(int n) { return n > 48 && n <= 384 ? 16 : 8; }
+inline bool plan_has_width(int pid, int n, int tx) {
+    return pid > 0 && (pid <= kBothWidths ? tx == 8 || tx == 16 : tx == plan_width(n));
 }
 
 // length of compiled plan PID (0 for an unknown PID)
@@ -604,10 +806,10 @@ __device__ __forceinline__ void col_stage_fixed(const T2* __restrict__ in, T2* _
             for (int t = 0; t < R; ++t) v[t] = p[t * M * TX];
         }
         const int jq = j / NS, k = j - jq * NS;
-        if constexpr (NS > 1) {
-            apply_twiddles<R, SIGN>(v, tw, k * TWS);
-        }
-        Bfly<R, SIGN, T2>::run(v);
+        if constexpr (NS > 1)
+            tw_bfly<R, SIGN>(v, tw, k * TWS, N);
+        else
+            Bfly<R, SIGN, T2>::run(v);
         const int base = jq * NS * R + k;
         if constexpr (LAST) {
 #pragma unroll
@@ -726,8 +928,10 @@ __device__ __forceinline__ void tile_stage_inplace(T2* S, const T2* __restrict__
         if (JOBS % NT == 0 || idx < JOBS) {
             const int f = idx / (TX * M), r = idx - f * (TX * M), col = r % TX, j = r / TX;
             const int jq = j / NS, k = j - jq * NS;
-            if constexpr (NS > 1) apply_twiddles<R, SIGN>(v[u], tw, k * TWS);
-            Bfly<R, SIGN, T2>::run(v[u]);
+            if constexpr (NS > 1)
+                tw_bfly<R, SIGN>(v[u], tw, k * TWS, N);
+            else
+                Bfly<R, SIGN, T2>::run(v[u]);
             T2* dst = S + f * (N * TX) + (jq * NS * R + k) * TX + col;
 #pragma unroll
             for (int t = 0; t < R; ++t) dst[t * NS * TX] = v[u][t];
@@ -796,11 +1000,11 @@ __device__ __forceinline__ void cols_fft(const AxisPlan& p, T2* P, T2* Q, Src sr
 
 // shared-memory buffers of a column pass of the compute type T at tile
 // width tx: one when the transform has at most two stages or runs a compiled
-// plan (FP32, tile width 8 or 16), else two
+// plan (FP32, the widths it is compiled for), else two
 template <typename T>
 inline int col_buffers(const AxisPlan& p, int tx) {
     if (p.nst <= 2) return 1;
-    const bool compiled = sizeof(T) == 4 && (tx == 8 || tx == 16) && fixed_plan_id(p) > 0;
+    const bool compiled = sizeof(T) == 4 && plan_has_width(fixed_plan_id(p), p.n, tx);
     return compiled ? 1 : 2;
 }
 

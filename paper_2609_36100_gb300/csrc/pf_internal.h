@@ -27,6 +27,9 @@ inline unsigned magic_u32(unsigned d) { return d <= 1 ? 0u : (unsigned)((0xfffff
 // radix schedule (8s first, then 4/2, 3s, 5s) and division magic of one axis
 bool make_axis_plan(int n, AxisPlan& p, bool prefer16 = false);
 bool make_axis_plan_radices(int n, const int* rad, int nr, AxisPlan& p);
+// untuned form of the FP32 elastic pass and its compiled plan (0: the axis plan)
+int default_elastic_form(const AxisPlan& pz);
+int default_elastic_plan(const AxisPlan& pz);
 // length of compiled (compile-time) plan `pid` (0 if unknown), and how many there are
 int compiled_plan_len(int pid);
 int compiled_plan_count();
@@ -61,8 +64,7 @@ struct Geo {
     int el_pid;              // compiled plan of the fused elastic pass (length nz), 0 = the z-axis plan,
                              // -1 = no fused stage (the one-kernel pass with the z-axis column transforms)
     int xf_off;              // 1: the FP32 x passes use the staged kernel instead of the fused one
-    int xf_inpl;             // 1: the FP32 fused x passes run every stage in one shared buffer (in place)
-    int xf_stg;              // 1: the FP32 fused right-hand-side x pass stages the stored real fields in shared memory
+    int xf_inpl, xf_stg;     // schedule slots kept for saved schedules; nothing reads them
     int el_unfused;          // form of the compiled-plan elastic pass: 0 fuses the last forward / first inverse
                              // stage, 1 runs every stage (and the contraction) over the three fields in place,
                              // 2 runs a cluster of three CTAs, one field each (FP32 contexts)
@@ -205,8 +207,15 @@ enum XMode {
 template <typename T>
 void launch_z_stage(const Geo& g, const Phys& ph, const double2* y, const StageTerms& st, double2* zout,
                     void* W, cudaStream_t s);
+template <typename T, int SIGN>
+void launch_y_pass_sign(const Geo& g, void* buf, int nf, cudaStream_t s);
 template <typename T>
-void launch_y_pass(const Geo& g, void* buf, int nf, int sign, cudaStream_t s);
+void launch_y_pass(const Geo& g, void* buf, int nf, int sign, cudaStream_t s) {
+    if (sign > 0)
+        launch_y_pass_sign<T, 1>(g, buf, nf, s);
+    else
+        launch_y_pass_sign<T, -1>(g, buf, nf, s);
+}
 // returns the number of CTAs launched (the WRMS mode writes one partial sum each)
 template <typename T>
 int launch_x_pass(const Geo& g, const Phys& ph, int mode, const void* in, void* out, void* R, const void* Rin,
@@ -246,7 +255,7 @@ void launch_stage_assemble(const Geo& g, const double2* y, const StageTerms& st,
                            cudaStream_t s);
 // in-place FFT along z of nf fields (sign +1 inverse)
 template <typename T>
-void launch_z_pass(const Geo& g, void* buf, int nf, int sign, cudaStream_t s);
+void launch_z_pass(const Geo& g, void* buf, int nf, cudaStream_t s);
 // batch round: coefficients from the member's step, controller, accepted-state copy
 void launch_batch_prep(const BatchConst& bc, MemberCtl* ctl, StageCoefDev* coef, cudaStream_t s);
 void launch_batch_ctl(const BatchConst& bc, MemberCtl* ctl, const double* wrms_sum, double scale, cudaStream_t s);

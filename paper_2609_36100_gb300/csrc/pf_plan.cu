@@ -1,16 +1,50 @@
 // Axis plans (radix schedules and division magic) and the x-pass CTA count.
+#include <vector>
+
 #include "pf_xpass.cuh"
 
 namespace pf {
 int compiled_plan_len(int pid) { return fixed_plan_len(pid); }
 int compiled_plan_count() { return kFixedPlans; }
 
-// plan from an explicit radix order (each radix in {2,3,4,5,8,16}, product n)
+// Form of the FP32 elastic pass that is run untuned (pf_internal.h lists
+// them).  The stages over three fields are the fastest single-CTA form (us a
+// launch against the fused one: 14.6 / 18.6 at 96, 23.1 / 24.7 at 128, 51.7 /
+// 53.7 at 160, 165 / 229 at 256) except where a radix-16 first stage meets a
+// last radix of at most 4, which the fused form holds in few registers (8.7 /
+// 9.9 at 64 = 16 4, 82 / 89 at 192 = 16 4 3).  A three-field tile of 8 columns no
+// longer fits beside another one above 512 points: the cluster form
+// (3.1 / 6.2 ms at 640).
+template <int PID = 1>
+static int elastic_form(int pid) {
+    if constexpr (PID > kFixedPlans) {
+        return 0;
+    } else {
+        if (pid != PID) return elastic_form<PID + 1>(pid);
+        using Rad = typename FixedPlan<PID>::Rad;
+        if (RadInfo<Rad>::count < 2) return 0;
+        if (FixedPlan<PID>::N > 512) return 2;
+        return RadInfo<Rad>::first == 16 && RadInfo<Rad>::last <= 4 ? 0 : 1;
+    }
+}
+int default_elastic_form(const AxisPlan& pz) { return elastic_form(fixed_plan_id(pz)); }
+
+// plan of the cluster form: one of those it is compiled for
+template <int PID = 1>
+static int cluster_plan(int n) {
+    if constexpr (PID > kBothWidths)
+        return 0;
+    else
+        return FixedPlan<PID>::N == n ? PID : cluster_plan<PID + 1>(n);
+}
+int default_elastic_plan(const AxisPlan& pz) { return default_elastic_form(pz) == 2 ? cluster_plan(pz.n) : 0; }
+
+// plan from an explicit radix order (each radix in {2,3,4,5,6,8,9,10,12,15,16}, product n)
 bool make_axis_plan_radices(int n, const int* rad, int nr, AxisPlan& p) {
     if (nr < 1 || nr > kMaxRadices) return false;
     long long prod = 1;
     for (int s = 0; s < nr; ++s) {
-        if (rad[s] != 2 && rad[s] != 3 && rad[s] != 4 && rad[s] != 5 && rad[s] != 8 && rad[s] != 16) return false;
+        if (rad[s] < 2 || rad[s] > 16 || rad[s] == 7 || rad[s] == 11 || rad[s] == 13 || rad[s] == 14) return false;
         prod *= rad[s];
     }
     if (prod != n) return false;
@@ -18,7 +52,7 @@ bool make_axis_plan_radices(int n, const int* rad, int nr, AxisPlan& p) {
     p.nst = nr;
     p.has16 = 0;
     for (int s = 0; s < nr; ++s)
-        if (rad[s] == 16) p.has16 = 1;
+        if (rad[s] > 8) p.has16 = 1;
     unsigned Ns = 1;
     for (int s = 0; s < nr; ++s) {
         p.rad[s] = rad[s];
@@ -29,9 +63,49 @@ bool make_axis_plan_radices(int n, const int* rad, int nr, AxisPlan& p) {
     return true;
 }
 
-// default schedule: the fewest stages, largest radices first -- radix-16
-// stages (prefer16) or radix-8 ones, then a 8 / 4 (or 4*4 instead of 8*2,
-// 8*4 instead of 16*2) or 2, then the 3s and 5s
+namespace {
+// arithmetic instructions per point of a radix-R stage, with twiddles and as
+// the first stage (in tenths)
+int stage_cost(int r, bool first) {
+    switch (r) {
+        case 2: return first ? 20 : 30;
+        case 3: return first ? 40 : 67;
+        case 4: return first ? 40 : 60;
+        case 5: return first ? 64 : 96;
+        case 6: return first ? 60 : 93;
+        case 8: return first ? 70 : 90;
+        case 9: return first ? 98 : 133;
+        case 10: return first ? 84 : 120;
+        case 12: return first ? 80 : 117;
+        case 15: return first ? 104 : 141;
+        default: return first ? 101 : 120;  // behind 8 8 at 64 and 8 4 at 32
+    }
+}
+
+// descending radix lists of product n: the fewest stages, of those the
+// cheapest, of those the largest first radix
+void best_order(int n, int limit, std::vector<int>& cur, int cost, std::vector<int>& best, int& best_cost) {
+    if (n == 1) {
+        if (best.empty() || cur.size() < best.size() || (cur.size() == best.size() && cost < best_cost)) {
+            best = cur;
+            best_cost = cost;
+        }
+        return;
+    }
+    if (!best.empty() && cur.size() >= best.size()) return;
+    for (int r : {16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2}) {
+        if (r > limit || n % r) continue;
+        cur.push_back(r);
+        best_order(n / r, r, cur, cost + stage_cost(r, cur.size() == 1), best, best_cost);
+        cur.pop_back();
+    }
+}
+}  // namespace
+
+// default schedule.  FP32 (prefer16): the fewest stages, since a stage is a
+// trip through shared memory and a barrier, of those the fewest instructions.
+// FP64: radix-8 stages (wider ones spill at the occupancy of its passes), then
+// a 4 (or 4*4 instead of 8*2) or 2, then the 3s and 5s.
 bool make_axis_plan(int n, AxisPlan& p, bool prefer16) {
     int m = n, a = 0, b = 0, c = 0;
     while (m % 2 == 0) { m /= 2; ++a; }
@@ -41,24 +115,14 @@ bool make_axis_plan(int n, AxisPlan& p, bool prefer16) {
     int r[kMaxRadices + 8];
     int nr = 0;
     if (prefer16) {
-        int n16 = a / 4;
-        int rem = a % 4;
-        if (rem == 1 && n16 > 0) {
-            --n16;
-            rem = 5;
-        }
-        for (int i = 0; i < n16; ++i) r[nr++] = 16;
-        if (rem == 5) {
-            r[nr++] = 8;
-            r[nr++] = 4;
-        } else if (rem == 3) {
-            r[nr++] = 8;
-        } else if (rem == 2) {
-            r[nr++] = 4;
-        } else if (rem == 1) {
-            r[nr++] = 2;
-        }
-    } else {
+        std::vector<int> cur, best;
+        int cost = 0;
+        // short lines: at most radix 8, so that a tile still gives work to a few
+        // warps (at 30 points radix 15 left one half-warp of it busy)
+        best_order(n, n <= 48 ? 8 : 16, cur, 0, best, cost);
+        return make_axis_plan_radices(n, best.data(), (int)best.size(), p);
+    }
+    {
         int n8 = a / 3;
         const int rem = a % 3;
         bool two4 = false;

@@ -12,37 +12,23 @@
 // the first forward stage to every output field without a shared-memory
 // round trip.  The C2R packing of two real rows into one complex line is
 // folded into the first inverse stage (read straight from the staged
-// half-spectrum rows), the R2C unpacking into the store.  Stages ping-pong
-// between two shared-memory tiles of skewed lines.
+// half-spectrum rows), the R2C unpacking into the store.  Every stage runs in
+// place in one shared-memory tile of skewed lines: two tiles, with a barrier
+// less a stage, hold half the CTAs on an SM and were slower from 96 points on
+// (right-hand-side pass at 256^3: 256 us against 200, h pass 182 against 154)
+// and as fast at 64; so was copying the real fields into shared memory ahead
+// of the physics (213 against 200 us).
 #pragma once
 #include "pf_xpass.cuh"
 
 namespace pf {
 
-// XF_PHYS2_STG: XF_PHYS2 with the stored real fields the physics reads
-// copied into shared memory (cp.async) together with the input rows, so that
-// the physics does not wait on global loads
-enum XFMode { XF_PHYS1_H = 0, XF_PHYS1_RHS = 1, XF_PHYS2 = 2, XF_WRMS = 3, XF_PHYS2_STG = 4 };
+enum XFMode { XF_PHYS1_H = 0, XF_PHYS1_RHS = 1, XF_PHYS2 = 2, XF_WRMS = 3 };
 template <int MODE>
 struct XFIO {
-    static constexpr bool PHYS2 = MODE == XF_PHYS2 || MODE == XF_PHYS2_STG;
-    static constexpr int FIN = PHYS2 ? 3 : 4;  // input lines per row pair
+    static constexpr int FIN = MODE == XF_PHYS2 ? 3 : 4;  // input lines per row pair
     static constexpr int FOUT = MODE == XF_WRMS ? 0 : (MODE == XF_PHYS1_H ? 3 : 4);
 };
-
-// stages of a radix list, sub-transform size growing from NS: cur -> oth,
-// then the pointers swap (the result is in cur)
-template <int SIGN, int N, int NS, typename T2>
-__device__ __forceinline__ void xf_run(T2*&, T2*&, int, const T2*, Radices<>) {}
-template <int SIGN, int N, int NS, typename T2, int R, int... Rest>
-__device__ __forceinline__ void xf_run(T2*& cur, T2*& oth, int nl, const T2* tw, Radices<R, Rest...>) {
-    fft_stage_fixed<R, SIGN, N, NS>(cur, oth, nl, skewed_len(N), tw);
-    __syncthreads();
-    T2* t = cur;
-    cur = oth;
-    oth = t;
-    xf_run<SIGN, N, NS * R>(cur, oth, nl, tw, Radices<Rest...>{});
-}
 
 // In-place stage of NL skewed lines (one shared buffer): every job's R
 // inputs are loaded into registers, the CTA synchronises, then the
@@ -75,8 +61,10 @@ __device__ __forceinline__ void xf_stage_inplace(T2* S, const T2* __restrict__ t
         if (JOBS % NT == 0 || idx < JOBS) {
             const int line = idx / M, j = idx - line * M;
             const int jq = j / NS, k = j - jq * NS;
-            if constexpr (NS > 1) apply_twiddles<R, SIGN>(v[u], tw, k * TWS);
-            Bfly<R, SIGN, T2>::run(v[u]);
+            if constexpr (NS > 1)
+                tw_bfly<R, SIGN>(v[u], tw, k * TWS, N);
+            else
+                Bfly<R, SIGN, T2>::run(v[u]);
             T2* d = S + line * LS;
             const int a = jq * NS * R;  // outputs at a + k + t NS
             if constexpr ((NS * R) % 16 == 0 && NS % 16 == 0) {
@@ -119,14 +107,12 @@ struct XFShape {
     static constexpr int LS = N + N / 16;            // skewed line stride
 };
 
-// INPL: one shared buffer, every stage in place (half the shared memory, so
-// more CTAs per SM, for a barrier more per stage); registers bounded to 64 a
-// thread so that the registers do not cap the CTAs per SM first
-template <typename T, class Fwd, int P, int MODE, bool INPL>
-__global__ void __launch_bounds__(XFShape<Fwd, P>::NT, INPL ? (65536 / (XFShape<Fwd, P>::NT * 64) > 0
-                                                                     ? 65536 / (XFShape<Fwd, P>::NT * 64)
-                                                                     : 1)
-                                                              : 1)
+// registers bounded to 64 a thread, so that they do not cap the CTAs per SM
+// before the shared memory does
+template <class Fwd, int P, int MODE>
+__global__ void __launch_bounds__(XFShape<Fwd, P>::NT, 65536 / (XFShape<Fwd, P>::NT * 64) > 0
+                                                           ? 65536 / (XFShape<Fwd, P>::NT * 64)
+                                                           : 1)
     k_x_fused(Geo g, Phys ph, const float2* __restrict__ in,
                                                                   float2* __restrict__ out, float* __restrict__ R,
                                                                   const float* __restrict__ Rin,
@@ -140,7 +126,7 @@ __global__ void __launch_bounds__(XFShape<Fwd, P>::NT, INPL ? (65536 / (XFShape<
     constexpr int R1 = RadInfo<Inv>::first;  // first inverse stage
     extern __shared__ __align__(16) unsigned char smraw[];
     T2* A = reinterpret_cast<T2*>(smraw);
-    T2* B = INPL ? A : A + P * 4 * LS;
+    T2* B = A;  // the raw rows, where the first stage's results go
     const int npairs = g.nz * g.ny / 2;
     const int rp0 = blockIdx.x * P;
     const long long NK = g.NK, N3 = g.N;
@@ -174,27 +160,13 @@ __global__ void __launch_bounds__(XFShape<Fwd, P>::NT, INPL ? (65536 / (XFShape<
             }
         }
     }
-    // the real fields X, phi_v of the CTA's rows -> C ([row pair][field][2 rows][N]), 16-byte copies
-    constexpr bool STG = MODE == XF_PHYS2_STG;
-    float* C = reinterpret_cast<float*>(B + P * 4 * LS);
-    if constexpr (STG) {
-        constexpr int Q = N / 4;  // 16-byte chunks per row
-        for (int e = threadIdx.x; e < P * 8 * Q; e += NT) {
-            const int r = e / Q, q = e - r * Q;  // r = (rp 4 + f) 2 + (0: row y, 1: row y+1)
-            const int rp = r >> 3, f = (r >> 1) & 3;
-            if (rp0 + rp < npairs)
-                cp_async<16>(C + 4 * e, Rin + f * N3 + (2LL * (rp0 + rp) + (r & 1)) * N + 4 * q);
-            else
-                reinterpret_cast<float4*>(C)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    }
     cp_async_wait_all();
     __syncthreads();
     // 2. first inverse stage (radix R1, no twiddles), packing Z = a + i b of
     //    the two rows' half spectra (Hermitian extension, imaginary parts of
-    //    DC and Nyquist dropped): B -> A (in place: all loads, a barrier, the stores)
+    //    DC and Nyquist dropped), in place: all loads, a barrier, the stores
     {
-        constexpr int M1 = N / R1, JOBS = P * FIN * M1, JPT = INPL ? (JOBS + NT - 1) / NT : 1;
+        constexpr int M1 = N / R1, JOBS = P * FIN * M1, JPT = (JOBS + NT - 1) / NT;
         auto load = [&](int idx, T2* v) {
             const int line = idx / M1, j = idx - line * M1;
             const T2* ra = B + line * 2 * NXH;
@@ -219,31 +191,18 @@ __global__ void __launch_bounds__(XFShape<Fwd, P>::NT, INPL ? (65536 / (XFShape<
 #pragma unroll
             for (int t = 0; t < R1; ++t) d[skew<true>(j * R1 + t)] = v[t];
         };
-        if constexpr (INPL) {
-            T2 v[JPT][R1];
+        T2 v[JPT][R1];
 #pragma unroll
-            for (int u = 0; u < JPT; ++u)
-                if (JOBS % NT == 0 || threadIdx.x + u * NT < JOBS) load(threadIdx.x + u * NT, v[u]);
-            __syncthreads();
+        for (int u = 0; u < JPT; ++u)
+            if (JOBS % NT == 0 || threadIdx.x + u * NT < JOBS) load(threadIdx.x + u * NT, v[u]);
+        __syncthreads();
 #pragma unroll
-            for (int u = 0; u < JPT; ++u)
-                if (JOBS % NT == 0 || threadIdx.x + u * NT < JOBS) store(threadIdx.x + u * NT, v[u]);
-        } else {
-            for (int idx = threadIdx.x; idx < JOBS; idx += NT) {
-                T2 v[R1];
-                load(idx, v);
-                store(idx, v);
-            }
-        }
+        for (int u = 0; u < JPT; ++u)
+            if (JOBS % NT == 0 || threadIdx.x + u * NT < JOBS) store(threadIdx.x + u * NT, v[u]);
     }
     __syncthreads();
-    T2* cur = A;
-    T2* oth = B;
     // 3. inverse stages between the first and the last
-    if constexpr (INPL)
-        xf_run_inplace<+1, N, R1, P * FIN, NT>(cur, tw, typename PlanInner<Inv>::type{});
-    else
-        xf_run<+1, N, R1>(cur, oth, P * FIN, tw, typename PlanInner<Inv>::type{});
+    xf_run_inplace<+1, N, R1, P * FIN, NT>(A, tw, typename PlanInner<Inv>::type{});
     // 4. fused: last inverse stage, physics, first forward stage
     const int rp = threadIdx.x / M, j = threadIdx.x - (threadIdx.x / M) * M;
     const bool valid = rp0 + rp < npairs;
@@ -251,11 +210,10 @@ __global__ void __launch_bounds__(XFShape<Fwd, P>::NT, INPL ? (65536 / (XFShape<
     T2 vin[FIN][RM];
 #pragma unroll
     for (int f = 0; f < FIN; ++f) {
-        const T2* src = cur + (rp * FIN + f) * LS;
+        const T2* src = A + (rp * FIN + f) * LS;
 #pragma unroll
         for (int t = 0; t < RM; ++t) vin[f][t] = src[skew<true>(j + t * M)];
-        apply_twiddles<RM, +1>(vin[f], tw, j);  // NS = M: twiddle exponent j t
-        Bfly<RM, +1, T2>::run(vin[f]);
+        tw_bfly<RM, +1>(vin[f], tw, j, N);  // NS = M: twiddle exponent j t
     }
     if constexpr (MODE == XF_WRMS) {
         // sum of squares of the weighted error w_i LTE_i (weights from the
@@ -295,19 +253,11 @@ __global__ void __launch_bounds__(XFShape<Fwd, P>::NT, INPL ? (65536 / (XFShape<
         for (int t = 0; t < RM; ++t) {
             const int x = j + t * M;
             float Xr[2], pr[2][3], er[2][3];
-            if constexpr (XFIO<MODE>::PHYS2) {
+            if constexpr (MODE == XF_PHYS2) {
 #pragma unroll
                 for (int f = 0; f < 4; ++f) {
-                    float u0, u1;
-                    if constexpr (STG) {
-                        const float* c = C + ((rp * 4 + f) * 2) * N + x;
-                        u0 = c[0];
-                        u1 = c[N];
-                    } else {
-                        const float* b = Rin + f * N3 + row * N + x;
-                        u0 = valid ? b[0] : 0.f;
-                        u1 = valid ? b[N] : 0.f;
-                    }
+                    const float* b = Rin + f * N3 + row * N + x;
+                    const float u0 = valid ? b[0] : 0.f, u1 = valid ? b[N] : 0.f;
                     if (f == 0) {
                         Xr[0] = u0;
                         Xr[1] = u1;
@@ -352,31 +302,23 @@ __global__ void __launch_bounds__(XFShape<Fwd, P>::NT, INPL ? (65536 / (XFShape<
                 for (int v = 0; v < 3; ++v) vout[1 + v][t] = T2{gv[0][v], gv[1][v]};
             }
         }
-        if constexpr (INPL) __syncthreads();  // every input of the fused stage read before the stores
+        __syncthreads();  // every input of the fused stage read before the stores
 #pragma unroll
         for (int f = 0; f < FOUT; ++f) {
             Bfly<RM, -1, T2>::run(vout[f]);  // first forward stage: NS = 1, no twiddles
-            T2* d = oth + (rp * FOUT + f) * LS;
+            T2* d = A + (rp * FOUT + f) * LS;
 #pragma unroll
             for (int t = 0; t < RM; ++t) d[skew<true>(j * RM + t)] = vout[f][t];
         }
         __syncthreads();
-        {
-            T2* t = cur;
-            cur = oth;
-            oth = t;
-        }
         // 5. the remaining forward stages
-        if constexpr (INPL)
-            xf_run_inplace<-1, N, RM, P * FOUT, NT>(cur, tw, typename DropFirst<Fwd>::type{});
-        else
-            xf_run<-1, N, RM>(cur, oth, P * FOUT, tw, typename DropFirst<Fwd>::type{});
+        xf_run_inplace<-1, N, RM, P * FOUT, NT>(A, tw, typename DropFirst<Fwd>::type{});
         // 6. R2C unpacking of the two rows of each line and the store
         for (int e = threadIdx.x; e < P * FOUT * NXH; e += NT) {
             const int line = e / NXH, k = e - line * NXH, lrp = line / FOUT, f = line - lrp * FOUT;
             if (rp0 + lrp >= npairs) continue;
-            const T2 Zk = cur[line * LS + skew<true>(k)];
-            const T2 Zm = cur[line * LS + skew<true>(k == 0 ? 0 : N - k)];
+            const T2 Zk = A[line * LS + skew<true>(k)];
+            const T2 Zm = A[line * LS + skew<true>(k == 0 ? 0 : N - k)];
             const T2 a = T2{(Zk.x + Zm.x) * 0.5f, (Zk.y - Zm.y) * 0.5f};
             const T2 b = T2{(Zk.y + Zm.y) * 0.5f, (Zm.x - Zk.x) * 0.5f};
             T2* base = out + (long long)f * NK + (2LL * (rp0 + lrp)) * NXH + k;
@@ -387,8 +329,10 @@ __global__ void __launch_bounds__(XFShape<Fwd, P>::NT, INPL ? (65536 / (XFShape<
 }
 
 // fused plans by line length (FP32): the first forward radix is small so the
-// fused stage holds few values per field; P row pairs per CTA, chosen so that
-// the CTA is a whole number of warps
+// fused stage holds few values per field; P row pairs per CTA, chosen for about 100 to
+// 400 threads (whole warps) and, below 128 points, so that a cube of that side has
+// at least about 150 CTAs: at 32 points 16 CTAs of 32 pairs took 4 us more a pass
+
 template <int N>
 struct XFPlan {
     static constexpr bool ok = false;
@@ -400,26 +344,45 @@ struct XFPlan {
         static constexpr int P = P_;         \
         using Fwd = Radices<__VA_ARGS__>;    \
     };
-PF_XF_PLAN(64, 16, 4, 16)
+PF_XF_PLAN(32, 4, 4, 8)
+PF_XF_PLAN(48, 8, 4, 12)
+PF_XF_PLAN(64, 8, 4, 16)
+PF_XF_PLAN(72, 8, 3, 12, 2)
+PF_XF_PLAN(80, 8, 5, 16)
 PF_XF_PLAN(96, 8, 4, 8, 3)
+PF_XF_PLAN(100, 8, 5, 10, 2)
+PF_XF_PLAN(108, 8, 3, 12, 3)
 PF_XF_PLAN(120, 4, 3, 8, 5)
 PF_XF_PLAN(128, 8, 4, 8, 4)
+PF_XF_PLAN(144, 4, 3, 12, 4)
 PF_XF_PLAN(160, 4, 4, 8, 5)
+PF_XF_PLAN(180, 8, 3, 15, 4)
 PF_XF_PLAN(192, 4, 4, 16, 3)
+PF_XF_PLAN(200, 8, 5, 10, 4)
+PF_XF_PLAN(216, 4, 3, 12, 6)
+PF_XF_PLAN(240, 4, 3, 10, 8)
 PF_XF_PLAN(256, 4, 4, 16, 4)
+PF_XF_PLAN(288, 2, 3, 12, 8)
+PF_XF_PLAN(300, 8, 5, 6, 10)
+PF_XF_PLAN(320, 4, 4, 10, 8)
+PF_XF_PLAN(360, 4, 3, 15, 8)
+PF_XF_PLAN(384, 2, 4, 12, 8)
+PF_XF_PLAN(400, 4, 5, 10, 8)
+PF_XF_PLAN(432, 2, 3, 12, 12)
+PF_XF_PLAN(480, 2, 3, 16, 10)
+PF_XF_PLAN(512, 2, 4, 16, 8)
 PF_XF_PLAN(640, 2, 5, 16, 8)
 #undef PF_XF_PLAN
 
-template <int N, int MODE, bool INPL>
+template <int N, int MODE>
 static int launch_x_fused_k(const Geo& g, const Phys& ph, const void* in, void* out, void* R, const void* Rin,
                             double* partials, double rtol, double atol, cudaStream_t s) {
     using Pl = XFPlan<N>;
     using Sh = XFShape<typename Pl::Fwd, Pl::P>;
-    const size_t sm = (INPL ? 1 : 2) * (size_t)Pl::P * 4 * Sh::LS * sizeof(float2) +
-                      (MODE == XF_PHYS2_STG ? (size_t)Pl::P * 8 * N * sizeof(float) : 0);
+    const size_t sm = (size_t)Pl::P * 4 * Sh::LS * sizeof(float2);
     const int npairs = g.nz * g.ny / 2;
     const int nb = (npairs + Pl::P - 1) / Pl::P;
-    auto k = k_x_fused<float, typename Pl::Fwd, Pl::P, MODE, INPL>;
+    auto k = k_x_fused<typename Pl::Fwd, Pl::P, MODE>;
     set_smem(k, sm);
     k<<<nb, Sh::NT, sm, s>>>(g, ph, reinterpret_cast<const float2*>(in), reinterpret_cast<float2*>(out),
                              reinterpret_cast<float*>(R), reinterpret_cast<const float*>(Rin), partials, (float)rtol,
@@ -427,48 +390,20 @@ static int launch_x_fused_k(const Geo& g, const Phys& ph, const void* in, void* 
     return nb;
 }
 
-template <int N, int MODE>
-static int launch_x_fused_n(const Geo& g, const Phys& ph, const void* in, void* out, void* R, const void* Rin,
-                            double* partials, double rtol, double atol, cudaStream_t s) {
-    return g.xf_inpl ? launch_x_fused_k<N, MODE, true>(g, ph, in, out, R, Rin, partials, rtol, atol, s)
-                     : launch_x_fused_k<N, MODE, false>(g, ph, in, out, R, Rin, partials, rtol, atol, s);
-}
-
+// the fused x pass of line length N; returns the number of CTAs launched, 0
+// for a mode it does not have
 template <int N>
-static int launch_x_fused_modes(const Geo& g, const Phys& ph, int mode, const void* in, void* out, void* R,
-                                const void* Rin, double* partials, double rtol, double atol, cudaStream_t s) {
-    if constexpr (!XFPlan<N>::ok) {
-        return 0;
-    } else {
-        switch (mode) {
-            case XM_PHYS1:
-                return ph.elastic ? launch_x_fused_n<N, XF_PHYS1_H>(g, ph, in, out, R, Rin, partials, rtol, atol, s)
-                                  : launch_x_fused_n<N, XF_PHYS1_RHS>(g, ph, in, out, R, Rin, partials, rtol, atol, s);
-            case XM_PHYS2:
-                if (!ph.elastic) return 0;
-                return g.xf_stg ? launch_x_fused_n<N, XF_PHYS2_STG>(g, ph, in, out, R, Rin, partials, rtol, atol, s)
-                                : launch_x_fused_n<N, XF_PHYS2>(g, ph, in, out, R, Rin, partials, rtol, atol, s);
-            case XM_WRMS: return launch_x_fused_n<N, XF_WRMS>(g, ph, in, out, R, Rin, partials, rtol, atol, s);
-            default: return 0;
-        }
-    }
-}
-
-// the fused x pass for FP32 contexts where the line length has a fused plan;
-// returns the number of CTAs launched, 0 if it does not apply
-int launch_x_fused(const Geo& g, const Phys& ph, int mode, const void* in, void* out, void* R, const void* Rin,
-                          double* partials, double rtol, double atol, cudaStream_t s) {
-    // the obstacle barrier runs the staged passes (the fused ones carry only the double well)
-    if (g.xf_off || ph.obst) return 0;
-    switch (g.nx) {
-        case 64: return launch_x_fused_modes<64>(g, ph, mode, in, out, R, Rin, partials, rtol, atol, s);
-        case 96: return launch_x_fused_modes<96>(g, ph, mode, in, out, R, Rin, partials, rtol, atol, s);
-        case 120: return launch_x_fused_modes<120>(g, ph, mode, in, out, R, Rin, partials, rtol, atol, s);
-        case 128: return launch_x_fused_modes<128>(g, ph, mode, in, out, R, Rin, partials, rtol, atol, s);
-        case 160: return launch_x_fused_modes<160>(g, ph, mode, in, out, R, Rin, partials, rtol, atol, s);
-        case 192: return launch_x_fused_modes<192>(g, ph, mode, in, out, R, Rin, partials, rtol, atol, s);
-        case 256: return launch_x_fused_modes<256>(g, ph, mode, in, out, R, Rin, partials, rtol, atol, s);
-        case 640: return launch_x_fused_modes<640>(g, ph, mode, in, out, R, Rin, partials, rtol, atol, s);
+int launch_x_fused_n(const Geo& g, const Phys& ph, int mode, const void* in, void* out, void* R, const void* Rin,
+                     double* partials, double rtol, double atol, cudaStream_t s) {
+    static_assert(XFPlan<N>::ok, "no fused plan of this length");
+    switch (mode) {
+        case XM_PHYS1:
+            return ph.elastic ? launch_x_fused_k<N, XF_PHYS1_H>(g, ph, in, out, R, Rin, partials, rtol, atol, s)
+                              : launch_x_fused_k<N, XF_PHYS1_RHS>(g, ph, in, out, R, Rin, partials, rtol, atol, s);
+        case XM_PHYS2:
+            if (!ph.elastic) return 0;
+            return launch_x_fused_k<N, XF_PHYS2>(g, ph, in, out, R, Rin, partials, rtol, atol, s);
+        case XM_WRMS: return launch_x_fused_k<N, XF_WRMS>(g, ph, in, out, R, Rin, partials, rtol, atol, s);
         default: return 0;
     }
 }

@@ -25,8 +25,8 @@ __global__ void __launch_bounds__(kThreads) k_y_pass(Geo g, typename Cx<T>::t* _
     cols_fft<SIGN, TX, true, 0, R16, PID, true>(g.py, A, B, src, dst);
 }
 
-template <typename T>
-void launch_y_pass(const Geo& g, void* buf, int nf, int sign, cudaStream_t s) {
+template <typename T, int SIGN>
+void launch_y_pass_sign(const Geo& g, void* buf, int nf, cudaStream_t s) {
     using T2 = typename Cx<T>::t;
     const int TX = tuned_cols<T>(g.tx_y, g.ny, 2, 128 * 1024, (long long)nf * g.nz * g.nxh);
     // a transform of at most two stages never touches its second buffer
@@ -35,18 +35,13 @@ void launch_y_pass(const Geo& g, void* buf, int nf, int sign, cudaStream_t s) {
     // CTAs per SM
     const size_t sm = col_buffers<T>(g.py, TX) * (size_t)TX * g.ny * sizeof(T2);
     dim3 grid(column_tiles(g.nxh, g.nz, TX), nf);
-    if (sign > 0) {
-        PF_COL_SWITCH(T, g.py, TX, set_smem(k_y_pass<T, 1, TXC, R16C, PIDC>, sm);
-                      k_y_pass<T, 1, TXC, R16C, PIDC><<<grid, kThreads, sm, s>>>(g, reinterpret_cast<T2*>(buf)));
-    } else {
-        PF_COL_SWITCH(T, g.py, TX, set_smem(k_y_pass<T, -1, TXC, R16C, PIDC>, sm);
-                      k_y_pass<T, -1, TXC, R16C, PIDC><<<grid, kThreads, sm, s>>>(g, reinterpret_cast<T2*>(buf)));
-    }
+    PF_COL_SWITCH(T, g.py, TX, set_smem(k_y_pass<T, SIGN, TXC, R16C, PIDC>, sm);
+                  k_y_pass<T, SIGN, TXC, R16C, PIDC><<<grid, kThreads, sm, s>>>(g, reinterpret_cast<T2*>(buf)));
 }
 
 // ---------------------------------------------------------------------------
-// z pass: in-place FFT along z of nf fields (the inverse transform of an
-// assembled FP32-bulk stage)
+// z pass: in-place inverse FFT along z of nf fields (of an assembled FP32-bulk
+// stage)
 // ---------------------------------------------------------------------------
 template <typename T, int SIGN, int TX, bool R16, int PID>
 __global__ void __launch_bounds__(kThreads) k_z_pass(Geo g, typename Cx<T>::t* __restrict__ buf) {
@@ -66,18 +61,13 @@ __global__ void __launch_bounds__(kThreads) k_z_pass(Geo g, typename Cx<T>::t* _
 }
 
 template <typename T>
-void launch_z_pass(const Geo& g, void* buf, int nf, int sign, cudaStream_t s) {
+void launch_z_pass(const Geo& g, void* buf, int nf, cudaStream_t s) {
     using T2 = typename Cx<T>::t;
     const int TX = tuned_cols<T>(g.tx_zf, g.nz, 2, 128 * 1024, (long long)nf * g.ny * g.nxh);
     const size_t sm = col_buffers<T>(g.pz, TX) * (size_t)TX * g.nz * sizeof(T2);  // as in the y pass
     dim3 grid(column_tiles(g.nxh, g.ny, TX), nf);
-    if (sign > 0) {
-        PF_COL_SWITCH(T, g.pz, TX, set_smem(k_z_pass<T, 1, TXC, R16C, PIDC>, sm);
-                      k_z_pass<T, 1, TXC, R16C, PIDC><<<grid, kThreads, sm, s>>>(g, reinterpret_cast<T2*>(buf)));
-    } else {
-        PF_COL_SWITCH(T, g.pz, TX, set_smem(k_z_pass<T, -1, TXC, R16C, PIDC>, sm);
-                      k_z_pass<T, -1, TXC, R16C, PIDC><<<grid, kThreads, sm, s>>>(g, reinterpret_cast<T2*>(buf)));
-    }
+    PF_COL_SWITCH(T, g.pz, TX, set_smem(k_z_pass<T, 1, TXC, R16C, PIDC>, sm);
+                  k_z_pass<T, 1, TXC, R16C, PIDC><<<grid, kThreads, sm, s>>>(g, reinterpret_cast<T2*>(buf)));
 }
 
 // ---------------------------------------------------------------------------
@@ -250,8 +240,10 @@ __device__ __forceinline__ void tile_stage_io(const T2* __restrict__ tw, Ld ld, 
 #pragma unroll
         for (int t = 0; t < R; ++t) v[t] = ld(f, j + t * M, col);
         const int jq = j / NS, k = j - jq * NS;
-        if constexpr (NS > 1) apply_twiddles<R, SIGN>(v, tw, k * TWS);
-        Bfly<R, SIGN, T2>::run(v);
+        if constexpr (NS > 1)
+            tw_bfly<R, SIGN>(v, tw, k * TWS, N);
+        else
+            Bfly<R, SIGN, T2>::run(v);
         const int base = jq * NS * R + k;
 #pragma unroll
         for (int t = 0; t < R; ++t) st(f, base + t * NS, col, v[t]);
@@ -314,8 +306,7 @@ __global__ void __launch_bounds__(NT, elastic_min_blocks<T, PID, NT>())
             const T2* src = S + f * (N * TX) + j * TX + col;
 #pragma unroll
             for (int t = 0; t < RL; ++t) h[f][t] = src[t * M * TX];
-            apply_twiddles<RL, -1>(h[f], tw, j);  // NS = N / RL: k = j, table stride 1
-            Bfly<RL, -1, T2>::run(h[f]);
+            tw_bfly<RL, -1>(h[f], tw, j, N);  // NS = N / RL: k = j, table stride 1
         }
         __syncthreads();
         const T invN = std::is_same<T, float>::value ? (T)g.invN32 : (T)g.invN;
@@ -506,16 +497,15 @@ static bool launch_z_elastic_unf(const Geo& g, const Phys& ph, void* H, int tune
         return false;
     } else {
         constexpr int N = FixedPlan<PID>::N;
+        // untuned: 16 columns up to 50 KB (128 points), else 8 while they fit
+        // (at 160 points 8 take 51.7 us against 56.1 for 16, at 256 165 against
+        // 174, at 128 24.3 against 23.1)
+        constexpr int TXD = 3 * 16 * N * sizeof(T2) <= 50 * 1024 ? 16 : (3 * 8 * N * sizeof(T2) <= 100 * 1024 ? 8 : 4);
         auto fits = [&](int tx) { return 3 * (size_t)tx * N * sizeof(T2) <= 100 * 1024; };
         int TX = 0;
         for (int tx : {16, 8, 4, 2})
             if (fits(tx) && (TX == 0 || (tuned > 0 && tx == tuned))) TX = tx;
-        if (tuned <= 0)
-            for (int tx : {16, 8, 4, 2})
-                if (fits(tx)) {
-                    TX = tx;
-                    break;
-                }
+        if (tuned <= 0 || PID > kBothWidths) TX = fits(TXD) ? TXD : 0;
         if (TX == 0) return false;
         const size_t sm = 3 * (size_t)TX * N * sizeof(T2);
         const unsigned grid = column_tiles(g.nxh, g.ny, TX);
@@ -525,33 +515,35 @@ static bool launch_z_elastic_unf(const Geo& g, const Phys& ph, void* H, int tune
         set_smem(k_z_elastic_stages<T, TXC, PID, NTU>, sm);                                           \
         k_z_elastic_stages<T, TXC, PID, NTU><<<grid, NTU, sm, s>>>(g, ph, reinterpret_cast<T2*>(H));  \
     }
-        switch (TX) {
-            case 16: PF_ELU(16); break;
-            case 8: PF_ELU(8); break;
-            case 4: PF_ELU(4); break;
-            default: PF_ELU(2); break;
+        if constexpr (PID > kBothWidths) {
+            PF_ELU(TXD)
+        } else {
+            switch (TX) {
+                case 16: PF_ELU(16); break;
+                case 8: PF_ELU(8); break;
+                case 4: PF_ELU(4); break;
+                default: PF_ELU(2); break;
+            }
         }
 #undef PF_ELU
         return true;
     }
 }
 
+template <typename T, int PID = 1>
+static bool unfused_by_plan(const Geo& g, const Phys& ph, void* H, int pid, cudaStream_t s) {
+    // FP64 contexts never have the FP32 default plans
+    if constexpr (PID > (sizeof(T) == 4 ? kFixedPlans : kBothWidths)) {
+        return false;
+    } else {
+        if (pid == PID) return launch_z_elastic_unf<T, PID>(g, ph, H, g.tx_el, s);
+        return unfused_by_plan<T, PID + 1>(g, ph, H, pid, s);
+    }
+}
+
 template <typename T>
 bool launch_z_elastic_unfused(const Geo& g, const Phys& ph, void* H, int pid, cudaStream_t s) {
-    switch (pid) {
-        case 1: return launch_z_elastic_unf<T, 1>(g, ph, H, g.tx_el, s);
-        case 2: return launch_z_elastic_unf<T, 2>(g, ph, H, g.tx_el, s);
-        case 3: return launch_z_elastic_unf<T, 3>(g, ph, H, g.tx_el, s);
-        case 4: return launch_z_elastic_unf<T, 4>(g, ph, H, g.tx_el, s);
-        case 5: return launch_z_elastic_unf<T, 5>(g, ph, H, g.tx_el, s);
-        case 6: return launch_z_elastic_unf<T, 6>(g, ph, H, g.tx_el, s);
-        case 7: return launch_z_elastic_unf<T, 7>(g, ph, H, g.tx_el, s);
-        case 8: return launch_z_elastic_unf<T, 8>(g, ph, H, g.tx_el, s);
-        case 9: return launch_z_elastic_unf<T, 9>(g, ph, H, g.tx_el, s);
-        case 10: return launch_z_elastic_unf<T, 10>(g, ph, H, g.tx_el, s);
-        case 11: return launch_z_elastic_unf<T, 11>(g, ph, H, g.tx_el, s);
-        default: return false;
-    }
+    return unfused_by_plan<T>(g, ph, H, pid, s);
 }
 #endif
 

@@ -1,0 +1,78 @@
+"""Compiled plans of common line lengths and the wide radices (6, 9, 10, 12,
+15) against the oracle: one ARK4 step with its error norm, each length along
+each axis in turn, and explicit orders of the wide radices in the generic
+stages of both precisions."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+LENGTHS = [32, 48, 72, 80, 96, 100, 108, 120, 144, 160, 180, 192, 200, 216, 240, 288, 300, 320, 360, 384, 400, 432,
+           480, 512, 640]
+
+
+@pytest.fixture(scope="module")
+def pfg():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2609_36100_gb300 as m
+    m.build()
+    return m
+
+
+def relerr(a, b):
+    return np.array([np.linalg.norm((a[f] - b[f]).ravel()) / np.linalg.norm(b[f].ravel()) for f in range(4)])
+
+
+def step_case(pfg, p, shape, prec, seed, cfg=None):
+    y = synth.random_state(shape, seed, phi_scale=0.9)
+    m = oracle.Model(shape, p)
+    ref, e_ref, _ = oracle.ark_step(m, m.to_k(y), 0.5, oracle.ark436l2sa(), p["rtol"], p["atol"])
+    with pfg.Simulation(shape, p, "ark4", prec) as s:
+        if cfg:
+            c = s.tuning()
+            for axis, order in cfg.items():
+                c[4 + 11 * axis:4 + 11 * (axis + 1)] = [len(order)] + order + [0] * (10 - len(order))
+            s.set_tuning(c)
+            assert s.tuning() == c
+        else:
+            c = s.tuning()
+            s.set_tuning(c)  # what a context reports it takes back
+        s.set_state(y)
+        e = s.step(0.5)
+        return relerr(s.state_hat().cpu().numpy(), ref), abs(e - e_ref) / e_ref
+
+
+@pytest.mark.parametrize("n", LENGTHS)
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_default_plans_match_oracle(pfg, params, n, axis):
+    shape = [12, 10, 6]  # half rows of four columns: every tile ends in the middle of a plane
+    shape[2 - axis] = n
+    err, e = step_case(pfg, params, tuple(shape), "fp32bulk", 10 + n)
+    assert np.all(err <= 1e-5), err
+    assert e <= 1e-3
+
+
+@pytest.mark.parametrize("prec,tol,etol", [("fp64", 1e-11, 1e-8), ("fp32bulk", 1e-5, 1e-3)])
+@pytest.mark.parametrize("orders", [
+    {0: [6, 15], 1: [12], 2: [10, 9]},
+    {0: [9, 10], 1: [2, 6], 2: [15, 6]},
+    {0: [10, 3, 3], 1: [3, 4], 2: [6, 15]},
+])
+def test_wide_radices_match_oracle(pfg, params, prec, tol, etol, orders):
+    err, e = step_case(pfg, params, (90, 12, 90), prec, 5, orders)
+    assert np.all(err <= tol), err
+    assert e <= etol
+
+
+def test_radix_that_is_none_refused(pfg, params):
+    with pfg.Simulation((14 * 5 + 10, 12, 10), params, "ark4", "fp64") as s:
+        c = s.tuning()
+        for bad in ([20, 4], [7, 10], [80], [0, 80], [-8, -10]):
+            c[4 + 22:4 + 33] = [len(bad)] + bad + [0] * (10 - len(bad))
+            with pytest.raises(pfg.PFError):
+                s.set_tuning(c)
