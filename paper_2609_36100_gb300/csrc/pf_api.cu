@@ -195,6 +195,8 @@ struct pf_ctx {
     Tableau tab;
     bool fp32 = false;
     Geo g{};
+    Geo g64{};  // g with the FP64 schedules: of the FP64 transforms of a FP32-bulk context
+    const Geo& geo64() const { return fp32 ? g64 : g; }
     Phys ph{};
     // stage bookkeeping
     bool need_fe[kMaxStages] = {};
@@ -223,10 +225,11 @@ struct pf_ctx {
     // phase-dependent stiffness (Hu-Chen iterations, FP64)
     bool inhom = false;
     HCConst hck{};
-    double* hc_tau = nullptr;      // eigenstress, real [8][N] (xx yy zz yz | xz xy, two padding fields)
-    double* hc_eu[2] = {};         // eps(u), real [8][N]: current and previous iterate
-    double2* hc_k = nullptr;       // k-space [8][NK] (tau^, then eps^(u))
-    double2* hc_ks = nullptr;      // partial-transform scratch [4][NK]
+    double* hc_pt = nullptr;       // C(r) and eps0 of the solve's fields, real [9][N]
+    double* hc_tau = nullptr;      // eigenstress, real [6][N] (xx yy zz yz xz xy)
+    double* hc_eu[2] = {};         // eps(u), real [6][N]: current and previous iterate
+    double2* hc_k = nullptr;       // k-space [6][NK] (tau^, then eps^(u))
+    double2* hc_ks = nullptr;      // partial-transform scratch [6][NK]
     double* hc_part = nullptr;     // per-block statistics [blocks][11]
     double* hc_ebar = nullptr;     // eps_bar on the device [6]
     double* hc_host = nullptr;     // pinned: statistics [blocks][11] and eps_bar [6]
@@ -392,6 +395,7 @@ void free_all(pf_ctx* c) {
     cudaFree(c->xsave);
     cudaFree(c->qtab);
     cudaFree(c->partials);
+    cudaFree(c->hc_pt);
     cudaFree(c->hc_tau);
     cudaFree(c->hc_eu[0]);
     cudaFree(c->hc_eu[1]);
@@ -466,43 +470,39 @@ struct ProfScope {
 // <= el_tol max |eps0| or el_max_iter solves; writes the driving
 // forces e_v into E ([3][N] of type TR, if not null) and the elastic energy
 // sum_r sigma:eps_el/2 (without the volume element) into *energy (if not
-// null).  Each transform is the FP64 four-field pipeline of set/get state.
+// null).  The transforms are those of set/get state, of the six components.
 template <typename TR>
 int hc_solve(pf_ctx* c, const void* R, void* E, double* energy) {
-    const Geo& g = c->g;
+    const Geo& g = c->geo64();
     const Phys& ph = c->ph;
     cudaStream_t s = c->stream;
     const HCConst& k = c->hck;
     const int nb = hc_blocks();
     const long long N = g.N, NK = g.NK;
     double* host = c->hc_host;
-    double* ebar_h = host + (size_t)nb * 11;
-    auto forward = [&](const double* real, double2* out) {  // 4 real fields -> normalised k-space
-        launch_x_pass<double>(g, ph, XM_R2C_REAL, nullptr, c->hc_ks, nullptr, nullptr, nullptr, 0, 0, real, nullptr, s);
-        launch_y_pass<double>(g, c->hc_ks, 4, -1, s);
-        launch_z_fwd<double>(g, ph, c->hc_ks, out, 0, s);
-    };
-    auto inverse = [&](const double2* in, double* real) {  // 4 k-space fields -> real
-        StageTerms none{};
-        launch_z_stage<double>(g, ph, in, none, nullptr, c->hc_ks, s);
-        launch_y_pass<double>(g, c->hc_ks, 4, +1, s);
-        launch_x_pass<double>(g, ph, XM_C2R_REAL, c->hc_ks, nullptr, nullptr, nullptr, nullptr, 0, 0, nullptr, real, s);
-    };
+    double* ebar_h = host + (size_t)nb * kHcStats;
     auto green = [&](double* eu) {
-        forward(c->hc_tau, c->hc_k);
-        forward(c->hc_tau + 4 * N, c->hc_k + 4 * NK);
+        for (int h = 0; h < 2; ++h)
+            launch_x_pass<double>(g, ph, XM_R2C_REAL3, nullptr, c->hc_ks + 3 * h * NK, nullptr, nullptr, nullptr, 0, 0,
+                                  c->hc_tau + 3 * h * N, nullptr, s);
+        launch_y_pass<double>(g, c->hc_ks, 6, -1, s);
+        launch_z_fwd<double>(g, ph, c->hc_ks, c->hc_k, 0, s, 6);
         launch_hc_green(g, k, c->hc_k, s);
-        inverse(c->hc_k, eu);
-        inverse(c->hc_k + 4 * NK, eu + 4 * N);
+        launch_z_pass<double>(g, c->hc_k, 6, s);
+        launch_y_pass<double>(g, c->hc_k, 6, +1, s);
+        for (int h = 0; h < 2; ++h)
+            launch_x_pass<double>(g, ph, XM_C2R_REAL3, c->hc_k + 3 * h * NK, nullptr, nullptr, nullptr, nullptr, 0, 0,
+                                  nullptr, eu + 3 * h * N, s);
     };
     // statistics -> eps_bar (host) and the change / scale
     auto stats = [&](const double* eu, const double* prev, double& change, double& scale) -> int {
-        launch_hc_stats<TR>(g, k, R, eu, prev, c->hc_part, s);
-        PF_CUDA(c, cudaMemcpyAsync(host, c->hc_part, (size_t)nb * 11 * sizeof(double), cudaMemcpyDeviceToHost, s));
+        launch_hc_stats(g, c->hc_pt, eu, prev, c->hc_part, s);
+        PF_CUDA(c, cudaMemcpyAsync(host, c->hc_part, (size_t)nb * kHcStats * sizeof(double), cudaMemcpyDeviceToHost, s));
         PF_CUDA(c, cudaStreamSynchronize(s));
-        double sum[11] = {};
+        double sum[kHcStats] = {};
         for (int b = 0; b < nb; ++b)
-            for (int q = 0; q < 11; ++q) sum[q] = q < 9 ? sum[q] + host[b * 11 + q] : std::fmax(sum[q], host[b * 11 + q]);
+            for (int q = 0; q < kHcStats; ++q)
+                sum[q] = q < 9 ? sum[q] + host[b * kHcStats + q] : std::fmax(sum[q], host[b * kHcStats + q]);
         double cav[3], sav[3], r[6];
         for (int a = 0; a < 3; ++a) cav[a] = sum[a] / (double)N;
         for (int a = 0; a < 6; ++a) r[a] = sum[3 + a] / (double)N;
@@ -519,6 +519,7 @@ int hc_solve(pf_ctx* c, const void* R, void* E, double* energy) {
         scale = sum[10];
         return PF_OK;
     };
+    launch_hc_point<TR>(g, k, R, c->hc_pt, c->hc_part, s);
     int cur = c->hc_cur;
     double change = 0.0, scale = 0.0;
     int it;
@@ -529,7 +530,7 @@ int hc_solve(pf_ctx* c, const void* R, void* E, double* energy) {
         if (int rc = stats(c->hc_eu[cur], nullptr, change, scale)) return rc;
         it = 0;
     } else {
-        launch_hc_tau<TR>(g, k, R, nullptr, nullptr, c->hc_tau, s);
+        launch_hc_tau(g, k, c->hc_pt, nullptr, nullptr, c->hc_tau, s);
         green(c->hc_eu[cur]);
         if (int rc = stats(c->hc_eu[cur], nullptr, change, scale)) return rc;
         it = 1;
@@ -538,7 +539,7 @@ int hc_solve(pf_ctx* c, const void* R, void* E, double* energy) {
     while (it < c->prm.el_max_iter) {
         const int prev = cur;
         cur ^= 1;
-        launch_hc_tau<TR>(g, k, R, c->hc_eu[prev], c->hc_ebar, c->hc_tau, s);
+        launch_hc_tau(g, k, c->hc_pt, c->hc_eu[prev], c->hc_ebar, c->hc_tau, s);
         green(c->hc_eu[cur]);
         if (int rc = stats(c->hc_eu[cur], c->hc_eu[prev], change, scale)) return rc;
         ++it;
@@ -547,9 +548,9 @@ int hc_solve(pf_ctx* c, const void* R, void* E, double* energy) {
     c->hc_iters = it;
     c->hc_cur = cur;
     c->hc_prev = c->prm.el_warm != 0;
-    if (E) launch_hc_force<TR>(g, k, R, c->hc_eu[cur], c->hc_ebar, E, s);
+    if (E) launch_hc_force<TR>(g, k, c->hc_pt, c->hc_eu[cur], c->hc_ebar, E, s);
     if (energy) {
-        launch_hc_energy<TR>(g, k, R, c->hc_eu[cur], c->hc_ebar, c->hc_part, s);
+        launch_hc_energy(g, c->hc_pt, c->hc_eu[cur], c->hc_ebar, c->hc_part, s);
         launch_reduce(c->hc_part, nb, 1.0, c->d_scalar + 2, s);
         PF_CUDA(c, cudaMemcpyAsync(c->h_scalar + 2, c->d_scalar + 2, sizeof(double), cudaMemcpyDeviceToHost, s));
         PF_CUDA(c, cudaStreamSynchronize(s));
@@ -973,20 +974,17 @@ int pf_create(const pf_grid* grid, const pf_params* params, void* cuda_stream, p
     if (energy_k_blocks(g) > c->npartials) c->npartials = energy_k_blocks(g);
     rc = rc ? rc : dalloc(c, &c->partials, (size_t)c->npartials * sizeof(double));
     if (c->inhom) {
-        const size_t n8 = 8 * (size_t)g.N * sizeof(double);
-        rc = rc ? rc : dalloc(c, &c->hc_tau, n8);
-        rc = rc ? rc : dalloc(c, &c->hc_eu[0], n8);
-        rc = rc ? rc : dalloc(c, &c->hc_eu[1], n8);
-        rc = rc ? rc : dalloc(c, &c->hc_k, 8 * (size_t)g.NK * sizeof(double2));
-        rc = rc ? rc : dalloc(c, &c->hc_ks, 4 * (size_t)g.NK * sizeof(double2));
-        rc = rc ? rc : dalloc(c, &c->hc_part, (size_t)hc_blocks() * 11 * sizeof(double));
+        const size_t n6 = 6 * (size_t)g.N * sizeof(double);
+        rc = rc ? rc : dalloc(c, &c->hc_pt, 9 * (size_t)g.N * sizeof(double));
+        rc = rc ? rc : dalloc(c, &c->hc_tau, n6);
+        rc = rc ? rc : dalloc(c, &c->hc_eu[0], n6);
+        rc = rc ? rc : dalloc(c, &c->hc_eu[1], n6);
+        rc = rc ? rc : dalloc(c, &c->hc_k, 6 * (size_t)g.NK * sizeof(double2));
+        rc = rc ? rc : dalloc(c, &c->hc_ks, 6 * (size_t)g.NK * sizeof(double2));
+        rc = rc ? rc : dalloc(c, &c->hc_part, (size_t)hc_blocks() * kHcStats * sizeof(double));
         rc = rc ? rc : dalloc(c, &c->hc_ebar, 6 * sizeof(double));
-        if (!rc && cudaMallocHost((void**)&c->hc_host, ((size_t)hc_blocks() * 11 + 8) * sizeof(double)) != cudaSuccess)
+        if (!rc && cudaMallocHost((void**)&c->hc_host, ((size_t)hc_blocks() * kHcStats + 8) * sizeof(double)) != cudaSuccess)
             rc = fail(c, PF_ENOMEM, "pinned host allocation failed");
-        // the padding fields of the second four-field group stay zero
-        if (!rc && (cudaMemset(c->hc_tau, 0, n8) != cudaSuccess || cudaMemset(c->hc_eu[0], 0, n8) != cudaSuccess ||
-                    cudaMemset(c->hc_eu[1], 0, n8) != cudaSuccess))
-            rc = fail(c, PF_ECUDA, "cudaMemset failed");
     }
     rc = rc ? rc : dalloc(c, &c->d_scalar, 4 * sizeof(double));
     if (!rc && cudaMallocHost((void**)&c->h_scalar, 4 * sizeof(double)) != cudaSuccess) {
@@ -1053,6 +1051,18 @@ int pf_create(const pf_grid* grid, const pf_params* params, void* cuda_stream, p
     g.kx32 = c->d_k32;
     g.ky32 = c->d_k32 + kx.size();
     g.kz32 = c->d_k32 + kx.size() + ky.size();
+    if (c->fp32) {
+        Geo& w = c->g64;
+        w = g;
+        AxisPlan* p64[3] = {&w.px, &w.py, &w.pz};
+        for (int a = 0; a < 3; ++a) {
+            make_axis_plan(ns[a], *p64[a], false);
+            p64[a]->tw64 = c->d_tw64[a];
+            p64[a]->tw32 = c->d_tw32[a];
+        }
+        w.el_unfused = w.el_pid = 0;
+        w.btab = nullptr;  // FP32 entries
+    }
     c->t = 0.0;
     c->h = params->h0;
     c->st.h = c->h;
@@ -1083,7 +1093,7 @@ static int check_finite(pf_ctx* c, const double* v, long long n, const char* whe
 int pf_set_state(pf_ctx* c, const double* fields, int on_device) {
     if (!c || !fields) return fail(c, PF_EINVAL, "pf_set_state: NULL argument");
     cudaSetDevice(c->dev);
-    const Geo& g = c->g;
+    const Geo& g = c->geo64();
     double* real = reinterpret_cast<double*>(fp64_scratch(c));
     const double* src = fields;
     if (!on_device) {
@@ -1106,7 +1116,7 @@ int pf_set_state(pf_ctx* c, const double* fields, int on_device) {
 int pf_get_state(pf_ctx* c, double* fields, int on_device) {
     if (!c || !fields) return fail(c, PF_EINVAL, "pf_get_state: NULL argument");
     cudaSetDevice(c->dev);
-    const Geo& g = c->g;
+    const Geo& g = c->geo64();
     StageTerms none{};
     launch_z_stage<double>(g, c->ph, c->y, none, nullptr, c->ynew, c->stream);
     launch_y_pass<double>(g, c->ynew, 4, +1, c->stream);
@@ -1176,7 +1186,7 @@ int pf_solve_implicit(pf_ctx* c, double gamma, const void* r_hat, void* z_hat) {
 // coefficients are restored unchanged, so its mean stays exact.
 static int project_obstacle(pf_ctx* c) {
     if (!c->ph.obst) return PF_OK;
-    const Geo& g = c->g;
+    const Geo& g = c->geo64();
     cudaStream_t s = c->stream;
     PF_CUDA(c, cudaMemcpyAsync(c->xsave, c->y, (size_t)g.NK * sizeof(double2), cudaMemcpyDeviceToDevice, s));
     StageTerms none{};
@@ -1555,7 +1565,7 @@ int pf_batch_advance(pf_ctx* const* ctxs, int n, double t_final, double rtol, do
 int pf_free_energy(pf_ctx* c, double* F_out) {
     if (!c || !F_out) return fail(c, PF_EINVAL, "pf_free_energy: NULL argument");
     cudaSetDevice(c->dev);
-    const Geo& g = c->g;
+    const Geo& g = c->geo64();
     cudaStream_t s = c->stream;
     double2* S1 = c->ynew;
     double2* S2 = fp64_scratch(c);

@@ -179,19 +179,20 @@ struct HCConst {
 void hc_constants(double C11, double C12, double C44, double C11v, double C12v, double C44v,
                   const double eps[3][6], HCConst& k);
 int hc_blocks();
+constexpr int kHcStats = 11;  // per-block statistics of a solve (see k_hc_point, k_hc_stats)
+// what a solve needs of the point's fields R: pt [9][N] = c11, c12, c44 of C(r), eps0 (xx yy zz yz xz xy)
 template <typename T>
-void launch_hc_tau(const Geo& g, const HCConst& k, const void* R, const double* eu, const double* ebar, double* tau,
-                   cudaStream_t s);
+void launch_hc_point(const Geo& g, const HCConst& k, const void* R, double* pt, double* part, cudaStream_t s);
+void launch_hc_tau(const Geo& g, const HCConst& k, const double* pt, const double* eu, const double* ebar,
+                   double* tau, cudaStream_t s);
 void launch_hc_green(const Geo& g, const HCConst& k, double2* hk, cudaStream_t s);
-template <typename T>
-void launch_hc_stats(const Geo& g, const HCConst& k, const void* R, const double* eu, const double* eu_prev,
-                     double* part, cudaStream_t s);
-template <typename T>
-void launch_hc_force(const Geo& g, const HCConst& k, const void* R, const double* eu, const double* ebar, void* E,
+void launch_hc_stats(const Geo& g, const double* pt, const double* eu, const double* eu_prev, double* part,
                      cudaStream_t s);
 template <typename T>
-void launch_hc_energy(const Geo& g, const HCConst& k, const void* R, const double* eu, const double* ebar,
-                      double* part, cudaStream_t s);
+void launch_hc_force(const Geo& g, const HCConst& k, const double* pt, const double* eu, const double* ebar, void* E,
+                     cudaStream_t s);
+void launch_hc_energy(const Geo& g, const double* pt, const double* eu, const double* ebar, double* part,
+                      cudaStream_t s);
 
 enum XMode {
     XM_PHYS1 = 0,      // C2R state -> real fields, h(phi) -> R2C (or the full RHS when elasticity is off)
@@ -200,6 +201,8 @@ enum XMode {
     XM_R2C_REAL = 3,   // real FP64 fields -> R2C (set_state)
     XM_C2R_REAL = 4,   // C2R -> real FP64 fields (get_state)
     XM_ENERGY = 5,     // C2R state -> local free-energy density partial sums + h -> R2C
+    XM_R2C_REAL3 = 7,  // XM_R2C_REAL and XM_C2R_REAL of three fields
+    XM_C2R_REAL3 = 8,
     XM_PHYS2R = 6      // real-space elastic potential (argument `in`, [3][N]) + stored real fields -> RHS -> R2C
 };
 

@@ -68,7 +68,7 @@ namespace {
 // the first stage (in tenths)
 int stage_cost(int r, bool first) {
     switch (r) {
-        case 2: return first ? 20 : 30;
+        case 2: return first ? 20 : 31;  // behind 4 4 in the place of 8 2
         case 3: return first ? 40 : 67;
         case 4: return first ? 40 : 60;
         case 5: return first ? 64 : 96;
@@ -83,67 +83,48 @@ int stage_cost(int r, bool first) {
 }
 
 // descending radix lists of product n: the fewest stages, of those the
-// cheapest, of those the largest first radix
-void best_order(int n, int limit, std::vector<int>& cur, int cost, std::vector<int>& best, int& best_cost) {
+// cheapest, of those the largest first radix; or the cheapest, of those the
+// fewest stages (by_cost)
+void best_order(int n, int limit, bool by_cost, std::vector<int>& cur, int cost, std::vector<int>& best,
+                int& best_cost) {
     if (n == 1) {
-        if (best.empty() || cur.size() < best.size() || (cur.size() == best.size() && cost < best_cost)) {
+        const int ns = (int)cur.size(), nb = (int)best.size();
+        const bool better = by_cost ? cost < best_cost || (cost == best_cost && ns < nb)
+                                    : ns < nb || (ns == nb && cost < best_cost);
+        if (best.empty() || better) {
             best = cur;
             best_cost = cost;
         }
         return;
     }
-    if (!best.empty() && cur.size() >= best.size()) return;
+    if (!by_cost && !best.empty() && cur.size() >= best.size()) return;
     for (int r : {16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2}) {
         if (r > limit || n % r) continue;
         cur.push_back(r);
-        best_order(n / r, r, cur, cost + stage_cost(r, cur.size() == 1), best, best_cost);
+        best_order(n / r, r, by_cost, cur, cost + stage_cost(r, cur.size() == 1), best, best_cost);
         cur.pop_back();
     }
 }
 }  // namespace
 
 // default schedule.  FP32 (prefer16): the fewest stages, since a stage is a
-// trip through shared memory and a barrier, of those the fewest instructions.
-// FP64: radix-8 stages (wider ones spill at the occupancy of its passes), then
-// a 4 (or 4*4 instead of 8*2) or 2, then the 3s and 5s.
+// trip through shared memory and a barrier, of those the fewest instructions;
+// short lines at most radix 8, so that a tile still gives work to a few warps
+// (at 30 points radix 15 left one half-warp of it busy).  FP64 passes take the
+// time of their FP64 instructions: the fewest of those, with radices of at most
+// 12 (wider ones spill).
 bool make_axis_plan(int n, AxisPlan& p, bool prefer16) {
-    int m = n, a = 0, b = 0, c = 0;
-    while (m % 2 == 0) { m /= 2; ++a; }
-    while (m % 3 == 0) { m /= 3; ++b; }
-    while (m % 5 == 0) { m /= 5; ++c; }
-    if (m != 1) return false;
-    int r[kMaxRadices + 8];
-    int nr = 0;
-    if (prefer16) {
-        std::vector<int> cur, best;
-        int cost = 0;
-        // short lines: at most radix 8, so that a tile still gives work to a few
-        // warps (at 30 points radix 15 left one half-warp of it busy)
-        best_order(n, n <= 48 ? 8 : 16, cur, 0, best, cost);
-        return make_axis_plan_radices(n, best.data(), (int)best.size(), p);
-    }
-    {
-        int n8 = a / 3;
-        const int rem = a % 3;
-        bool two4 = false;
-        if (rem == 1 && n8 > 0) {
-            --n8;
-            two4 = true;
-        }
-        for (int i = 0; i < n8; ++i) r[nr++] = 8;
-        if (two4) {
-            r[nr++] = 4;
-            r[nr++] = 4;
-        } else if (rem == 2) {
-            r[nr++] = 4;
-        } else if (rem == 1) {
-            r[nr++] = 2;
-        }
-    }
-    for (int i = 0; i < b; ++i) r[nr++] = 3;
-    for (int i = 0; i < c; ++i) r[nr++] = 5;
-    if (nr > kMaxRadices) return false;
-    return make_axis_plan_radices(n, r, nr, p);
+    int m = n;
+    for (int q : {2, 3, 5})
+        while (m % q == 0) m /= q;
+    if (n < 2 || m != 1) return false;
+    std::vector<int> cur, best;
+    int cost = 0;
+    if (prefer16)
+        best_order(n, n <= 48 ? 8 : 16, false, cur, 0, best, cost);
+    else
+        best_order(n, 12, true, cur, 0, best, cost);
+    return make_axis_plan_radices(n, best.data(), (int)best.size(), p);
 }
 
 int x_pass_blocks(const Geo& g, int f64) {

@@ -194,7 +194,7 @@ __device__ __forceinline__ void r2c_store(const Geo& g, const T2* S, int ls, int
 }
 
 template <typename T, bool R16, int PID>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 3) k_x_pass(Geo g, Phys ph, int mode, const typename Cx<T>::t* __restrict__ in,
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : (R16 ? 2 : 3)) k_x_pass(Geo g, Phys ph, int mode, const typename Cx<T>::t* __restrict__ in,
                                                      typename Cx<T>::t* __restrict__ out, T* __restrict__ R,
                                                      const T* __restrict__ Rin, double* __restrict__ partials,
                                                      double rtol, double atol, const double* __restrict__ real_in,
@@ -215,14 +215,16 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 3) k_x_pass(Geo
 
     // ---- input: C2R of the incoming half-spectrum lines, or packed real rows
     int Fin = 0;
-    if (mode == XM_PHYS1 || mode == XM_WRMS || mode == XM_C2R_REAL || mode == XM_ENERGY) Fin = 4;
+    const int FR = mode == XM_R2C_REAL3 || mode == XM_C2R_REAL3 ? 3 : 4;  // fields of the plain transforms
+    if (mode == XM_PHYS1 || mode == XM_WRMS || mode == XM_ENERGY) Fin = 4;
+    if (mode == XM_C2R_REAL || mode == XM_C2R_REAL3) Fin = FR;
     if (mode == XM_PHYS2) Fin = ph.elastic ? 3 : 0;
     const T* Ereal = mode == XM_PHYS2R ? reinterpret_cast<const T*>(in) : nullptr;
     T2* RS = S0;  // real-space lines (a + i b)
-    if (mode == XM_R2C_REAL) {
+    if (mode == XM_R2C_REAL || mode == XM_R2C_REAL3) {
 #pragma unroll 4
-        for (int e = threadIdx.x; e < P * 4 * nx; e += blockDim.x) {
-            const int line = L.divn(e), x = e - line * nx, rp = line >> 2, f = line & 3;
+        for (int e = threadIdx.x; e < P * FR * nx; e += blockDim.x) {
+            const int line = L.divn(e), x = e - line * nx, rp = FR == 4 ? line >> 2 : line / 3, f = line - rp * FR;
             T2 Z = T2{0, 0};
             if (rp0 + rp < npairs) {
                 const long long row = 2LL * (rp0 + rp);
@@ -232,8 +234,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 3) k_x_pass(Geo
             S0[line * ls + skew<true>(x)] = Z;
         }
         __syncthreads();
-        T2* res = x_fft<-1, PID, R16>(S0, S1, g.px, 4 * P, ls);
-        r2c_store<NX>(g, res, ls, 4, P, rp0, npairs, out);
+        T2* res = x_fft<-1, PID, R16>(S0, S1, g.px, FR * P, ls);
+        r2c_store<NX>(g, res, ls, FR, P, rp0, npairs, out);
         return;
     }
     if (Fin > 0) {
@@ -247,9 +249,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 3) k_x_pass(Geo
     }
     T2* OS = (RS == S0) ? S1 : S0;  // output lines
 
-    if (mode == XM_C2R_REAL) {
-        for (int e = threadIdx.x; e < P * 4 * nx; e += blockDim.x) {
-            const int line = L.divn(e), x = e - line * nx, rp = line >> 2, f = line & 3;
+    if (mode == XM_C2R_REAL || mode == XM_C2R_REAL3) {
+        for (int e = threadIdx.x; e < P * FR * nx; e += blockDim.x) {
+            const int line = L.divn(e), x = e - line * nx, rp = FR == 4 ? line >> 2 : line / 3, f = line - rp * FR;
             if (rp0 + rp >= npairs) continue;
             const long long row = 2LL * (rp0 + rp);
             const T2 z = RS[line * ls + skew<true>(x)];

@@ -5,11 +5,18 @@
 #include "pf_common.cuh"
 
 namespace pf {
+// FP64 passes with radices above 8 would take 130 registers a thread and leave
+// one CTA on an SM, nothing to transform while it loads: bounded to two
+template <typename T, bool R16>
+constexpr int col_min_blocks() {
+    return sizeof(T) == 8 && R16 ? 2 : 0;  // 0: no bound (1 would let the FP32 passes take registers of occupancy)
+}
+
 // ---------------------------------------------------------------------------
 // y pass: in-place complex FFT along y of nf fields
 // ---------------------------------------------------------------------------
 template <typename T, int SIGN, int TX, bool R16, int PID>
-__global__ void __launch_bounds__(kThreads) k_y_pass(Geo g, typename Cx<T>::t* __restrict__ buf) {
+__global__ void __launch_bounds__(kThreads, col_min_blocks<T, R16>()) k_y_pass(Geo g, typename Cx<T>::t* __restrict__ buf) {
     PF_SKIP_INACTIVE(g);
     using T2 = typename Cx<T>::t;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -41,10 +48,10 @@ void launch_y_pass_sign(const Geo& g, void* buf, int nf, cudaStream_t s) {
 
 // ---------------------------------------------------------------------------
 // z pass: in-place inverse FFT along z of nf fields (of an assembled FP32-bulk
-// stage)
+// stage, of the strain components of the Hu-Chen solve)
 // ---------------------------------------------------------------------------
 template <typename T, int SIGN, int TX, bool R16, int PID>
-__global__ void __launch_bounds__(kThreads) k_z_pass(Geo g, typename Cx<T>::t* __restrict__ buf) {
+__global__ void __launch_bounds__(kThreads, col_min_blocks<T, R16>()) k_z_pass(Geo g, typename Cx<T>::t* __restrict__ buf) {
     PF_SKIP_INACTIVE(g);
     using T2 = typename Cx<T>::t;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -77,7 +84,7 @@ void launch_z_pass(const Geo& g, void* buf, int nf, cudaStream_t s) {
 //   mode 2: same scaling -> FP64                                  (ABI f^E)
 // ---------------------------------------------------------------------------
 template <typename T, typename OT2, int TX, bool R16, int PID>
-__global__ void __launch_bounds__(kThreads) k_z_fwd(Geo g, Phys ph, const typename Cx<T>::t* __restrict__ W,
+__global__ void __launch_bounds__(kThreads, col_min_blocks<T, R16>()) k_z_fwd(Geo g, Phys ph, const typename Cx<T>::t* __restrict__ W,
                                                     OT2* __restrict__ out, int mode) {
     PF_SKIP_INACTIVE(g);
     using T2 = typename Cx<T>::t;
