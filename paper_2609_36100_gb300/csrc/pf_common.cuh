@@ -397,6 +397,22 @@ __device__ __forceinline__ void cp_async_wait_all() {
                 PF_PID_CASE1(34, __VA_ARGS__) \
                 PF_PID_CASE1(35, __VA_ARGS__) \
                 PF_PID_CASE1(36, __VA_ARGS__) \
+                PF_PID_CASE1(37, __VA_ARGS__) \
+                PF_PID_CASE1(38, __VA_ARGS__) \
+                PF_PID_CASE1(39, __VA_ARGS__) \
+                PF_PID_CASE1(40, __VA_ARGS__) \
+                PF_PID_CASE1(41, __VA_ARGS__) \
+                PF_PID_CASE1(42, __VA_ARGS__) \
+                PF_PID_CASE1(43, __VA_ARGS__) \
+                PF_PID_CASE1(44, __VA_ARGS__) \
+                PF_PID_CASE1(45, __VA_ARGS__) \
+                PF_PID_CASE1(46, __VA_ARGS__) \
+                PF_PID_CASE1(47, __VA_ARGS__) \
+                PF_PID_CASE1(48, __VA_ARGS__) \
+                PF_PID_CASE1(49, __VA_ARGS__) \
+                PF_PID_CASE1(50, __VA_ARGS__) \
+                PF_PID_CASE1(51, __VA_ARGS__) \
+                PF_PID_CASE1(52, __VA_ARGS__) \
                 default: break; \
             } \
         } \

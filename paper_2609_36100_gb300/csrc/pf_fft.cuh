@@ -691,7 +691,8 @@ __device__ void fft_cols(const AxisPlan& p, T2* P, T2* Q, Src src, Dst dst) {
 // Plans compiled with a constant length and radix order (PID > 0), shared by
 // the line (x) and column (y, z) transforms; any other plan runs the generic
 // stages (PID 0).  The list: PIDs 1 to 11 every pass compiles, at both tile
-// widths; from 12 on the default FP32 plans of common sizes up to 640, which the
+// widths; from 12 on the default FP32 plans of every even length from 24 to 512 and of
+// 640 that is not among those, which the
 // y and z passes compile at their default tile width and the elastic pass in
 // the form with every stage over the three fields.
 // ---------------------------------------------------------------------------
@@ -717,33 +718,49 @@ PF_FIXED_PLAN(8, 96, 8, 4, 3)
 PF_FIXED_PLAN(9, 120, 8, 3, 5)
 PF_FIXED_PLAN(10, 192, 16, 4, 3)
 PF_FIXED_PLAN(11, 640, 16, 8, 5)
-PF_FIXED_PLAN(12, 32, 8, 4)
-PF_FIXED_PLAN(13, 48, 8, 6)
-PF_FIXED_PLAN(14, 72, 12, 6)
-PF_FIXED_PLAN(15, 80, 10, 8)
-PF_FIXED_PLAN(16, 96, 12, 8)
-PF_FIXED_PLAN(17, 100, 10, 10)
-PF_FIXED_PLAN(18, 108, 12, 9)
-PF_FIXED_PLAN(19, 120, 15, 8)
-PF_FIXED_PLAN(20, 144, 12, 12)
-PF_FIXED_PLAN(21, 160, 16, 10)
-PF_FIXED_PLAN(22, 180, 15, 12)
-PF_FIXED_PLAN(23, 192, 16, 12)
-PF_FIXED_PLAN(24, 200, 10, 10, 2)
-PF_FIXED_PLAN(25, 216, 12, 6, 3)
-PF_FIXED_PLAN(26, 240, 16, 15)
-PF_FIXED_PLAN(27, 288, 12, 12, 2)
-PF_FIXED_PLAN(28, 300, 15, 10, 2)
-PF_FIXED_PLAN(29, 320, 10, 8, 4)
-PF_FIXED_PLAN(30, 360, 15, 12, 2)
-PF_FIXED_PLAN(31, 384, 12, 8, 4)
-PF_FIXED_PLAN(32, 400, 10, 10, 4)
-PF_FIXED_PLAN(33, 432, 12, 12, 3)
-PF_FIXED_PLAN(34, 480, 15, 8, 4)
-PF_FIXED_PLAN(35, 512, 8, 8, 8)
-PF_FIXED_PLAN(36, 640, 10, 8, 8)
+PF_FIXED_PLAN(12, 24, 6, 4)
+PF_FIXED_PLAN(13, 30, 6, 5)
+PF_FIXED_PLAN(14, 32, 8, 4)
+PF_FIXED_PLAN(15, 36, 6, 6)
+PF_FIXED_PLAN(16, 40, 8, 5)
+PF_FIXED_PLAN(17, 48, 8, 6)
+PF_FIXED_PLAN(18, 50, 10, 5)
+PF_FIXED_PLAN(19, 54, 9, 6)
+PF_FIXED_PLAN(20, 60, 15, 4)
+PF_FIXED_PLAN(21, 72, 12, 6)
+PF_FIXED_PLAN(22, 80, 10, 8)
+PF_FIXED_PLAN(23, 90, 15, 6)
+PF_FIXED_PLAN(24, 96, 12, 8)
+PF_FIXED_PLAN(25, 100, 10, 10)
+PF_FIXED_PLAN(26, 108, 12, 9)
+PF_FIXED_PLAN(27, 120, 15, 8)
+PF_FIXED_PLAN(28, 144, 12, 12)
+PF_FIXED_PLAN(29, 150, 15, 10)
+PF_FIXED_PLAN(30, 160, 16, 10)
+PF_FIXED_PLAN(31, 162, 9, 6, 3)
+PF_FIXED_PLAN(32, 180, 15, 12)
+PF_FIXED_PLAN(33, 192, 16, 12)
+PF_FIXED_PLAN(34, 200, 10, 10, 2)
+PF_FIXED_PLAN(35, 216, 12, 6, 3)
+PF_FIXED_PLAN(36, 240, 16, 15)
+PF_FIXED_PLAN(37, 250, 10, 5, 5)
+PF_FIXED_PLAN(38, 270, 15, 6, 3)
+PF_FIXED_PLAN(39, 288, 12, 12, 2)
+PF_FIXED_PLAN(40, 300, 15, 10, 2)
+PF_FIXED_PLAN(41, 320, 10, 8, 4)
+PF_FIXED_PLAN(42, 324, 12, 9, 3)
+PF_FIXED_PLAN(43, 360, 15, 12, 2)
+PF_FIXED_PLAN(44, 384, 12, 8, 4)
+PF_FIXED_PLAN(45, 400, 10, 10, 4)
+PF_FIXED_PLAN(46, 432, 12, 12, 3)
+PF_FIXED_PLAN(47, 450, 15, 15, 2)
+PF_FIXED_PLAN(48, 480, 15, 8, 4)
+PF_FIXED_PLAN(49, 486, 9, 9, 6)
+PF_FIXED_PLAN(50, 500, 10, 10, 5)
+PF_FIXED_PLAN(51, 512, 8, 8, 8)
+PF_FIXED_PLAN(52, 640, 10, 8, 8)
 #undef PF_FIXED_PLAN
-constexpr int kFixedPlans = 36;
+constexpr int kFixedPlans = 52;
 
 template <int... Rs>
 inline bool plan_is(const AxisPlan& p, int n, Radices<Rs...>) {

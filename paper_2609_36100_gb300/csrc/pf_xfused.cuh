@@ -345,7 +345,10 @@ struct XFPlan {
         using Fwd = Radices<__VA_ARGS__>;    \
     };
 PF_XF_PLAN(32, 4, 4, 8)
+PF_XF_PLAN(36, 8, 3, 12)
+PF_XF_PLAN(40, 4, 5, 8)
 PF_XF_PLAN(48, 8, 4, 12)
+PF_XF_PLAN(60, 8, 3, 4, 5)
 PF_XF_PLAN(64, 8, 4, 16)
 PF_XF_PLAN(72, 8, 3, 12, 2)
 PF_XF_PLAN(80, 8, 5, 16)

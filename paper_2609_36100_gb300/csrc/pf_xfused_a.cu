@@ -7,11 +7,12 @@ namespace pf {
     template int launch_x_fused_n<N_>(const Geo&, const Phys&, int, const void*, void*, void*, const void*, \
                                       double*, double, double, cudaStream_t);
 PF_XF_INST(32)
-PF_XF_INST(80)
-PF_XF_INST(120)
-PF_XF_INST(180)
-PF_XF_INST(240)
-PF_XF_INST(320)
-PF_XF_INST(432)
+PF_XF_INST(60)
+PF_XF_INST(96)
+PF_XF_INST(128)
+PF_XF_INST(192)
+PF_XF_INST(256)
+PF_XF_INST(360)
+PF_XF_INST(480)
 #undef PF_XF_INST
 }  // namespace pf

@@ -6,12 +6,13 @@ namespace pf {
 #define PF_XF_INST(N_)                                                                                       \
     template int launch_x_fused_n<N_>(const Geo&, const Phys&, int, const void*, void*, void*, const void*, \
                                       double*, double, double, cudaStream_t);
-PF_XF_INST(48)
-PF_XF_INST(96)
-PF_XF_INST(128)
-PF_XF_INST(192)
-PF_XF_INST(256)
-PF_XF_INST(360)
-PF_XF_INST(480)
+PF_XF_INST(36)
+PF_XF_INST(64)
+PF_XF_INST(100)
+PF_XF_INST(144)
+PF_XF_INST(200)
+PF_XF_INST(288)
+PF_XF_INST(384)
+PF_XF_INST(512)
 #undef PF_XF_INST
 }  // namespace pf

@@ -6,12 +6,13 @@ namespace pf {
 #define PF_XF_INST(N_)                                                                                       \
     template int launch_x_fused_n<N_>(const Geo&, const Phys&, int, const void*, void*, void*, const void*, \
                                       double*, double, double, cudaStream_t);
-PF_XF_INST(64)
-PF_XF_INST(100)
-PF_XF_INST(144)
-PF_XF_INST(200)
-PF_XF_INST(288)
-PF_XF_INST(384)
-PF_XF_INST(512)
+PF_XF_INST(40)
+PF_XF_INST(72)
+PF_XF_INST(108)
+PF_XF_INST(160)
+PF_XF_INST(216)
+PF_XF_INST(300)
+PF_XF_INST(400)
+PF_XF_INST(640)
 #undef PF_XF_INST
 }  // namespace pf

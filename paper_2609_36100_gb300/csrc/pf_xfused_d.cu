@@ -6,12 +6,12 @@ namespace pf {
 #define PF_XF_INST(N_)                                                                                       \
     template int launch_x_fused_n<N_>(const Geo&, const Phys&, int, const void*, void*, void*, const void*, \
                                       double*, double, double, cudaStream_t);
-PF_XF_INST(72)
-PF_XF_INST(108)
-PF_XF_INST(160)
-PF_XF_INST(216)
-PF_XF_INST(300)
-PF_XF_INST(400)
-PF_XF_INST(640)
+PF_XF_INST(48)
+PF_XF_INST(80)
+PF_XF_INST(120)
+PF_XF_INST(180)
+PF_XF_INST(240)
+PF_XF_INST(320)
+PF_XF_INST(432)
 #undef PF_XF_INST
 }  // namespace pf

@@ -16,11 +16,12 @@ int launch_x_fused(const Geo& g, const Phys& ph, int mode, const void* in, void*
     switch (g.nx) {
 #define PF_XF(N_) \
     case N_: return launch_x_fused_n<N_>(g, ph, mode, in, out, R, Rin, partials, rtol, atol, s);
-        PF_XF(32) PF_XF(48) PF_XF(64) PF_XF(72) PF_XF(80) PF_XF(96)
-        PF_XF(100) PF_XF(108) PF_XF(120) PF_XF(128) PF_XF(144) PF_XF(160)
-        PF_XF(180) PF_XF(192) PF_XF(200) PF_XF(216) PF_XF(240) PF_XF(256)
-        PF_XF(288) PF_XF(300) PF_XF(320) PF_XF(360) PF_XF(384) PF_XF(400)
-        PF_XF(432) PF_XF(480) PF_XF(512) PF_XF(640)
+        PF_XF(32) PF_XF(36) PF_XF(40) PF_XF(48) PF_XF(60) PF_XF(64)
+        PF_XF(72) PF_XF(80) PF_XF(96) PF_XF(100) PF_XF(108) PF_XF(120)
+        PF_XF(128) PF_XF(144) PF_XF(160) PF_XF(180) PF_XF(192) PF_XF(200)
+        PF_XF(216) PF_XF(240) PF_XF(256) PF_XF(288) PF_XF(300) PF_XF(320)
+        PF_XF(360) PF_XF(384) PF_XF(400) PF_XF(432) PF_XF(480) PF_XF(512)
+        PF_XF(640)
 #undef PF_XF
         default: return 0;
     }

@@ -10,8 +10,8 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
-LENGTHS = [32, 48, 72, 80, 96, 100, 108, 120, 144, 160, 180, 192, 200, 216, 240, 288, 300, 320, 360, 384, 400, 432,
-           480, 512, 640]
+LENGTHS = [24, 30, 32, 36, 40, 48, 50, 54, 60, 72, 80, 90, 96, 100, 108, 120, 144, 150, 160, 162, 180, 192, 200, 216, 240,
+           250, 270, 288, 300, 320, 324, 360, 384, 400, 432, 450, 480, 486, 500, 512, 640]
 
 
 @pytest.fixture(scope="module")
@@ -76,3 +76,14 @@ def test_radix_that_is_none_refused(pfg, params):
             c[4 + 22:4 + 33] = [len(bad)] + bad + [0] * (10 - len(bad))
             with pytest.raises(pfg.PFError):
                 s.set_tuning(c)
+
+
+@pytest.mark.parametrize("n", [30, 50, 96, 100, 108, 120, 150, 180, 240])
+def test_fp64_default_plans_match_oracle(pfg, params, n):
+    """FP64 plans of the fewest instructions, along every axis."""
+    for axis in range(3):
+        shape = [12, 10, 6]
+        shape[2 - axis] = n
+        err, e = step_case(pfg, params, tuple(shape), "fp64", 20 + n)
+        assert np.all(err <= 1e-11), (axis, err)
+        assert e <= 1e-8
