@@ -238,6 +238,22 @@ struct pf_ctx {
     bool hc_prev = false;          // hc_eu[hc_cur] can start the next solve (warm start)
     double* d_scalar = nullptr;
     double* h_scalar = nullptr;  // pinned
+    // A step as a graph, for grids whose kernels are as short as the gaps
+    // between launches: one per state buffer (an accepted step swaps them) and
+    // with or without the error estimate, its step size in coefficients the
+    // launch copies in.  Built after kGraphAfter steps of a context.
+    struct StepGraph {
+        cudaGraphExec_t exec = nullptr;
+        const double2* y = nullptr;
+        bool lte = false;
+        double rtol = 0.0, atol = 0.0;
+    };
+    StepGraph graphs[4];
+    int steps_run = 0, graphs_built = 0;
+    bool graphs_off = false;
+    StageCoefDev* d_coef = nullptr;  // [kMaxStages + 2]
+    StageCoefDev* h_coef = nullptr;  // pinned
+    cudaStream_t cap = nullptr;      // captured on (the legacy default stream cannot be)
     // integrator state
     double t = 0.0, h = 0.0;
     double e_prev = 1.0;
@@ -370,7 +386,18 @@ void derive_phys(const pf_params& p, Phys& ph) {
         }
 }
 
+void drop_graphs(pf_ctx* c) {
+    for (auto& gr : c->graphs) {
+        if (gr.exec) cudaGraphExecDestroy(gr.exec);
+        gr = {};
+    }
+}
+
 void free_all(pf_ctx* c) {
+    drop_graphs(c);
+    if (c->cap) cudaStreamDestroy(c->cap);
+    cudaFree(c->d_coef);
+    if (c->h_coef) cudaFreeHost(c->h_coef);
     cudaFree(c->d_kx);
     cudaFree(c->d_ky);
     cudaFree(c->d_kz);
@@ -737,8 +764,86 @@ int enqueue_step(pf_ctx* c, double dt, bool want_lte, const StageCoefDev* dcoef 
     return check_launch(c, "step kernels");
 }
 
+// Steps of up to 160^3 points run as a graph from the kGraphAfter-th on: the
+// gaps between 60 launches were 2.2 us each (1.1 of 12.9 ms for eight steps at
+// 128^3, most of a step at 32^3).  Capturing and instantiating costs about a
+// millisecond and is left to contexts that step on; larger grids would gain
+// under 1 %.
+constexpr int kGraphAfter = 16;
+constexpr long long kGraphPoints = 160LL * 160 * 160;
+constexpr int kGraphsMost = 16;  // rebuilt for other tolerances that often, then no more
+
+// a graph of the step from c->y, or null where the step is launched directly
+cudaGraphExec_t step_graph(pf_ctx* c, bool lte) {
+    if (c->graphs_off || c->prof_on || c->inhom || c->g.N > kGraphPoints || ++c->steps_run <= kGraphAfter)
+        return nullptr;
+    pf_ctx::StepGraph* slot = nullptr;
+    for (auto& gr : c->graphs) {
+        if (gr.exec && gr.y == c->y && gr.lte == lte) {
+            if (!lte || (gr.rtol == c->prm.rtol && gr.atol == c->prm.atol)) return gr.exec;
+            cudaGraphExecDestroy(gr.exec);
+            gr = {};
+        }
+        if (!gr.exec && !slot) slot = &gr;
+    }
+    const int ncoef = c->tab.s + 2;
+    cudaError_t e = !slot || ++c->graphs_built > kGraphsMost ? cudaErrorNotSupported : cudaSuccess;
+    if (e == cudaSuccess && !c->d_coef) e = cudaMalloc((void**)&c->d_coef, ncoef * sizeof(StageCoefDev));
+    if (e == cudaSuccess && !c->h_coef) {
+        e = cudaMallocHost((void**)&c->h_coef, ncoef * sizeof(StageCoefDev));
+        if (e == cudaSuccess) std::memset(c->h_coef, 0, ncoef * sizeof(StageCoefDev));
+    }
+    if (e == cudaSuccess && !c->cap) e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeRelaxed);
+    cudaGraph_t graph = nullptr;
+    if (e == cudaSuccess) {
+        const cudaStream_t user = c->stream;
+        c->stream = c->cap;
+        e = cudaMemcpyAsync(c->d_coef, c->h_coef, ncoef * sizeof(StageCoefDev), cudaMemcpyHostToDevice, c->cap);
+        const int rc = c->fp32 ? enqueue_step<float>(c, 1.0, lte, c->d_coef) : enqueue_step<double>(c, 1.0, lte, c->d_coef);
+        c->stream = user;
+        const cudaError_t e2 = cudaStreamEndCapture(c->cap, &graph);
+        if (e == cudaSuccess) e = rc ? cudaErrorUnknown : e2;
+    }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&slot->exec, graph, 0);
+    if (graph) cudaGraphDestroy(graph);
+    if (e != cudaSuccess) {  // the step is launched directly, now and from now on
+        cudaGetLastError();
+        if (slot) slot->exec = nullptr;
+        c->graphs_off = true;
+        return nullptr;
+    }
+    slot->y = c->y;
+    slot->lte = lte;
+    slot->rtol = c->prm.rtol;
+    slot->atol = c->prm.atol;
+    return slot->exec;
+}
+
 int step_once(pf_ctx* c, double dt, bool want_lte, double* e_out) {
-    int rc = c->fp32 ? enqueue_step<float>(c, dt, want_lte) : enqueue_step<double>(c, dt, want_lte);
+    int rc = PF_OK;
+    if (cudaGraphExec_t exec = step_graph(c, want_lte && c->tab.embedded)) {
+        const Tableau& tb = c->tab;
+        StageCoefDev co[kMaxStages + 2];
+        std::memset(co, 0, sizeof co);
+        for (int i = 0; i < tb.s; ++i)
+            fill_coef(co[i], i, tb.AI[i], tb.AE[i], dt, dt * tb.AI[i][i], dt * c->gdiag);
+        double dI[kMaxStages], dE[kMaxStages];
+        for (int j = 0; j < kMaxStages; ++j) {
+            dI[j] = tb.embedded ? tb.bI[j] - tb.btI[j] : 0.0;
+            dE[j] = tb.embedded ? tb.bE[j] - tb.btE[j] : 0.0;
+        }
+        fill_coef(co[tb.s], tb.s, tb.bI, tb.bE, dt, 0.0, 0.0);
+        fill_coef(co[tb.s + 1], tb.s, dI, dE, dt, 0.0, 0.0);
+        if (std::memcmp(co, c->h_coef, (tb.s + 2) * sizeof(StageCoefDev)) != 0) {
+            // an earlier step that was not waited for may still have to copy them
+            PF_CUDA(c, cudaStreamSynchronize(c->stream));
+            std::memcpy(c->h_coef, co, (tb.s + 2) * sizeof(StageCoefDev));
+        }
+        PF_CUDA(c, cudaGraphLaunch(exec, c->stream));
+    } else {
+        rc = c->fp32 ? enqueue_step<float>(c, dt, want_lte) : enqueue_step<double>(c, dt, want_lte);
+    }
     if (rc) return rc;
     int nrhs = 0;
     for (int i = 0; i < c->tab.s; ++i) nrhs += c->need_fe[i] ? 1 : 0;
@@ -1702,6 +1807,7 @@ int pf_set_tuning(pf_ctx* c, const int* cfg, int n) {
         *pl[a] = p;
     }
     c->g = g;
+    drop_graphs(c);  // their launches are of the old schedule
     return PF_OK;
 }
 

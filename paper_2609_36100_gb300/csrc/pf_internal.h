@@ -126,6 +126,29 @@ struct StageCoefDev {
     float gh, gl, qgh, qgl;
 };
 
+// coefficients of a stage (rows aI, aE of n entries) or of the completion
+__host__ __device__ inline void fill_coef(StageCoefDev& c, int n, const double* aI, const double* aE, double dt,
+                                          double gam, double qgam) {
+    for (int j = 0; j < kMaxStages; ++j) {
+        const double ci = j < n ? dt * aI[j] : 0.0;
+        const double ce = j < n ? dt * aE[j] : 0.0;
+        c.cI[j] = ci;
+        c.cE[j] = ce;
+        const float h = (float)ce;
+        c.cEh[j] = h;
+        c.cEl[j] = (float)(ce - (double)h);
+        const float hi = (float)ci;
+        c.cIh[j] = hi;
+        c.cIl[j] = (float)(ci - (double)hi);
+    }
+    c.gamma = gam;
+    c.qgamma = qgam;
+    c.gh = (float)gam;
+    c.gl = (float)(gam - (double)c.gh);
+    c.qgh = (float)qgam;
+    c.qgl = (float)(qgam - (double)c.qgh);
+}
+
 // Coefficients of one stage assembly / step completion pass.
 struct StageTerms {
     int n;                             // number of previous-stage terms

@@ -287,54 +287,48 @@ void launch_lambda_table(const Geo& g, const Phys& ph, double* lam, float2* lamd
 // ---------------------------------------------------------------------------
 // batch round kernels (one thread each, or a grid-stride copy)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void fill_coef(StageCoefDev& c, int n, const double* aI, const double* aE, double dt,
-                                          double gam, double qgam) {
-    for (int j = 0; j < kMaxStages; ++j) {
-        const double ci = j < n ? dt * aI[j] : 0.0;
-        const double ce = j < n ? dt * aE[j] : 0.0;
-        c.cI[j] = ci;
-        c.cE[j] = ce;
-        const float h = (float)ce;
-        c.cEh[j] = h;
-        c.cEl[j] = (float)(ce - (double)h);
-        const float hi = (float)ci;
-        c.cIh[j] = hi;
-        c.cIl[j] = (float)(ci - (double)hi);
-    }
-    c.gamma = gam;
-    c.qgamma = qgam;
-    c.gh = (float)gam;
-    c.gl = (float)(gam - (double)c.gh);
-    c.qgh = (float)qgam;
-    c.qgl = (float)(qgam - (double)c.qgh);
-}
-
 // step size of this round's attempt (clipped to t_final) and the stage /
-// completion coefficients built from it, as the host driver builds them
-__global__ void k_batch_prep(BatchConst bc, MemberCtl* __restrict__ ctl, StageCoefDev* __restrict__ coef) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// completion coefficients built from it, as the host driver builds them: a
+// thread per coefficient set (one thread for all of them took 26 us, the
+// longest kernel of a round of a 32^3 member)
+__global__ void __launch_bounds__(32) k_batch_prep(BatchConst bc, MemberCtl* __restrict__ ctl,
+                                                   StageCoefDev* __restrict__ coef) {
     MemberCtl& m = *ctl;
     if (!m.active) return;
+    const int i = threadIdx.x;
     const double dt = fmin(m.h, bc.t_final - m.t);
-    m.dt = dt;
-    for (int i = 0; i < bc.s; ++i)
+    if (i == 0) m.dt = dt;
+    if (i < bc.s) {
         fill_coef(coef[i], i, bc.AI[i], bc.AE[i], dt, dt * bc.AI[i][i], dt * bc.gdiag);
-    double dI[kMaxStages], dE[kMaxStages];
-    for (int j = 0; j < kMaxStages; ++j) {
-        dI[j] = bc.embedded ? bc.bI[j] - bc.btI[j] : 0.0;
-        dE[j] = bc.embedded ? bc.bE[j] - bc.btE[j] : 0.0;
+    } else if (i == bc.s) {
+        fill_coef(coef[i], bc.s, bc.bI, bc.bE, dt, 0.0, 0.0);
+    } else if (i == bc.s + 1) {
+        double dI[kMaxStages], dE[kMaxStages];
+        for (int j = 0; j < kMaxStages; ++j) {
+            dI[j] = bc.embedded ? bc.bI[j] - bc.btI[j] : 0.0;
+            dE[j] = bc.embedded ? bc.bE[j] - bc.btE[j] : 0.0;
+        }
+        fill_coef(coef[i], bc.s, dI, dE, dt, 0.0, 0.0);
     }
-    fill_coef(coef[bc.s], bc.s, bc.bI, bc.bE, dt, 0.0, 0.0);
-    fill_coef(coef[bc.s + 1], bc.s, dI, dE, dt, 0.0, 0.0);
 }
 
 // accept / reject and the next step size (same PI rule as the host driver)
-__global__ void k_batch_ctl(BatchConst bc, MemberCtl* __restrict__ ctl, const double* __restrict__ wsum, double scale) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// accept / reject's three powers on a lane each, side by side
+__global__ void __launch_bounds__(32) k_batch_ctl(BatchConst bc, MemberCtl* __restrict__ ctl,
+                                                  const double* __restrict__ wsum, double scale) {
     MemberCtl& m = *ctl;
-    m.accepted_now = 0;
-    if (!m.active) return;
+    const int active = m.active;
     const double e = bc.embedded ? sqrt(wsum[0] * scale) : 0.0;
+    const double ee = e < 1e-10 ? 1e-10 : e;
+    double pw = 0.0;
+    if (bc.embedded && active)
+        pw = threadIdx.x == 0 ? ee : (threadIdx.x == 1 ? m.e_prev : e);
+    if (bc.embedded && active && threadIdx.x < 3)
+        pw = pow(pw, (threadIdx.x == 0 ? -bc.k1 : (threadIdx.x == 1 ? bc.k2 : -1.0)) / bc.q);
+    const double pw_prev = __shfl_sync(0xffffffffu, pw, 1), pw_rej = __shfl_sync(0xffffffffu, pw, 2);
+    if (threadIdx.x != 0) return;
+    m.accepted_now = 0;
+    if (!active) return;
     m.e_last = e;
     m.n_rhs += bc.nrhs;
     const bool ok = isfinite(e) && e <= 1.0;
@@ -347,8 +341,7 @@ __global__ void k_batch_ctl(BatchConst bc, MemberCtl* __restrict__ ctl, const do
         m.accepted_now = 1;
         m.ypar ^= 1;
         if (bc.embedded) {
-            const double ee = e < 1e-10 ? 1e-10 : e;
-            double eta = bc.safety * pow(ee, -bc.k1 / bc.q) * pow(m.e_prev, bc.k2 / bc.q);
+            double eta = bc.safety * pw * pw_prev;
             const double cap = m.after_reject ? 1.0 : bc.eta_max;
             eta = fmin(cap, fmax(bc.eta_min, eta));
             m.e_prev = ee;
@@ -365,7 +358,7 @@ __global__ void k_batch_ctl(BatchConst bc, MemberCtl* __restrict__ ctl, const do
             return;
         }
         m.after_reject = 1;
-        hn = isfinite(e) ? h * fmax(bc.eta_rej, bc.safety * pow(e, -1.0 / bc.q)) : h * 0.25;
+        hn = isfinite(e) ? h * fmax(bc.eta_rej, bc.safety * pw_rej) : h * 0.25;
     }
     m.h = fmin(fmax(hn, bc.h_min), bc.h_max);
     if (!(m.t < bc.t_final * (1 - 1e-14))) m.active = 0;
