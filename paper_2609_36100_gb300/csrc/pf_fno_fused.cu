@@ -29,7 +29,7 @@ constexpr int kSMs = 152;
 constexpr int kSmemMax = 227 * 1024;
 constexpr int kMaxModes = 16;  // x modes a lane group of the row kernels covers
 constexpr int kMaxRow = 256;   // points of a row
-constexpr int kFoldIter = (kMaxRow / 2 + 31) / 32;
+constexpr int kFoldIter = (kMaxRow / 2 + 31) / 32;  // pairs of positions a lane folds: 4, or 2 (rows of up to 128)
 
 __host__ __device__ inline int up(int a, int b) { return (a + b - 1) / b * b; }
 // padded half row, row pitch (16-byte units odd: rows 0..7 fall on different
@@ -335,29 +335,31 @@ __device__ __forceinline__ void row_forward(const RowArgs& a, long long row, con
 // val(channel, x, value, pre(channel, x)).  The two positions that are their
 // own mirrors, 0 and n/2, share a lane.  CB channels at a time: first every
 // pre (a load, say), then the values.
-template <int CB, int W, class G, class F>
+template <int FI, int CB, int W, class G, class F>
 __device__ __forceinline__ void row_fold(float* A, int RS, int nx, int C, Team<W> tm, G pre, F val) {
     const int lane = threadIdx.x & 31, HP = half_pad(nx), Hx = nx / 2 + 1, XL = (nx + 1) / 2;
     const bool even = (nx & 1) == 0;
     for (int c0 = CB * tm.part; c0 < C; c0 += CB * W) {
-        float v[CB][kFoldIter], u[CB][kFoldIter];
+        float v[CB][FI], u[CB][FI];
         using P = decltype(pre(0, 0));
-        P pv[CB][kFoldIter], pu[CB][kFoldIter];
+        P pv[CB][FI], pu[CB][FI];
 #pragma unroll
-        for (int b = 0; b < CB; ++b)
+        for (int q = 0; q < FI; ++q) {
+            if (32 * q >= XL) break;  // the same for every lane: no instructions for positions no row has
+            const int x = lane + 32 * q, y = x ? nx - x : nx / 2;
 #pragma unroll
-            for (int q = 0; q < kFoldIter; ++q) {
-                const int x = lane + 32 * q, y = x ? nx - x : nx / 2;
+            for (int b = 0; b < CB; ++b)
                 if (c0 + b < C && x < XL) {
                     pv[b][q] = pre(c0 + b, x);
                     if (x || even) pu[b][q] = pre(c0 + b, y);
                 }
-            }
+        }
 #pragma unroll
-        for (int b = 0; b < CB; ++b)
+        for (int q = 0; q < FI; ++q) {
+            if (32 * q >= XL) break;
+            const int x = lane + 32 * q, y = x ? nx - x : nx / 2;
 #pragma unroll
-            for (int q = 0; q < kFoldIter; ++q) {
-                const int x = lane + 32 * q, y = x ? nx - x : nx / 2;
+            for (int b = 0; b < CB; ++b) {
                 v[b][q] = u[b][q] = 0.f;
                 if (c0 + b < C && x < XL) {
                     const float* r = A + (c0 + b) * RS;
@@ -365,13 +367,15 @@ __device__ __forceinline__ void row_fold(float* A, int RS, int nx, int C, Team<W
                     if (x || even) u[b][q] = val(c0 + b, y, r[y], pu[b][q]);
                 }
             }
+        }
         __syncwarp();
 #pragma unroll
         for (int b = 0; b < CB; ++b) {
             if (c0 + b >= C) break;
             float* r = A + (c0 + b) * RS;
 #pragma unroll
-            for (int q = 0; q < kFoldIter; ++q) {
+            for (int q = 0; q < FI; ++q) {
+                if (32 * q >= XL) break;
                 const int x = lane + 32 * q;
                 if (x < XL) {
                     r[x] = x ? v[b][q] + u[b][q] : v[b][q];
@@ -429,7 +433,7 @@ __global__ void __launch_bounds__(256) k_fno_lift_modes(RowArgs a) {
             for (int f = 0; f < 4; ++f) cp4(A + f * RS + x, a.x + f * a.N + row * nx + x, true);
         cp_wait();
         __syncwarp();
-        row_fold<4>(
+        row_fold<kFoldIter, 4>(
             A, RS, nx, 4, Team<1>{0, 0}, [](int, int) { return 0; }, [](int, int, float v, int) { return v; });
         const int f = lane & 3;
         for (int k = lane >> 2; k < a.m; k += 8) {
@@ -459,7 +463,7 @@ __global__ void __launch_bounds__(256) k_fno_lift_modes(RowArgs a) {
 
 constexpr int kTeam = 2;  // warps of a row
 
-template <int CP, int MP>
+template <int CP, int MP, int FI>
 __global__ void __launch_bounds__(640, 1) k_fno_row(RowArgs a) {
     extern __shared__ __align__(16) float sm[];
     const RowSmem L = row_smem(a.nx, CP, MP);
@@ -498,14 +502,14 @@ __global__ void __launch_bounds__(640, 1) k_fno_row(RowArgs a) {
             continue;
         }
         if (a.dense) {
-            row_fold<2>(
+            row_fold<FI, 2>(
                 A, RS, nx, C, tm, [](int, int) { return 0; },
                 [&](int c, int x, float v, int) {
                     a.z[(long long)c * a.N + r0 + x] = v;
                     return gelu_fast(v);
                 });
         } else {
-            row_fold<2>(
+            row_fold<FI, 2>(
                 A, RS, nx, C, tm, [](int, int) { return 0; }, [](int, int, float v, int) { return v; });
         }
         row_forward<CP, MP>(a, row, A, RS, T, sm + L.tf, sm + L.tf + MP * HP, tm);
@@ -515,7 +519,7 @@ __global__ void __launch_bounds__(640, 1) k_fno_row(RowArgs a) {
 // Partial sums of a block of k_fno_row_bwd: [C C] V, [C] v, [4 C] P, [C] p
 __host__ __device__ inline int row_part_len(int C) { return C * C + 6 * C; }
 
-template <int CP, int MP>
+template <int CP, int MP, int FI>
 __global__ void __launch_bounds__(512, 1) k_fno_row_bwd(RowArgs a) {
     extern __shared__ __align__(16) float sm[];
     const RowSmem L = row_smem(a.nx, CP, MP);
@@ -558,17 +562,28 @@ __global__ void __launch_bounds__(512, 1) k_fno_row_bwd(RowArgs a) {
         cp_wait();
         tm.sync();
         // gradient of V: dz a^T over the row's points, a in fragments straight from global memory
+        const float* zp = first ? nullptr : a.zprev + (g < C ? (long long)g * a.N : 0) + r0;
         for (int k0 = 16 * tm.part; k0 < nx; k0 += 16 * kTeam) {
             const int p = k0 + 2 * t;
             float av[NT][4];
             if (!first) {
 #pragma unroll
-                for (int j = 0; j < NT; ++j)
+                for (int j = 0; j < NT; ++j) {
+                    const bool dc = j * 8 + g < C;
+                    const float* z = zp + (dc ? (long long)(j * 8) * a.N : 0);
+                    if (a.vec) {  // p even, pairs 8-byte aligned, and nx even
+                        const float2 lo = dc && p < nx ? *reinterpret_cast<const float2*>(z + p) : make_float2(0.f, 0.f);
+                        const float2 hi =
+                            dc && p + 8 < nx ? *reinterpret_cast<const float2*>(z + p + 8) : make_float2(0.f, 0.f);
+                        av[j][0] = lo.x, av[j][1] = lo.y, av[j][2] = hi.x, av[j][3] = hi.y;
+                    } else {
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const int d = j * 8 + g, q = p + (r & 1) + ((r & 2) ? 8 : 0);
-                        av[j][r] = d < C && q < nx ? a.zprev[(long long)d * a.N + r0 + q] : 0.f;
+                        for (int r = 0; r < 4; ++r) {
+                            const int q = p + (r & 1) + ((r & 2) ? 8 : 0);
+                            av[j][r] = dc && q < nx ? z[q] : 0.f;
+                        }
                     }
+                }
 #pragma unroll
                 for (int j = 0; j < NT; ++j)
 #pragma unroll
@@ -627,7 +642,7 @@ __global__ void __launch_bounds__(512, 1) k_fno_row_bwd(RowArgs a) {
             tm.sync();
             continue;
         }
-        row_fold<4>(
+        row_fold<FI, 2>(
             A, RS, nx, C, tm, [&](int c, int x) { return a.zprev[(long long)c * a.N + r0 + x]; },
             [&](int c, int x, float v, float z) {
                 const float d = v * gelu_fast_g(z);
@@ -885,7 +900,13 @@ __global__ void __launch_bounds__(256) k_mix_modes_bwd(const float2* __restrict_
 // ---------------------------------------------------------------------------
 // projection: tiles of 64 points; a warp owns 16 of the H rows.
 // ---------------------------------------------------------------------------
-constexpr int kPts = 64, kPS = 68;
+// points of a tile and the pitch of its rows: 8 (mod 32), so that the 8-byte
+// reads of a fragment along the points (rows g) and, with the rows of a k tile
+// taken in the order t, t + 4, t + 8, t + 12 (krow), the 4-byte ones across the
+// rows are free of bank conflicts
+constexpr int kPts = 64, kPS = 72;
+// row of a k tile behind slot 2 t + i (i = 0, 1) and 2 t + 8 + i (i = 2, 3) of lane t
+__device__ __forceinline__ int krow(int t, int i) { return t + 4 * i; }
 __host__ __device__ inline int proj_part_len(int C, int H) { return H * C + 5 * H + 4; }
 struct ProjArgs {
     const float *a, *tgt, *Q1, *q1, *Q2, *q2;
@@ -924,23 +945,23 @@ __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
         const int lane = e & 31, tile = e >> 5, g = lane >> 2, t = lane & 3;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            const int mm = g + ((r & 1) ? 8 : 0), kk = 2 * t + ((r & 2) ? 8 : 0);
+            const int mm = g + ((r & 1) ? 8 : 0), k0 = krow(t, r & 2), k1 = krow(t, (r & 2) + 1);
             const int mt = tile / KT, kt = tile - mt * KT;
-            split2(q1v(mt * 16 + mm, kt * 16 + kk), q1v(mt * 16 + mm, kt * 16 + kk + 1), w1[tile * 256 + lane * 4 + r],
+            split2(q1v(mt * 16 + mm, kt * 16 + k0), q1v(mt * 16 + mm, kt * 16 + k1), w1[tile * 256 + lane * 4 + r],
                    w1[tile * 256 + 128 + lane * 4 + r]);
             if (TRAIN) {
                 const int ct = tile / NW, ht = tile - ct * NW;
-                split2(q1v(ht * 16 + kk, ct * 16 + mm), q1v(ht * 16 + kk + 1, ct * 16 + mm),
+                split2(q1v(ht * 16 + k0, ct * 16 + mm), q1v(ht * 16 + k1, ct * 16 + mm),
                        wt[tile * 256 + lane * 4 + r], wt[tile * 256 + 128 + lane * 4 + r]);
             }
         }
     }
     for (int e = threadIdx.x; e < NW * 32; e += blockDim.x) {
-        const int g = (e & 31) >> 2, h = (e >> 5) * 16 + 2 * (e & 3);
+        const int g = (e & 31) >> 2, h = (e >> 5) * 16 + (e & 3);
         auto v = [&](int hh) -> float { return g < 4 && hh < H ? p.Q2[g * H + hh] : 0.f; };
         uint4 w;
-        split2(v(h), v(h + 1), w.x, w.z);
-        split2(v(h + 8), v(h + 9), w.y, w.w);
+        split2(v(h), v(h + 4), w.x, w.z);
+        split2(v(h + 8), v(h + 12), w.y, w.w);
         w2[e] = w;
     }
     for (int e = threadIdx.x; e < HP; e += blockDim.x) {
@@ -1010,10 +1031,10 @@ __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
                 float acc[4] = {b0, b0, b1, b1};
 #pragma unroll
                 for (int k = 0; k < KT; ++k) {
-                    const float* b = sa + (k * 16 + 2 * t) * kPS + n * 8 + g;
+                    const float* b = sa + (k * 16 + t) * kPS + n * 8 + g;
                     unsigned bh0, bl0, bh1, bl1;
-                    split2(b[0], b[kPS], bh0, bl0);
-                    split2(b[8 * kPS], b[9 * kPS], bh1, bl1);
+                    split2(b[0], b[4 * kPS], bh0, bl0);
+                    split2(b[8 * kPS], b[12 * kPS], bh1, bl1);
                     mma3(acc, ah[k], al[k], bh0, bh1, bl0, bl1);
                 }
                 float hv[4];
@@ -1039,10 +1060,10 @@ __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
             float acc[2][4] = {{b, b, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
             for (int k = 0; k < NW; ++k) {
-                const float* hb = sh + (k * 16 + 2 * t) * kPS + n * 8 + g;
+                const float* hb = sh + (k * 16 + t) * kPS + n * 8 + g;
                 unsigned bh0, bl0, bh1, bl1;
-                split2(hb[0], hb[kPS], bh0, bl0);
-                split2(hb[8 * kPS], hb[9 * kPS], bh1, bl1);
+                split2(hb[0], hb[4 * kPS], bh0, bl0);
+                split2(hb[8 * kPS], hb[12 * kPS], bh1, bl1);
                 const uint4 w = w2[k * 32 + lane];
                 const unsigned ah[4] = {w.x, 0u, w.y, 0u}, al[4] = {w.z, 0u, w.w, 0u};
                 mma3(acc[k & 1], ah, al, bh0, bh1, bl0, bl1);
@@ -1087,73 +1108,73 @@ __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
                 mma3(gQ2, ah, al, bh0, bh1, bl0, bl1);
             }
             __syncwarp();
-            // dh = GELU' (Q2^T d out) over h
+            // dh = GELU' (Q2^T d out) over h, and the gradient of Q1, dh a^T over
+            // the tile's points: two column tiles of dh are an A fragment as
+            // they stand in the registers
             {
                 const float4 qa = *reinterpret_cast<const float4*>(sq2 + 4 * (h0 + g));
                 const float4 qb = *reinterpret_cast<const float4*>(sq2 + 4 * (h0 + g + 8));
 #pragma unroll
-                for (int n = 0; n < NT; ++n) {
-                    const float* d = sd + n * 8 + 2 * t;
-                    const float2 d0 = *reinterpret_cast<const float2*>(d), d1 = *reinterpret_cast<const float2*>(d + kPS);
-                    const float2 d2 = *reinterpret_cast<const float2*>(d + 2 * kPS);
-                    const float2 d3 = *reinterpret_cast<const float2*>(d + 3 * kPS);
-                    const float v0 = gp[n][0] * (qa.x * d0.x + qa.y * d1.x + qa.z * d2.x + qa.w * d3.x);
-                    const float v1 = gp[n][1] * (qa.x * d0.y + qa.y * d1.y + qa.z * d2.y + qa.w * d3.y);
-                    const float v2 = gp[n][2] * (qb.x * d0.x + qb.y * d1.x + qb.z * d2.x + qb.w * d3.x);
-                    const float v3 = gp[n][3] * (qb.x * d0.y + qb.y * d1.y + qb.z * d2.y + qb.w * d3.y);
-                    gq1[0] += v0 + v1;
-                    gq1[1] += v2 + v3;
-                    float* o = sh + (h0 + g) * kPS + n * 8 + 2 * t;
-                    *reinterpret_cast<float2*>(o) = make_float2(v0, v1);
-                    *reinterpret_cast<float2*>(o + 8 * kPS) = make_float2(v2, v3);
+                for (int k = 0; k < NT / 2; ++k) {
+                    unsigned ah[4], al[4];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int n = 2 * k + u;
+                        const float* d = sd + n * 8 + 2 * t;
+                        const float2 d0 = *reinterpret_cast<const float2*>(d);
+                        const float2 d1 = *reinterpret_cast<const float2*>(d + kPS);
+                        const float2 d2 = *reinterpret_cast<const float2*>(d + 2 * kPS);
+                        const float2 d3 = *reinterpret_cast<const float2*>(d + 3 * kPS);
+                        const float v0 = gp[n][0] * (qa.x * d0.x + qa.y * d1.x + qa.z * d2.x + qa.w * d3.x);
+                        const float v1 = gp[n][1] * (qa.x * d0.y + qa.y * d1.y + qa.z * d2.y + qa.w * d3.y);
+                        const float v2 = gp[n][2] * (qb.x * d0.x + qb.y * d1.x + qb.z * d2.x + qb.w * d3.x);
+                        const float v3 = gp[n][3] * (qb.x * d0.y + qb.y * d1.y + qb.z * d2.y + qb.w * d3.y);
+                        gq1[0] += v0 + v1;
+                        gq1[1] += v2 + v3;
+                        float* o = sh + (h0 + g) * kPS + n * 8 + 2 * t;
+                        *reinterpret_cast<float2*>(o) = make_float2(v0, v1);
+                        *reinterpret_cast<float2*>(o + 8 * kPS) = make_float2(v2, v3);
+                        split2(v0, v1, ah[2 * u], al[2 * u]);
+                        split2(v2, v3, ah[2 * u + 1], al[2 * u + 1]);
+                    }
+#pragma unroll
+                    for (int j = 0; j < CP / 8; ++j) {
+                        const float* b = sa + (j * 8 + g) * kPS + k * 16 + 2 * t;
+                        const float2 u0 = *reinterpret_cast<const float2*>(b);
+                        const float2 u1 = *reinterpret_cast<const float2*>(b + 8);
+                        unsigned bh0, bl0, bh1, bl1;
+                        split2(u0.x, u0.y, bh0, bl0);
+                        split2(u1.x, u1.y, bh1, bl1);
+                        mma3(gQ1[j], ah, al, bh0, bh1, bl0, bl1);
+                    }
                 }
             }
             __syncthreads();
-            // gradient of Q1: dh a^T over the tile's points
-#pragma unroll
-            for (int k = 0; k < kPts / 16; ++k) {
-                unsigned ah[4], al[4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const float2 u = *reinterpret_cast<const float2*>(sh + (h0 + g + ((r & 1) ? 8 : 0)) * kPS + k * 16 +
-                                                                      2 * t + ((r & 2) ? 8 : 0));
-                    split2(u.x, u.y, ah[r], al[r]);
-                }
-#pragma unroll
-                for (int j = 0; j < CP / 8; ++j) {
-                    const float* b = sa + (j * 8 + g) * kPS + k * 16 + 2 * t;
-                    const float2 u0 = *reinterpret_cast<const float2*>(b), u1 = *reinterpret_cast<const float2*>(b + 8);
-                    unsigned bh0, bl0, bh1, bl1;
-                    split2(u0.x, u0.y, bh0, bl0);
-                    split2(u1.x, u1.y, bh1, bl1);
-                    mma3(gQ1[j], ah, al, bh0, bh1, bl0, bl1);
-                }
-            }
-            // da = Q1^T dh, column tiles over the warps
-#pragma unroll
-            for (int v = 0; v < NT / NW; ++v) {
-                const int n = warp + v * NW;
-                float acc[KT][4] = {};
-#pragma unroll
+            // da = Q1^T dh: a warp takes 16 channels of NT KT / NW column tiles
+            {
+                constexpr int NG = NW / KT, NU = NT / NG;
+                const int i = warp % KT, ng = warp / KT;
+                float acc[NU][4] = {};
+#pragma unroll 4
                 for (int k = 0; k < NW; ++k) {
-                    const float* b = sh + (k * 16 + 2 * t) * kPS + n * 8 + g;
-                    unsigned bh0, bl0, bh1, bl1;
-                    split2(b[0], b[kPS], bh0, bl0);
-                    split2(b[8 * kPS], b[9 * kPS], bh1, bl1);
+                    const uint4 hv = *reinterpret_cast<const uint4*>(wt + (i * NW + k) * 256 + lane * 4);
+                    const uint4 lv = *reinterpret_cast<const uint4*>(wt + (i * NW + k) * 256 + 128 + lane * 4);
+                    const unsigned ah[4] = {hv.x, hv.y, hv.z, hv.w}, al[4] = {lv.x, lv.y, lv.z, lv.w};
 #pragma unroll
-                    for (int i = 0; i < KT; ++i) {
-                        const uint4 hv = *reinterpret_cast<const uint4*>(wt + (i * NW + k) * 256 + lane * 4);
-                        const uint4 lv = *reinterpret_cast<const uint4*>(wt + (i * NW + k) * 256 + 128 + lane * 4);
-                        const unsigned ah[4] = {hv.x, hv.y, hv.z, hv.w}, al[4] = {lv.x, lv.y, lv.z, lv.w};
-                        mma3(acc[i], ah, al, bh0, bh1, bl0, bl1);
+                    for (int u = 0; u < NU; ++u) {
+                        const float* b = sh + (k * 16 + t) * kPS + (ng * NU + u) * 8 + g;
+                        unsigned bh0, bl0, bh1, bl1;
+                        split2(b[0], b[4 * kPS], bh0, bl0);
+                        split2(b[8 * kPS], b[12 * kPS], bh1, bl1);
+                        mma3(acc[u], ah, al, bh0, bh1, bl0, bl1);
                     }
                 }
 #pragma unroll
-                for (int i = 0; i < KT; ++i)
+                for (int u = 0; u < NU; ++u)
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
-                        const int c = i * 16 + g + ((r & 2) ? 8 : 0), q = n * 8 + 2 * t + (r & 1);
-                        if (c < C && q < np) p.da[(long long)c * p.N + p0 + q] = acc[i][r];
+                        const int c = i * 16 + g + ((r & 2) ? 8 : 0), q = (ng * NU + u) * 8 + 2 * t + (r & 1);
+                        if (c < C && q < np) p.da[(long long)c * p.N + p0 + q] = acc[u][r];
                     }
             }
         }
@@ -1259,8 +1280,11 @@ cudaError_t row_launch(const FnoFusedDims& d, RowArgs& a, bool bwd, cudaStream_t
     cudaError_t e = cudaSuccess;
     with_modes(d.m, [&](auto M) {
         constexpr int MP = decltype(M)::value;
-        auto k = bwd ? (CP == 16 ? k_fno_row_bwd<16, MP> : k_fno_row_bwd<32, MP>)
-                     : (CP == 16 ? k_fno_row<16, MP> : k_fno_row<32, MP>);
+        const bool shortr = d.nx <= 128;
+        auto k = bwd ? (CP == 16 ? (shortr ? k_fno_row_bwd<16, MP, 2> : k_fno_row_bwd<16, MP, kFoldIter>)
+                                 : (shortr ? k_fno_row_bwd<32, MP, 2> : k_fno_row_bwd<32, MP, kFoldIter>))
+                     : (CP == 16 ? (shortr ? k_fno_row<16, MP, 2> : k_fno_row<16, MP, kFoldIter>)
+                                 : (shortr ? k_fno_row<32, MP, 2> : k_fno_row<32, MP, kFoldIter>));
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
         if (e == cudaSuccess) k<<<(int)grid, 32 * kTeam * nw, sm, s>>>(a);
     });
