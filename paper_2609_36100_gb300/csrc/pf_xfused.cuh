@@ -30,12 +30,23 @@ struct XFIO {
     static constexpr int FOUT = MODE == XF_WRMS ? 0 : (MODE == XF_PHYS1_H ? 3 : 4);
 };
 
-// In-place stage of NL skewed lines (one shared buffer): every job's R
-// inputs are loaded into registers, the CTA synchronises, then the
-// butterflies are formed and stored, and the CTA synchronises again.
-template <int R, int SIGN, int N, int NS, int NL, int NT, typename T2>
+// Lines are skewed (one empty slot after every 16 elements) or not, as their
+// plan says.  Power-of-two lengths are: their stages read and write with
+// power-of-two strides.  Most others are not: an odd first radix is free of
+// most conflicts as it stands, and with N / R no multiple of 16 the skew costs
+// two integer instructions an element (right-hand-side pass at 480 points 1714
+// us skewed, 1596 not; h pass 1516 and 1309).
+template <int N, bool SKEW>
+struct XFLine {
+    static constexpr int LS = SKEW ? N + N / 16 : N + 2;  // stride: at least the two raw rows of a line
+};
+
+// In-place stage of NL lines (one shared buffer): every job's R inputs are
+// loaded into registers, the CTA synchronises, then the butterflies are formed
+// and stored, and the CTA synchronises again.
+template <int R, int SIGN, int N, int NS, int NL, int NT, bool SK, typename T2>
 __device__ __forceinline__ void xf_stage_inplace(T2* S, const T2* __restrict__ tw) {
-    constexpr int M = N / R, TWS = N / (NS * R), JOBS = NL * M, JPT = (JOBS + NT - 1) / NT, LS = N + N / 16;
+    constexpr int M = N / R, TWS = N / (NS * R), JOBS = NL * M, JPT = (JOBS + NT - 1) / NT, LS = XFLine<N, SK>::LS;
     T2 v[JPT][R];
 #pragma unroll
     for (int u = 0; u < JPT; ++u) {
@@ -43,7 +54,10 @@ __device__ __forceinline__ void xf_stage_inplace(T2* S, const T2* __restrict__ t
         if (JOBS % NT == 0 || idx < JOBS) {
             const int line = idx / M, j = idx - line * M;
             const T2* s = S + line * LS;
-            if constexpr (M % 16 == 0) {
+            if constexpr (!SK) {
+#pragma unroll
+                for (int t = 0; t < R; ++t) v[u][t] = s[j + t * M];
+            } else if constexpr (M % 16 == 0) {
                 // skew(j + t M) = skew(j) + t (M + M/16)
                 const T2* sj = s + skew<true>(j);
 #pragma unroll
@@ -67,7 +81,11 @@ __device__ __forceinline__ void xf_stage_inplace(T2* S, const T2* __restrict__ t
                 Bfly<R, SIGN, T2>::run(v[u]);
             T2* d = S + line * LS;
             const int a = jq * NS * R;  // outputs at a + k + t NS
-            if constexpr ((NS * R) % 16 == 0 && NS % 16 == 0) {
+            if constexpr (!SK) {
+                T2* dk = d + a + k;
+#pragma unroll
+                for (int t = 0; t < R; ++t) dk[t * NS] = v[u][t];
+            } else if constexpr ((NS * R) % 16 == 0 && NS % 16 == 0) {
                 T2* dk = d + skew<true>(a) + skew<true>(k);
 #pragma unroll
                 for (int t = 0; t < R; ++t) dk[t * (NS + NS / 16)] = v[u][t];
@@ -89,37 +107,37 @@ __device__ __forceinline__ void xf_stage_inplace(T2* S, const T2* __restrict__ t
     }
     __syncthreads();
 }
-template <int SIGN, int N, int NS, int NL, int NT, typename T2>
+template <int SIGN, int N, int NS, int NL, int NT, bool SK, typename T2>
 __device__ __forceinline__ void xf_run_inplace(T2*, const T2*, Radices<>) {}
-template <int SIGN, int N, int NS, int NL, int NT, typename T2, int R, int... Rest>
+template <int SIGN, int N, int NS, int NL, int NT, bool SK, typename T2, int R, int... Rest>
 __device__ __forceinline__ void xf_run_inplace(T2* S, const T2* tw, Radices<R, Rest...>) {
-    xf_stage_inplace<R, SIGN, N, NS, NL, NT>(S, tw);
-    xf_run_inplace<SIGN, N, NS * R, NL, NT>(S, tw, Radices<Rest...>{});
+    xf_stage_inplace<R, SIGN, N, NS, NL, NT, SK>(S, tw);
+    xf_run_inplace<SIGN, N, NS * R, NL, NT, SK>(S, tw, Radices<Rest...>{});
 }
 
-template <class Fwd, int P>
+template <class Fwd, int P, bool SK>
 struct XFShape {
     static constexpr int N = RadProd<Fwd>::value;
     static constexpr int RM = RadInfo<Fwd>::first;  // radix of the fused stages
     static constexpr int M = N / RM;                 // butterflies per line in the fused stages
     static constexpr int NT = P * M;                 // one thread per (row pair, butterfly)
     static_assert(NT % 32 == 0 && NT <= 1024, "whole warps, at most 1024 threads");
-    static constexpr int LS = N + N / 16;            // skewed line stride
+    static constexpr int LS = XFLine<N, SK>::LS;     // line stride
 };
 
 // registers bounded to 64 a thread, so that they do not cap the CTAs per SM
 // before the shared memory does
-template <class Fwd, int P, int MODE>
-__global__ void __launch_bounds__(XFShape<Fwd, P>::NT, 65536 / (XFShape<Fwd, P>::NT * 64) > 0
-                                                           ? 65536 / (XFShape<Fwd, P>::NT * 64)
-                                                           : 1)
+template <class Fwd, int P, bool SK, int MODE>
+__global__ void __launch_bounds__(XFShape<Fwd, P, SK>::NT, 65536 / (XFShape<Fwd, P, SK>::NT * 64) > 0
+                                                               ? 65536 / (XFShape<Fwd, P, SK>::NT * 64)
+                                                               : 1)
     k_x_fused(Geo g, Phys ph, const float2* __restrict__ in,
                                                                   float2* __restrict__ out, float* __restrict__ R,
                                                                   const float* __restrict__ Rin,
                                                                   double* __restrict__ partials, float rt, float at) {
     PF_SKIP_INACTIVE(g);
     using T2 = float2;
-    using Sh = XFShape<Fwd, P>;
+    using Sh = XFShape<Fwd, P, SK>;
     constexpr int N = Sh::N, RM = Sh::RM, M = Sh::M, NT = Sh::NT, LS = Sh::LS, NXH = N / 2 + 1;
     constexpr int FIN = XFIO<MODE>::FIN, FOUT = XFIO<MODE>::FOUT;
     using Inv = Reversed<Fwd>;
@@ -189,7 +207,7 @@ __global__ void __launch_bounds__(XFShape<Fwd, P>::NT, 65536 / (XFShape<Fwd, P>:
             Bfly<R1, +1, T2>::run(v);
             T2* d = A + line * LS;
 #pragma unroll
-            for (int t = 0; t < R1; ++t) d[skew<true>(j * R1 + t)] = v[t];
+            for (int t = 0; t < R1; ++t) d[skew<SK>(j * R1 + t)] = v[t];
         };
         T2 v[JPT][R1];
 #pragma unroll
@@ -202,7 +220,7 @@ __global__ void __launch_bounds__(XFShape<Fwd, P>::NT, 65536 / (XFShape<Fwd, P>:
     }
     __syncthreads();
     // 3. inverse stages between the first and the last
-    xf_run_inplace<+1, N, R1, P * FIN, NT>(A, tw, typename PlanInner<Inv>::type{});
+    xf_run_inplace<+1, N, R1, P * FIN, NT, SK>(A, tw, typename PlanInner<Inv>::type{});
     // 4. fused: last inverse stage, physics, first forward stage
     const int rp = threadIdx.x / M, j = threadIdx.x - (threadIdx.x / M) * M;
     const bool valid = rp0 + rp < npairs;
@@ -212,7 +230,7 @@ __global__ void __launch_bounds__(XFShape<Fwd, P>::NT, 65536 / (XFShape<Fwd, P>:
     for (int f = 0; f < FIN; ++f) {
         const T2* src = A + (rp * FIN + f) * LS;
 #pragma unroll
-        for (int t = 0; t < RM; ++t) vin[f][t] = src[skew<true>(j + t * M)];
+        for (int t = 0; t < RM; ++t) vin[f][t] = src[skew<SK>(j + t * M)];
         tw_bfly<RM, +1>(vin[f], tw, j, N);  // NS = M: twiddle exponent j t
     }
     if constexpr (MODE == XF_WRMS) {
@@ -308,17 +326,17 @@ __global__ void __launch_bounds__(XFShape<Fwd, P>::NT, 65536 / (XFShape<Fwd, P>:
             Bfly<RM, -1, T2>::run(vout[f]);  // first forward stage: NS = 1, no twiddles
             T2* d = A + (rp * FOUT + f) * LS;
 #pragma unroll
-            for (int t = 0; t < RM; ++t) d[skew<true>(j * RM + t)] = vout[f][t];
+            for (int t = 0; t < RM; ++t) d[skew<SK>(j * RM + t)] = vout[f][t];
         }
         __syncthreads();
         // 5. the remaining forward stages
-        xf_run_inplace<-1, N, RM, P * FOUT, NT>(A, tw, typename DropFirst<Fwd>::type{});
+        xf_run_inplace<-1, N, RM, P * FOUT, NT, SK>(A, tw, typename DropFirst<Fwd>::type{});
         // 6. R2C unpacking of the two rows of each line and the store
         for (int e = threadIdx.x; e < P * FOUT * NXH; e += NT) {
             const int line = e / NXH, k = e - line * NXH, lrp = line / FOUT, f = line - lrp * FOUT;
             if (rp0 + lrp >= npairs) continue;
-            const T2 Zk = A[line * LS + skew<true>(k)];
-            const T2 Zm = A[line * LS + skew<true>(k == 0 ? 0 : N - k)];
+            const T2 Zk = A[line * LS + skew<SK>(k)];
+            const T2 Zm = A[line * LS + skew<SK>(k == 0 ? 0 : N - k)];
             const T2 a = T2{(Zk.x + Zm.x) * 0.5f, (Zk.y - Zm.y) * 0.5f};
             const T2 b = T2{(Zk.y + Zm.y) * 0.5f, (Zm.x - Zk.x) * 0.5f};
             T2* base = out + (long long)f * NK + (2LL * (rp0 + lrp)) * NXH + k;
@@ -328,64 +346,68 @@ __global__ void __launch_bounds__(XFShape<Fwd, P>::NT, 65536 / (XFShape<Fwd, P>:
     }
 }
 
-// fused plans by line length (FP32): the first forward radix is small so the
-// fused stage holds few values per field; P row pairs per CTA, chosen for about 100 to
-// 400 threads (whole warps) and, below 128 points, so that a cube of that side has
-// at least about 150 CTAs: at 32 points 16 CTAs of 32 pairs took 4 us more a pass
-
+// Fused plans by line length (FP32): row pairs per CTA, whether the lines are
+// skewed, and the radices.  The first forward radix is small, so that the fused
+// stage holds few values per field; the row pairs give 100 to 400 threads (whole
+// warps) and, below 128 points, at least about 150 CTAs for a cube of that side
+// (at 32 points 16 CTAs of 32 pairs took 4 us more a pass).  Of the orders tried
+// the fastest: an odd first radix and the power of two next (480 = 5 8 12: 1177
+// and 1455 us for the h and the right-hand-side pass, 5 12 8: 1309 and 1596, 3 16
+// 10: 1385 and 1633).
 template <int N>
 struct XFPlan {
     static constexpr bool ok = false;
 };
-#define PF_XF_PLAN(N_, P_, ...)              \
+#define PF_XF_PLAN(N_, P_, SK_, ...)         \
     template <>                              \
     struct XFPlan<N_> {                      \
         static constexpr bool ok = true;     \
         static constexpr int P = P_;         \
+        static constexpr bool SK = SK_;      \
         using Fwd = Radices<__VA_ARGS__>;    \
     };
-PF_XF_PLAN(32, 4, 4, 8)
-PF_XF_PLAN(36, 8, 3, 12)
-PF_XF_PLAN(40, 4, 5, 8)
-PF_XF_PLAN(48, 8, 4, 12)
-PF_XF_PLAN(60, 8, 3, 4, 5)
-PF_XF_PLAN(64, 8, 4, 16)
-PF_XF_PLAN(72, 8, 3, 12, 2)
-PF_XF_PLAN(80, 8, 5, 16)
-PF_XF_PLAN(96, 8, 4, 8, 3)
-PF_XF_PLAN(100, 8, 5, 10, 2)
-PF_XF_PLAN(108, 8, 3, 12, 3)
-PF_XF_PLAN(120, 4, 3, 8, 5)
-PF_XF_PLAN(128, 8, 4, 8, 4)
-PF_XF_PLAN(144, 4, 3, 12, 4)
-PF_XF_PLAN(160, 4, 4, 8, 5)
-PF_XF_PLAN(180, 8, 3, 15, 4)
-PF_XF_PLAN(192, 4, 4, 16, 3)
-PF_XF_PLAN(200, 8, 5, 10, 4)
-PF_XF_PLAN(216, 4, 3, 12, 6)
-PF_XF_PLAN(240, 4, 3, 10, 8)
-PF_XF_PLAN(256, 4, 4, 16, 4)
-PF_XF_PLAN(288, 2, 3, 12, 8)
-PF_XF_PLAN(300, 8, 5, 6, 10)
-PF_XF_PLAN(320, 4, 4, 10, 8)
-PF_XF_PLAN(360, 4, 3, 15, 8)
-PF_XF_PLAN(384, 2, 4, 12, 8)
-PF_XF_PLAN(400, 4, 5, 10, 8)
-PF_XF_PLAN(432, 2, 3, 12, 12)
-PF_XF_PLAN(480, 2, 3, 16, 10)
-PF_XF_PLAN(512, 2, 4, 16, 8)
-PF_XF_PLAN(640, 2, 5, 16, 8)
+PF_XF_PLAN(32, 4, true, 2, 4, 4)
+PF_XF_PLAN(36, 8, false, 3, 12)
+PF_XF_PLAN(40, 4, false, 5, 8)
+PF_XF_PLAN(48, 8, false, 3, 16)
+PF_XF_PLAN(60, 8, false, 3, 4, 5)
+PF_XF_PLAN(64, 8, true, 4, 16)
+PF_XF_PLAN(72, 8, false, 3, 8, 3)
+PF_XF_PLAN(80, 8, true, 5, 16)
+PF_XF_PLAN(96, 8, true, 4, 8, 3)
+PF_XF_PLAN(100, 8, false, 5, 4, 5)
+PF_XF_PLAN(108, 8, false, 3, 12, 3)
+PF_XF_PLAN(120, 4, false, 3, 8, 5)
+PF_XF_PLAN(128, 8, true, 4, 8, 4)
+PF_XF_PLAN(144, 4, false, 3, 8, 6)
+PF_XF_PLAN(160, 4, false, 4, 8, 5)
+PF_XF_PLAN(180, 8, false, 5, 12, 3)
+PF_XF_PLAN(192, 4, true, 4, 16, 3)
+PF_XF_PLAN(200, 4, false, 5, 8, 5)
+PF_XF_PLAN(216, 4, false, 3, 12, 6)
+PF_XF_PLAN(240, 4, false, 5, 8, 6)
+PF_XF_PLAN(256, 4, true, 4, 16, 4)
+PF_XF_PLAN(288, 2, false, 3, 8, 12)
+PF_XF_PLAN(300, 8, false, 5, 6, 10)
+PF_XF_PLAN(320, 2, false, 5, 8, 8)
+PF_XF_PLAN(360, 4, false, 5, 8, 9)
+PF_XF_PLAN(384, 2, true, 4, 12, 8)
+PF_XF_PLAN(400, 4, false, 5, 8, 10)
+PF_XF_PLAN(432, 2, false, 3, 12, 12)
+PF_XF_PLAN(480, 2, false, 5, 8, 12)
+PF_XF_PLAN(512, 2, true, 4, 16, 8)
+PF_XF_PLAN(640, 2, true, 5, 16, 8)
 #undef PF_XF_PLAN
 
 template <int N, int MODE>
 static int launch_x_fused_k(const Geo& g, const Phys& ph, const void* in, void* out, void* R, const void* Rin,
                             double* partials, double rtol, double atol, cudaStream_t s) {
     using Pl = XFPlan<N>;
-    using Sh = XFShape<typename Pl::Fwd, Pl::P>;
+    using Sh = XFShape<typename Pl::Fwd, Pl::P, Pl::SK>;
     const size_t sm = (size_t)Pl::P * 4 * Sh::LS * sizeof(float2);
     const int npairs = g.nz * g.ny / 2;
     const int nb = (npairs + Pl::P - 1) / Pl::P;
-    auto k = k_x_fused<typename Pl::Fwd, Pl::P, MODE>;
+    auto k = k_x_fused<typename Pl::Fwd, Pl::P, Pl::SK, MODE>;
     set_smem(k, sm);
     k<<<nb, Sh::NT, sm, s>>>(g, ph, reinterpret_cast<const float2*>(in), reinterpret_cast<float2*>(out),
                              reinterpret_cast<float*>(R), reinterpret_cast<const float*>(Rin), partials, (float)rtol,
