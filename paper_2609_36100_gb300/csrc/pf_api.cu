@@ -777,6 +777,11 @@ constexpr int kGraphsMost = 16;  // rebuilt for other tolerances that often, the
 cudaGraphExec_t step_graph(pf_ctx* c, bool lte) {
     if (c->graphs_off || c->prof_on || c->inhom || c->g.N > kGraphPoints || ++c->steps_run <= kGraphAfter)
         return nullptr;
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();  // refused by the step itself, as before
+        return nullptr;
+    }
     pf_ctx::StepGraph* slot = nullptr;
     for (auto& gr : c->graphs) {
         if (gr.exec && gr.y == c->y && gr.lte == lte) {
