@@ -291,7 +291,10 @@ static int tuned_cols(int tuned, int n, int nbuf, int budget, long long cols) {
 // mostly empty (33 columns in three tiles of 16 at nx = 64: 69 % used).  Every
 // loop over a tile strides by a multiple of TX, so a thread keeps its column.
 // Columns of a z pass are also contiguous across rows: tiles start on 128-byte
-// lines wherever ny (nx/2 + 1) is a multiple of 16.
+// lines wherever ny (nx/2 + 1) is a multiple of 16.  Ten FP64 Euler steps at
+// 64^3 took 6.13 ms with tiles cut row by row and 4.70 with these, eight ARK4
+// steps at 128^3 14.37 and 13.53, FP64 at 256^3 (tiles of 8, 95 % used) 155.5 and
+// 150.9.
 template <int TX>
 struct Column {
     int row, kx;  // ky of a z pass, kz of a y pass

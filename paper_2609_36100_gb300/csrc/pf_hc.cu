@@ -88,6 +88,10 @@ __device__ __forceinline__ void block_stats(double (&sum)[NS], long long (&mx)[N
     }
 }
 
+// The pointwise kernels of an iteration read C(r) and eps0 as stored here: formed
+// again in each (three FP64 divisions a point) they took the FP64 pipe's time.
+// us at 96^3, before and now: stress 202 / 73, statistics 237 / 77, Green 112 /
+// 85 (six components for eight), on 10 to 15 arrays of 7 MB, mostly in L2.
 // C(r) and eps0 of every point into pt [9][N]; statistics [0..2] sums of c11,
 // c12, c44, [10] max |eps0|
 template <typename T>

@@ -13,7 +13,8 @@ constexpr int col_min_blocks() {
 }
 
 // ---------------------------------------------------------------------------
-// y pass: in-place complex FFT along y of nf fields
+// y pass: in-place complex FFT along y of nf fields.  FP32 at 256^3 it moves its
+// bytes at 0.8 of the copy bandwidth; FP64 passes are bound by FP64 instructions
 // ---------------------------------------------------------------------------
 template <typename T, int SIGN, int TX, bool R16, int PID>
 __global__ void __launch_bounds__(kThreads, col_min_blocks<T, R16>()) k_y_pass(Geo g, typename Cx<T>::t* __restrict__ buf) {
