@@ -721,22 +721,32 @@ __global__ void __launch_bounds__(512, 1) k_fno_row_bwd(RowArgs a) {
 // P_k = sum_j E cos, Q_k = sum_j O sin give F(+-k) = P_k -+ i Q_k, a quarter
 // of the products of the plain contraction.  tab[j][k] = (cos, sin), k <= m.
 // A thread takes a column of the contiguous inner index and all modes of it in
-// registers, so rows come in whole: 25 us forward and 11 back along y at 128^3,
-// 12 modes, C = 32 (a thread per output read its J values again for every mode).
+// registers, so rows come in whole (a thread per output read its J values again
+// for every mode).  Along z there are few columns (144 blocks of 64 at 24 y
+// modes), so forward four threads share a column's positions: 15.7 us a launch
+// at 128^3, 12 modes, C = 32, mean of y and z, where one thread a column took
+// 24.9; back 11.
 // ---------------------------------------------------------------------------
+constexpr int kDftCols = 64;   // columns of a block
+constexpr int kDftParts = 4;   // parts of the positions, each summed by kDftCols threads
 template <int MP>
-__global__ void __launch_bounds__(64) k_dft_modes(const float2* __restrict__ in, float2* __restrict__ out,
-                                                  const float2* __restrict__ tab, int J, int m, int I) {
-    extern __shared__ __align__(16) float2 st[];  // [J/2 + 1][MP + 2]
+constexpr size_t dft_sum_bytes() {  // two parts' sums P, Q
+    return (kDftParts / 2) * 2 * (MP + 1) * kDftCols * sizeof(float2);
+}
+template <int MP>
+__global__ void __launch_bounds__(kDftCols* kDftParts) k_dft_modes(const float2* __restrict__ in, float2* __restrict__ out,
+                                                                   const float2* __restrict__ tab, int J, int m, int I) {
+    extern __shared__ __align__(16) float2 st[];  // [J/2 + 1][MP + 2]; then the sums of two parts
     constexpr int TP = MP + 2;
     for (int e = threadIdx.x; e < (J / 2 + 1) * TP; e += blockDim.x) {
         const int j = e / TP, k = e - j * TP;
         st[e] = k <= m ? tab[j * (m + 1) + k] : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= I) return;
-    const float2* src = in + (long long)blockIdx.y * J * I + i;
+    const int col = threadIdx.x % kDftCols, part = threadIdx.x / kDftCols;
+    const int i = blockIdx.x * kDftCols + col;
+    const bool ok = i < I;
+    const float2* src = in + (long long)blockIdx.y * J * I + (ok ? i : 0);
     float2 P[MP + 1], Q[MP + 1];
 #pragma unroll
     for (int k = 0; k <= MP; ++k) P[k] = Q[k] = make_float2(0.f, 0.f);
@@ -759,27 +769,49 @@ __global__ void __launch_bounds__(64) k_dft_modes(const float2* __restrict__ in,
         }
     };
     const float2 z = make_float2(0.f, 0.f);
-    add(0, src[0], z);
-    const int pairs = (J - 1) / 2;
-    int j = 1;
+    const int pairs = (J - 1) / 2, per = (pairs + kDftParts - 1) / kDftParts;
+    const int end = min(pairs, (part + 1) * per);
+    if (part == 0) add(0, src[0], z);
+    if (part == kDftParts - 1 && (J & 1) == 0) add(J / 2, src[(long long)(J / 2) * I], z);
     // eight pairs' loads in flight: a thread's trips to memory, not its
     // products, set the time
-    for (; j + 7 <= pairs; j += 8) {
+    for (int j = 1 + part * per; j <= end; j += 8) {
         float2 a[8], b[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            a[u] = src[(long long)(j + u) * I];
-            b[u] = src[(long long)(J - j - u) * I];
+            const bool in_part = j + u <= end;
+            a[u] = in_part ? src[(long long)(j + u) * I] : z;
+            b[u] = in_part ? src[(long long)(J - j - u) * I] : z;
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-            add(j + u, make_float2(a[u].x + b[u].x, a[u].y + b[u].y), make_float2(a[u].x - b[u].x, a[u].y - b[u].y));
+            if (j + u <= end)
+                add(j + u, make_float2(a[u].x + b[u].x, a[u].y + b[u].y), make_float2(a[u].x - b[u].x, a[u].y - b[u].y));
     }
-    for (; j <= pairs; ++j) {
-        const float2 a = src[(long long)j * I], b = src[(long long)(J - j) * I];
-        add(j, make_float2(a.x + b.x, a.y + b.y), make_float2(a.x - b.x, a.y - b.y));
+    // the upper half of the parts hands its sums to the lower one
+#pragma unroll
+    for (int n = kDftParts / 2; n > 0; n /= 2) {
+        __syncthreads();  // the table, or the sums before, are read
+        if (part >= n && part < 2 * n) {
+            float2* d = st + (size_t)(part - n) * 2 * (MP + 1) * kDftCols + col;
+#pragma unroll
+            for (int k = 0; k <= MP; ++k) {
+                d[(2 * k) * kDftCols] = P[k];
+                d[(2 * k + 1) * kDftCols] = Q[k];
+            }
+        }
+        __syncthreads();
+        if (part < n) {
+            const float2* d = st + (size_t)part * 2 * (MP + 1) * kDftCols + col;
+#pragma unroll
+            for (int k = 0; k <= MP; ++k) {
+                const float2 p = d[(2 * k) * kDftCols], q = d[(2 * k + 1) * kDftCols];
+                P[k] = make_float2(P[k].x + p.x, P[k].y + p.y);
+                Q[k] = make_float2(Q[k].x + q.x, Q[k].y + q.y);
+            }
+        }
     }
-    if ((J & 1) == 0) add(J / 2, src[(long long)(J / 2) * I], z);
+    if (part > 0 || !ok) return;
     float2* dst = out + (long long)blockIdx.y * 2 * m * I + i;
 #pragma unroll
     for (int k = 0; k <= MP; ++k) {
@@ -1346,10 +1378,11 @@ cudaError_t project_launch(const FnoFusedDims& d, ProjArgs& p, int* blocks, cuda
 void dft_fwd(const float2* in, float2* out, const float2* tab, int J, int m, int I, int O, cudaStream_t s) {
     with_modes(m, [&](auto M) {
         constexpr int MP = decltype(M)::value;
-        const size_t sm = (size_t)(J / 2 + 1) * (MP + 2) * sizeof(float2);
+        size_t sm = (size_t)(J / 2 + 1) * (MP + 2) * sizeof(float2);
+        if (sm < dft_sum_bytes<MP>()) sm = dft_sum_bytes<MP>();
         if (sm > 48 * 1024)
             cudaFuncSetAttribute(k_dft_modes<MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k_dft_modes<MP><<<dim3((I + 63) / 64, O), 64, sm, s>>>(in, out, tab, J, m, I);
+        k_dft_modes<MP><<<dim3((I + kDftCols - 1) / kDftCols, O), kDftCols * kDftParts, sm, s>>>(in, out, tab, J, m, I);
     });
 }
 void dft_inv(const float2* in, float2* out, const float2* tab, int J, int m, int I, int O, cudaStream_t s) {
