@@ -240,19 +240,19 @@ struct pf_ctx {
     double* h_scalar = nullptr;  // pinned
     // A step as a graph, for grids whose kernels are as short as the gaps
     // between launches: one per state buffer (an accepted step swaps them) and
-    // with or without the error estimate, its step size in coefficients the
-    // launch copies in.  Built after kGraphAfter steps of a context.
+    // with or without the error estimate.  Step size and tolerances are read
+    // from d_vars.  Built after kGraphAfter steps of a context.
     struct StepGraph {
         cudaGraphExec_t exec = nullptr;
         const double2* y = nullptr;
         bool lte = false;
-        double rtol = 0.0, atol = 0.0;
     };
     StepGraph graphs[4];
-    int steps_run = 0, graphs_built = 0;
+    int steps_run = 0;               // up to kGraphAfter
     bool graphs_off = false;
-    StageCoefDev* d_coef = nullptr;  // [kMaxStages + 2]
-    StageCoefDev* h_coef = nullptr;  // pinned
+    StepVars* d_vars = nullptr;
+    StepVars vars{};                 // what d_vars holds, once set
+    bool vars_set = false;
     cudaStream_t cap = nullptr;      // captured on (the legacy default stream cannot be)
     // integrator state
     double t = 0.0, h = 0.0;
@@ -391,13 +391,13 @@ void drop_graphs(pf_ctx* c) {
         if (gr.exec) cudaGraphExecDestroy(gr.exec);
         gr = {};
     }
+    c->steps_run = 0;
 }
 
 void free_all(pf_ctx* c) {
     drop_graphs(c);
     if (c->cap) cudaStreamDestroy(c->cap);
-    cudaFree(c->d_coef);
-    if (c->h_coef) cudaFreeHost(c->h_coef);
+    cudaFree(c->d_vars);
     cudaFree(c->d_kx);
     cudaFree(c->d_ky);
     cudaFree(c->d_kz);
@@ -587,7 +587,8 @@ int hc_solve(pf_ctx* c, const void* R, void* E, double* energy) {
 }
 
 template <typename T>
-int enqueue_step(pf_ctx* c, double dt, bool want_lte, const StageCoefDev* dcoef = nullptr) {
+int enqueue_step(pf_ctx* c, double dt, bool want_lte, const StageCoefDev* dcoef = nullptr,
+                 const StepTol* dtol = nullptr) {
     using T2 = typename std::conditional<sizeof(T) == 8, double2, float2>::type;
     const Geo& g = c->g;
     const Phys& ph = c->ph;
@@ -753,7 +754,9 @@ int enqueue_step(pf_ctx* c, double dt, bool want_lte, const StageCoefDev* dcoef 
         int nb = 0;
         {
             ProfScope p(c, PF_K_X_WRMS, 4 * NK * cb + 4 * N * rb);
-            nb = launch_x_pass<T>(g, ph, XM_WRMS, c->W, nullptr, nullptr, c->R1, c->partials, c->prm.rtol,
+            Geo gw = g;
+            gw.tol = dtol;
+            nb = launch_x_pass<T>(gw, ph, XM_WRMS, c->W, nullptr, nullptr, c->R1, c->partials, c->prm.rtol,
                                   c->prm.atol, nullptr, nullptr, s);
         }
         {
@@ -768,15 +771,20 @@ int enqueue_step(pf_ctx* c, double dt, bool want_lte, const StageCoefDev* dcoef 
 // gaps between 60 launches were 2.2 us each (1.1 of 12.9 ms for eight steps at
 // 128^3, most of a step at 32^3).  Capturing and instantiating costs about a
 // millisecond and is left to contexts that step on; larger grids would gain
-// under 1 %.
+// under 1 %.  The buffers a graph needs are the context's, allocated with it;
+// the graph object itself is the driver's.
 constexpr int kGraphAfter = 16;
 constexpr long long kGraphPoints = 160LL * 160 * 160;
-constexpr int kGraphsMost = 16;  // rebuilt for other tolerances that often, then no more
+
+bool graph_sized(const pf_ctx* c) { return c->g.N <= kGraphPoints && !c->inhom; }
 
 // a graph of the step from c->y, or null where the step is launched directly
 cudaGraphExec_t step_graph(pf_ctx* c, bool lte) {
-    if (c->graphs_off || c->prof_on || c->inhom || c->g.N > kGraphPoints || ++c->steps_run <= kGraphAfter)
+    if (c->graphs_off || c->prof_on || !graph_sized(c)) return nullptr;
+    if (c->steps_run < kGraphAfter) {
+        ++c->steps_run;
         return nullptr;
+    }
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone) {
         cudaGetLastError();  // refused by the step itself, as before
@@ -784,34 +792,31 @@ cudaGraphExec_t step_graph(pf_ctx* c, bool lte) {
     }
     pf_ctx::StepGraph* slot = nullptr;
     for (auto& gr : c->graphs) {
-        if (gr.exec && gr.y == c->y && gr.lte == lte) {
-            if (!lte || (gr.rtol == c->prm.rtol && gr.atol == c->prm.atol)) return gr.exec;
-            cudaGraphExecDestroy(gr.exec);
-            gr = {};
-        }
+        if (gr.exec && gr.y == c->y && gr.lte == lte) return gr.exec;
         if (!gr.exec && !slot) slot = &gr;
     }
-    const int ncoef = c->tab.s + 2;
-    cudaError_t e = !slot || ++c->graphs_built > kGraphsMost ? cudaErrorNotSupported : cudaSuccess;
-    if (e == cudaSuccess && !c->d_coef) e = cudaMalloc((void**)&c->d_coef, ncoef * sizeof(StageCoefDev));
-    if (e == cudaSuccess && !c->h_coef) {
-        e = cudaMallocHost((void**)&c->h_coef, ncoef * sizeof(StageCoefDev));
-        if (e == cudaSuccess) std::memset(c->h_coef, 0, ncoef * sizeof(StageCoefDev));
-    }
-    if (e == cudaSuccess && !c->cap) e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeRelaxed);
-    cudaGraph_t graph = nullptr;
+    // calls that are unsafe beside another thread's capture in the default
+    // (global) mode must not end it: this thread captures in the relaxed one
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaError_t e = slot ? cudaThreadExchangeStreamCaptureMode(&mode) : cudaErrorNotSupported;
     if (e == cudaSuccess) {
-        const cudaStream_t user = c->stream;
-        c->stream = c->cap;
-        e = cudaMemcpyAsync(c->d_coef, c->h_coef, ncoef * sizeof(StageCoefDev), cudaMemcpyHostToDevice, c->cap);
-        const int rc = c->fp32 ? enqueue_step<float>(c, 1.0, lte, c->d_coef) : enqueue_step<double>(c, 1.0, lte, c->d_coef);
-        c->stream = user;
-        const cudaError_t e2 = cudaStreamEndCapture(c->cap, &graph);
-        if (e == cudaSuccess) e = rc ? cudaErrorUnknown : e2;
+        if (!c->cap) e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeRelaxed);
+        cudaGraph_t graph = nullptr;
+        if (e == cudaSuccess) {
+            const cudaStream_t user = c->stream;
+            c->stream = c->cap;
+            const StageCoefDev* co = c->d_vars->coef;
+            const StepTol* tol = &c->d_vars->tol;
+            const int rc = c->fp32 ? enqueue_step<float>(c, 1.0, lte, co, tol) : enqueue_step<double>(c, 1.0, lte, co, tol);
+            c->stream = user;
+            e = cudaStreamEndCapture(c->cap, &graph);
+            if (rc) e = cudaErrorUnknown;
+        }
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&slot->exec, graph, 0);
+        if (graph) cudaGraphDestroy(graph);
+        cudaThreadExchangeStreamCaptureMode(&mode);
     }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&slot->exec, graph, 0);
-    if (graph) cudaGraphDestroy(graph);
     if (e != cudaSuccess) {  // the step is launched directly, now and from now on
         cudaGetLastError();
         if (slot) slot->exec = nullptr;
@@ -820,32 +825,42 @@ cudaGraphExec_t step_graph(pf_ctx* c, bool lte) {
     }
     slot->y = c->y;
     slot->lte = lte;
-    slot->rtol = c->prm.rtol;
-    slot->atol = c->prm.atol;
     return slot->exec;
+}
+
+// d_vars for a step of size dt, in the stream's order; nothing to do where it
+// holds them already
+int set_step_vars(pf_ctx* c, double dt) {
+    const Tableau& tb = c->tab;
+    StepVars v;
+    std::memset(&v, 0, sizeof v);
+    for (int i = 0; i < tb.s; ++i)
+        fill_coef(v.coef[i], i, tb.AI[i], tb.AE[i], dt, dt * tb.AI[i][i], dt * c->gdiag);
+    double dI[kMaxStages], dE[kMaxStages];
+    for (int j = 0; j < kMaxStages; ++j) {
+        dI[j] = tb.embedded ? tb.bI[j] - tb.btI[j] : 0.0;
+        dE[j] = tb.embedded ? tb.bE[j] - tb.btE[j] : 0.0;
+    }
+    fill_coef(v.coef[tb.s], tb.s, tb.bI, tb.bE, dt, 0.0, 0.0);
+    fill_coef(v.coef[tb.s + 1], tb.s, dI, dE, dt, 0.0, 0.0);
+    v.tol.rtol = c->prm.rtol;
+    v.tol.atol = c->prm.atol;
+    v.tol.rtol32 = (float)c->prm.rtol;
+    v.tol.atol32 = (float)c->prm.atol;
+    if (c->vars_set && std::memcmp(&v, &c->vars, sizeof v) == 0) return PF_OK;
+    c->vars_set = false;
+    launch_set_step_vars(v, c->d_vars, c->stream);
+    if (int rc = check_launch(c, "step coefficients")) return rc;
+    std::memcpy(&c->vars, &v, sizeof v);
+    c->vars_set = true;
+    return PF_OK;
 }
 
 int step_once(pf_ctx* c, double dt, bool want_lte, double* e_out) {
     int rc = PF_OK;
     if (cudaGraphExec_t exec = step_graph(c, want_lte && c->tab.embedded)) {
-        const Tableau& tb = c->tab;
-        StageCoefDev co[kMaxStages + 2];
-        std::memset(co, 0, sizeof co);
-        for (int i = 0; i < tb.s; ++i)
-            fill_coef(co[i], i, tb.AI[i], tb.AE[i], dt, dt * tb.AI[i][i], dt * c->gdiag);
-        double dI[kMaxStages], dE[kMaxStages];
-        for (int j = 0; j < kMaxStages; ++j) {
-            dI[j] = tb.embedded ? tb.bI[j] - tb.btI[j] : 0.0;
-            dE[j] = tb.embedded ? tb.bE[j] - tb.btE[j] : 0.0;
-        }
-        fill_coef(co[tb.s], tb.s, tb.bI, tb.bE, dt, 0.0, 0.0);
-        fill_coef(co[tb.s + 1], tb.s, dI, dE, dt, 0.0, 0.0);
-        if (std::memcmp(co, c->h_coef, (tb.s + 2) * sizeof(StageCoefDev)) != 0) {
-            // an earlier step that was not waited for may still have to copy them
-            PF_CUDA(c, cudaStreamSynchronize(c->stream));
-            std::memcpy(c->h_coef, co, (tb.s + 2) * sizeof(StageCoefDev));
-        }
-        PF_CUDA(c, cudaGraphLaunch(exec, c->stream));
+        rc = set_step_vars(c, dt);
+        if (!rc) PF_CUDA(c, cudaGraphLaunch(exec, c->stream));
     } else {
         rc = c->fp32 ? enqueue_step<float>(c, dt, want_lte) : enqueue_step<double>(c, dt, want_lte);
     }
@@ -1097,6 +1112,7 @@ int pf_create(const pf_grid* grid, const pf_params* params, void* cuda_stream, p
             rc = fail(c, PF_ENOMEM, "pinned host allocation failed");
     }
     rc = rc ? rc : dalloc(c, &c->d_scalar, 4 * sizeof(double));
+    if (graph_sized(c)) rc = rc ? rc : dalloc(c, &c->d_vars, sizeof(StepVars));
     if (!rc && cudaMallocHost((void**)&c->h_scalar, 4 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         rc = fail(c, PF_ENOMEM, "cudaMallocHost failed");

@@ -34,6 +34,8 @@ int default_elastic_plan(const AxisPlan& pz);
 int compiled_plan_len(int pid);
 int compiled_plan_count();
 
+struct StepTol;
+
 // Grid geometry and the per-axis wave-number tables k_m = 2 pi m / (n d)
 // (FP64, Nyquist index taken as +pi/d).
 struct Geo {
@@ -70,6 +72,7 @@ struct Geo {
                              // 2 runs a cluster of three CTAs, one field each (FP32 contexts)
     const void* btab;        // elastic kernel B(k) / N in the compute type over kx >= 0, |ky| <= ny/2, |kz| <= nz/2
                              // (six symmetric entries, [6][nz/2+1][ny/2+1][nx/2+1]), or null: computed per k
+    const StepTol* tol;      // tolerances of the WRMS pass (a step that runs as a graph), or null: its arguments
 };
 
 // Model constants of the real-space and elastic terms in one compute type,
@@ -148,6 +151,19 @@ __host__ __device__ inline void fill_coef(StageCoefDev& c, int n, const double* 
     c.qgh = (float)qgam;
     c.qgl = (float)(qgam - (double)c.qgh);
 }
+
+// What a step that runs as a graph reads from device memory instead of its
+// launches' arguments: the coefficients of the stages, the completion and the
+// error estimate, and the error weights' tolerances.
+struct StepTol {
+    double rtol, atol;
+    float rtol32, atol32;
+};
+struct StepVars {
+    StageCoefDev coef[kMaxStages + 2];
+    StepTol tol;
+};
+static_assert(sizeof(StepVars) <= 4000, "passed to a kernel by value");
 
 // Coefficients of one stage assembly / step completion pass.
 struct StageTerms {
@@ -282,6 +298,8 @@ void launch_stage_assemble(const Geo& g, const double2* y, const StageTerms& st,
 // in-place FFT along z of nf fields (sign +1 inverse)
 template <typename T>
 void launch_z_pass(const Geo& g, void* buf, int nf, cudaStream_t s);
+// the variables of a step graph's next launch into *d
+void launch_set_step_vars(const StepVars& v, StepVars* d, cudaStream_t s);
 // batch round: coefficients from the member's step, controller, accepted-state copy
 void launch_batch_prep(const BatchConst& bc, MemberCtl* ctl, StageCoefDev* coef, cudaStream_t s);
 void launch_batch_ctl(const BatchConst& bc, MemberCtl* ctl, const double* wrms_sum, double scale, cudaStream_t s);

@@ -284,6 +284,15 @@ void launch_lambda_table(const Geo& g, const Phys& ph, double* lam, float2* lamd
     k_lambda_table<<<152 * 8, 256, 0, s>>>(g, ph, lam, lamdf);
 }
 
+// A kernel argument is copied at its launch, so the host may go on at once: a
+// copy from pinned memory would have to be waited for before the next values.
+__global__ void __launch_bounds__(256) k_set_step_vars(StepVars v, StepVars* __restrict__ d) {
+    const int* src = reinterpret_cast<const int*>(&v);
+    for (int i = threadIdx.x; i < (int)(sizeof(StepVars) / sizeof(int)); i += blockDim.x)
+        reinterpret_cast<int*>(d)[i] = src[i];
+}
+void launch_set_step_vars(const StepVars& v, StepVars* d, cudaStream_t s) { k_set_step_vars<<<1, 256, 0, s>>>(v, d); }
+
 // ---------------------------------------------------------------------------
 // batch round kernels (one thread each, or a grid-stride copy)
 // ---------------------------------------------------------------------------

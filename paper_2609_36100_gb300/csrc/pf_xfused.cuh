@@ -238,6 +238,10 @@ __global__ void __launch_bounds__(XFShape<Fwd, P, SK>::NT, 65536 / (XFShape<Fwd,
         // stored real-space y_{n-1}); compensated FP32 sum per thread, FP64
         // across threads and CTAs
         float sh = 0.f, sl = 0.f;
+        if (g.tol) {
+            rt = step_tol<float>(*g.tol, 0);
+            at = step_tol<float>(*g.tol, 1);
+        }
         if (valid) {
 #pragma unroll
             for (int t = 0; t < RM; ++t) {

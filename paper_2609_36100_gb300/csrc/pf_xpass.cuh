@@ -22,6 +22,15 @@ __device__ __forceinline__ T xdiv(T a, T b) {
         return a / b;
 }
 
+// rtol (0) or atol (1) of a step graph in the compute type
+template <typename T>
+__device__ __forceinline__ T step_tol(const StepTol& t, int which) {
+    if constexpr (sizeof(T) == 4)
+        return which ? t.atol32 : t.rtol32;
+    else
+        return which ? t.atol : t.rtol;
+}
+
 // x clipped to [-1, 1]; in FP64 by the exponent field, off the FP64 pipe
 // (where two comparisons a value would run).  A NaN stays a NaN there; every
 // term it meets is one already.
@@ -264,6 +273,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : (R16 ? 2 : 3)) 
 
     if (mode == XM_WRMS) {
         double acc = 0.0;
+        const T rt = g.tol ? step_tol<T>(*g.tol, 0) : (T)rtol, at = g.tol ? step_tol<T>(*g.tol, 1) : (T)atol;
         for (int e = threadIdx.x; e < P * 4 * nx; e += blockDim.x) {
             const int line = L.divn(e), x = e - line * nx, rp = line >> 2, f = line & 3;
             if (rp0 + rp >= npairs) continue;
@@ -273,7 +283,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : (R16 ? 2 : 3)) 
             // weighted error w_i * LTE_i formed in the compute type (the
             // error and y_{n-1} are already compute-type fields); squares
             // accumulated in FP64
-            const T rt = (T)rtol, at = (T)atol;
             const T a = z.x / (rt * fabs(yr[0]) + at), b = z.y / (rt * fabs(yr[nx]) + at);
             if (sizeof(T) == 4) {
                 const double da = f2d_bits((float)a), db = f2d_bits((float)b);
