@@ -1083,15 +1083,6 @@ int pf_create(const pf_grid* grid, const pf_params* params, void* cuda_stream, p
     rc = rc ? rc : dalloc(c, &c->R1, 4 * (size_t)g.N * tsz);
     rc = rc ? rc : dalloc(c, &c->lam, nk4 * sizeof(double));
     if (c->fp32) rc = rc ? rc : dalloc(c, &c->lamdf, nk4 * sizeof(float2));
-    // elastic-kernel table: homogeneous modulus, diagonal eigenstrains (B even
-    // in each wave-number component), at most 1 GB (FP32: 794 MB at 640^3; FP64:
-    // 103 MB at 256^3)
-    bool diag = true;
-    for (int v = 0; v < 3; ++v)
-        for (int a = 3; a < 6; ++a) diag = diag && params->eps_star[v][a] == 0.0;
-    const long long tabn = (long long)(g.nz / 2 + 1) * (g.ny / 2 + 1) * g.nxh;
-    if (c->ph.elastic && !c->inhom && diag && 6 * tabn * (long long)tsz <= (1LL << 30))
-        rc = rc ? rc : dalloc(c, &c->btab, 6 * (size_t)tabn * tsz);
     rc = rc ? rc : dalloc(c, &c->qtab, nk4 * sizeof(double));
     if (params->barrier == 1) rc = rc ? rc : dalloc(c, &c->xsave, (size_t)g.NK * sizeof(double2));
     // worst case over any tuned rows-per-CTA setting (one row pair per CTA)
@@ -1116,6 +1107,19 @@ int pf_create(const pf_grid* grid, const pf_params* params, void* cuda_stream, p
     if (!rc && cudaMallocHost((void**)&c->h_scalar, 4 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         rc = fail(c, PF_ENOMEM, "cudaMallocHost failed");
+    }
+    // elastic-kernel table: homogeneous modulus, diagonal eigenstrains (B even
+    // in each wave-number component), at most 1 GB (FP32: 794 MB at 640^3; FP64:
+    // 103 MB at 256^3).  The passes form B per wave vector without it, so a
+    // device that has no room left for it still takes the context.
+    bool diag = true;
+    for (int v = 0; v < 3; ++v)
+        for (int a = 3; a < 6; ++a) diag = diag && params->eps_star[v][a] == 0.0;
+    const long long tabn = (long long)(g.nz / 2 + 1) * (g.ny / 2 + 1) * g.nxh;
+    if (!rc && c->ph.elastic && !c->inhom && diag && 6 * tabn * (long long)tsz <= (1LL << 30) &&
+        cudaMalloc(&c->btab, 6 * (size_t)tabn * tsz) != cudaSuccess) {
+        cudaGetLastError();
+        c->btab = nullptr;
     }
     if (rc) {
         std::snprintf(g_create_err, sizeof g_create_err, "%s", c->err);
