@@ -226,7 +226,7 @@ struct pf_ctx {
     bool inhom = false;
     HCConst hck{};
     double* hc_pt = nullptr;       // C(r) and eps0 of the solve's fields, real [9][N]
-    double* hc_tau = nullptr;      // eigenstress, real [6][N] (xx yy zz yz xz xy)
+    double* hc_tau = nullptr;      // eigenstress, real [6][N] (xx yy zz yz xz xy), in the place of hc_k
     double* hc_eu[2] = {};         // eps(u), real [6][N]: current and previous iterate
     double2* hc_k = nullptr;       // k-space [6][NK] (tau^, then eps^(u))
     double2* hc_ks = nullptr;      // partial-transform scratch [6][NK]
@@ -423,7 +423,6 @@ void free_all(pf_ctx* c) {
     cudaFree(c->qtab);
     cudaFree(c->partials);
     cudaFree(c->hc_pt);
-    cudaFree(c->hc_tau);
     cudaFree(c->hc_eu[0]);
     cudaFree(c->hc_eu[1]);
     cudaFree(c->hc_k);
@@ -1092,11 +1091,13 @@ int pf_create(const pf_grid* grid, const pf_params* params, void* cuda_stream, p
     if (c->inhom) {
         const size_t n6 = 6 * (size_t)g.N * sizeof(double);
         rc = rc ? rc : dalloc(c, &c->hc_pt, 9 * (size_t)g.N * sizeof(double));
-        rc = rc ? rc : dalloc(c, &c->hc_tau, n6);
         rc = rc ? rc : dalloc(c, &c->hc_eu[0], n6);
         rc = rc ? rc : dalloc(c, &c->hc_eu[1], n6);
         rc = rc ? rc : dalloc(c, &c->hc_k, 6 * (size_t)g.NK * sizeof(double2));
         rc = rc ? rc : dalloc(c, &c->hc_ks, 6 * (size_t)g.NK * sizeof(double2));
+        // the x pass has read tau when the z pass writes hc_k, and tau is
+        // formed anew after the last read of hc_k
+        c->hc_tau = reinterpret_cast<double*>(c->hc_k);
         rc = rc ? rc : dalloc(c, &c->hc_part, (size_t)hc_blocks() * kHcStats * sizeof(double));
         rc = rc ? rc : dalloc(c, &c->hc_ebar, 6 * sizeof(double));
         if (!rc && cudaMallocHost((void**)&c->hc_host, ((size_t)hc_blocks() * kHcStats + 8) * sizeof(double)) != cudaSuccess)

@@ -1,4 +1,5 @@
-"""Device memory of a context: the elastic-kernel table is taken where there is room for it."""
+"""Device memory of a context: the elastic-kernel table is taken where there is room for it, and the phase-dependent
+stiffness takes 33 real fields."""
 import numpy as np
 import pytest
 
@@ -52,3 +53,19 @@ def test_context_without_room_for_the_elastic_table(pfg, params, prec, tol):
         free_bytes()
     for f in range(4):
         assert np.linalg.norm(got[f] - ref[f]) <= tol * np.linalg.norm(ref[f])
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32bulk"])
+def test_phase_dependent_stiffness_buffers(pfg, params, prec):
+    n = 128
+    p = dict(params, eps_star=[[0.0] * 6] * 3)
+    q = dict(params, el_inhom=1, C11_v=325.0, C12_v=176.0, C44_v=144.0)
+    with pfg.Simulation((n, n, n), p, "euler", prec):
+        pass
+    size = []
+    for r in (p, q):
+        before = free_bytes()
+        with pfg.Simulation((n, n, n), r, "euler", prec):
+            size.append(before - free_bytes())
+    # 33 fields of real points, 12 of them as half spectra (n + 2 in n), and a share of the driver's 2 MB pages
+    assert size[1] - size[0] <= 36 * 8 * n ** 3
