@@ -967,11 +967,20 @@ struct ProjArgs {
     long long N;
     float sc;  // 2 / (4 N)
 };
-template <int CP, int NW, bool TRAIN>
+template <int CP, int NW, bool TRAIN, bool FULL>
 constexpr int proj_smem() {
     constexpr int HP = 16 * NW, KT = CP / 16;
-    return (2 * CP * kPS + HP * kPS + 4 * kPS + NW * 128 + 4 * HP + HP + 4 + NW * KT * 256 +
+    return (2 * CP * kPS + HP * kPS + 4 * kPS + NW * 128 + 4 * HP + HP + 4 + (FULL ? HP * (CP + 4) : NW * KT * 256) +
             (TRAIN ? NW * KT * 256 : 0)) * 4;
+}
+
+// Hidden widths whose row tiles are no power of two (33 to 48, 65 to 112) have
+// the product Q1 a in FP32, the others in BF16 parts: so it is in the kernels
+// of one operation each (dense_mma has forms for 1, 2, 4 and 8 row tiles), and
+// which of the two paths a size runs says nothing about its precision.
+__host__ __device__ constexpr bool proj_full(int H) {
+    const int tiles = (H + 15) / 16;
+    return (tiles & (tiles - 1)) != 0;
 }
 
 // The products of a tile run on the tensor cores (1031 us forward and backward
@@ -980,7 +989,7 @@ constexpr int proj_smem() {
 // the instructions around them, GELU of its H x 64 hidden values first, and the
 // shared memory those pass through.  The next tile's columns of a are copied in
 // while this one is worked on.
-template <int CP, int NW, bool TRAIN>
+template <int CP, int NW, bool TRAIN, bool FULL>
 __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
     constexpr int HP = 16 * NW, KT = CP / 16, NT = kPts / 8;
     extern __shared__ __align__(16) float sm[];
@@ -991,8 +1000,10 @@ __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
     float* sq2 = sd + 4 * kPS + NW * 128;  // [HP][4]
     float* sq1 = sq2 + 4 * HP;             // [HP]
     float* sb2 = sq1 + HP;                 // [4]
-    unsigned* w1 = reinterpret_cast<unsigned*>(sb2 + 4);  // Q1 fragments [NW][KT]
-    unsigned* wt = w1 + NW * KT * 256;                    // Q1^T fragments [KT][NW]
+    unsigned* w1 = reinterpret_cast<unsigned*>(sb2 + 4);  // Q1 fragments [NW][KT], or (FULL) Q1 itself
+    float* f1 = sb2 + 4;                                  // [HP][FS]
+    constexpr int FS = CP + 4;
+    unsigned* wt = w1 + (FULL ? HP * FS : NW * KT * 256);  // Q1^T fragments [KT][NW]
     const int C = p.C, H = p.H;
     auto q1v = [&](int h, int c) -> float { return h < H && c < C ? p.Q1[h * C + c] : 0.f; };
     for (int e = threadIdx.x; e < NW * KT * 32; e += blockDim.x) {
@@ -1001,8 +1012,9 @@ __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
         for (int r = 0; r < 4; ++r) {
             const int mm = g + ((r & 1) ? 8 : 0), k0 = krow(t, r & 2), k1 = krow(t, (r & 2) + 1);
             const int mt = tile / KT, kt = tile - mt * KT;
-            split2(q1v(mt * 16 + mm, kt * 16 + k0), q1v(mt * 16 + mm, kt * 16 + k1), w1[tile * 256 + lane * 4 + r],
-                   w1[tile * 256 + 128 + lane * 4 + r]);
+            if constexpr (!FULL)
+                split2(q1v(mt * 16 + mm, kt * 16 + k0), q1v(mt * 16 + mm, kt * 16 + k1), w1[tile * 256 + lane * 4 + r],
+                       w1[tile * 256 + 128 + lane * 4 + r]);
             if (TRAIN) {
                 const int ct = tile / NW, ht = tile - ct * NW;
                 split2(q1v(ht * 16 + k0, ct * 16 + mm), q1v(ht * 16 + k1, ct * 16 + mm),
@@ -1010,6 +1022,8 @@ __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
             }
         }
     }
+    if constexpr (FULL)
+        for (int e = threadIdx.x; e < HP * CP; e += blockDim.x) f1[e / CP * FS + e % CP] = q1v(e / CP, e % CP);
     for (int e = threadIdx.x; e < NW * 32; e += blockDim.x) {
         const int g = (e & 31) >> 2, h = (e >> 5) * 16 + (e & 3);
         auto v = [&](int hh) -> float { return g < 4 && hh < H ? p.Q2[g * H + hh] : 0.f; };
@@ -1071,26 +1085,9 @@ __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
         // h = GELU(Q1 a + q1) of this warp's rows; its derivative stays in registers
         float gp[TRAIN ? NT : 1][4];
         {
-            unsigned ah[KT][4], al[KT][4];
-#pragma unroll
-            for (int k = 0; k < KT; ++k) {
-                const uint4 hv = *reinterpret_cast<const uint4*>(w1 + (warp * KT + k) * 256 + lane * 4);
-                const uint4 lv = *reinterpret_cast<const uint4*>(w1 + (warp * KT + k) * 256 + 128 + lane * 4);
-                ah[k][0] = hv.x, ah[k][1] = hv.y, ah[k][2] = hv.z, ah[k][3] = hv.w;
-                al[k][0] = lv.x, al[k][1] = lv.y, al[k][2] = lv.z, al[k][3] = lv.w;
-            }
             const float b0 = sq1[h0 + g], b1 = sq1[h0 + g + 8];
-#pragma unroll
-            for (int n = 0; n < NT; ++n) {
-                float acc[4] = {b0, b0, b1, b1};
-#pragma unroll
-                for (int k = 0; k < KT; ++k) {
-                    const float* b = sa + (k * 16 + t) * kPS + n * 8 + g;
-                    unsigned bh0, bl0, bh1, bl1;
-                    split2(b[0], b[4 * kPS], bh0, bl0);
-                    split2(b[8 * kPS], b[12 * kPS], bh1, bl1);
-                    mma3(acc, ah[k], al[k], bh0, bh1, bl0, bl1);
-                }
+            // column tile n of the pre-activations: GELU into sh
+            auto hidden = [&](int n, const float (&acc)[4]) {
                 float hv[4];
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
@@ -1103,6 +1100,52 @@ __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
                 float* o = sh + (h0 + g) * kPS + n * 8 + 2 * t;
                 *reinterpret_cast<float2*>(o) = make_float2(hv[0], hv[1]);
                 *reinterpret_cast<float2*>(o + 8 * kPS) = make_float2(hv[2], hv[3]);
+            };
+            if constexpr (FULL) {
+                const float *q0 = f1 + (h0 + g) * FS, *q8 = q0 + 8 * FS;
+                constexpr int NB = 4;  // column tiles at a time
+#pragma unroll
+                for (int n0 = 0; n0 < NT; n0 += NB) {
+                    float acc[NB][4];
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) acc[u][0] = acc[u][1] = b0, acc[u][2] = acc[u][3] = b1;
+#pragma unroll 4
+                    for (int c = 0; c < C; ++c) {
+                        const float w0 = q0[c], w8 = q8[c];
+#pragma unroll
+                        for (int u = 0; u < NB; ++u) {
+                            const float2 v = *reinterpret_cast<const float2*>(sa + c * kPS + (n0 + u) * 8 + 2 * t);
+                            acc[u][0] = fmaf(w0, v.x, acc[u][0]);
+                            acc[u][1] = fmaf(w0, v.y, acc[u][1]);
+                            acc[u][2] = fmaf(w8, v.x, acc[u][2]);
+                            acc[u][3] = fmaf(w8, v.y, acc[u][3]);
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) hidden(n0 + u, acc[u]);
+                }
+            } else {
+                unsigned ah[KT][4], al[KT][4];
+#pragma unroll
+                for (int k = 0; k < KT; ++k) {
+                    const uint4 hv = *reinterpret_cast<const uint4*>(w1 + (warp * KT + k) * 256 + lane * 4);
+                    const uint4 lv = *reinterpret_cast<const uint4*>(w1 + (warp * KT + k) * 256 + 128 + lane * 4);
+                    ah[k][0] = hv.x, ah[k][1] = hv.y, ah[k][2] = hv.z, ah[k][3] = hv.w;
+                    al[k][0] = lv.x, al[k][1] = lv.y, al[k][2] = lv.z, al[k][3] = lv.w;
+                }
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                    float acc[4] = {b0, b0, b1, b1};
+#pragma unroll
+                    for (int k = 0; k < KT; ++k) {
+                        const float* b = sa + (k * 16 + t) * kPS + n * 8 + g;
+                        unsigned bh0, bl0, bh1, bl1;
+                        split2(b[0], b[4 * kPS], bh0, bl0);
+                        split2(b[8 * kPS], b[12 * kPS], bh1, bl1);
+                        mma3(acc, ah[k], al[k], bh0, bh1, bl0, bl1);
+                    }
+                    hidden(n, acc);
+                }
             }
         }
         __syncthreads();
@@ -1353,16 +1396,23 @@ cudaError_t project_launch(const FnoFusedDims& d, ProjArgs& p, int* blocks, cuda
     p.sc = 2.0f / (float)(4 * d.N);
     const long long tiles = (d.N + kPts - 1) / kPts;
     cudaError_t e = cudaSuccess;
-    auto go = [&](auto cp, auto nwc) {
+    auto launch = [&](auto cp, auto nwc, auto full) {
         constexpr int CP = decltype(cp)::value, NW = decltype(nwc)::value;
-        constexpr int sm = proj_smem<CP, NW, TRAIN>();
-        auto k = k_fno_project<CP, NW, TRAIN>;
+        constexpr bool FULL = decltype(full)::value;
+        constexpr int sm = proj_smem<CP, NW, TRAIN, FULL>();
+        auto k = k_fno_project<CP, NW, TRAIN, FULL>;
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
         if (e != cudaSuccess) return;
         const int per = 2;  // 93 KB a block at C = 32, H = 128
         const long long grid = tiles < per * kSMs ? tiles : per * kSMs;
         if (blocks) *blocks = (int)grid;
         k<<<(int)grid, 32 * NW, sm, s>>>(p);
+    };
+    auto go = [&](auto cp, auto nwc) {
+        if (proj_full(d.H))
+            launch(cp, nwc, std::true_type{});
+        else
+            launch(cp, nwc, std::false_type{});
     };
     using I16 = std::integral_constant<int, 16>;
     using I32 = std::integral_constant<int, 32>;

@@ -135,6 +135,38 @@ def test_fused_layers_vs_oracle(pfg, shape, dims):
         net.close()
 
 
+@pytest.mark.parametrize("C,H", [(32, 40), (16, 48), (32, 65), (18, 80), (32, 100), (8, 112)])
+def test_hidden_product_in_fp32(pfg, C, H):
+    """Hidden widths whose row tiles are no power of two form Q1 a in FP32 (BF16 mode).  Pre-activations are small
+    differences of a large product and a large bias, of factors close to 1 + 2^-8, which BF16 rounds most: the product of
+    the two remainders, 2^-16 of every term, is what the split form leaves out.  FP32 sums lose at most (C + 2) 2^-24 of
+    the terms' sum."""
+    import torch
+    shape = (8, 10, 36)
+    d = ofno.Dims(shape, C=C, m=2, H=H, L=1)
+    rng = np.random.default_rng(H)
+    theta = ofno.init_params(d, 11)
+    P = ofno.unpack(d, theta)
+    P["W0"][...] = 0.0
+    P["P"][...] = np.eye(4)[np.arange(C) % 4]  # a_1 = the inputs copied into the channels, exact also in BF16 parts
+    P["V0"][...] = np.eye(C)
+    P["Q1"][...] = 64.0 * (1 + 2.0 ** -8 - rng.integers(1, 64, (H, C)) * 2.0 ** -22)
+    P["q1"][...] = -P["Q1"].sum(1) * (1 + 2.0 ** -8 - 4 * 2.0 ** -14)
+    P["Q2"][...] = rng.uniform(0.5, 1.0, (4, H)) / H
+    theta = theta.astype(np.float32).astype(np.float64)
+    x = 1 + 2.0 ** -8 - rng.integers(1, 8, (4,) + shape) * 2.0 ** -14
+    out_ref = ofno.forward(d, theta, x)
+    net = pfg.FNO(shape, C=C, modes=2, H=H, L=1, bf16=True)
+    try:
+        net.set_params(theta.astype(np.float32))
+        out = net.forward(torch.from_numpy(x.astype(np.float32)).cuda()).cpu().numpy().astype(np.float64)
+    finally:
+        net.close()
+    # GELU' is at most 1.13, the weights of Q2 sum to less than 1, and the output product is the split one
+    bound = 1.13 * (C + 2) * 2.0 ** -24 * 64.3 * C + 2.0 ** -16
+    assert np.abs(out - out_ref).max() <= bound, (np.abs(out - out_ref).max(), bound)
+
+
 def test_adam_training_reduces_loss(pfg):
     import torch
     d = odims()
