@@ -287,7 +287,10 @@ int fail(pf_ctx* c, int code, const char* fmt, ...) {
 #define PF_CUDA(ctx, call)                                                                        \
     do {                                                                                          \
         cudaError_t e_ = (call);                                                                  \
-        if (e_ != cudaSuccess) return fail(ctx, PF_ECUDA, "%s: %s", #call, cudaGetErrorString(e_)); \
+        if (e_ != cudaSuccess) {                                                                  \
+            cudaGetLastError(); /* reported here, not by the next call's check */                 \
+            return fail(ctx, PF_ECUDA, "%s: %s", #call, cudaGetErrorString(e_));                  \
+        }                                                                                         \
     } while (0)
 
 cudaEvent_t prof_event(pf_ctx* c) {
