@@ -1091,11 +1091,9 @@ __global__ void __launch_bounds__(32 * NW, 2) k_fno_project(ProjArgs p) {
                 float hv[4];
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    const float z = acc[r];
-                    float e;
-                    const float cdf = gauss_cdf(z, e);
-                    hv[r] = z * cdf;
-                    if (TRAIN) gp[n][r] = fmaf(z * 0.39894228f, e, cdf);
+                    const GaussTail gt = gauss_tail(acc[r]);
+                    hv[r] = gelu_of(acc[r], gt);
+                    if (TRAIN) gp[n][r] = gelu_deriv_of(acc[r], gt);
                 }
                 float* o = sh + (h0 + g) * kPS + n * 8 + 2 * t;
                 *reinterpret_cast<float2*>(o) = make_float2(hv[0], hv[1]);
