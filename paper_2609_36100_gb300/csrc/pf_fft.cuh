@@ -241,18 +241,36 @@ struct Bfly<9, SIGN, T2> {
 // Twiddled butterfly of a power-of-two radix with the twiddles merged into its
 // radix-2 levels (decimation in time): X_k = E_k + c_k O_k, X_{k+R/2} = E_k -
 // c_k O_k with c_k = w w_R^k, E and O the halves over the even and the odd
-// inputs with w^2 in the place of w.  a + c b is four FMAs and a - c b = 2 a -
-// (a + c b) two more, so a radix-16 butterfly with its 15 twiddles is 192
-// instructions (238 with products first: 4 a twiddle, 160 for the butterfly
-// and its constants), a radix-8 one 72 (84), a radix-4 one 24 (28).  c_{k+R/4}
-// is c_k turned by a quarter, so R/2 twiddles are read, all of them rounded
-// table entries: w^(R/2), ..., w^2, w and their eighth and sixteenth turns.
+// inputs with w^2 in the place of w.  c_{k+R/4} is c_k turned by a quarter, so
+// R/2 twiddles are read, all of them rounded table entries: w^(R/2), ..., w^2, w
+// and their eighth and sixteenth turns.
+//
+// FP64: a + c b is four FMAs and a - c b = 2 a - (a + c b) two more, so a radix-8
+// butterfly with its twiddles is 72 instructions (84 with products first: 4 a
+// twiddle), a radix-4 one 24 (28): FP64 passes run at that pipe's rate.  The
+// difference inherits the sum's rounding.  Against 80-bit arithmetic an ARK4
+// step errs by 3.4e-16 at 64^3 and 3.7e-16 at 96^3 (4.3e-16 and 4.0e-16 with
+// products first and the physics of that form), a transform there and back by
+// 4.7e-16 on average over 19 lengths from 30 to 256 (4.8e-16; 4.7 / 4.1 at 96,
+// 5.1 / 4.4 at 192, 4.2 / 4.7 at 60, 4.5 / 5.1 at 150).
+//
+// FP32: a - c b is four FMAs of its own.  With the difference of the sum the
+// rounding of the stages' right-hand sides, which the error estimate is made
+// of, showed in it: at 256^3 and a step of 0.25 the estimate was 3.1e-3 too
+// large, where it had been 2.7e-3 with products first; now 2.6e-3 (at 32^3 1.28e-2,
+// 0.93e-2, 0.92e-2; at 96^3 6.6e-3, 5.1e-3, 5.1e-3).  It costs 1 % of a step at 256^3
+// and 480^3 and 3 % at 128^3.  A radix-8 butterfly multiplies first, with the
+// powers but w, w^2, w^4 formed by products (100 instructions, 3 loads): as exact
+// and 1 % of a step at 96^3 cheaper than merged.
 // ---------------------------------------------------------------------------
 template <typename T2>
 __device__ __forceinline__ void bf2_tw(T2& a, T2& b, T2 c) {
     using T = decltype(a.x);
     const T sx = fma(c.x, b.x, fma(-c.y, b.y, a.x)), sy = fma(c.x, b.y, fma(c.y, b.x, a.y));
-    b = T2{fma((T)2, a.x, -sx), fma((T)2, a.y, -sy)};
+    if constexpr (sizeof(T) == 4)
+        b = T2{fma(-c.x, b.x, fma(c.y, b.y, a.x)), fma(-c.x, b.y, fma(-c.y, b.x, a.y))};
+    else
+        b = T2{fma((T)2, a.x, -sx), fma((T)2, a.y, -sy)};
     a = T2{sx, sy};
 }
 // X[0..3] (natural order) of the inputs x[0], x[S], x[2S], x[3S] in place of
@@ -295,6 +313,18 @@ __device__ __forceinline__ void tw_bfly(T2* v, const T2* __restrict__ tw, int st
         bf2_tw(v[0], v[1], ld(st));
     } else if constexpr (R == 4) {
         bf4_tw<SIGN>(v[0], v[1], v[2], v[3], ld(st), ld(2 * st));
+    } else if constexpr (R == 8 && sizeof(T2) == 8) {
+        auto mul = [](T2& x, T2 w) { x = cmul(x, w); };
+        const T2 w1 = ld(st), w2 = ld(2 * st), w4 = ld(4 * st);
+        mul(v[1], w1);
+        mul(v[2], w2);
+        const T2 w3 = cmul(w2, w1);
+        mul(v[3], w3);
+        mul(v[4], w4);
+        mul(v[5], cmul(w4, w1));
+        mul(v[6], cmul(w4, w2));
+        mul(v[7], cmul(w4, w3));
+        Bfly<R, SIGN, T2>::run(v);
     } else if constexpr (R == 8) {
         bf8_tw<SIGN>(v, ld(st), ld(st + n / 8), ld(2 * st), ld(4 * st));
     } else if constexpr (R == 16) {
@@ -325,8 +355,7 @@ __device__ __forceinline__ void tw_bfly(T2* v, const T2* __restrict__ tw, int st
 }
 
 // butterfly of a generic (run-time plan) stage: FP64 stages, bound by the FP64
-// pipe, merge the twiddles; FP32 ones, bound by address arithmetic, gained
-// nothing from it (a second form of every radix: 480^3 1 % slower) and multiply
+// pipe, merge the twiddles; FP32 ones are bound by address arithmetic and multiply
 template <int R, int SIGN, typename T2>
 __device__ __forceinline__ void generic_bfly(T2* v, const T2* __restrict__ tw, int st, int n, bool turn) {
     if (sizeof(T2) == 16 && turn) {

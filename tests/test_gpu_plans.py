@@ -87,3 +87,20 @@ def test_fp64_default_plans_match_oracle(pfg, params, n):
         err, e = step_case(pfg, params, tuple(shape), "fp64", 20 + n)
         assert np.all(err <= 1e-11), (axis, err)
         assert e <= 1e-8
+
+
+@pytest.mark.parametrize("n,limit", [(96, 5.0e-4), (128, 3.27e-4)])
+def test_noise_of_the_fp32_error_estimate(pfg, params, n, limit):
+    """What FP32 rounding of the right-hand sides adds to the error estimate, per unit of the step: sqrt(e32^2 - e64^2)
+    / dt for steps so short that the true estimate is smaller.  The limits are 4 to 5 % above what transforms that
+    multiply by the twiddles first (one rounded table entry an input, plain butterflies) give: 4.75e-4 and 3.15e-4."""
+    v = []
+    for seed in (1, 2, 3):
+        y = synth.ic_spheres(n, 4, 3.0, 5.0, seed, params)
+        e = []
+        for prec in ("fp64", "fp32bulk"):
+            with pfg.Simulation((n, n, n), params, "ark4", prec) as s:
+                s.set_state(y)
+                e.append([s.step(dt) for dt in (0.02, 0.05)])
+        v += [np.sqrt(b * b - a * a) / dt for a, b, dt in zip(e[0], e[1], (0.02, 0.05))]
+    assert np.mean(v) <= limit, v
