@@ -77,6 +77,38 @@ def test_forward_and_gradients_vs_oracle(pfg, bf16, tol_out, tol_g):
         net.close()
 
 
+@pytest.mark.parametrize("C", [5, 6])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_mix_of_odd_and_even_channels(pfg, C, bf16):
+    """Spectral weights that start on a pair of floats (even C) and between two (odd C), in the kernels of one operation
+    each: FP32 sums throughout, spectral weights that BF16 holds exactly."""
+    import torch
+    shape = (8, 8, 12)
+    d = ofno.Dims(shape, C=C, m=3, H=16, L=2)
+    theta = ofno.init_params(d, 3).astype(np.float32)
+    P = ofno.unpack(d, theta)
+    for l in range(d.L):
+        w = torch.from_numpy(P["W%d" % l] * np.float32(20.0))
+        P["W%d" % l][...] = w.bfloat16().float().numpy()
+    rng = np.random.default_rng(2)
+    x, tgt = rng.standard_normal((4,) + shape), rng.standard_normal((4,) + shape) * 0.1
+    x, tgt = x.astype(np.float32).astype(np.float64), tgt.astype(np.float32).astype(np.float64)
+    out_ref, acts = ofno.forward(d, theta.astype(np.float64), x, cache=True)
+    g_ref = ofno.backward(d, theta.astype(np.float64), acts, out_ref, tgt)
+    net = pfg.FNO(shape, C=C, modes=3, H=16, L=2, bf16=bf16)
+    try:
+        net.set_params(theta)
+        out = net.forward(torch.from_numpy(x.astype(np.float32)).cuda()).cpu().numpy()
+        tol = 7 * 2.0 ** -16 if bf16 else 1e-5  # 2 L + 3 split products, or FP32 sums
+        assert np.linalg.norm(out - out_ref) <= tol * np.linalg.norm(out_ref)
+        net.backward(torch.from_numpy(tgt.astype(np.float32)).cuda())
+        errs = per_tensor(d, net.grads().astype(np.float64), g_ref)
+        bad = {k: v for k, v in errs.items() if k[0] == "W" and v > 10 * tol}
+        assert not bad, bad
+    finally:
+        net.close()
+
+
 # the fused layers' edges: the shortest and longest rows, odd rows and sides, padded channels, modes and hidden widths,
 # one mode, one layer, modes up to the Nyquist plane of an axis
 @pytest.mark.parametrize("shape,dims", [
