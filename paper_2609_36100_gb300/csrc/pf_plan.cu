@@ -108,11 +108,13 @@ void best_order(int n, int limit, bool by_cost, std::vector<int>& cur, int cost,
 }  // namespace
 
 // default schedule.  FP32 (prefer16): the fewest stages, since a stage is a
-// trip through shared memory and a barrier, of those the fewest instructions;
-// short lines at most radix 8, so that a tile still gives work to a few warps
-// (at 30 points radix 15 left one half-warp of it busy).  FP64 passes take the
-// time of their FP64 instructions: the fewest of those, with radices of at most
-// 12 (wider ones spill).
+// trip through shared memory and a barrier, of those the fewest instructions.
+// FP64 passes take the time of their FP64 instructions: the fewest of those,
+// with radices of at most 12 (wider ones spill).  Lines of up to 48 points in
+// both precisions at most radix 8, so that a tile still gives work to a few
+// warps (FP32, 30 points: radix 15 left one half-warp of it busy; FP64 step of
+// a cube, ms: 30 = 10 3 1.20 and 6 5 0.96, 36 = 12 3 1.61 and 6 6 1.28, 40 = 10 4
+// 1.66 and 5 4 2 1.31, 48 = 12 4 1.66 and 6 4 2 1.40).
 bool make_axis_plan(int n, AxisPlan& p, bool prefer16) {
     int m = n;
     for (int q : {2, 3, 5})
@@ -120,10 +122,7 @@ bool make_axis_plan(int n, AxisPlan& p, bool prefer16) {
     if (n < 2 || m != 1) return false;
     std::vector<int> cur, best;
     int cost = 0;
-    if (prefer16)
-        best_order(n, n <= 48 ? 8 : 16, false, cur, 0, best, cost);
-    else
-        best_order(n, 12, true, cur, 0, best, cost);
+    best_order(n, n <= 48 ? 8 : (prefer16 ? 16 : 12), !prefer16, cur, 0, best, cost);
     return make_axis_plan_radices(n, best.data(), (int)best.size(), p);
 }
 

@@ -78,7 +78,17 @@ def test_radix_that_is_none_refused(pfg, params):
                 s.set_tuning(c)
 
 
-@pytest.mark.parametrize("n", [30, 50, 96, 100, 108, 120, 150, 180, 240])
+@pytest.mark.parametrize("n", [24, 30, 32, 36, 40, 48])
+@pytest.mark.parametrize("prec", ["fp64", "fp32bulk"])
+def test_short_lines_have_no_wide_radices(pfg, params, n, prec):
+    with pfg.Simulation((n, n, n), params, "euler", prec) as s:
+        c = s.tuning()
+    for axis in range(3):
+        count, order = c[4 + 11 * axis], c[5 + 11 * axis:5 + 11 * axis + c[4 + 11 * axis]]
+        assert count > 0 and np.prod(order) == n and max(order) <= 8, order
+
+
+@pytest.mark.parametrize("n", [24, 30, 32, 36, 40, 48, 50, 96, 100, 108, 120, 150, 180, 240])
 def test_fp64_default_plans_match_oracle(pfg, params, n):
     """FP64 plans of the fewest instructions, along every axis."""
     for axis in range(3):
