@@ -28,7 +28,7 @@ def relerr(a, b):
     return np.array([np.linalg.norm((a[f] - b[f]).ravel()) / np.linalg.norm(b[f].ravel()) for f in range(4)])
 
 
-def step_case(pfg, p, shape, prec, seed, cfg=None):
+def step_case(pfg, p, shape, prec, seed, cfg=None, widths=0):
     y = synth.random_state(shape, seed, phi_scale=0.9)
     m = oracle.Model(shape, p)
     ref, e_ref, _ = oracle.ark_step(m, m.to_k(y), 0.5, oracle.ark436l2sa(), p["rtol"], p["atol"])
@@ -41,6 +41,7 @@ def step_case(pfg, p, shape, prec, seed, cfg=None):
             assert s.tuning() == c
         else:
             c = s.tuning()
+            c[1] = c[37] = widths  # y pass, z passes (0: untuned)
             s.set_tuning(c)  # what a context reports it takes back
         s.set_state(y)
         e = s.step(0.5)
@@ -55,6 +56,41 @@ def test_default_plans_match_oracle(pfg, params, n, axis):
     err, e = step_case(pfg, params, tuple(shape), "fp32bulk", 10 + n)
     assert np.all(err <= 1e-5), err
     assert e <= 1e-3
+
+
+@pytest.mark.parametrize("n", [n for n in LENGTHS if 48 < n <= 384])
+@pytest.mark.parametrize("axis", [1, 2])
+def test_wide_tiles_match_oracle(pfg, params, n, axis):
+    """The column passes at 16 columns a tile, the width the plans of these lengths are compiled for and grids of real
+    size run: the small grids of test_default_plans_match_oracle have too few columns for it and run the generic stages.
+    24 or 40 columns a field, so the last tile is half empty."""
+    assert 2 * 16 * n * 8 <= 128 * 1024  # what the library caps a tuned width by
+    shape = (n, 10, 6) if axis == 2 else (6, n, 6)
+    err, e = step_case(pfg, params, shape, "fp32bulk", 30 + n, widths=16)
+    assert np.all(err <= 1e-5), err
+    assert e <= 1e-3
+
+
+@pytest.mark.parametrize("shape", [(108, 48, 80), (48, 150, 80), (36, 40, 180)])
+def test_untuned_wide_tiles_match_oracle(pfg, params, shape):
+    """Enough columns (4 fields of 1620 and more) for an untuned tile of 16."""
+    err, e = step_case(pfg, params, shape, "fp32bulk", 7)
+    assert np.all(err <= 1e-5), err
+    assert e <= 1e-3
+
+
+LONG = [540, 576, 600, 640, 648, 720, 750, 768, 800, 810, 864, 900, 960, 972, 1000, 1024]
+
+
+@pytest.mark.parametrize("n", LONG)
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("prec,tol,etol", [("fp64", 1e-11, 1e-8), ("fp32bulk", 1e-5, 1e-3)])
+def test_long_default_plans_match_oracle(pfg, params, n, axis, prec, tol, etol):
+    shape = [6, 10, 6]
+    shape[2 - axis] = n
+    err, e = step_case(pfg, params, tuple(shape), prec, 50 + n)
+    assert np.all(err <= tol), err
+    assert e <= etol
 
 
 @pytest.mark.parametrize("prec,tol,etol", [("fp64", 1e-11, 1e-8), ("fp32bulk", 1e-5, 1e-3)])
