@@ -105,14 +105,14 @@ def gelu_grad(z):
 def fwd_dft(d, a):
     """a[c, z, y, x] real -> A[c, kz, ky, kx] over the retained modes."""
     Mx, My, Mz, _ = dft_matrices(d)
-    return np.einsum("az,by,cx,nzyx->nabc", Mz, My, Mx, a)
+    return np.einsum("az,by,cx,nzyx->nabc", Mz, My, Mx, a, optimize=True)  # an axis at a time
 
 
 def inv_re(d, O, weighted=True, scale=True):
     """Re( sum_k c_k O(k) e^{ik.r} ), c_k = w_kx / N (weighted, scaled)."""
     Mx, My, Mz, w = dft_matrices(d)
     Ow = O * (w[None, None, None, :] if weighted else 1.0)
-    r = np.einsum("az,by,cx,nabc->nzyx", np.conj(Mz), np.conj(My), np.conj(Mx), Ow).real
+    r = np.einsum("az,by,cx,nabc->nzyx", np.conj(Mz), np.conj(My), np.conj(Mx), Ow, optimize=True).real
     return r / d.N if scale else r
 
 

@@ -119,6 +119,11 @@ def test_mix_of_odd_and_even_channels(pfg, C, bf16):
     ((26, 27, 63), dict(C=2, modes=13, H=64, L=1)),
     ((8, 9, 150), dict(C=30, modes=4, H=65, L=2)),
     ((7, 9, 40), dict(C=5, modes=3, H=20, L=2)),  # odd channel counts run the unfused kernels
+    # more rows than one sweep of the row kernels' teams (152 blocks of ten forward, eight backward; four or five of long
+    # rows), more tiles than the projection has blocks (304), more rows than the lift's warps (4864)
+    ((40, 42, 36), dict(C=32, modes=4, H=128, L=2)),
+    ((28, 30, 256), dict(C=32, modes=13, H=64, L=2)),
+    ((72, 70, 32), dict(C=8, modes=2, H=100, L=2)),
 ])
 def test_fused_layers_vs_oracle(pfg, shape, dims):
     """Spectral weights that BF16 holds exactly, so that only the products' split (about 2^-16 relative for each of the
