@@ -125,7 +125,8 @@ typedef struct {
 } pf_stats;
 
 /* Create a context on `cuda_stream` (a cudaStream_t, NULL = legacy default
- * stream).  Validates sizes and parameters, allocates all device buffers,
+ * stream).  Validates sizes and parameters, allocates all device buffers (a
+ * table of the elastic kernel, at most 1 GB, only where there is room for it),
  * builds FFT plans and twiddle tables (FP64, computed on the host).
  * Returns PF_EUNSUPPORTED for non-smooth/odd sizes. */
 int pf_create(const pf_grid* grid, const pf_params* params, void* cuda_stream, pf_ctx** out);
@@ -158,7 +159,11 @@ int pf_rhs_explicit(pf_ctx* ctx, const void* y_hat, void* fE_hat);
  * Device complex128 vectors in ABI layout; r and z may alias. FP64. */
 int pf_solve_implicit(pf_ctx* ctx, double gamma, const void* r_hat, void* z_hat);
 
-/* One fixed step of size dt from the current state (always accepted).  If the
+/* Steps of grids of up to 160^3 points run as a CUDA graph from a context's
+ * seventeenth on (counted anew after pf_set_tuning; not with el_inhom or under
+ * the profiler); the driver keeps the graphs' own memory.
+ *
+ * One fixed step of size dt from the current state (always accepted).  If the
  * method has an embedding and `lte_wrms_out` is non-NULL, the WRMS norm of
  * the local error estimate (real space, all four fields, weights from the
  * previous solution) is written there; else 0. */

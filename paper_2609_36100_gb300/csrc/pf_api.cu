@@ -195,6 +195,7 @@ struct pf_ctx {
     Tableau tab;
     bool fp32 = false;
     Geo g{};
+    int tune41 = 0, tune42 = 0;  // schedule slots that choose nothing any more, kept for saved schedules
     Geo g64{};  // g with the FP64 schedules: of the FP64 transforms of a FP32-bulk context
     const Geo& geo64() const { return fp32 ? g64 : g; }
     Phys ph{};
@@ -1799,8 +1800,8 @@ int pf_get_tuning(pf_ctx* c, int* cfg, int n) {
     cfg[38] = c->g.el_pid;
     cfg[39] = c->g.xf_off;
     cfg[40] = c->g.el_unfused;
-    cfg[41] = c->g.xf_stg;
-    cfg[42] = c->g.xf_inpl;
+    cfg[41] = c->tune41;
+    cfg[42] = c->tune42;
     plan_to_cfg(c->g.px, cfg + 4);
     plan_to_cfg(c->g.py, cfg + 4 + 11);
     plan_to_cfg(c->g.pz, cfg + 4 + 22);
@@ -1822,8 +1823,6 @@ int pf_set_tuning(pf_ctx* c, const int* cfg, int n) {
     g.xf_off = cfg[39] != 0;
     if (cfg[40] < 0 || cfg[40] > 2) return fail(c, PF_EINVAL, "pf_set_tuning: bad elastic form %d", cfg[40]);
     g.el_unfused = cfg[40];
-    g.xf_stg = cfg[41] != 0;
-    g.xf_inpl = cfg[42] != 0;
     AxisPlan* pl[3] = {&g.px, &g.py, &g.pz};
     const int ns[3] = {g.nx, g.ny, g.nz};
     for (int a = 0; a < 3; ++a) {
@@ -1836,14 +1835,18 @@ int pf_set_tuning(pf_ctx* c, const int* cfg, int n) {
         *pl[a] = p;
     }
     c->g = g;
+    c->tune41 = cfg[41] != 0;
+    c->tune42 = cfg[42] != 0;
     drop_graphs(c);  // their launches are of the old schedule
     return PF_OK;
 }
 
 namespace {
 
-// distinct orders of the radix multisets that factor n with the fewest (and
-// one more) stages, at most `cap` of them
+// distinct orders of the radix multisets of 2, 3, 4, 5, 8 and 16 that factor n
+// with the fewest (and one more) stages of the powers of two, at most `cap` of
+// them; the order a context has (wider radices among them) stays unless one of
+// these is faster
 std::vector<std::vector<int>> radix_orders(int n, size_t cap) {
     int m = n, a = 0, b = 0, cc = 0;
     while (m % 2 == 0) { m /= 2; ++a; }

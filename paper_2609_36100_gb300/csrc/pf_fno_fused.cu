@@ -470,7 +470,6 @@ constexpr int kTeam = 2;  // warps of a row
 // issuing, of the products along x, GELU and the split into BF16 parts.  A row
 // of all channels fills 20 KB, so ten rows an SM: with one warp a row that left
 // two and a half warps a scheduler (402 us, with erff); two warps share a row.
-
 template <int CP, int MP, int FI>
 __global__ void __launch_bounds__(640, 1) k_fno_row(RowArgs a) {
     extern __shared__ __align__(16) float sm[];
@@ -527,13 +526,12 @@ __global__ void __launch_bounds__(640, 1) k_fno_row(RowArgs a) {
 // Partial sums of a block of k_fno_row_bwd: [C C] V, [C] v, [4 C] P, [C] p
 __host__ __device__ inline int row_part_len(int C) { return C * C + 6 * C; }
 
-template <int CP, int MP, int FI>
-
 // A layer backward: the gradient of its pre-activation in place of the next
 // one's, the weights' partial sums over the block's rows.  It moves 3 [C][N]
 // arrays (118 us at 128^3, C = 32) in 438 us, half the cycles issuing: two row
 // tiles a team leave eight teams an SM, and 128 registers a thread.  810 us with
 // a warp a row, 590 with the fold of long rows kept in registers for short ones.
+template <int CP, int MP, int FI>
 __global__ void __launch_bounds__(512, 1) k_fno_row_bwd(RowArgs a) {
     extern __shared__ __align__(16) float sm[];
     const RowSmem L = row_smem(a.nx, CP, MP);
@@ -1451,10 +1449,14 @@ void dft_inv(const float2* in, float2* out, const float2* tab, int J, int m, int
 
 }  // namespace
 
-// The rule: one warp row of every channel has to fit a warp's share of shared
-// memory (C <= 32, rows of 32 to 256 points), a lane group's registers cover
-// the modes (m <= 16) and the projection's row tiles the hidden width (H <= 128).
-// Shorter rows leave most lanes of a warp idle; longer ones few warps an SM.
+// The rule: a row of every channel has to fit the shared memory of its two warps
+// (C <= 32, rows of 32 to 256 points), a lane group's registers cover the modes
+// (m <= 16) and the projection's row tiles the hidden width (H <= 128).  Shorter
+// rows leave most lanes of a warp idle; longer ones few rows an SM.
+// Nothing bounds the lengths along y and z: their tables fit a block's shared
+// memory up to 3227 points at 13 to 16 modes and 9683 at up to 4, and longer
+// ones fail at the launch, as in the unfused kernels, whose matrices stay within
+// 48 KB (2 m n <= 6144: 236 points at 13 modes).
 // With an odd C the spectral weights are not aligned to (re, im) pairs.
 bool fno_fused_ok(const FnoFusedDims& d) {
     return d.C <= 32 && d.C % 2 == 0 && d.H <= 128 && d.m <= kMaxModes && d.nx >= 32 && d.nx <= kMaxRow && d.nz <= 65535;

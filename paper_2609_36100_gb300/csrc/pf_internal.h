@@ -66,7 +66,6 @@ struct Geo {
     int el_pid;              // compiled plan of the fused elastic pass (length nz), 0 = the z-axis plan,
                              // -1 = no fused stage (the one-kernel pass with the z-axis column transforms)
     int xf_off;              // 1: the FP32 x passes use the staged kernel instead of the fused one
-    int xf_inpl, xf_stg;     // schedule slots kept for saved schedules; nothing reads them
     int el_unfused;          // form of the compiled-plan elastic pass: 0 fuses the last forward / first inverse
                              // stage, 1 runs every stage (and the contraction) over the three fields in place,
                              // 2 runs a cluster of three CTAs, one field each (FP32 contexts)
@@ -286,9 +285,8 @@ void launch_stage_pointwise(const Geo& g, const Phys& ph, const double2* y, cons
                             double2* zout, cudaStream_t s);
 void launch_solve(const Geo& g, const Phys& ph, double gamma, const double2* r, double2* z, cudaStream_t s);
 void launch_lambda_table(const Geo& g, const Phys& ph, double* lam, float2* lamdf, cudaStream_t s);
-// FP32 table of the elastic kernel B_vq(k)/N (diagonal eigenstrains: B is
-// even in each wave-number component, so |ky| and |kz| index it)
-// table of the elastic kernel in double (fp64) or float
+// table of the elastic kernel B_vq(k)/N in double (fp64) or float (diagonal
+// eigenstrains: B is even in each wave-number component, so |ky| and |kz| index it)
 void launch_btab(const Geo& g, const Phys& ph, void* btab, bool fp64, cudaStream_t s);
 void launch_clamp_phi(double* real, long long N, cudaStream_t s);
 // FP32-bulk stage assembly as a streaming pass (double-float z_i out, FP32

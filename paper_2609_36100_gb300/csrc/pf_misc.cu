@@ -321,8 +321,8 @@ __global__ void __launch_bounds__(32) k_batch_prep(BatchConst bc, MemberCtl* __r
     }
 }
 
-// accept / reject and the next step size (same PI rule as the host driver)
-// accept / reject's three powers on a lane each, side by side
+// accept / reject and the next step size (same PI rule as the host driver), its
+// three powers on a lane each, side by side
 __global__ void __launch_bounds__(32) k_batch_ctl(BatchConst bc, MemberCtl* __restrict__ ctl,
                                                   const double* __restrict__ wsum, double scale) {
     MemberCtl& m = *ctl;

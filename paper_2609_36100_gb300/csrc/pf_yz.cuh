@@ -540,7 +540,10 @@ static bool launch_z_elastic_unf(const Geo& g, const Phys& ph, void* H, int tune
 
 template <typename T, int PID = 1>
 static bool unfused_by_plan(const Geo& g, const Phys& ph, void* H, int pid, cudaStream_t s) {
-    // FP64 contexts never have the FP32 default plans
+    // FP64 contexts can have plans above kBothWidths (96 = 12 8, 100 = 10 10, 144 =
+    // 12 12 by default); no elastic pass is compiled for them in FP64, and forms 0
+    // and 1 both run k_z_elastic (all passes together, a FP64 ARK4 step of 96^3 takes
+    // 6.4 ms so; 10.1 with 8 4 3, its compiled elastic pass and products first)
     if constexpr (PID > (sizeof(T) == 4 ? kFixedPlans : kBothWidths)) {
         return false;
     } else {
