@@ -254,14 +254,16 @@ struct Bfly<9, SIGN, T2> {
 // 4.7e-16 on average over 19 lengths from 30 to 256 (4.8e-16; 4.7 / 4.1 at 96,
 // 5.1 / 4.4 at 192, 4.2 / 4.7 at 60, 4.5 / 5.1 at 150).
 //
-// FP32: a - c b is four FMAs of its own.  With the difference of the sum the
-// rounding of the stages' right-hand sides, which the error estimate is made
-// of, showed in it: at 256^3 and a step of 0.25 the estimate was 3.1e-3 too
-// large, where it had been 2.7e-3 with products first; now 2.6e-3 (at 32^3 1.28e-2,
-// 0.93e-2, 0.92e-2; at 96^3 6.6e-3, 5.1e-3, 5.1e-3).  It costs 1 % of a step at 256^3
-// and 480^3 and 3 % at 128^3.  A radix-8 butterfly multiplies first, with the
-// powers but w, w^2, w^4 formed by products (100 instructions, 3 loads): as exact
-// and 1 % of a step at 96^3 cheaper than merged.
+// FP32: a - c b is four FMAs of its own in radices 2 and 16 (16: 256 instructions;
+// 238 with products first, but 15 loads for 8).  Radices 4 and 8 multiply first,
+// radix 8 with the powers but w, w^2, w^4 formed by products (100 instructions, 3
+// loads).  With the difference taken from the sum in all of them, the rounding
+// of the stages' right-hand sides, which the error estimate is made of, grew by
+// 8 to 13 %: at 256^3 and a step of 0.25 the estimate was 3.1e-3 too large where
+// it had been 2.7e-3 with products first; now 2.6e-3 (at 128^3 5.0e-3, 4.3e-3, 4.3e-3;
+// at 96^3 6.6e-3, 5.1e-3, 5.2e-3; at 64^3 1.12e-2, 1.09e-2, 1.00e-2).  It costs 1.3 % of a
+// step at 256^3, 1.1 % at 128^3, 0.6 % at 480^3.  Radices 2 to 8 merged with a
+// difference of their own: 128^3 1.7 % slower, 256^3 0.3 % faster.
 // ---------------------------------------------------------------------------
 template <typename T2>
 __device__ __forceinline__ void bf2_tw(T2& a, T2& b, T2 c) {
@@ -311,9 +313,11 @@ __device__ __forceinline__ void tw_bfly(T2* v, const T2* __restrict__ tw, int st
     };
     if constexpr (R == 2) {
         bf2_tw(v[0], v[1], ld(st));
-    } else if constexpr (R == 4) {
+    } else if constexpr (R == 4 && sizeof(T2) == 16) {
         bf4_tw<SIGN>(v[0], v[1], v[2], v[3], ld(st), ld(2 * st));
-    } else if constexpr (R == 8 && sizeof(T2) == 8) {
+    } else if constexpr (R == 8 && sizeof(T2) == 16) {
+        bf8_tw<SIGN>(v, ld(st), ld(st + n / 8), ld(2 * st), ld(4 * st));
+    } else if constexpr (R == 8) {
         auto mul = [](T2& x, T2 w) { x = cmul(x, w); };
         const T2 w1 = ld(st), w2 = ld(2 * st), w4 = ld(4 * st);
         mul(v[1], w1);
@@ -325,8 +329,6 @@ __device__ __forceinline__ void tw_bfly(T2* v, const T2* __restrict__ tw, int st
         mul(v[6], cmul(w4, w2));
         mul(v[7], cmul(w4, w3));
         Bfly<R, SIGN, T2>::run(v);
-    } else if constexpr (R == 8) {
-        bf8_tw<SIGN>(v, ld(st), ld(st + n / 8), ld(2 * st), ld(4 * st));
     } else if constexpr (R == 16) {
         T2 e[8] = {v[0], v[2], v[4], v[6], v[8], v[10], v[12], v[14]};
         T2 o[8] = {v[1], v[3], v[5], v[7], v[9], v[11], v[13], v[15]};
