@@ -6,10 +6,17 @@
 
 namespace pf {
 // FP64 passes with radices above 8 would take 130 registers a thread and leave
-// one CTA on an SM, nothing to transform while it loads: bounded to two
-template <typename T, bool R16>
+// one CTA on an SM, nothing to transform while it loads: bounded to two.  The
+// FP32 inverse z pass of 16 16 would take 74 and leave three: bounded to four
+// (91 us a launch at 256^3 where three took 97).
+template <typename T, bool R16, int PID = 0>
 constexpr int col_min_blocks() {
-    return sizeof(T) == 8 && R16 ? 2 : 0;  // 0: no bound (1 would let the FP32 passes take registers of occupancy)
+    if (sizeof(T) == 8 && R16) return 2;
+    if constexpr (PID > 0)
+        if (sizeof(T) == 4 && RadInfo<typename FixedPlan<PID>::Rad>::first == 16 &&
+            RadInfo<typename FixedPlan<PID>::Rad>::last == 16)
+            return 4;
+    return 0;  // no bound (1 would let the FP32 passes take registers of occupancy)
 }
 
 // ---------------------------------------------------------------------------
@@ -52,7 +59,7 @@ void launch_y_pass_sign(const Geo& g, void* buf, int nf, cudaStream_t s) {
 // stage, of the strain components of the Hu-Chen solve)
 // ---------------------------------------------------------------------------
 template <typename T, int SIGN, int TX, bool R16, int PID>
-__global__ void __launch_bounds__(kThreads, col_min_blocks<T, R16>()) k_z_pass(Geo g, typename Cx<T>::t* __restrict__ buf) {
+__global__ void __launch_bounds__(kThreads, col_min_blocks<T, R16, PID>()) k_z_pass(Geo g, typename Cx<T>::t* __restrict__ buf) {
     PF_SKIP_INACTIVE(g);
     using T2 = typename Cx<T>::t;
     extern __shared__ __align__(16) unsigned char smraw[];
