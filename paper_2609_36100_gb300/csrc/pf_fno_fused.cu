@@ -528,7 +528,7 @@ __host__ __device__ inline int row_part_len(int C) { return C * C + 6 * C; }
 
 // A layer backward: the gradient of its pre-activation in place of the next
 // one's, the weights' partial sums over the block's rows.  It moves 3 [C][N]
-// arrays (118 us at 128^3, C = 32) in 438 us, half the cycles issuing: two row
+// arrays (118 us at 128^3, C = 32) in 449 us, half the cycles issuing: two row
 // tiles a team leave eight teams an SM, and 128 registers a thread.  810 us with
 // a warp a row, 590 with the fold of long rows kept in registers for short ones.
 template <int CP, int MP, int FI>
@@ -975,15 +975,18 @@ constexpr int proj_smem() {
 // Hidden widths whose row tiles are no power of two (33 to 48, 65 to 112) have
 // the product Q1 a in FP32, the others in BF16 parts: so it is in the kernels
 // of one operation each (dense_mma has forms for 1, 2, 4 and 8 row tiles), and
-// which of the two paths a size runs says nothing about its precision.
+// which of the two paths a size runs says nothing about its precision.  A forward
+// pass at 64^3, C = 20, H = 100, 12 modes, four layers takes 441 us so, 423 with
+// BF16 parts; at 160x160x40, C = 16, H = 112 1122 and 1029.
 __host__ __device__ constexpr bool proj_full(int H) {
     const int tiles = (H + 15) / 16;
     return (tiles & (tiles - 1)) != 0;
 }
 
-// The products of a tile run on the tensor cores (1031 us forward and backward
-// at 128^3, C = 32, H = 128, 1708 with the output and its weight gradient as
-// scalar loops; 395 us forward at 160x96x120).  What bounds the kernel is
+// The products of a tile run on the tensor cores (1110 us forward and backward
+// at 128^3, C = 32, H = 128, 1031 with GELU's derivative from the tail alone, 1708
+// with the output and its weight gradient as scalar loops as well; 394 us forward
+// at 160x96x120).  What bounds the kernel is
 // the instructions around them, GELU of its H x 64 hidden values first, and the
 // shared memory those pass through.  The next tile's columns of a are copied in
 // while this one is worked on.

@@ -15,7 +15,8 @@
 // half-spectrum rows), the R2C unpacking into the store.  Every stage runs in
 // place in one shared-memory tile of skewed lines: two tiles, with a barrier
 // less a stage, hold half the CTAs on an SM and were slower from 96 points on
-// (right-hand-side pass at 256^3: 256 us against 200, h pass 182 against 154)
+// (right-hand-side pass at 256^3: 256 us against 200, h pass 182 against 154 then,
+// 201 and 161 with the stages as they are now)
 // and as fast at 64; so was copying the real fields into shared memory ahead
 // of the physics (213 against 200 us).
 #pragma once
