@@ -14,11 +14,10 @@
 // folded into the first inverse stage (read straight from the staged
 // half-spectrum rows), the R2C unpacking into the store.  Every stage runs in
 // place in one shared-memory tile of skewed lines: two tiles, with a barrier
-// less a stage, hold half the CTAs on an SM and were slower from 96 points on
-// (right-hand-side pass at 256^3: 256 us against 200, h pass 182 against 154 then,
-// 201 and 161 with the stages as they are now)
-// and as fast at 64; so was copying the real fields into shared memory ahead
-// of the physics (213 against 200 us).
+// less a stage, hold half the CTAs on an SM and were as fast at 64 points and
+// slower from 96 on (right-hand-side pass at 256^3: 256 us against 200, h pass 182
+// against 154 then, 201 and 161 with the stages as they are now); so was copying
+// the real fields into shared memory ahead of the physics (213 against 200 us).
 #pragma once
 #include "pf_xpass.cuh"
 
